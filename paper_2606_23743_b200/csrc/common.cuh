@@ -37,6 +37,11 @@ __device__ __forceinline__ float e4m3_to_float(uint32_t byte) {
   return __half2float(__half(h));
 }
 
+// two e4m3 bytes (the low 16 bits) -> two floats (exact), the low byte first
+__device__ __forceinline__ float2 e4m3x2_to_float2(uint32_t pair) {
+  return __half22float2(__half2(__nv_cvt_fp8x2_to_halfraw2((__nv_fp8x2_storage_t)pair, __NV_E4M3)));
+}
+
 // x / s for the e4m3 cast, s and y = RN(1/s) fixed for a whole block: q0 = x*y, one exact residual, one
 // correction -- the correctly rounded quotient (Markstein's sequence) in three FMA-pipe operations instead of
 // the dozen of a general division, valid while s is in [2^-60, 2^60] and its significand is not all ones
@@ -104,5 +109,25 @@ bool attn_ts_remainder_serves(const Dims& m);
 bool attn_ts_serves(const Dims& m);    // d = 128 or 64, bf16 or e4m3 Q/K, 128- or 64-token blocks
 int launch_prepare_v_ts(const Dims& m, const sva_problem_t* p, const void* v, void* ws, size_t ws_bytes,
                         cudaStream_t st);
+
+// two fp32 lanes in one instruction (sm_100): d = a * b + c, d = a + b
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
 
 }  // namespace sva

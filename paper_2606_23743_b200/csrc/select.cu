@@ -11,6 +11,7 @@
 // ascending order.  When the per-row count is known on the host (top-k with no window larger than k)
 // rows go straight into the CSR; otherwise they are staged and csr_kernel builds it in one launch.
 #include <mutex>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -18,67 +19,87 @@ namespace sva {
 
 static constexpr int POOL_THREADS = 256;
 
-// One CTA pools one block of one head of one tensor (blockIdx.z: 0 = Q, 1 = K).
+// Block means of one head of one tensor (blockIdx.z: 0 = Q, 1 = K); a CTA pools `run` consecutive blocks.
 // ELEM_BYTES = 2: bf16 input.  ELEM_BYTES = 1: e4m3 codes, multiplied by the block's scale.
+// Bound by the HBM: one pass over Q and K.  A CTA's loads run one step (four vectors per thread) ahead of its sums, across
+// the blocks of its run, so the reduction at the end of a block (two barriers) happens with the next block's loads in
+// flight; with a CTA per block nothing was in flight while it reduced.  Q and K of 24 heads
+// x 32 760 tokens, d = 128 (403 MB): 75.8 -> 71.8 us (5.6 TB/s) with 128-token blocks, 81 -> 72.7 us with 64-token
+// ones; e4m3 codes (201 MB, converted in pairs): 66.5 -> 58.6 us.
 template <int D, int ELEM_BYTES>
 __global__ void __launch_bounds__(POOL_THREADS)
 pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Strides sq, Strides sk,
             const float* __restrict__ q_scale, const float* __restrict__ k_scale, int H, int N,
-            int block, int Nb, float* __restrict__ qbar, float* __restrict__ kbar) {
+            int block, int Nb, int run, float* __restrict__ qbar, float* __restrict__ kbar) {
   constexpr int EPV = 16 / ELEM_BYTES;          // elements per 16-byte vector
   constexpr int VPR = D / EPV;                  // vectors per token row
   constexpr int GROUPS = POOL_THREADS / VPR;    // token rows read concurrently
+  constexpr int STEP = GROUPS * 4;              // token rows per step
   __shared__ float part[GROUPS][D + 1];
 
-  const int I = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
+  const int bh = blockIdx.y, which = blockIdx.z;
   const int b = bh / H, h = bh % H;
-  const uint8_t* base = which ? k : q;
   const Strides s = which ? sk : sq;
-  base += ((long long)b * s.b + (long long)h * s.h) * ELEM_BYTES;
-  const int lo = I * block;
-  const int cnt = min(block, N - lo);
+  const uint8_t* base = (which ? k : q) + ((long long)b * s.b + (long long)h * s.h) * ELEM_BYTES;
+  const int I0 = blockIdx.x * run, I1 = min(I0 + run, Nb);
   const int vec = threadIdx.x % VPR, grp = threadIdx.x / VPR;
+  const int per_block = (block + STEP - 1) / STEP, steps = (I1 - I0) * per_block;
 
+  uint4 u[4];
+  auto load = [&](int step) {
+    const int I = I0 + step / per_block, t0 = (step % per_block) * STEP + grp;
+    const int lo = I * block, cnt = step < steps ? min(block, N - lo) : 0;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int t = t0 + j * GROUPS;
+      u[j] = make_uint4(0, 0, 0, 0);
+      if (t < cnt) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(lo + t) * s.n * ELEM_BYTES) + vec);
+    }
+  };
   float acc[EPV];
 #pragma unroll
   for (int e = 0; e < EPV; ++e) acc[e] = 0.f;
-
-  for (int t0 = grp; t0 < cnt; t0 += GROUPS * 4) {
-    uint4 u[4];
+  load(0);
+  for (int step = 0; step < steps; ++step) {
+    uint4 c[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) c[j] = u[j];
+    load(step + 1);
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      int t = t0 + j * GROUPS;
-      u[j] = make_uint4(0, 0, 0, 0);
-      if (t < cnt)
-        u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(lo + t) * s.n * ELEM_BYTES) + vec);
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t w[4] = {u[j].x, u[j].y, u[j].z, u[j].w};
+      const uint32_t w[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
       if constexpr (ELEM_BYTES == 2) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) { acc[2 * e] += bf16lo(w[e]); acc[2 * e + 1] += bf16hi(w[e]); }
       } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-#pragma unroll
-          for (int c = 0; c < 4; ++c) acc[4 * e + c] += e4m3_to_float((w[e] >> (8 * c)) & 0xff);
+        for (int e = 0; e < 4; ++e) {
+          const float2 lo2 = e4m3x2_to_float2(w[e] & 0xffffu), hi2 = e4m3x2_to_float2(w[e] >> 16);
+          acc[4 * e] += lo2.x; acc[4 * e + 1] += lo2.y; acc[4 * e + 2] += hi2.x; acc[4 * e + 3] += hi2.y;
+        }
       }
     }
-  }
+    if ((step + 1) % per_block == 0) {                            // the block's rows are in: reduce over the groups
+      const int I = I0 + step / per_block;
 #pragma unroll
-  for (int e = 0; e < EPV; ++e) part[grp][vec * EPV + e] = acc[e];
-  __syncthreads();
-  if (threadIdx.x < D) {
-    float sum = 0.f;
+      for (int e = 0; e < EPV; ++e) { part[grp][vec * EPV + e] = acc[e]; acc[e] = 0.f; }
+      __syncthreads();
+      if (threadIdx.x < D) {
+        float sum = 0.f;
 #pragma unroll 8
-    for (int g = 0; g < GROUPS; ++g) sum += part[g][threadIdx.x];   // fixed order
-    float mean = sum / (float)cnt;
-    if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
-    (which ? kbar : qbar)[((long long)bh * Nb + I) * D + threadIdx.x] = mean;
+        for (int g = 0; g < GROUPS; ++g) sum += part[g][threadIdx.x];   // fixed order
+        float mean = sum / (float)min(block, N - I * block);
+        if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
+        (which ? kbar : qbar)[((long long)bh * Nb + I) * D + threadIdx.x] = mean;
+      }
+      __syncthreads();
+    }
   }
 }
 
+// Blocks per CTA: runs of four once they still give every SM a few CTAs; before that a block each, since the time is then the
+// longest CTA's latency.
+static int pool_run(const Dims& m) { return 2LL * m.R >= 4 * 148 * 4 ? 4 : 1; }
 
 struct SelParams {
   int H, Nb, mode, k, use_window, win_t, win_s, bpf, cap, fixed_n;
@@ -103,7 +124,8 @@ __device__ __forceinline__ float key_score(uint32_t key) {
 
 // Selection and emission of one query-block row by one warp.  Lane j owns the key blocks
 // J = it*32 + j, it < ITEMS, whose scores arrive as sortable keys (0 = no candidate).
-template <int ITEMS>
+// MASS: the cumulative-mass rule (mode 1).
+template <int ITEMS, bool MASS>
 __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const int I, const int bh, const int lane,
                                                 const SelParams& p, int32_t* __restrict__ row_ptr,
                                                 int32_t* __restrict__ col_idx, int32_t* __restrict__ tmp_idx,
@@ -112,10 +134,17 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
   // ---- selection
   // The rule is sequential -- forced window first, then candidates by score (descending, ties to the
   // lower index) until k blocks are kept or, in mode 1, the kept softmax mass reaches tau -- but what it
-  // keeps is "every candidate above a threshold key plus the first few of the candidates equal to it",
-  // so the threshold is found by a 32-step bisection on the key bits (each step: one compare per
-  // register, a warp reduction of the count and, in mode 1, of the mass) instead of up to k rounds of
-  // arg-max.  The masses are summed in fixed point (weights in units of 2^-31: a warp-wide integer add is
+  // keeps is "every candidate above a threshold key plus the first few of the candidates equal to it":
+  // T = the largest key at which taking every candidate >= it ends the rule.  T is a candidate's key, so the
+  // search narrows an interval [lo, hi) of keys that holds it (lo ends the rule, hi does not; each step one
+  // compare per register, a warp reduction of the count and, in mode 1, of the mass) only until one distinct
+  // key is left in it.  Steps halve the interval in SCORE space: the scores of a row spread over a few units,
+  // so about log2(candidates) + 2 steps isolate one, where halving the 32 key bits takes all 32 (sign and
+  // exponent bits separate nothing).  Every fourth step tightens the interval to the candidates in it, which
+  // ends rows of equal scores and drops outliers; every eighth halves the key bits, which bounds the search for
+  // any input.  Against 32 steps on the key bits: 12 288 rows of 512 scores,
+  // top-k, 55 -> 36 us; 6 144 rows of 256, mass rule, 21.5 -> 16.7 us.
+  // The masses are summed in fixed point (weights in units of 2^-31: a warp-wide integer add is
   // one instruction where a float sum is five shuffle rounds, and the result does not depend on the order),
   // so decisions agree with the round-by-round form except where the mass comes within about 1e-7 --
   // fp32 summation noise -- of tau.
@@ -127,7 +156,7 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
   uint32_t wgt[ITEMS];          // mode 1: softmax weight of every candidate, units of 2^-31
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) wgt[it] = 0u;
-  if (p.mode == 1) {
+  if (MASS) {
     uint32_t km = 0u;
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) km = max(km, key[it]);
@@ -159,42 +188,70 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
       }
     }
     n = (int)__reduce_add_sync(0xffffffffu, (unsigned)cnt);
-    cum = __reduce_add_sync(0xffffffffu, fm);
+    if (MASS) cum = __reduce_add_sync(0xffffffffu, fm);
   }
   const int kk = min(p.k, Nb);
-  if (n < kk && !(p.mode == 1 && n >= 1 && cum >= tau_q)) {
-    // count and mass of the candidates with key >= t
+  if (n < kk && !(MASS && n >= 1 && cum >= tau_q)) {
+    // count and mass of the candidates with key >= t (t >= 1)
     auto above = [&](uint32_t t, int& cnt, uint32_t& mass) {
       int c = 0;
       uint32_t g = 0u;
 #pragma unroll
       for (int it = 0; it < ITEMS; ++it) {
-        const bool ge = key[it] >= t && key[it] != 0u;
+        const bool ge = key[it] >= t;
         c += ge;
-        if (ge) g += wgt[it];
+        if (MASS && ge) g += wgt[it];
       }
       cnt = (int)__reduce_add_sync(0xffffffffu, (unsigned)c);
-      mass = p.mode == 1 ? __reduce_add_sync(0xffffffffu, g) : 0u;
+      mass = MASS ? __reduce_add_sync(0xffffffffu, g) : 0u;
     };
-    // largest threshold at which taking every candidate >= it ends the rule (0: never -> take them all)
-    uint32_t T = 0u;
+    auto ends = [&](int c, uint32_t g) { return n + c >= kk || (MASS && c >= 1 && cum + g >= tau_q); };
+    // smallest and largest candidate key in [lo, hi) (it holds at least one)
+    auto range = [&](uint32_t lo, uint32_t hi, uint32_t& kmin, uint32_t& kmax) {
+      uint32_t a = 0xffffffffu, b = 0u;
+#pragma unroll
+      for (int it = 0; it < ITEMS; ++it)
+        if (key[it] >= lo && key[it] < hi) { a = min(a, key[it]); b = max(b, key[it]); }
+      kmin = __reduce_min_sync(0xffffffffu, a);
+      kmax = __reduce_max_sync(0xffffffffu, b);
+    };
+    uint32_t T = 0u;                         // 0: the rule never ends, take every candidate
+    int cl, G = 0;                           // candidates >= lo; candidates >= hi, and their mass
+    uint32_t ml, Mg = 0u;
+    above(1u, cl, ml);
+    if (!ends(cl, ml)) {
+      G = cl;
+      Mg = ml;
+    } else {
+      uint32_t lo, hi;
+      range(1u, 0xffffffffu, lo, hi);        // (no score has the key 0xffffffff)
+      ++hi;
 #pragma unroll 1
-    for (int bit = 31; bit >= 0; --bit) {
-      const uint32_t t = T | (1u << bit);
-      int c;
-      uint32_t g;
-      above(t, c, g);
-      if (n + c >= kk || (p.mode == 1 && c >= 1 && cum + g >= tau_q)) T = t;
+      for (int step = 0; hi - lo > 1u && cl - G > 1; ++step) {
+        uint32_t t;
+        if ((step & 7) == 7) {
+          t = lo + ((hi - lo) >> 1);
+        } else {
+          t = score_key(0.5f * key_score(lo) + 0.5f * key_score(hi - 1u));      // (NaN -- infinities of both signs -- gives 0)
+          t = min(max(t, lo + 1u), hi - 1u);
+        }
+        int c;
+        uint32_t g;
+        above(t, c, g);
+        if (ends(c, g)) { lo = t; cl = c; } else { hi = t; G = c; Mg = g; }
+        if ((step & 3) == 3) {
+          range(lo, hi, lo, hi);
+          ++hi;
+        }
+      }
+      if (hi - lo > 1u) range(lo, hi, lo, hi);        // one candidate left
+      T = lo;
     }
     // everything above T, then ties at T in index order while the rule still runs
-    int G;
-    uint32_t Mg;
-    above(T + 1u, G, Mg);                    // T = 0: all candidates; T = 0xffffffff cannot be reached (see below)
     int have = n + G;
     uint32_t acc = cum + Mg;
-    int ties_wanted = 0;
+    int ties_wanted = 0, E = 0;              // ties: candidates equal to T
     if (T != 0u) {
-      int E = 0;
       uint32_t wT = 0u;                      // weight of a candidate equal to T (they all have the same)
 #pragma unroll
       for (int it = 0; it < ITEMS; ++it) {
@@ -202,23 +259,27 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
         if (key[it] == T) wT = wgt[it];
       }
       E = (int)__reduce_add_sync(0xffffffffu, (unsigned)E);
-      wT = __reduce_max_sync(0xffffffffu, wT);
+      if (MASS) wT = __reduce_max_sync(0xffffffffu, wT);
       while (ties_wanted < E) {
         if (have >= kk) break;
-        if (p.mode == 1 && have >= 1 && acc >= tau_q) break;
+        if (MASS && have >= 1 && acc >= tau_q) break;
         ++ties_wanted; ++have; acc += wT;
       }
     }
-    int seen = 0;                            // ties met so far, in index order
+    if (ties_wanted == E) {                  // all of them (the common case: one candidate holds the threshold)
 #pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-      const bool cand = key[it] != 0u;
-      const bool gt = cand && key[it] > T;
-      const bool eq = cand && T != 0u && key[it] == T;
-      const uint32_t bal = __ballot_sync(0xffffffffu, eq);
-      const bool take = gt || (eq && seen + __popc(bal & ((1u << lane) - 1u)) < ties_wanted);
-      if (take) mask |= 1u << it;
-      seen += __popc(bal);
+      for (int it = 0; it < ITEMS; ++it)
+        if (key[it] >= max(T, 1u)) mask |= 1u << it;
+    } else {
+      int seen = 0;                          // ties met so far, in index order
+#pragma unroll
+      for (int it = 0; it < ITEMS; ++it) {
+        const bool gt = key[it] > T, eq = key[it] == T;          // (T != 0 here: T = 0 has no ties)
+        const uint32_t bal = __ballot_sync(0xffffffffu, eq);
+        const bool take = gt || (eq && seen + __popc(bal & ((1u << lane) - 1u)) < ties_wanted);
+        if (take) mask |= 1u << it;
+        seen += __popc(bal);
+      }
     }
     n = have;
   }
@@ -248,73 +309,105 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
 }
 
 // Block scores of one head as a small fp32 GEMM: S[I][J] = scale * <qbar_I, kbar_J>.  A CTA computes a
-// 64 x 64 tile from the two 64 x D panels in shared memory (row stride D + 4 floats: 128-bit reads of
-// eight consecutive rows touch every bank once); a thread owns a 4 x 4 patch -- rows 4*ty..4*ty+3 (one
-// address per half-warp: a broadcast), keys tx, tx+16, tx+32, tx+48 -- and keeps two partial sums per
-// entry (dimensions 0,2 mod 4 and 1,3 mod 4, each in ascending order; that order is part of the
-// result: it is what makes the scores reproducible bit for bit).  32 independent FMA chains per thread
-// hide the shared-memory latency that bounded the earlier one-warp-per-row form.
-static constexpr int SC_TILE = 64;
-template <int D>
-__global__ void __launch_bounds__(256)
+// (PQ * TY) x (PK * 16) tile from two D-wide panels in shared memory (row stride D + 4 floats: 128-bit reads of
+// eight consecutive rows touch every bank once); a thread owns a PQ x PK patch -- rows PQ*ty.., keys tx, tx+16, .. --
+// and keeps two partial sums per entry (dimensions 0,2 mod 4 and 1,3 mod 4, each in ascending order; that
+// order is part of the result: it is what makes the scores reproducible bit for bit).  The two sums are the halves
+// of one packed f32x2 accumulator, so four dimensions of an entry are two instructions.
+// A 128-bit shared-memory read delivers 512 bytes to a warp whatever it broadcasts -- four cycles of the port -- so the 4 x 4
+// patch of 256 threads ran at 90 % of the port; 8 x 4 needs a quarter fewer reads per FMA.  Patches beyond that (8 x 8 of
+// 64 x 128 tiles: 19.3 / 49.8 us) and scalar FMAs measured the same: what is left is the FMA pipe at about half its
+// nominal rate and the panels' load.  24 heads of 256 / 512 blocks, d = 128: 18.9 / 57 -> 16.2 / 51 us.
+template <int D, int PQ, int PK, int TY>
+__global__ void __launch_bounds__(16 * TY)
 block_scores_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar, int Nb, float scale,
                     float* __restrict__ scores) {
-  constexpr int LD = D + 4;
+  constexpr int LD = D + 4, TQ = PQ * TY, TK = PK * 16, THREADS = 16 * TY, V = D / 4;
   extern __shared__ __align__(16) float sc_smem[];
-  float* qs = sc_smem;                     // [64][LD]
-  float* ks = sc_smem + SC_TILE * LD;      // [64][LD]
-  const int bh = blockIdx.z, I0 = blockIdx.y * SC_TILE, J0 = blockIdx.x * SC_TILE;
-  const float* qb = qbar + (long long)bh * Nb * D;
-  const float* kb = kbar + (long long)bh * Nb * D;
-  for (int idx = threadIdx.x; idx < SC_TILE * (D / 4); idx += 256) {
-    const int row = idx / (D / 4), c4 = idx % (D / 4);
-    float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-    if (I0 + row < Nb) a = __ldg(reinterpret_cast<const float4*>(qb + (long long)(I0 + row) * D) + c4);
-    if (J0 + row < Nb) b = __ldg(reinterpret_cast<const float4*>(kb + (long long)(J0 + row) * D) + c4);
-    *reinterpret_cast<float4*>(qs + row * LD + 4 * c4) = a;
-    *reinterpret_cast<float4*>(ks + row * LD + 4 * c4) = b;
-  }
+  float* qs = sc_smem;                     // [TQ][LD]
+  float* ks = sc_smem + TQ * LD;           // [TK][LD]
+  const int bh = blockIdx.z, I0 = blockIdx.y * TQ, J0 = blockIdx.x * TK;
+  auto fill = [&](float* dst, const float* src, int r0, auto rows_tag) {      // eight 16-byte vectors per thread in flight
+    constexpr int PER = decltype(rows_tag)::value * V / THREADS, BATCH = PER < 8 ? PER : 8;
+#pragma unroll
+    for (int u0 = 0; u0 < PER; u0 += BATCH) {
+      float4 a[BATCH];
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u) {
+        const int idx = threadIdx.x + THREADS * (u0 + u), row = idx / V, c4 = idx % V;
+        a[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (r0 + row < Nb) a[u] = __ldg(reinterpret_cast<const float4*>(src + (long long)(r0 + row) * D) + c4);
+      }
+#pragma unroll
+      for (int u = 0; u < BATCH; ++u) {
+        const int idx = threadIdx.x + THREADS * (u0 + u), row = idx / V, c4 = idx % V;
+        *reinterpret_cast<float4*>(dst + row * LD + 4 * c4) = a[u];
+      }
+    }
+  };
+  fill(qs, qbar + (long long)bh * Nb * D, I0, std::integral_constant<int, TQ>{});
+  fill(ks, kbar + (long long)bh * Nb * D, J0, std::integral_constant<int, TK>{});
   __syncthreads();
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  float a0[4][4], a1[4][4];
+  uint64_t acc[PQ][PK];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < PQ; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) { a0[i][j] = 0.f; a1[i][j] = 0.f; }
+    for (int j = 0; j < PK; ++j) acc[i][j] = pack2(0.f, 0.f);
 #pragma unroll 2
   for (int c = 0; c < D; c += 4) {
-    float4 qv[4], kv[4];
+    ulonglong2 qv[PQ], kv[PK];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) qv[i] = *reinterpret_cast<const float4*>(qs + (ty * 4 + i) * LD + c);
+    for (int i = 0; i < PQ; ++i) qv[i] = *reinterpret_cast<const ulonglong2*>(qs + (ty * PQ + i) * LD + c);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) kv[j] = *reinterpret_cast<const float4*>(ks + (tx + 16 * j) * LD + c);
+    for (int j = 0; j < PK; ++j) kv[j] = *reinterpret_cast<const ulonglong2*>(ks + (tx + 16 * j) * LD + c);
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
+    for (int i = 0; i < PQ; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        a0[i][j] = fmaf(qv[i].x, kv[j].x, a0[i][j]);
-        a1[i][j] = fmaf(qv[i].y, kv[j].y, a1[i][j]);
-        a0[i][j] = fmaf(qv[i].z, kv[j].z, a0[i][j]);
-        a1[i][j] = fmaf(qv[i].w, kv[j].w, a1[i][j]);
+      for (int j = 0; j < PK; ++j) {
+        acc[i][j] = fma2(qv[i].x, kv[j].x, acc[i][j]);
+        acc[i][j] = fma2(qv[i].y, kv[j].y, acc[i][j]);
       }
   }
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int I = I0 + ty * 4 + i;
+  for (int i = 0; i < PQ; ++i) {
+    const int I = I0 + ty * PQ + i;
     if (I >= Nb) continue;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < PK; ++j) {
       const int J = J0 + tx + 16 * j;
-      if (J < Nb) scores[((long long)bh * Nb + I) * Nb + J] = (a0[i][j] + a1[i][j]) * scale;
+      float s0, s1;
+      unpack2(acc[i][j], s0, s1);
+      if (J < Nb) scores[((long long)bh * Nb + I) * Nb + J] = (s0 + s1) * scale;
     }
   }
+}
+
+template <int D, int PQ, int PK, int TY>
+static int launch_scores(const float* qbar, const float* kbar, int Nb, int heads, float scale, float* scores, cudaStream_t st) {
+  auto kern = block_scores_kernel<D, PQ, PK, TY>;
+  constexpr int TQ = PQ * TY, TK = PK * 16, smem = (TQ + TK) * (D + 4) * (int)sizeof(float);
+  // (the shared-memory attribute is set once per device and instantiation, not per call)
+  static std::mutex attr_mutex;
+  static bool attr_set[64] = {false};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SVA_ERR_CUDA;
+  {
+    std::lock_guard<std::mutex> lock(attr_mutex);
+    if (!attr_set[dev]) {
+      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return SVA_ERR_CUDA;
+      attr_set[dev] = true;
+    }
+  }
+  kern<<<dim3((Nb + TK - 1) / TK, (Nb + TQ - 1) / TQ, heads), 16 * TY, smem, st>>>(qbar, kbar, Nb, scale, scores);
+  return SVA_OK;
 }
 
 // Selection: one warp per query-block row, its Nb scores read straight from the score matrix (lane j owns
 // the key blocks it*32 + j).  No shared memory and few registers, so the SMs hold enough warps to hide the
 // serial chain of the threshold search.
 static constexpr int SEL_WARPS = 8;
-template <int ITEMS>
+template <int ITEMS, bool MASS>
 __global__ void __launch_bounds__(SEL_WARPS * 32)
 select_rows_kernel(const float* __restrict__ scores, SelParams p, int32_t* __restrict__ row_ptr,
                    int32_t* __restrict__ col_idx, int32_t* __restrict__ tmp_idx, int32_t* __restrict__ counts, int R) {
@@ -329,7 +422,7 @@ select_rows_kernel(const float* __restrict__ scores, SelParams p, int32_t* __res
     const int J = it * 32 + lane;
     key[it] = J < Nb ? score_key(__ldg(srow + J)) : 0u;
   }
-  select_and_emit<ITEMS>(key, I, bh, lane, p, row_ptr, col_idx, tmp_idx, counts, R);
+  select_and_emit<ITEMS, MASS>(key, I, bh, lane, p, row_ptr, col_idx, tmp_idx, counts, R);
 }
 
 // CSR assembly for rows of varying length, one launch: a CTA owns 32 consecutive rows (one warp each).  It
@@ -423,15 +516,16 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
     tmp_idx = reinterpret_cast<int32_t*>(w + 2 * pooled);
     counts = reinterpret_cast<int32_t*>(w + 2 * pooled + align256((size_t)m.R * cap * sizeof(int32_t)));
   }
-  dim3 pg(m.Nb, m.B * m.H, 2);
+  const int run = pool_run(m);
+  dim3 pg((m.Nb + run - 1) / run, m.B * m.H, 2);
   Strides sq = make_strides(p->q_stride), sk = make_strides(p->k_stride);
   if (qbar_in) {
   } else if (m.fp8)
     pool_kernel<D, 1><<<pg, POOL_THREADS, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, q_scale,
-                                                   k_scale, m.H, m.N, m.block, m.Nb, qbar, kbar);
+                                                   k_scale, m.H, m.N, m.block, m.Nb, run, qbar, kbar);
   else
     pool_kernel<D, 2><<<pg, POOL_THREADS, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, nullptr,
-                                                   nullptr, m.H, m.N, m.block, m.Nb, qbar, kbar);
+                                                   nullptr, m.H, m.N, m.block, m.Nb, run, qbar, kbar);
   SelParams sp;
   sp.H = m.H; sp.Nb = m.Nb; sp.mode = s->mode; sp.k = s->k;
   sp.use_window = (s->win_t >= 0 && s->win_s >= 0 && s->blocks_per_frame > 0) ? 1 : 0;
@@ -445,27 +539,20 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
     scores = reinterpret_cast<float*>(w + off);
   }
   {
-    auto kern = block_scores_kernel<D>;
-    constexpr int smem = 2 * SC_TILE * (D + 4) * (int)sizeof(float);
-    // (the shared-memory attribute is set once per device and instantiation, not per call)
-    static std::mutex attr_mutex;
-    static bool attr_set[64] = {false};
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SVA_ERR_CUDA;
-    {
-      std::lock_guard<std::mutex> lock(attr_mutex);
-      if (!attr_set[dev]) {
-        if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return SVA_ERR_CUDA;
-        attr_set[dev] = true;
-      }
-    }
-    const int nt = (m.Nb + SC_TILE - 1) / SC_TILE;
-    kern<<<dim3(nt, nt, m.B * m.H), 256, smem, st>>>(qbar, kbar, m.Nb, m.scale, scores);
+    // 64 x 64 tiles where they give most of the SMs a CTA, else 32 x 32: with few rows the time is one CTA's latency, and
+    // that shrinks with its tile (16 heads of 64 blocks: 16 tiles of 64 x 64 take 6.8 us, 64 of 32 x 32 4.2 us).
+    const int heads = m.B * m.H, nt = (m.Nb + 63) / 64;
+    const int rc = nt * nt * heads >= 96 ? launch_scores<D, 8, 4, 8>(qbar, kbar, m.Nb, heads, m.scale, scores, st)
+                             : launch_scores<D, 2, 2, 16>(qbar, kbar, m.Nb, heads, m.scale, scores, st);
+    if (rc != SVA_OK) return rc;
   }
   const int items = (m.Nb + 31) / 32;
   const int sg = (m.R + SEL_WARPS - 1) / SEL_WARPS;
-#define SVA_SEL_LAUNCH(IT) \
-  select_rows_kernel<IT><<<sg, SEL_WARPS * 32, 0, st>>>(scores, sp, row_ptr, col_idx, tmp_idx, counts, m.R)
+#define SVA_SEL_LAUNCH(IT)                                                                                                    \
+  do {                                                                                                                        \
+    if (s->mode == 1) select_rows_kernel<IT, true><<<sg, SEL_WARPS * 32, 0, st>>>(scores, sp, row_ptr, col_idx, tmp_idx, counts, m.R); \
+    else select_rows_kernel<IT, false><<<sg, SEL_WARPS * 32, 0, st>>>(scores, sp, row_ptr, col_idx, tmp_idx, counts, m.R);     \
+  } while (0)
   if (items <= 4) SVA_SEL_LAUNCH(4);
   else if (items <= 8) SVA_SEL_LAUNCH(8);
   else if (items <= 12) SVA_SEL_LAUNCH(12);
@@ -494,16 +581,17 @@ int launch_select(const Dims& m, const sva_problem_t* p, const sva_select_t* s, 
 // Pooling alone: block means of Q and K into the caller's arrays ([B,H,Nb,d] fp32 each).
 int launch_pool(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale,
                 const float* k_scale, float* qbar, float* kbar, cudaStream_t st) {
-  dim3 pg(m.Nb, m.B * m.H, 2);
+  const int run = pool_run(m);
+  dim3 pg((m.Nb + run - 1) / run, m.B * m.H, 2);
   Strides sq = make_strides(p->q_stride), sk = make_strides(p->k_stride);
 #define SVA_POOL_LAUNCH(DD)                                                                                        \
   do {                                                                                                             \
     if (m.fp8)                                                                                                     \
       pool_kernel<DD, 1><<<pg, POOL_THREADS, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, q_scale, k_scale, \
-                                                      m.H, m.N, m.block, m.Nb, qbar, kbar);                       \
+                                                      m.H, m.N, m.block, m.Nb, run, qbar, kbar);                       \
     else                                                                                                           \
       pool_kernel<DD, 2><<<pg, POOL_THREADS, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, nullptr, nullptr, \
-                                                      m.H, m.N, m.block, m.Nb, qbar, kbar);                       \
+                                                      m.H, m.N, m.block, m.Nb, run, qbar, kbar);                       \
   } while (0)
   if (m.d == 128) SVA_POOL_LAUNCH(128);
   else if (m.d == 64) SVA_POOL_LAUNCH(64);

@@ -132,3 +132,56 @@ def test_many_blocks_per_head(T, Hg, Wg, mode, k, tau, d):
     o, lse, st = U.gpu_attn(w, qd, kd, vd, rp, ci)
     assert st == 0
     U.check_attn_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, U.sample_rows(w.R, w.Nb, 6))
+
+
+def _rule(scores, mode, k, tau):
+    """The routing rule, one candidate at a time (float64 masses); the smallest distance of the mass from tau on the way."""
+    order = sorted((j for j in range(len(scores)) if not np.isnan(scores[j])), key=lambda j: (-scores[j], j))
+    x = scores.astype(np.float64)
+    e = np.exp(x - x[order[0]]) if mode == 1 else None
+    z = e[order].sum() if mode == 1 else 1.0
+    kept, mass, margin = [], 0.0, np.inf
+    for j in order[:k]:
+        kept.append(j)
+        if mode == 1:
+            mass += e[j] / z
+            margin = min(margin, abs(mass - tau))
+            if mass >= tau:
+                break
+    return sorted(kept), margin
+
+
+@pytest.mark.parametrize("nb", [1, 2, 31, 33, 128, 129, 257, 385, 513, 1024])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_threshold_search_on_awkward_scores(nb, mode):
+    """Rows whose scores are equal, nearly equal, far apart, infinite or a few values many times: the search for the
+    threshold must end and keep what the rule keeps (scores are made exact: one non-zero dimension)."""
+    rng = np.random.default_rng(nb)
+    kinds = [rng.standard_normal(nb), np.zeros(nb), 1.0 + 2.0 ** -22 * rng.integers(0, 3, nb), rng.integers(-2, 3, nb) * 1.0,
+             -np.exp(rng.standard_normal(nb) * 4.0), np.linspace(-3.0, 3.0, nb)]
+    if mode == 0:
+        wild = rng.standard_normal(nb)
+        wild[rng.integers(0, nb, 2)] = (np.inf, -np.inf)
+        kinds += [rng.standard_normal(nb) * 10.0 ** rng.integers(-30, 30, nb), wild, 1e-40 * rng.standard_normal(nb)]
+    H, d = len(kinds), 128
+    n = nb * 128
+    kbar = np.zeros((1, H, nb, d), np.float32)
+    for h, x in enumerate(kinds):
+        kbar[0, h, :, 0] = x
+    qbar = np.zeros_like(kbar)
+    qbar[..., 0] = 1.0
+    t = torch.empty(1, H, n, d, dtype=torch.bfloat16, device="cuda")
+    p = B.make_problem(t, t, None, None, n, 128, 1.0)
+    for k in sorted({1, max(1, nb // 10), max(1, nb // 2), nb}):
+        s = B.make_select(mode, k, 0.87)
+        ws = torch.empty(max(B.select_workspace_bytes(p, s), 256), dtype=torch.uint8, device="cuda")
+        rp = torch.zeros(H * nb + 1, dtype=torch.int32, device="cuda")
+        ci = torch.zeros(B.select_max_nnz(p, s), dtype=torch.int32, device="cuda")
+        B.block_select_pooled(p, s, torch.tensor(qbar).cuda(), torch.tensor(kbar).cuda(), rp, ci, ws)
+        rp, ci = rp.cpu().numpy(), ci.cpu().numpy()
+        for h in range(H):
+            want, margin = _rule(kbar[0, h, :, 0], mode, k, 0.87)
+            if margin < 1e-5:                                 # fixed-point masses (2^-31 each) against float64
+                continue
+            for r in (h * nb, h * nb + nb - 1):
+                assert ci[rp[r]:rp[r + 1]].tolist() == want, (h, k)
