@@ -337,16 +337,18 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);        // entries of the row's own list
           if (r < prm.R) { e0 = list_block<B64, REM>(prm, beg, 0, n_own); if (n > 1) e1 = list_block<B64, REM>(prm, beg, 1, n_own); }
           if (!F4 && !B64 && r < prm.R) {
-            // the row's Q tile will be fetched about a row from now: start it on its way into the L2
-            const int I = r % Nb, bh0 = r / Nb, rows = min(BS, prm.N - I * BS);
+            // the row's Q tile will be fetched about a row from now: start it on its way into the L2.  Token rows that are not
+            // contiguous ([B,N,H,d], a packed projection) go as a tensor prefetch: with a plain one per token row this lane
+            // spent about 9 000 cycles per row in which no K tile was on its way (32 760 tokens x 24 heads, 40 blocks kept:
+            // 3.08 M cycles where [B,H,N,d] took 2.69 M; now the same).
+            const int I = r % Nb, bh0 = r / Nb;
             const uint32_t eb = F8 ? 1u : 2u, row_bytes = (uint32_t)prm.d * eb;
-            const uint8_t* qrow = reinterpret_cast<const uint8_t*>(prm.q) +
-                                  ((long long)(bh0 / prm.H) * prm.sq.b + (long long)(bh0 % prm.H) * prm.sq.h +
-                                   (long long)I * BS * prm.sq.n) * eb;
             if (prm.sq.n * (long long)eb == (long long)row_bytes) {
-              bulk_prefetch_l2(qrow, (uint32_t)rows * row_bytes);
+              const long long q0 = (long long)(bh0 / prm.H) * prm.sq.b + (long long)(bh0 % prm.H) * prm.sq.h + (long long)I * BS * prm.sq.n;
+              bulk_prefetch_l2(reinterpret_cast<const uint8_t*>(prm.q) + q0 * eb, (uint32_t)min(BS, prm.N - I * BS) * row_bytes);
             } else {
-              for (int t = 0; t < rows; ++t) bulk_prefetch_l2(qrow + (long long)t * prm.sq.n * eb, row_bytes);
+              tma_prefetch_4d(&tm_q, 0, I * BS, bh0 % prm.H, bh0 / prm.H);
+              if (!F8) tma_prefetch_4d(&tm_q, 64, I * BS, bh0 % prm.H, bh0 / prm.H);
             }
           }
           rowq[8 * slot] = r;
