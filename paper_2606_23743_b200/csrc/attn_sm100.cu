@@ -100,7 +100,9 @@ struct TsParams {
   int n1;                     // first-order tiles after them: 0 (order 0), 1, or 2 with 64-token blocks (one per query block)
   const float* mu;            // first-order term: the reference mu_I of every query block's weights, [R of the CSR]
   int np;                     // pooled tiles per head = ceil(Nb / 128); 0 = no remainder
-  int rem_mask;               // 1: the K producer leaves a bit mask of every row's kept blocks in shared memory (Nb <= 1024)
+  int rem_mask;               // 1: the kept blocks of a row are at hand as a bit mask (Nb <= 1024): 128-token blocks, left in
+                              // shared memory by the K producer; 64-token blocks, in kept_mask by pair_lists_kernel
+  const uint4* kept_mask;     // 64-token blocks: [tile row][query block A, B][8 chunks of 128 key blocks]
   float log2_block;           // log2(tokens per block): a block mean stands for that many keys
   float tail_bias;            // (log2(keys of the last block) - log2_block) / scale_log2: added to the last block's pooled logit
   long long* prof;            // tuning aid, normally null: entry 319 receives the longest CTA's cycle count
@@ -193,6 +195,39 @@ __device__ __forceinline__ uint32_t list_block(const TsParams& prm, int beg, int
   if (prm.row_ptr == nullptr) return (uint32_t)j;
   const int J = __ldg(prm.col_idx + beg + j);
   return (J < 0 || J >= prm.Nb) ? 0u : (uint32_t)J;
+}
+
+// -inf into the columns [from, to) of this warp's lanes; to is a multiple of 8.  Eight columns per store: with one per store
+// (about 30 cycles each) a tile of 10 block means out of 128 took 3 500 cycles to mask; 138 blocks per head, remainder of
+// order 1: 1.05 -> 0.90 M cycles.  Not inlined: rare, and the tile loop is bound by its instruction stream.  (64-token
+// blocks keep single stores for a ragged half of at most 63 keys: with this call there 2.41 -> 2.47 M cycles.)
+__device__ __noinline__ void tmem_fill_ninf(uint32_t from, uint32_t to) {
+#pragma unroll 1
+  for (; from & 7u; ++from) tmem_st1(from, 0xff800000u);
+#pragma unroll 1
+  for (; from < to; from += 8) tmem_st8_same(from, 0xff800000u);
+}
+
+// The remainder stands for the DROPPED blocks only: in a tile of block means (S in tensor memory at s_tmem, chunk pc of 128
+// blocks) the blocks that query block rq keeps become -inf, one warp-wide TMEM store each (they are the same for a whole
+// warp).  This form looks them up in the CSR (no bit mask: more than 1024 key blocks, or a workspace without room for the
+// masks); called by whole warps.
+__device__ __noinline__ void mask_pooled_from_csr(const int32_t* row_ptr, const int32_t* col_idx, int rq, int nnz_total, int Nb,
+                                                  int pc, uint32_t s_tmem) {
+  const int lane = threadIdx.x & 31;
+  const int cb = __ldg(row_ptr + rq);
+  int ce = __ldg(row_ptr + rq + 1);
+  if (cb < 0 || ce < cb || ce - cb > Nb || ce > nnz_total) ce = cb;              // corrupt pair (reported elsewhere)
+#pragma unroll 1
+  for (int t0 = cb; t0 < ce; t0 += 32) {                         // 32 entries at a time, one per lane
+    const int Jl = t0 + lane < ce ? __ldg(col_idx + t0 + lane) : -1;
+    uint32_t hit = __ballot_sync(0xffffffffu, Jl >= 0 && Jl < Nb && (Jl >> 7) == pc);
+    while (hit) {
+      const int Jk = __shfl_sync(0xffffffffu, Jl, __ffs(hit) - 1);
+      hit &= hit - 1;
+      tmem_st1(s_tmem + (Jk & 127), 0xff800000u);
+    }
+  }
 }
 
 // Persistent kernel.  Rows are handed out in their natural order from one device-wide counter (so the
@@ -629,6 +664,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         mbar_arrive(bar_q_ready);
         return;
       }
+      tc_fence_after();
       if (F8) tmem_st16(q_tmem, qv); else tmem_st32(q_tmem, qv);
       tc_wait_st();
       tc_fence_before();
@@ -653,6 +689,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         if (!F8) tma_load_4d(sbase + OFF_QS, &tm_q, bar_qs, 64, I * BS, bh % prm.H, bh / prm.H);
       }
       if (!mbar_wait(bar_qs, use & 1u, abort_flag, prm.status)) return false;
+      tc_fence_after();
 #pragma unroll
       for (int ps = 0; ps < (F8 ? 1 : 2); ++ps) {
         // 128-byte rows, 16-byte chunks swizzled by row % 8
@@ -713,8 +750,13 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         if (w < n) load_ks(J);
       }
       const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);      // entries of the row's own list
-      // One tile of the row (KIND 0: a kept key block, 1: a tile of block means, 2: the first-order tile).  The
-      // kinds are separate instantiations, so the hot one carries none of the remainder's code; false: a wait ran out.
+      // One tile of the row: a kept key block, or (REM) a tile of block means.  128-token blocks: one copy of the body per kind
+      // (KIND 0, 1), so that the kept blocks' instruction stream carries none of the remainder's; 64-token blocks (KIND 2): one
+      // body for both, told apart by j -- there two copies made the groups, whose warps take different kinds at the same
+      // time, stream both through the instruction cache (24 heads x 512 blocks, 51 kept, order 0: 3.42 M cycles with two
+      // copies, 3.19 with one; with 128-token blocks and 256 of them one copy is 3 % slower).  What only block means need is
+      // kept small or out of line: the mask, and an addend (the logarithm of the keys a mean stands for).
+      // false: a wait ran out.
       auto tile = [&](auto kind_tag, const int j) -> bool {
         constexpr int KIND = decltype(kind_tag)::value;
         const uint32_t mine = cnt[w] + (uint32_t)(j >> 1);            // my barriers' phase index for block j
@@ -722,15 +764,11 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         // valid keys of the tile's two 64-key halves (64-token blocks: a half whose key block this
         // thread's query block does not keep counts as 0; uniform over a warp)
         int v0, v1;
-        constexpr bool pooled = REM && KIND == 1;                     // a tile of block means (the remainder)
+        const bool pooled = REM && (KIND == 2 ? j >= n_own : KIND == 1);                        // a tile of block means (the remainder)
         const int pc = (int)(J & 0xffffu);                            // ... and which 128 blocks it holds
-        constexpr bool fo = REM && KIND == 2;                         // the first-order tile: P = scaled q, "V^T" = A^T
-        if (fo) {
-          v0 = B64 ? 64 : BS; v1 = B64 ? 64 : 0;
-        } else if (pooled) {
-          const int vn = min(BS, prm.Nb - BS * pc);                   // blocks that exist in this tile
-          v0 = B64 ? min(64, vn) : vn;
-          v1 = B64 ? max(vn - 64, 0) : 0;
+        if (REM && pooled) {
+          v0 = B64 ? 64 : BS;                                         // (blocks that do not exist are masked below)
+          v1 = B64 ? 64 : 0;
         } else if (B64) {
           const int u0 = (int)(J & 0x3fffu), u1 = (int)((J >> 16) & 0x3fffu);
           v0 = ((J >> (14 + qh)) & 1u) ? (u0 == prm.Nb - 1 ? tail_keys : 64) : 0;
@@ -743,6 +781,12 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         if (j + 2 < n) {                                               // one entry ahead
           J = list_block<B64, REM>(prm, lbeg, j + 2, n_own);
           if (F8) load_ks(J);
+        }
+        uint4 kept = make_uint4(0u, 0u, 0u, 0u);
+        if (REM && pooled && prm.rem_mask) {                          // four words for this tile's 128 blocks
+          if (B64) {
+            kept = __ldg(prm.kept_mask + ((long long)r * 2 + qh) * 8 + pc);
+          }
         }
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 0);
         if (!mbar_wait(bar_s_full + 8 * w, mine & 1u, abort_flag, prm.status)) return false;
@@ -762,60 +806,47 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
               for (int e = 64 + v1; e < BS; ++e) tmem_st1(s_tmem + e, 0xff800000u);
             }
           } else {
-#pragma unroll 1
-            for (int e = v0; e < BS; ++e) tmem_st1(s_tmem + e, 0xff800000u);
+            tmem_fill_ninf(s_tmem + v0, s_tmem + BS);
           }
           tc_wait_st();
         }
         if (REM && pooled) {
-          // The remainder stands for the DROPPED blocks only: the blocks this thread's query block keeps become
-          // -inf (one warp-wide TMEM store each; the row's CSR entries are the same for a whole warp), and the
-          // ragged last block's mean stands for fewer keys than the others.
-          if (RMASK && prm.rem_mask) {
-            // (the K producer left the kept blocks of this row as a bit mask: four words for this tile's 128 blocks)
+          if (RMASK && prm.rem_mask) {                                // (left by the K producer)
             const volatile uint32_t* mk = reinterpret_cast<const volatile uint32_t*>(smem + OFF_KMASK) +
                                           (rows_done & 7u) * 32 + 4 * pc;
-#pragma unroll 1
+            kept = make_uint4(mk[0], mk[1], mk[2], mk[3]);
+          }
+          if (prm.rem_mask) {
+#pragma unroll
             for (int kw = 0; kw < 4; ++kw) {
-              uint32_t mword = mk[kw];
+              uint32_t mword = kw == 0 ? kept.x : kw == 1 ? kept.y : kw == 2 ? kept.z : kept.w;
+#pragma unroll 1
               while (mword) {
                 const int bit = __ffs(mword) - 1;
                 mword &= mword - 1u;
                 tmem_st1(s_tmem + 32 * kw + bit, 0xff800000u);
               }
             }
+          } else {
+            mask_pooled_from_csr(prm.row_ptr, prm.col_idx, B64 ? bh * prm.Nb + min(2 * I + qh, prm.Nb - 1) : r, nnz_total, prm.Nb,
+                                 pc, s_tmem);
           }
-          const int rq = B64 ? bh * prm.Nb + min(2 * I + qh, prm.Nb - 1) : r;      // my query block's CSR row
-          int cb = 0, ce = 0;                                          // (more than 1024 key blocks: from the CSR itself)
-          if (!(RMASK && prm.rem_mask)) { cb = __ldg(prm.row_ptr + rq); ce = __ldg(prm.row_ptr + rq + 1); }
-          if (cb < 0 || ce < cb || ce - cb > prm.Nb || ce > nnz_total) ce = cb;      // corrupt pair (reported elsewhere)
-#pragma unroll 1
-          for (int t0 = cb; t0 < ce; t0 += 32) {                       // 32 entries at a time, one per lane
-            const int Jl = t0 + lane < ce ? __ldg(prm.col_idx + t0 + lane) : -1;
-            uint32_t hit = __ballot_sync(0xffffffffu, Jl >= 0 && Jl < prm.Nb && (Jl >> 7) == pc);
-            while (hit) {
-              const int Jk = __shfl_sync(0xffffffffu, Jl, __ffs(hit) - 1);
-              hit &= hit - 1;
-              tmem_st1(s_tmem + (Jk & 127), 0xff800000u);
-            }
-          }
-          if (tail_keys < KB && ((prm.Nb - 1) >> 7) == pc) {
+          if (prm.Nb - BS * pc < BS) tmem_fill_ninf(s_tmem + prm.Nb - BS * pc, s_tmem + BS);
+          if (tail_keys < KB && ((prm.Nb - 1) >> 7) == pc) {          // the ragged last block's mean stands for fewer keys
             tc_wait_st();
             const uint32_t col = s_tmem + ((prm.Nb - 1) & 127);
             const float x = __uint_as_float(tmem_ld1(col));
             tc_wait_ld();
-            tmem_st1(col, __float_as_uint(x + prm.tail_bias));          // (-inf stays -inf)
+            tmem_st1(col, __float_as_uint(x + prm.tail_bias));        // (-inf stays -inf)
           }
           tc_wait_st();
         }
         uint32_t sv[128];
-        if (!(REM && fo)) {                                           // (a first-order tile's S is a dummy: not read)
-          tmem_ld32(s_tmem + 0, sv + 0);
-          tmem_ld32(s_tmem + 32, sv + 32);
-          tc_wait_ld();
-          tmem_ld32(s_tmem + 64, sv + 64);
-          tmem_ld32(s_tmem + 96, sv + 96);
-        }
+        tmem_ld32(s_tmem + 0, sv + 0);
+        tmem_ld32(s_tmem + 32, sv + 32);
+        tc_wait_ld();
+        tmem_ld32(s_tmem + 64, sv + 64);
+        tmem_ld32(s_tmem + 96, sv + 96);
         float mxa = -INFINITY, mxb = -INFINITY, mxc = -INFINITY, mxd = -INFINITY;
         float mx0, mx1;
         if (!B64) {
@@ -828,7 +859,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             mxd = max3(mxd, __uint_as_float(sv[e + 6]), __uint_as_float(sv[e + 7]));
           }
         }
-        if (!(REM && fo)) tc_wait_ld();
+        tc_wait_ld();
         tc_fence_before();
         mbar_arrive(bar_s_free + 8 * w);                     // the S issuer may refill this buffer
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 2);
@@ -855,9 +886,9 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         }
         // (e4m3 with 64-token blocks: each half has its own scale; a half that is not kept stays -inf)
         // (a pooled logit carries + log2(keys per block): a block mean stands for that many keys)
-        const float mx = (REM && fo) ? -INFINITY
-                       : (B64 && F8) ? fmaxf(v0 > 0 ? mx0 * c : -INFINITY, v1 > 0 ? mx1 * c1 : -INFINITY)
-                                     : fmaxf(mx0, mx1) * c + ((REM && pooled) ? prm.log2_block : 0.f);
+        const float bias = REM && pooled ? prm.log2_block : 0.f;
+        const float mx = (B64 && F8) ? fmaxf(v0 > 0 ? mx0 * c : -INFINITY, v1 > 0 ? mx1 * c1 : -INFINITY)
+                                     : REM ? fmaxf(mx0, mx1) * c + bias : fmaxf(mx0, mx1) * c;
         // reference exponent left by block j-1 (other group)
         float m_prev = -INFINITY;
         if (j > 0) {
@@ -892,7 +923,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         // (64-token blocks: -inf instead of -m for a half that is not kept, or while the row has seen no
         // kept key yet, makes those P exactly 0 at no cost)
         float nm = -m_new, nmh1 = -m_new;
-        if (REM && pooled) { nm += prm.log2_block; nmh1 = nm; }
+        if (REM) { nm += bias; nmh1 = nm; }
         if (B64) {
           if (m_new == -INFINITY || v0 == 0) nm = -INFINITY;
           if (m_new == -INFINITY || v1 == 0) nmh1 = -INFINITY;
@@ -900,24 +931,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const uint64_t c2 = pack2(c, c), nm2 = pack2(nm, nm), nm2h1 = B64 ? pack2(nmh1, nmh1) : nm2;
         const uint64_t c2h1 = (B64 && F8) ? pack2(c1, c1) : c2;
         uint64_t sum2 = pack2(0.f, 0.f);
-        if (REM && fo) {
-          // P'[i][c] = scale * q_i[c] * exp(mu - m): the row's own query values, for the rows of the query block this
-          // tile belongs to (64-token blocks: the other half of the tile row gets zeros); nothing joins the row sum
-          const int qb = B64 ? min(2 * I + qh, prm.Nb - 1) : I;
-          const bool mine_rows = (qi < prm.N) && (!B64 || qh == (int)(J & 1u)) && m_new != -INFINITY;
-          const float f = mine_rows ? prm.scale_log2 * 0.6931471805599453f *
-                                          ex2(__ldg(prm.mu + (long long)bh * prm.Nb + qb) * 1.4426950408889634f - m_new)
-                                    : 0.f;
-          const uint4* src = reinterpret_cast<const uint4*>(prm.q + (long long)bb * prm.sq.b + (long long)hh * prm.sq.h +
-                                                            (long long)min(qi, prm.N - 1) * prm.sq.n);
-#pragma unroll
-          for (int e = 0; e < 16; ++e) {
-            const uint4 u = __ldg(src + e);
-            const uint32_t wd[4] = {u.x, u.y, u.z, u.w};
-#pragma unroll
-            for (int t = 0; t < 4; ++t) sv[4 * e + t] = pack_bf16(bf16lo(wd[t]) * f, bf16hi(wd[t]) * f);
-          }
-        } else if (!(prm.debug & 1)) {
+        if (!(prm.debug & 1)) {
 #pragma unroll
           for (int e = 0; e < 128; e += 2) {
             float x0, x1;
@@ -947,10 +961,51 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 6);
         return true;
       };
-      for (int j = w; j < n && ok; j += 2) {
-        if (!REM || j < n_own) ok = tile(std::integral_constant<int, 0>{}, j);
-        else if (j < n_own + prm.np) ok = tile(std::integral_constant<int, 1>{}, j);
-        else ok = tile(std::integral_constant<int, 2>{}, j);
+      // A first-order tile: P = the row's own query values, scaled, and "V" = A_I.  Its S is a dummy; nothing joins the row sum.
+      // P'[i][c] = scale * q_i[c] * exp(mu - m) for the rows of the query block it belongs to (64-token blocks: the other
+      // half of the tile row gets zeros).  Q is still in tensor memory (the next row's is written after this P is out).
+      auto first_order_tile = [&](const int j) -> bool {
+        const uint32_t mine = cnt[w] + (uint32_t)(j >> 1), prev = cnt[w ^ 1] + (uint32_t)((j - 1) >> 1);
+        const uint32_t J_now = J;
+        if (j + 2 < n) J = list_block<B64, REM>(prm, lbeg, j + 2, n_own);
+        if (!mbar_wait(bar_s_full + 8 * w, mine & 1u, abort_flag, prm.status)) return false;
+        mbar_arrive(bar_s_free + 8 * w);
+        if (!mbar_wait(bar_ref + 8 * (w ^ 1), prev & 1u, abort_flag, prm.status)) return false;
+        const float m_now = ref[(w ^ 1) * 128 + row];                 // (j > 0: the row has at least one tile of block means)
+        ref[w * 128 + row] = m_now;
+        mbar_arrive(bar_ref + 8 * w);
+        if (m_now != m_mine) { l *= ex2(m_mine - m_now); m_mine = m_now; }
+        const int qb = B64 ? min(2 * I + qh, prm.Nb - 1) : I;
+        const bool mine_rows = (qi < prm.N) && (!B64 || qh == (int)(J_now & 1u)) && m_now != -INFINITY;
+        const float f = mine_rows ? prm.scale_log2 * 0.6931471805599453f *
+                                        ex2(__ldg(prm.mu + (long long)bh * prm.Nb + qb) * 1.4426950408889634f - m_now)
+                                  : 0.f;
+        if (!mbar_wait(bar_pv_done + 8 * (w ^ 1), prev & 1u, abort_flag, prm.status)) return false;
+        tc_fence_after();
+#pragma unroll 1
+        for (int cc = 0; cc < D / 2; cc += 16) {
+          uint32_t qv[16];
+          tmem_ld16(tmem_base + lane_addr + COL_Q + cc, qv);
+          tc_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 16; ++e) qv[e] = pack_bf16(bf16lo(qv[e]) * f, bf16hi(qv[e]) * f);
+          tmem_st16(p_tmem + cc, qv);
+        }
+        tc_wait_st();
+        tc_fence_before();
+        mbar_arrive(bar_p_full + 8 * w);
+        return true;
+      };
+      const int n_tiles = REM ? n - prm.n1 : n;                       // (then come the first-order tiles)
+      int j = w;
+      if (REM && !B64) {
+        for (; j < n_own && ok; j += 2) ok = tile(std::integral_constant<int, 0>{}, j);
+        for (; j < n_tiles && ok; j += 2) ok = tile(std::integral_constant<int, 1>{}, j);
+      } else {
+        for (; j < n_tiles && ok; j += 2) ok = tile(std::integral_constant<int, REM ? 2 : 0>{}, j);
+      }
+      if (REM) {
+        for (; j < n && ok; j += 2) ok = first_order_tile(j);
       }
       if (!ok) break;
       if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 7);
@@ -973,6 +1028,9 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         // The row's last S tile (the other group's) has been computed, and with it every S of the row: Q is free.
         // (Its barrier's previous phase completed before the S tile this group has just worked on, or in an earlier row.)
         if (!mbar_wait(bar_s_full + 8 * wl, last & 1u, abort_flag, prm.status)) { ok = false; break; }
+        // (... and a last tile of first order has read it.  Its barrier's previous phase completed before P V of the tile two
+        // before it, which this group has waited for.)
+        if (REM && prm.n1 > 0 && !mbar_wait(bar_p_full + 8 * wl, last & 1u, abort_flag, prm.status)) { ok = false; break; }
         if (r_next < prm.R && !copy_q(r_next, rows_done + 1u)) { ok = false; break; }
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 8);
       }
@@ -1100,7 +1158,7 @@ constexpr int PAIR_WARPS = 8;
 __global__ void __launch_bounds__(PAIR_WARPS * 32)
 pair_lists_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, int Nb, int Nt, int R2,
                   int32_t* __restrict__ tile_cnt, int32_t* __restrict__ tile_beg, uint32_t* __restrict__ tile_desc,
-                  long long cap, int32_t* __restrict__ status) {
+                  long long cap, uint32_t* __restrict__ kept_mask, int32_t* __restrict__ status) {
   __shared__ uint32_t bm[PAIR_WARPS][2][32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int t = blockIdx.x * PAIR_WARPS + w;
@@ -1126,6 +1184,10 @@ pair_lists_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict
   if ((bad || bad_idx) && status) atomicOr(status, SVA_DEV_BAD_INDEX);
   __syncwarp();
   const uint32_t a = bm[w][0][lane], b = bm[w][1][lane];
+  if (kept_mask) {                                            // (an odd Nb: the absent query block computes as the last one)
+    kept_mask[(size_t)t * 64 + lane] = a;
+    kept_mask[(size_t)t * 64 + 32 + lane] = hasB ? b : a;
+  }
   uint32_t u = a | b;
   int incl = __popc(u);
 #pragma unroll
@@ -1313,10 +1375,17 @@ size_t remainder1_bytes(const Dims& m);
 int launch_remainder1(const Dims& m, const sva_problem_t* p, const void* k, const void* v, const float* scores,
                       const int32_t* row_ptr, const int32_t* col_idx, void* buf, const __nv_bfloat16** at_out,
                       const float** mu_out, int32_t* status, cudaStream_t st, bool natural);
-// (order 1 adds the buffers of the first-order term behind those of order 0)
+// (order 1 adds the buffers of the first-order term behind those of order 0; 64-token blocks: then the tile rows' kept-block
+// masks, for which a smaller workspace is accepted too -- the kernel then looks the kept blocks up in the CSR)
+static size_t remainder_base_bytes(const Dims& m, int order) {
+  return ts_layout(m, !(g_debug_ts & 32)).total_rem + (order >= 1 ? remainder1_bytes(m) : 0);
+}
+static size_t kept_mask_bytes(const Dims& m) {
+  return m.block == 64 && m.Nb <= 1024 ? (size_t)m.B * m.H * ((m.Nb + 1) / 2) * 256 : 0;
+}
 size_t attn_ts_remainder_workspace_bytes(const Dims& m, int order) {
   if (!attn_ts_remainder_serves(m)) return 0;
-  return ts_layout(m, !(g_debug_ts & 32)).total_rem + (order >= 1 ? remainder1_bytes(m) : 0);
+  return remainder_base_bytes(m, order) + kept_mask_bytes(m);
 }
 
 // What the one-call entry points need: they read V where it lies, so only the row counters (and the tile lists of
@@ -1380,7 +1449,7 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
   if (rem) {
     if (remainder_order > 1 || !attn_ts_remainder_serves(m_in) || !row_ptr || !v) return SVA_ERR_UNSUPPORTED;
     if (remainder_order == 1 && !block_scores) return SVA_ERR_INVALID_ARG;
-    if (ws_bytes < attn_ts_remainder_workspace_bytes(m_in, remainder_order)) return SVA_ERR_WORKSPACE;
+    if (ws_bytes < remainder_base_bytes(m_in, remainder_order)) return SVA_ERR_WORKSPACE;
   }
   // dense attention does not depend on the block size: 64-token blocks run as 128-token blocks
   Dims m = m_in;
@@ -1477,7 +1546,9 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
   prm.scale_log2 = m.scale * 1.4426950408889634f;
   prm.next_row = reinterpret_cast<int32_t*>(wsb + L.counter_off);
   prm.np = rem ? L.np : 0;
-  prm.rem_mask = (rem && !b64 && m.Nb <= 1024 && !(g_debug_ts & 128)) ? 1 : 0;
+  const size_t mask_off = rem ? remainder_base_bytes(m, remainder_order) : 0;
+  prm.rem_mask = (rem && m.Nb <= 1024 && !(g_debug_ts & 128) && ws_bytes >= mask_off + kept_mask_bytes(m)) ? 1 : 0;
+  prm.kept_mask = b64 && prm.rem_mask ? reinterpret_cast<const uint4*>(wsb + mask_off) : nullptr;
   prm.n1 = (rem && remainder_order == 1) ? (b64 ? 2 : 1) : 0;
   prm.mu = mu_dev;
   prm.log2_block = log2f((float)m.block);
@@ -1491,7 +1562,8 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
     if (row_ptr) {                      // (dense, e4m3 only: the kernel makes up the tile lists itself)
       pair_lists_kernel<<<(L.R2 + PAIR_WARPS - 1) / PAIR_WARPS, PAIR_WARPS * 32, 0, st>>>(
           row_ptr, col_idx, m.Nb, L.Nt, L.R2, reinterpret_cast<int32_t*>(wsb + L.cnt_off),
-          reinterpret_cast<int32_t*>(wsb + L.beg_off), reinterpret_cast<uint32_t*>(wsb + L.desc_off), L.cap, status);
+          reinterpret_cast<int32_t*>(wsb + L.beg_off), reinterpret_cast<uint32_t*>(wsb + L.desc_off), L.cap,
+          const_cast<uint32_t*>(reinterpret_cast<const uint32_t*>(prm.kept_mask)), status);
       if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
     }
     if (rem) return vmn ? launch_ts<true, false, true, false, true>(L.R2, tk, tv, to, tkp, tvp, tat, tq, prm, st)

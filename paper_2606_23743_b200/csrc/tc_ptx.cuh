@@ -180,6 +180,9 @@ __device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t* v) {
 __device__ __forceinline__ void tmem_st1(uint32_t taddr, uint32_t v) {       // one column of this warp's 32 lanes
   asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(v) : "memory");
 }
+__device__ __forceinline__ void tmem_st8_same(uint32_t taddr, uint32_t v) {  // eight columns of this warp's 32 lanes, one value
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %1, %1, %1, %1, %1, %1, %1};" ::"r"(taddr), "r"(v) : "memory");
+}
 __device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {             // one column of this warp's 32 lanes
   uint32_t v;
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(taddr) : "memory");

@@ -295,3 +295,15 @@ def test_wait_that_runs_out_is_reported_and_the_context_survives():
     o, lse, st = U.gpu_attn(w, *data, rp, ci)
     assert st == 0
     U.check_attn_vs_oracle(w, *bits, rp, ci, o, lse, list(range(w.R)))
+
+
+@pytest.mark.parametrize("block,tail", [(128, t) for t in (1, 7, 8, 9, 63, 64, 65, 121, 127)] + [(64, 1), (64, 9), (64, 63)])
+def test_ragged_last_key_block(block, tail):
+    """Keys beyond N are masked from any column on (whole groups of eight columns and single ones)."""
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=1, Wg=3 * block + tail, block=block, k=4)
+    (q, k, v), (qb, kb, vb) = U.host_inputs(w)
+    qd, kd, vd = U.dev(q), U.dev(k), U.dev(v)
+    rp, ci, _ = U.gpu_select(w, qd, kd)
+    o, lse, st = U.gpu_attn(w, qd, kd, vd, rp, ci)
+    assert st == 0
+    U.check_attn_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, list(range(w.R)))

@@ -222,3 +222,39 @@ def test_random_configurations_of_the_remainder(seed):
             if order == 0:
                 vmax = float(np.abs(oracle.bf16_to_f64(vb)).max())
                 assert mag <= 1.01 * vmax, (what, mag, vmax)                             # inside the hull of V
+
+
+@pytest.mark.parametrize("order", [0, 1])
+def test_workspace_without_the_kept_block_masks(order):
+    """64-token blocks: a workspace without room for the masks (256 bytes per tile row at its end) still serves, with the
+    same result; a byte less than that does not."""
+    w = CASES["b64_ragged_tail"]
+    (q, k, v), _ = U.host_inputs(w)
+    qd, kd, vd = U.dev(q), U.dev(k), U.dev(v)
+    rp, ci, scores = U.gpu_select(w, qd, kd, want_scores=order == 1)
+    want, want_lse, st = gpu_remainder(w, qd, kd, vd, rp, ci, order, scores=scores)
+    assert st == 0
+    o = torch.full_like(want, 7.0)
+    lse = torch.full_like(want_lse, 7.0)
+    status = torch.zeros(1, dtype=torch.int32, device="cuda")
+    p = B.make_problem(qd, kd, vd, o, w.N, w.block)
+    small = B.attn_remainder_workspace_bytes(p, order) - w.B * w.H * ((w.Nb + 1) // 2) * 256
+    ws = torch.full((small,), 0xFF, dtype=torch.uint8, device="cuda")
+    B.block_sparse_attn_remainder_fwd(p, qd, kd, vd, rp, ci, o, lse, status, order, ws, scores)
+    assert int(status.item()) == 0
+    assert torch.equal(o, want) and torch.equal(lse, want_lse)
+    with pytest.raises(B.SvaError):
+        B.block_sparse_attn_remainder_fwd(p, qd, kd, vd, rp, ci, o, lse, status, order, ws[:small - 1], scores)
+
+
+@pytest.mark.parametrize("block", [128, 64])
+@pytest.mark.parametrize("nb", [127, 129, 136, 191, 255])
+def test_ragged_tile_of_block_means(nb, block):
+    """The last tile of block means holds 127, 1, 8, 63 or 127 of 128: what does not exist is masked, from any column on."""
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=nb, Wg=block, block=block, k=5)
+    (q, k, v), (qb, kb, vb) = U.host_inputs(w)
+    qd, kd, vd = U.dev(q), U.dev(k), U.dev(v)
+    rp, ci, _ = U.gpu_select(w, qd, kd)
+    o, lse, st = gpu_remainder(w, qd, kd, vd, rp, ci)
+    assert st == 0
+    check_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, [0, 1, nb // 2, nb - 2, nb - 1])
