@@ -1166,49 +1166,52 @@ pair_lists_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict
   const int bh = t / Nt, I2 = t % Nt;
   const int rA = bh * Nb + 2 * I2;
   const bool hasB = 2 * I2 + 1 < Nb;
-  bm[w][0][lane] = 0u;
-  bm[w][1][lane] = 0u;
-  __syncwarp();
   const int begA = __ldg(row_ptr + rA), endA = __ldg(row_ptr + rA + 1);
   const int endB = hasB ? __ldg(row_ptr + rA + 2) : endA;
   const int nnz_bound = __ldg(row_ptr + (R2 / Nt) * Nb);      // row_ptr[R]: the entries the CSR says it has
   const bool bad = begA < 0 || endA < begA || endB < endA || endA - begA > Nb || endB - endA > Nb || endB > nnz_bound;
-  bool bad_idx = false;
-  if (!bad) {
-    for (int e = begA + lane; e < endB; e += 32) {
-      const int J = __ldg(col_idx + e);
-      if (J < 0 || J >= Nb) { bad_idx = true; continue; }
-      atomicOr(&bm[w][e < endA ? 0 : 1][J >> 5], 1u << (J & 31));
+  bool bad_idx = false, too_long = false;
+  const long long start = ((long long)(bad ? 0 : begA) + t + 1) / 2;
+  uint16_t* ent = reinterpret_cast<uint16_t*>(tile_desc) + 2 * start;
+  int total = 0;                                              // members of the union so far
+  for (int base = 0; base < Nb; base += 1024) {               // the bitmaps hold 1024 key blocks at a time
+    bm[w][0][lane] = 0u;
+    bm[w][1][lane] = 0u;
+    __syncwarp();
+    if (!bad) {
+      for (int e = begA + lane; e < endB; e += 32) {
+        const int J = __ldg(col_idx + e);
+        if (J < 0 || J >= Nb) { bad_idx = true; continue; }
+        if (J >= base && J - base < 1024) atomicOr(&bm[w][e < endA ? 0 : 1][(J - base) >> 5], 1u << (J & 31));
+      }
     }
-  }
-  if ((bad || bad_idx) && status) atomicOr(status, SVA_DEV_BAD_INDEX);
-  __syncwarp();
-  const uint32_t a = bm[w][0][lane], b = bm[w][1][lane];
-  if (kept_mask) {                                            // (an odd Nb: the absent query block computes as the last one)
-    kept_mask[(size_t)t * 64 + lane] = a;
-    kept_mask[(size_t)t * 64 + 32 + lane] = hasB ? b : a;
-  }
-  uint32_t u = a | b;
-  int incl = __popc(u);
+    __syncwarp();
+    const uint32_t a = bm[w][0][lane], b = bm[w][1][lane];
+    if (kept_mask) {                                          // (an odd Nb: the absent query block computes as the last one)
+      kept_mask[(size_t)t * 64 + lane] = a;
+      kept_mask[(size_t)t * 64 + 32 + lane] = hasB ? b : a;
+    }
+    uint32_t u = a | b;
+    int incl = __popc(u);
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const int x = __shfl_up_sync(0xffffffffu, incl, o);
-    if (lane >= o) incl += x;
-  }
-  const int total = __shfl_sync(0xffffffffu, incl, 31);
-  long long start = ((long long)(bad ? 0 : begA) + t + 1) / 2;
-  int ntile = (total + 1) / 2;
-  if (start + ntile > cap) { ntile = 0; if (lane == 0 && status) atomicOr(status, SVA_DEV_BAD_INDEX); }
-  if (ntile > 0) {
-    uint16_t* ent = reinterpret_cast<uint16_t*>(tile_desc) + 2 * start;
-    int p = incl - __popc(u);
-    while (u) {
-      const int bit = __ffs(u) - 1;
-      u &= u - 1;
-      ent[p++] = (uint16_t)((lane * 32 + bit) | (((a >> bit) & 1u) << 14) | (((b >> bit) & 1u) << 15));
+    for (int o = 1; o < 32; o <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += x;
     }
-    if (lane == 0 && (total & 1)) ent[total] = 0;          // odd union: the last tile's second half is nobody's
+    int p = total + incl - __popc(u);
+    total += __shfl_sync(0xffffffffu, incl, 31);
+    too_long = too_long || start + (total + 1) / 2 > cap;
+    if (!too_long) {
+      while (u) {
+        const int bit = __ffs(u) - 1;
+        u &= u - 1;
+        ent[p++] = (uint16_t)((base + lane * 32 + bit) | (((a >> bit) & 1u) << 14) | (((b >> bit) & 1u) << 15));
+      }
+    }
   }
+  if ((bad || bad_idx || too_long) && status) atomicOr(status, SVA_DEV_BAD_INDEX);
+  const int ntile = too_long ? 0 : (total + 1) / 2;
+  if (lane == 0 && ntile > 0 && (total & 1)) ent[total] = 0;   // odd union: the last tile's second half is nobody's
   if (lane == 0) {
     tile_cnt[t] = ntile;
     tile_beg[t] = (int32_t)start;

@@ -307,3 +307,21 @@ def test_ragged_last_key_block(block, tail):
     o, lse, st = U.gpu_attn(w, qd, kd, vd, rp, ci)
     assert st == 0
     U.check_attn_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, list(range(w.R)))
+
+
+def test_b64_more_than_1024_key_blocks():
+    """64-token blocks, 1 031 of them (a CSR of the caller's own: the routing call stops at 1 024): the tile lists are put
+    together 1 024 key blocks at a time, and entries on both sides of that line keep their order."""
+    nb = 1031
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=nb, Wg=64, block=64, k=6)
+    (q, k, v), (qb, kb, vb) = U.host_inputs(w)
+    rng = np.random.default_rng(5)
+    lists = [np.sort(rng.choice(nb, rng.integers(0, 9), replace=False)) for _ in range(nb)]
+    lists[0], lists[1], lists[2] = np.array([1023, 1024, 1030]), np.array([0, 1024]), np.array([], dtype=int)
+    rp = torch.tensor(np.concatenate([[0], np.cumsum([len(x) for x in lists])]), dtype=torch.int32).cuda()
+    ci = torch.tensor(np.concatenate(lists), dtype=torch.int32).cuda()
+    o, lse, st = U.gpu_attn(w, U.dev(q), U.dev(k), U.dev(v), rp, ci)
+    assert st == 0
+    rows = [r for r in [0, 1, 3] + list(range(4, nb, 41)) + [nb - 1] if len(lists[r])]
+    U.check_attn_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, rows)
+    assert (o[0, 0, 128:192] == 0).all()                       # the empty list's rows
