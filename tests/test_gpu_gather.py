@@ -86,3 +86,28 @@ def test_attention_over_a_pruned_token_subset():
     torch.cuda.synchronize()
     kept = torch.zeros(w_full.N, dtype=torch.bool); kept[idx[0].long()] = True
     assert torch.equal(full[0][:, kept.cuda()], o[0, :, :M]) and (full[0][:, (~kept).cuda()] == 7.0).all()
+
+
+@pytest.mark.parametrize("H,d,dtype", [(1, 128, torch.bfloat16), (4, 64, torch.bfloat16), (5, 16, torch.uint8), (7, 24, torch.bfloat16),
+                                       (2, 2080, torch.bfloat16), (9, 128, torch.float32)])
+@pytest.mark.parametrize("tokens_first", [False, True])
+def test_row_sizes_and_head_counts(H, d, dtype, tokens_first):
+    """Rows of 1, 3, 8, 16, 32 and 260 vectors, head counts around the four a thread moves, [B,H,N,d] and [B,N,H,d]."""
+    g = torch.Generator().manual_seed(d + H)
+    Bq, N, M = 2, 203, 101
+    shape = (Bq, N, H, d) if tokens_first else (Bq, H, N, d)
+    x = torch.randint(0, 200, shape, generator=g).to(dtype).cuda()
+    x = x.transpose(1, 2) if tokens_first else x
+    idx = torch.stack([torch.randperm(N, generator=g)[:M] for _ in range(Bq)]).to(torch.int32).cuda()
+    out = torch.zeros(Bq, H, M, d, dtype=dtype, device="cuda")
+    st = torch.zeros(1, dtype=torch.int32, device="cuda")
+    B.gather_tokens(x, idx, out, st)
+    want = torch.stack([x[b][:, idx[b].long()] for b in range(Bq)])
+    assert torch.equal(out, want)
+    back = torch.zeros(shape, dtype=dtype, device="cuda")
+    back = back.transpose(1, 2) if tokens_first else back
+    B.scatter_tokens(out, idx, back, st)
+    ref = torch.zeros_like(back)
+    for b in range(Bq):
+        ref[b][:, idx[b].long()] = want[b]
+    assert torch.equal(back, ref) and int(st.item()) == 0
