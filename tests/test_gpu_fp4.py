@@ -115,3 +115,20 @@ def test_fp4_full_size_and_distance_to_bf16_attention():
     a, b = o[:, :, :w.N].float(), o16[:, :, :w.N].float()
     print(f"4-bit vs bf16 attention on the same CSR: rel_l2 {float(torch.linalg.vector_norm(a - b) / torch.linalg.vector_norm(b)):.3f}")
     assert torch.isfinite(a).all()
+
+
+@pytest.mark.parametrize("exponent", [-120, -92, -89, -60, -20, 0, 40, 100])     # (finite: |x| < 8 * 2^100)
+def test_quantiser_bytes_at_extreme_magnitudes(exponent):
+    """Tensors scaled by a power of two, with tokens far below the largest: scales from the short division, and from true
+    divisions where it would not be exact (tiny blocks, tensor scales outside 2^-60 .. 2^60), are the oracle's bytes."""
+    w = shrink(WORKLOADS["medium"], H=2, T=1, Hg=4, Wg=50)                           # N = 200
+    (q, k, v), _ = U.host_inputs(w)
+    span = torch.exp2(-(torch.arange(w.N, dtype=torch.float32) % 37))[None, None, :, None]
+    q = (q[:, :, :w.N].float() * span * 2.0 ** exponent).to(torch.bfloat16)
+    k = (k[:, :, :w.N].float() * span.flip(2) * 2.0 ** exponent).to(torch.bfloat16)
+    q4, k4, qsf, ksf, qg, kg = gpu_quantize4(w, U.dev(q), U.dev(k))
+    for x, g4, gsf, gg in ((q, q4, qsf, qg), (k, k4, ksf, kg)):
+        codes, sfs, g = nvfp4.quantize(bf16_bits(x), w.N)
+        np.testing.assert_array_equal(gg.cpu().numpy().reshape(w.B, w.H), g)
+        np.testing.assert_array_equal(untile_sf(gsf, w.Nb).reshape(w.B, w.H, w.Nb * 128, 8)[:, :, :w.N], sfs[:, :, :w.N])
+        np.testing.assert_array_equal(g4.cpu().numpy().reshape(w.B, w.H, w.Nb * 128, 64)[:, :, :w.N], codes[:, :, :w.N])
