@@ -318,6 +318,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_base_p;
+  const int zero = grid_dep_wait();            // (the set-up above overlaps the end of the kernel before)
   constexpr uint32_t IDESC = instr_desc(128, 128, 1, false);   // bf16 x bf16 -> fp32, A and B K-major
   constexpr uint32_t IDESC_QK = F8 ? instr_desc(128, 128, 0, false) : IDESC;   // e4m3 x e4m3 for S in the e4m3 variant
   constexpr int KTILE = F8 ? TILE / 2 : TILE;                  // bytes of one K tile
@@ -346,7 +347,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         int s = 0;
         uint32_t ph = 0;
         bool ok = true;
-        const int nnz_bound = (!B64 && prm.row_ptr) ? __ldg(prm.row_ptr + prm.R) : 0;
+        const int nnz_bound = (!B64 && prm.row_ptr) ? __ldg(prm.row_ptr + prm.R + zero) : 0;
         for (uint32_t i = 0; ok; ++i) {
           // ---- row scheduling: draw the next row with a non-empty list and publish it
           const uint32_t slot = i % QD;
@@ -626,7 +627,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const uint32_t p_tmem = tmem_base + lane_addr + COL_P;
     const uint32_t q_tmem = tmem_base + lane_addr + COL_Q + (F8 ? 16 : 32) * w;
     const int tail_keys = prm.N - (prm.Nb - 1) * KB;         // valid keys of the last key block
-    const int nnz_total = (REM && prm.row_ptr) ? __ldg(prm.row_ptr + (prm.R / prm.Nt) * prm.Nb) : 0;   // row_ptr[R of the CSR]
+    const int nnz_total = (REM && prm.row_ptr) ? __ldg(prm.row_ptr + (prm.R / prm.Nt) * prm.Nb + zero) : 0;   // row_ptr[R of the CSR]
     const int qh = row >> 6;                                 // 64-token blocks: which query block of the tile I am in
     float c = prm.scale_log2;      // e4m3 variant: times the scales of the query block and of the key block, per block
     float c1 = prm.scale_log2;     // e4m3 with 64-token blocks: the same for the tile's second key block
@@ -1108,6 +1109,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 __global__ void __launch_bounds__(256)
 transpose_v_kernel(const __nv_bfloat16* __restrict__ v, Strides sv, __nv_bfloat16* __restrict__ vt, int H, int N,
                    int Nb, int d, int kb, int32_t* __restrict__ row_counter) {
+  const int zero = grid_dep_wait();
   // d = 64: the tile still has 128 d-rows; the CTAs of the upper half (d0 >= d) write zeros
   // the attention kernel that follows draws its rows from this counter
   if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) {
@@ -1115,7 +1117,7 @@ transpose_v_kernel(const __nv_bfloat16* __restrict__ v, Strides sv, __nv_bfloat1
     row_counter[1] = 0;     // CTAs that have finished drawing
   }
   __shared__ __nv_bfloat16 tile[64][66];            // [d][key], padded
-  const int n0 = blockIdx.x * 64, d0 = blockIdx.y * 64, bh = blockIdx.z;
+  const int n0 = blockIdx.x * 64, d0 = blockIdx.y * 64, bh = blockIdx.z + zero;
   const int b = bh / H, h = bh % H;
   const __nv_bfloat16* src = v + (long long)b * sv.b + (long long)h * sv.h;
   {
@@ -1145,6 +1147,13 @@ transpose_v_kernel(const __nv_bfloat16* __restrict__ v, Strides sv, __nv_bfloat1
   }
 }
 
+// The row counters of an attention call that no other kernel prepares.  (A kernel and not a memset: between kernels the next
+// one's launch overlaps.)
+__global__ void zero_counters_kernel(int32_t* __restrict__ row_counter) {
+  grid_dep_launch();
+  if (threadIdx.x < 2) row_counter[threadIdx.x + grid_dep_wait()] = 0;
+}
+
 // ------------------------------------------------------------------ 64-token blocks: tile lists
 // The MMA tile is 128 x 128, so with 64-token blocks one tile row is two adjacent query blocks (A, B)
 // and one tile two key blocks.  Per tile row this kernel merges the two CSR rows into the ascending
@@ -1158,17 +1167,20 @@ constexpr int PAIR_WARPS = 8;
 __global__ void __launch_bounds__(PAIR_WARPS * 32)
 pair_lists_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx, int Nb, int Nt, int R2,
                   int32_t* __restrict__ tile_cnt, int32_t* __restrict__ tile_beg, uint32_t* __restrict__ tile_desc,
-                  long long cap, uint32_t* __restrict__ kept_mask, int32_t* __restrict__ status) {
+                  long long cap, uint32_t* __restrict__ kept_mask, int32_t* __restrict__ row_counter,
+                  int32_t* __restrict__ status) {
   __shared__ uint32_t bm[PAIR_WARPS][2][32];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t = blockIdx.x * PAIR_WARPS + w;
+  grid_dep_launch();
+  const int zero = grid_dep_wait(), t = blockIdx.x * PAIR_WARPS + w + zero;
+  if (t == 0 && lane < 2) row_counter[lane] = 0;              // the attention kernel that follows draws its rows from it
   if (t >= R2) return;
   const int bh = t / Nt, I2 = t % Nt;
   const int rA = bh * Nb + 2 * I2;
   const bool hasB = 2 * I2 + 1 < Nb;
   const int begA = __ldg(row_ptr + rA), endA = __ldg(row_ptr + rA + 1);
   const int endB = hasB ? __ldg(row_ptr + rA + 2) : endA;
-  const int nnz_bound = __ldg(row_ptr + (R2 / Nt) * Nb);      // row_ptr[R]: the entries the CSR says it has
+  const int nnz_bound = __ldg(row_ptr + (R2 / Nt) * Nb + zero);      // row_ptr[R]: the entries the CSR says it has
   const bool bad = begA < 0 || endA < begA || endB < endA || endA - begA > Nb || endB - endA > Nb || endB > nnz_bound;
   bool bad_idx = false, too_long = false;
   const long long start = ((long long)(bad ? 0 : begA) + t + 1) / 2;
@@ -1219,41 +1231,65 @@ pair_lists_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict
 }
 
 // ------------------------------------------------------------------ remainder: block means of K and V
-// One CTA per (block J, head, tensor): the mean over the existing tokens of the block, fp32 accumulation in a
-// fixed order, rounded to bf16.  K means go to kp [B*H][Nbp][128] (rows >= Nb stay zero: the launcher clears the
-// buffer), V means transposed to vtp [B*H][np][128 d][128 blocks], the layout of a V^T tile.
+// The mean over the existing tokens of a block, fp32 accumulation in a fixed order, rounded to bf16.  K means go to kp
+// [B*H][Nbp][128] (rows >= Nb zero), V means likewise (v_rows) or transposed to vtp [B*H][np][128 d][128 blocks], the
+// layout of a V^T tile.  HBM-bound; a CTA takes `run` consecutive blocks of one head of K or V, the next loads in flight while
+// it reduces (as the routing's pooling does; 24 heads x 32 760 tokens in 64-token blocks: 79 -> 72 us).
 __global__ void __launch_bounds__(256)
 pool_kv_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, Strides sk, Strides sv,
-               int H, int N, int block, int Nb, int Nbp, __nv_bfloat16* __restrict__ kp,
-               __nv_bfloat16* __restrict__ vtp, int v_rows) {
+               int H, int N, int block, int Nb, int Nbp, int run, __nv_bfloat16* __restrict__ kp,
+               __nv_bfloat16* __restrict__ vtp, int v_rows, int32_t* __restrict__ row_counter) {
   __shared__ float part[16][ts::D + 1];
-  const int J = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
+  const int zero = grid_dep_wait(), bh = blockIdx.y + zero, which = blockIdx.z;
+  // the attention kernel that follows draws its rows from this counter
+  if (blockIdx.x == 0 && blockIdx.y == 0 && which == 0 && threadIdx.x < 2) row_counter[threadIdx.x] = 0;
   const int b = bh / H, h = bh % H;
   const Strides s = which ? sv : sk;
   const __nv_bfloat16* base = (which ? v : k) + (long long)b * s.b + (long long)h * s.h;
-  const int lo = J * block, cnt = min(block, N - lo);
+  const int J0 = blockIdx.x * run, J1 = min(J0 + run, Nbp);
   const int vec = threadIdx.x & 15, grp = threadIdx.x >> 4;          // 16 vectors of 8 elements per row, 16 rows at a time
+  const int per_block = block / 64, steps = (J1 - J0) * per_block;   // 64 rows per step
+  uint4 u[4];
+  auto load = [&](int step) {
+    const int lo = (J0 + step / per_block) * block + (step % per_block) * 64;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int t = lo + 16 * j + grp;
+      u[j] = make_uint4(0u, 0u, 0u, 0u);
+      if (step < steps && t < N) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)t * s.n) + vec);
+    }
+  };
   float acc[8];
 #pragma unroll
   for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-  for (int t = grp; t < cnt; t += 16) {
-    const uint4 u = __ldg(reinterpret_cast<const uint4*>(base + (long long)(lo + t) * s.n) + vec);
-    const uint32_t wd[4] = {u.x, u.y, u.z, u.w};
+  load(0);
+  for (int step = 0; step < steps; ++step) {
+    uint4 c[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) { acc[2 * e] += bf16lo(wd[e]); acc[2 * e + 1] += bf16hi(wd[e]); }
-  }
+    for (int j = 0; j < 4; ++j) c[j] = u[j];
+    load(step + 1);
 #pragma unroll
-  for (int e = 0; e < 8; ++e) part[grp][vec * 8 + e] = acc[e];
-  __syncthreads();
-  if (threadIdx.x < ts::D) {
-    float sum = 0.f;
+    for (int j = 0; j < 4; ++j) {
+      const uint32_t wd[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
 #pragma unroll
-    for (int g = 0; g < 16; ++g) sum += part[g][threadIdx.x];
-    const __nv_bfloat16 mean = __float2bfloat16_rn(sum / (float)cnt);
-    if (which == 0 || v_rows)                                 // (v_rows: the means of V laid out like those of K)
-      (which ? vtp : kp)[((long long)bh * Nbp + J) * ts::D + threadIdx.x] = mean;
-    else
-      vtp[(((long long)bh * (Nbp >> 7) + (J >> 7)) * ts::D + threadIdx.x) * BS + (J & 127)] = mean;
+      for (int e = 0; e < 4; ++e) { acc[2 * e] += bf16lo(wd[e]); acc[2 * e + 1] += bf16hi(wd[e]); }
+    }
+    if ((step + 1) % per_block != 0) continue;
+    const int J = J0 + step / per_block;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) { part[grp][vec * 8 + e] = acc[e]; acc[e] = 0.f; }
+    __syncthreads();
+    if (threadIdx.x < ts::D) {
+      float sum = 0.f;
+#pragma unroll
+      for (int g = 0; g < 16; ++g) sum += part[g][threadIdx.x];
+      const __nv_bfloat16 mean = J < Nb ? __float2bfloat16_rn(sum / (float)min(block, N - J * block)) : __float2bfloat16_rn(0.f);
+      if (which == 0 || v_rows)                                 // (v_rows: the means of V laid out like those of K)
+        (which ? vtp : kp)[((long long)bh * Nbp + J) * ts::D + threadIdx.x] = mean;
+      else
+        vtp[(((long long)bh * (Nbp >> 7) + (J >> 7)) * ts::D + threadIdx.x) * BS + (J & 127)] = mean;
+    }
+    __syncthreads();
   }
 }
 
@@ -1330,8 +1366,7 @@ static int launch_ts(int rows, const CUtensorMap& tk, const CUtensorMap& tv, con
     sms = g_ts_sms[dev];
   }
   const int grid = rows < sms ? rows : sms;        // persistent: one CTA per SM, rows drawn from a counter
-  kern<<<grid, ts::THREADS, ts::SMEM_BYTES, st>>>(tk, tv, to, tkp, tvp, tat, tq, prm);
-  return cudaGetLastError() == cudaSuccess ? SVA_OK : SVA_ERR_CUDA;
+  return launch_dep(kern, grid, ts::THREADS, ts::SMEM_BYTES, st, tk, tv, to, tkp, tvp, tat, tq, prm);
 }
 
 // Workspace layout: transposed V tiles | row counter (256 bytes) | 64-token blocks only: tile_cnt[R2],
@@ -1434,9 +1469,8 @@ int launch_prepare_v_ts(const Dims& m, const sva_problem_t* p, const void* v, vo
   const TsLayout L = ts_layout(m);
   const Strides sv = make_strides(p->v_stride);
   dim3 tg((m.Nb * m.block + 63) / 64, ts::D / 64, m.B * m.H);    // every key slot of every tile, also those beyond N (zeros)
-  transpose_v_kernel<<<tg, 256, 0, st>>>((const __nv_bfloat16*)v, sv, (__nv_bfloat16*)ws, m.H, m.N, m.Nb, m.d, m.block,
-                                         reinterpret_cast<int32_t*>(static_cast<uint8_t*>(ws) + L.counter_off));
-  return cudaGetLastError() == cudaSuccess ? SVA_OK : SVA_ERR_CUDA;
+  return launch_dep(transpose_v_kernel, tg, 256, 0, st, (const __nv_bfloat16*)v, sv, (__nv_bfloat16*)ws, m.H, m.N, m.Nb, m.d, m.block,
+                    reinterpret_cast<int32_t*>(static_cast<uint8_t*>(ws) + L.counter_off));
 }
 
 // v == nullptr: the workspace has been prepared by launch_prepare_v_ts (once per attention call).
@@ -1478,11 +1512,15 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
   if ((rc = make_map_ts(&tk, k, m.d, m.N, m.H, m.B, (cuuint64_t)sk.n * eb, (cuuint64_t)sk.h * eb, (cuuint64_t)sk.b * eb,
                         m.block, eb)) != SVA_OK)
     return rc;
-  // transposed V: per (b,h) a [Nb*128 rows][block keys] matrix, key block J = rows J*128 .. J*128+127
-  const cuuint64_t vrows = (cuuint64_t)m.Nb * ts::D;
-  if ((rc = make_map_ts(&tv, ws, m.block, vrows, m.H, m.B, (cuuint64_t)m.block * 2, vrows * m.block * 2,
-                        vrows * m.block * 2 * m.H, BS)) != SVA_OK)
-    return rc;
+  if (vmn) {
+    const Strides sv = make_strides(p->v_stride);
+    rc = make_map_ts(&tv, v, m.d, m.N, m.H, m.B, (cuuint64_t)sv.n * 2, (cuuint64_t)sv.h * 2, (cuuint64_t)sv.b * 2, m.block);
+  } else {
+    // transposed V: per (b,h) a [Nb*128 rows][block keys] matrix, key block J = rows J*128 .. J*128+127
+    const cuuint64_t vrows = (cuuint64_t)m.Nb * ts::D;
+    rc = make_map_ts(&tv, ws, m.block, vrows, m.H, m.B, (cuuint64_t)m.block * 2, vrows * m.block * 2, vrows * m.block * 2 * m.H, BS);
+  }
+  if (rc != SVA_OK) return rc;
   tkp = tk; tvp = tv; tat = tv;  // (placeholders when there is no remainder: the kernel never touches them)
   // Q as 128-row tiles, like K (128-token blocks: a row's Q reaches the kernel by TMA; otherwise unused)
   CUtensorMap tq = tk;
@@ -1505,11 +1543,11 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
     // block means of K ([Nbp rows][128], rows >= Nb zero) and of V (transposed tiles), then their maps
     __nv_bfloat16* kp = reinterpret_cast<__nv_bfloat16*>(wsb + L.kp_off);
     __nv_bfloat16* vtp = reinterpret_cast<__nv_bfloat16*>(wsb + L.vtp_off);
-    if (cudaMemsetAsync(kp, 0, 2 * L.pooled_bytes, st) != cudaSuccess) return SVA_ERR_CUDA;
-    pool_kv_kernel<<<dim3(m.Nb, m.B * m.H, 2), 256, 0, st>>>((const __nv_bfloat16*)k, (const __nv_bfloat16*)v, sk,
-                                                            make_strides(p->v_stride), m.H, m.N, m.block, m.Nb, L.Nbp, kp, vtp,
-                                                            vmn ? 1 : 0);
-    if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
+    const int run = 2LL * m.R >= 4 * 148 * 4 ? 4 : 1;              // (a block per CTA while there are few)
+    if ((rc = launch_dep(pool_kv_kernel, dim3((L.Nbp + run - 1) / run, m.B * m.H, 2), 256, 0, st, (const __nv_bfloat16*)k,
+                         (const __nv_bfloat16*)v, sk, make_strides(p->v_stride), m.H, m.N, m.block, m.Nb, L.Nbp, run, kp, vtp, vmn ? 1 : 0,
+                         reinterpret_cast<int32_t*>(wsb + L.counter_off))) != SVA_OK)
+      return rc;
     const cuuint64_t prow = (cuuint64_t)L.Nbp;
     if ((rc = make_map_ts(&tkp, kp, ts::D, prow, m.H, m.B, (cuuint64_t)ts::D * 2, prow * ts::D * 2,
                           prow * ts::D * 2 * m.H, BS)) != SVA_OK)
@@ -1519,19 +1557,16 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
       return rc;
   }
   if (vmn) {
-    const Strides sv = make_strides(p->v_stride);
-    if ((rc = make_map_ts(&tv, v, m.d, m.N, m.H, m.B, (cuuint64_t)sv.n * 2, (cuuint64_t)sv.h * 2, (cuuint64_t)sv.b * 2,
-                          m.block)) != SVA_OK)
+    // (block means and tile lists are made by kernels that also put the row counters to 0)
+    if (!rem && !(b64 && row_ptr) && (rc = launch_dep(zero_counters_kernel, 1, 32, 0, st, reinterpret_cast<int32_t*>(wsb + L.counter_off))) != SVA_OK)
       return rc;
-    if (!rem) tvp = tv;
-    if (cudaMemsetAsync(wsb + L.counter_off, 0, 256, st) != cudaSuccess) return SVA_ERR_CUDA;
   } else if (v) {
     // (the transposed copy is laid out for the block size of this launch)
     const Strides sv = make_strides(p->v_stride);
     dim3 tg((m.Nb * m.block + 63) / 64, ts::D / 64, m.B * m.H);    // every key slot of every tile, also those beyond N (zeros)
-    transpose_v_kernel<<<tg, 256, 0, st>>>((const __nv_bfloat16*)v, sv, (__nv_bfloat16*)ws, m.H, m.N, m.Nb, m.d, m.block,
-                                           reinterpret_cast<int32_t*>(wsb + L.counter_off));
-    if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
+    if ((rc = launch_dep(transpose_v_kernel, tg, 256, 0, st, (const __nv_bfloat16*)v, sv, (__nv_bfloat16*)ws, m.H, m.N, m.Nb, m.d, m.block,
+                         reinterpret_cast<int32_t*>(wsb + L.counter_off))) != SVA_OK)
+      return rc;
   } else if (m.block != m_in.block) {
     return SVA_ERR_UNSUPPORTED;     // a workspace prepared for 64-token blocks cannot serve the dense path
   }
@@ -1563,11 +1598,11 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
   prm.debug = g_debug_ts;
   if (b64) {
     if (row_ptr) {                      // (dense, e4m3 only: the kernel makes up the tile lists itself)
-      pair_lists_kernel<<<(L.R2 + PAIR_WARPS - 1) / PAIR_WARPS, PAIR_WARPS * 32, 0, st>>>(
-          row_ptr, col_idx, m.Nb, L.Nt, L.R2, reinterpret_cast<int32_t*>(wsb + L.cnt_off),
-          reinterpret_cast<int32_t*>(wsb + L.beg_off), reinterpret_cast<uint32_t*>(wsb + L.desc_off), L.cap,
-          const_cast<uint32_t*>(reinterpret_cast<const uint32_t*>(prm.kept_mask)), status);
-      if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
+      if ((rc = launch_dep(pair_lists_kernel, (L.R2 + PAIR_WARPS - 1) / PAIR_WARPS, PAIR_WARPS * 32, 0, st, row_ptr, col_idx, m.Nb, L.Nt,
+                           L.R2, reinterpret_cast<int32_t*>(wsb + L.cnt_off), reinterpret_cast<int32_t*>(wsb + L.beg_off),
+                           reinterpret_cast<uint32_t*>(wsb + L.desc_off), L.cap,
+                           const_cast<uint32_t*>(reinterpret_cast<const uint32_t*>(prm.kept_mask)), prm.next_row, status)) != SVA_OK)
+        return rc;
     }
     if (rem) return vmn ? launch_ts<true, false, true, false, true>(L.R2, tk, tv, to, tkp, tvp, tat, tq, prm, st)
                         : launch_ts<true, false, true>(L.R2, tk, tv, to, tkp, tvp, tat, tq, prm, st);
@@ -1608,7 +1643,7 @@ int launch_attn_ts_fp4(const Dims& m, const sva_problem_t* p, const void* q4, co
   if ((rc = make_map_ts(&tv, v, m.d, m.N, m.H, m.B, (cuuint64_t)sv.n * 2, (cuuint64_t)sv.h * 2, (cuuint64_t)sv.b * 2,
                         BS)) != SVA_OK)
     return rc;
-  if (cudaMemsetAsync(wsb + L.counter_off, 0, 256, st) != cudaSuccess) return SVA_ERR_CUDA;
+  if ((rc = launch_dep(zero_counters_kernel, 1, 32, 0, st, reinterpret_cast<int32_t*>(wsb + L.counter_off))) != SVA_OK) return rc;
   TsParams prm = {};
   prm.q = nullptr; prm.sq = Strides{0, 0, 0};
   prm.q_scale = q_g; prm.k_scale = k_g;

@@ -20,7 +20,7 @@ token_move_kernel(const uint8_t* __restrict__ src, Strides ss, uint8_t* __restri
                   int32_t* __restrict__ status) {
   const int vpr = row_bytes / 16;                       // 16-byte vectors per row
   const int groups = (H + MOVE_HEADS - 1) / MOVE_HEADS;
-  const int b = blockIdx.y, h0 = (int)(blockIdx.x % groups) * MOVE_HEADS;
+  const int b = blockIdx.y + grid_dep_wait(), h0 = (int)(blockIdx.x % groups) * MOVE_HEADS;
   const int r = threadIdx.x / vpr, m = (int)(blockIdx.x / groups) * tokens_per_cta + r;
   if (r >= tokens_per_cta || m >= M) return;
   const int t = __ldg(idx + (long long)b * M + m);
@@ -51,13 +51,8 @@ int launch_token_move(bool scatter, const void* src, const int64_t ss[3], void* 
   const long long tiles = (long long)((M + tokens_per_cta - 1) / tokens_per_cta) * ((H + MOVE_HEADS - 1) / MOVE_HEADS);
   if (tiles > 0x7fffffffLL) return SVA_ERR_UNSUPPORTED;
   const dim3 grid((unsigned)tiles, (unsigned)B);
-  if (scatter)
-    token_move_kernel<true><<<grid, 256, 0, st>>>((const uint8_t*)src, make_strides(ss), (uint8_t*)dst, make_strides(sd),
-                                                  idx, H, M, n_full, row_bytes, elem_bytes, tokens_per_cta, status);
-  else
-    token_move_kernel<false><<<grid, 256, 0, st>>>((const uint8_t*)src, make_strides(ss), (uint8_t*)dst, make_strides(sd),
-                                                   idx, H, M, n_full, row_bytes, elem_bytes, tokens_per_cta, status);
-  return cudaGetLastError() == cudaSuccess ? SVA_OK : SVA_ERR_CUDA;
+  return launch_dep(scatter ? token_move_kernel<true> : token_move_kernel<false>, grid, 256, 0, st, (const uint8_t*)src,
+                    make_strides(ss), (uint8_t*)dst, make_strides(sd), idx, H, M, n_full, row_bytes, elem_bytes, tokens_per_cta, status);
 }
 
 }  // namespace sva

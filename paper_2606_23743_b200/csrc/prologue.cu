@@ -45,7 +45,7 @@ prologue_kernel(const PrologueParams prm) {
   __shared__ float s_scale, s_rcp;
   __shared__ int s_fast;
 
-  const int I = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
+  const int zero = grid_dep_wait(), I = blockIdx.x, bh = blockIdx.y + zero, which = blockIdx.z;
   const int b = bh / prm.H, h = bh % prm.H;
   const Strides s = which ? prm.sk : prm.sq;
   const long long head_off = (long long)b * s.b + (long long)h * s.h;
@@ -56,12 +56,12 @@ prologue_kernel(const PrologueParams prm) {
   uint8_t* __restrict__ dst = (which ? prm.ko : prm.qo) + head_off * 2;
   const float* __restrict__ cosn = prm.cosn;
   const float* __restrict__ sinn = prm.sinn;
-  const int lo = I * prm.block, cnt = min(prm.block, prm.N - lo);
+  const int lo = I * prm.block + zero, cnt = min(prm.block, prm.N - lo);
   const int vec = threadIdx.x % VPR, grp = threadIdx.x / VPR;
 
   float g[8];
   {
-    const float4* gp = reinterpret_cast<const float4*>((which ? prm.gk : prm.gq) + vec * 8);
+    const float4* gp = reinterpret_cast<const float4*>((which ? prm.gk : prm.gq) + vec * 8 + zero);
     const float4 g0 = __ldg(gp), g1 = __ldg(gp + 1);
     g[0] = g0.x; g[1] = g0.y; g[2] = g0.z; g[3] = g0.w; g[4] = g1.x; g[5] = g1.y; g[6] = g1.z; g[7] = g1.w;
   }
@@ -185,14 +185,8 @@ int launch_prologue(const Dims& m, const sva_problem_t* p, const void* q, const 
   prm.H = m.H; prm.N = m.N; prm.block = m.block; prm.Nb = m.Nb;
   dim3 g(m.Nb, m.B * m.H, 2);
   const bool codes = q8 != nullptr;
-  if (m.d == 128) {
-    if (codes) prologue_kernel<128, 128, true><<<g, PT, 0, st>>>(prm);
-    else prologue_kernel<128, 128, false><<<g, PT, 0, st>>>(prm);
-  } else {
-    if (codes) prologue_kernel<64, 128, true><<<g, PT, 0, st>>>(prm);
-    else prologue_kernel<64, 128, false><<<g, PT, 0, st>>>(prm);
-  }
-  return cudaGetLastError() == cudaSuccess ? SVA_OK : SVA_ERR_CUDA;
+  if (m.d == 128) return launch_dep(codes ? prologue_kernel<128, 128, true> : prologue_kernel<128, 128, false>, g, PT, 0, st, prm);
+  return launch_dep(codes ? prologue_kernel<64, 128, true> : prologue_kernel<64, 128, false>, g, PT, 0, st, prm);
 }
 
 }  // namespace sva

@@ -18,7 +18,7 @@ __global__ void __launch_bounds__(QT)
 block_sum_kernel(const uint8_t* __restrict__ k, Strides sk, float* __restrict__ part, int H, int N, int block, int Nb) {
   constexpr int VPR = D / 8, GROUPS = QT / VPR;
   __shared__ float acc[GROUPS][D];
-  const int I = blockIdx.x, bh = blockIdx.y;
+  const int I = blockIdx.x, bh = blockIdx.y + grid_dep_wait();
   const uint8_t* src = k + ((long long)(bh / H) * sk.b + (long long)(bh % H) * sk.h) * 2;
   const int lo = I * block, cnt = min(block, N - lo);
   const int vec = threadIdx.x % VPR, grp = threadIdx.x / VPR;
@@ -41,7 +41,8 @@ block_sum_kernel(const uint8_t* __restrict__ k, Strides sk, float* __restrict__ 
 
 // mean[bh*D + c] = (sum over blocks, in index order) / N                        (grid BH, D threads)
 __global__ void mean_key_kernel(const float* __restrict__ part, float* __restrict__ mean, int Nb, int D, int N) {
-  const int bh = blockIdx.x, c = threadIdx.x;
+  grid_dep_launch();
+  const int bh = blockIdx.x + grid_dep_wait(), c = threadIdx.x;
   const float* src = part + (long long)bh * Nb * D + c;
   float t = 0.f;
   int I = 0;
@@ -70,7 +71,7 @@ quantize_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, St
   __shared__ float s_scale, s_rcp;
   __shared__ int s_fast;
 
-  const int I = blockIdx.x, bh = blockIdx.y, which = blockIdx.z;
+  const int I = blockIdx.x, bh = blockIdx.y + grid_dep_wait(), which = blockIdx.z;
   const int b = bh / H, h = bh % H;
   const Strides s = which ? sk : sq;
   const long long head_off = (long long)b * s.b + (long long)h * s.h;
@@ -171,21 +172,15 @@ int launch_quantize(const Dims& m, const sva_problem_t* p, const void* q, const 
   if (!((m.d == 128 || m.d == 64) && m.block <= 128)) return SVA_ERR_UNSUPPORTED;
   if (k_mean) {
     dim3 g1(m.Nb, m.B * m.H);
-    if (m.d == 128)
-      block_sum_kernel<128><<<g1, QT, 0, st>>>((const uint8_t*)k, sk, (float*)ws, m.H, m.N, m.block, m.Nb);
-    else
-      block_sum_kernel<64><<<g1, QT, 0, st>>>((const uint8_t*)k, sk, (float*)ws, m.H, m.N, m.block, m.Nb);
-    if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
-    mean_key_kernel<<<m.B * m.H, m.d, 0, st>>>((const float*)ws, k_mean, m.Nb, m.d, m.N);
-    if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
+    int rc = launch_dep(m.d == 128 ? block_sum_kernel<128> : block_sum_kernel<64>, g1, QT, 0, st, (const uint8_t*)k, sk, (float*)ws, m.H,
+                        m.N, m.block, m.Nb);
+    if (rc == SVA_OK) rc = launch_dep(mean_key_kernel, m.B * m.H, m.d, 0, st, (const float*)ws, k_mean, m.Nb, m.d, m.N);
+    if (rc != SVA_OK) return rc;
   }
-#define SVA_QUANT_LAUNCH(DD, SM)                                                                            \
-  quantize_kernel<DD, 128, SM><<<g, QT, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, (uint8_t*)q8, \
-                                                 (uint8_t*)k8, qs, ks, m.H, m.N, m.block, m.Nb, k_mean, lse_shift, m.scale)
-  if (m.d == 128) { if (k_mean) SVA_QUANT_LAUNCH(128, true); else SVA_QUANT_LAUNCH(128, false); }
-  else { if (k_mean) SVA_QUANT_LAUNCH(64, true); else SVA_QUANT_LAUNCH(64, false); }
-#undef SVA_QUANT_LAUNCH
-  return cudaGetLastError() == cudaSuccess ? SVA_OK : SVA_ERR_CUDA;
+  auto kern = m.d == 128 ? (k_mean ? quantize_kernel<128, 128, true> : quantize_kernel<128, 128, false>)
+                         : (k_mean ? quantize_kernel<64, 128, true> : quantize_kernel<64, 128, false>);
+  return launch_dep(kern, g, QT, 0, st, (const uint8_t*)q, (const uint8_t*)k, sq, sk, (uint8_t*)q8, (uint8_t*)k8, qs, ks, m.H, m.N,
+                    m.block, m.Nb, k_mean, lse_shift, m.scale);
 }
 
 }  // namespace sva

@@ -25,7 +25,7 @@ static constexpr int Q4_THREADS = 256;
 __global__ void __launch_bounds__(Q4_THREADS)
 amax_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, Strides sq, Strides sk, int H, int N,
             int BH, int run, uint32_t* __restrict__ amax) {
-  const int bh = blockIdx.y, which = blockIdx.z;
+  const int bh = blockIdx.y + grid_dep_wait(), which = blockIdx.z;
   const Strides s = which ? sk : sq;
   const __nv_bfloat16* base = (which ? k : q) + (long long)(bh / H) * s.b + (long long)(bh % H) * s.h;
   const int lo = blockIdx.x * run * 128, hi = min(lo + run * 128, N);
@@ -79,7 +79,7 @@ quantize4_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
                  int N, int Nb, int BH, const uint32_t* __restrict__ amax, uint8_t* __restrict__ q4,
                  uint8_t* __restrict__ k4, uint8_t* __restrict__ q_sf, uint8_t* __restrict__ k_sf, float* __restrict__ q_g,
                  float* __restrict__ k_g) {
-  const int I = gridDim.x - 1 - blockIdx.x, bh = gridDim.y - 1 - blockIdx.y, which = 1 - blockIdx.z;
+  const int I = gridDim.x - 1 - blockIdx.x, bh = gridDim.y - 1 - blockIdx.y + grid_dep_wait(), which = 1 - blockIdx.z;
   const Strides s = which ? sk : sq;
   const __nv_bfloat16* base = (which ? k : q) + (long long)(bh / H) * s.b + (long long)(bh % H) * s.h;
   uint8_t* codes = (which ? k4 : q4) + ((long long)bh * Nb + I) * 128 * 64;
@@ -161,13 +161,11 @@ int launch_quantize4(const Dims& m, const sva_problem_t* p, const void* q, const
   if (cudaMemsetAsync(amax, 0, (size_t)2 * BH * sizeof(uint32_t), st) != cudaSuccess) return SVA_ERR_CUDA;
   const Strides sq = make_strides(p->q_stride), sk = make_strides(p->k_stride);
   const int run = 2LL * m.R >= 4 * 148 * 4 ? 4 : 1;           // (a block per CTA while there are few)
-  amax_kernel<<<dim3((m.Nb + run - 1) / run, BH, 2), Q4_THREADS, 0, st>>>((const __nv_bfloat16*)q, (const __nv_bfloat16*)k, sq, sk,
-                                                                        m.H, m.N, BH, run, amax);
-  if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
-  quantize4_kernel<<<dim3(m.Nb, BH, 2), Q4_THREADS, 0, st>>>((const __nv_bfloat16*)q, (const __nv_bfloat16*)k, sq, sk, m.H, m.N,
-                                                           m.Nb, BH, amax, (uint8_t*)q4, (uint8_t*)k4, (uint8_t*)q_sf,
-                                                           (uint8_t*)k_sf, q_g, k_g);
-  return cudaGetLastError() == cudaSuccess ? SVA_OK : SVA_ERR_CUDA;
+  const int rc = launch_dep(amax_kernel, dim3((m.Nb + run - 1) / run, BH, 2), Q4_THREADS, 0, st, (const __nv_bfloat16*)q,
+                            (const __nv_bfloat16*)k, sq, sk, m.H, m.N, BH, run, amax);
+  if (rc != SVA_OK) return rc;
+  return launch_dep(quantize4_kernel, dim3(m.Nb, BH, 2), Q4_THREADS, 0, st, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, sq, sk,
+                    m.H, m.N, m.Nb, BH, amax, (uint8_t*)q4, (uint8_t*)k4, (uint8_t*)q_sf, (uint8_t*)k_sf, q_g, k_g);
 }
 
 }  // namespace sva

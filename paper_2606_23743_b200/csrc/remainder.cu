@@ -53,6 +53,7 @@ cov_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUt
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  grid_dep_wait();
   if (threadIdx.x == 0) {
     mbar_expect_tx(bar_full, 4u * panel);
     tma_load_4d(sbase, &tm_k, bar_full, 0, J * block, hh, bb);
@@ -121,10 +122,11 @@ __global__ void __launch_bounds__(256)
 weights_kernel(const float* __restrict__ scores, const int32_t* __restrict__ row_ptr, const int32_t* __restrict__ col_idx,
                int R, int Nb, int Nbw, __nv_bfloat16* __restrict__ w, float* __restrict__ mu) {
   const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * 8 + (threadIdx.x >> 5);
+  grid_dep_launch();
+  const int zero = grid_dep_wait(), r = blockIdx.x * 8 + (threadIdx.x >> 5) + zero;
   if (r >= R) return;
   const float* srow = scores + (long long)r * Nb;
-  const int nnz = __ldg(row_ptr + R);
+  const int nnz = __ldg(row_ptr + R + zero);
   int cb = __ldg(row_ptr + r), ce = __ldg(row_ptr + r + 1);
   if (cb < 0 || ce < cb || ce - cb > Nb || ce > nnz) ce = cb;          // corrupt pair: treated as keeping nothing
   // first pass: the maximum over the dropped blocks (the row's kept list is ascending: walk it alongside)
@@ -183,6 +185,7 @@ aggregate_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = tmem_base_s;
+  grid_dep_wait();
   bool ok = true;
   if (threadIdx.x == 0) {
     const uint32_t idesc = instr_desc(128, 128, 1, true);
@@ -313,13 +316,12 @@ int launch_remainder1(const Dims& m, const sva_problem_t* p, const void* k, cons
   }
   const int smem_cov = 2 * rem::TILE + 1024, smem_agg = 128 * 128 + 2 * 64 * 128 + 1024;
   if (cudaFuncSetAttribute(cov_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_cov) != cudaSuccess) return SVA_ERR_CUDA;
-  if (natural) cov_kernel<<<dim3(m.Nb, m.B * m.H), 128, smem_cov, st>>>(tv, tk, m.H, m.N, m.block, m.Nb, ct, status);
-  else cov_kernel<<<dim3(m.Nb, m.B * m.H), 128, smem_cov, st>>>(tk, tv, m.H, m.N, m.block, m.Nb, ct, status);
-  if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
-  weights_kernel<<<(m.R + 7) / 8, 256, 0, st>>>(scores, row_ptr, col_idx, m.R, m.Nb, Nbw, w, mu);
-  if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
-  aggregate_kernel<<<dim3(rem::D, (m.Nb + 127) / 128, m.B * m.H), 128, smem_agg, st>>>(tw, tc, m.Nb, Nbw, at, status);
-  if (cudaGetLastError() != cudaSuccess) return SVA_ERR_CUDA;
+  if ((rc = launch_dep(cov_kernel, dim3(m.Nb, m.B * m.H), 128, smem_cov, st, natural ? tv : tk, natural ? tk : tv, m.H, m.N, m.block, m.Nb,
+                       ct, status)) != SVA_OK)
+    return rc;
+  if ((rc = launch_dep(weights_kernel, (m.R + 7) / 8, 256, 0, st, scores, row_ptr, col_idx, m.R, m.Nb, Nbw, w, mu)) != SVA_OK) return rc;
+  if ((rc = launch_dep(aggregate_kernel, dim3(rem::D, (m.Nb + 127) / 128, m.B * m.H), 128, smem_agg, st, tw, tc, m.Nb, Nbw, at, status)) != SVA_OK)
+    return rc;
   *at_out = at;
   *mu_out = mu;
   return SVA_OK;

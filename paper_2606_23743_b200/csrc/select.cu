@@ -37,7 +37,7 @@ pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Stride
   constexpr int STEP = GROUPS * 4;              // token rows per step
   __shared__ float part[GROUPS][D + 1];
 
-  const int bh = blockIdx.y, which = blockIdx.z;
+  const int bh = blockIdx.y + grid_dep_wait(), which = blockIdx.z;
   const int b = bh / H, h = bh % H;
   const Strides s = which ? sk : sq;
   const uint8_t* base = (which ? k : q) + ((long long)b * s.b + (long long)h * s.h) * ELEM_BYTES;
@@ -326,7 +326,8 @@ block_scores_kernel(const float* __restrict__ qbar, const float* __restrict__ kb
   extern __shared__ __align__(16) float sc_smem[];
   float* qs = sc_smem;                     // [TQ][LD]
   float* ks = sc_smem + TQ * LD;           // [TK][LD]
-  const int bh = blockIdx.z, I0 = blockIdx.y * TQ, J0 = blockIdx.x * TK;
+  grid_dep_launch();
+  const int bh = blockIdx.z + grid_dep_wait(), I0 = blockIdx.y * TQ, J0 = blockIdx.x * TK;
   auto fill = [&](float* dst, const float* src, int r0, auto rows_tag) {      // eight 16-byte vectors per thread in flight
     constexpr int PER = decltype(rows_tag)::value * V / THREADS, BATCH = PER < 8 ? PER : 8;
 #pragma unroll
@@ -399,8 +400,7 @@ static int launch_scores(const float* qbar, const float* kbar, int Nb, int heads
       attr_set[dev] = true;
     }
   }
-  kern<<<dim3((Nb + TK - 1) / TK, (Nb + TQ - 1) / TQ, heads), 16 * TY, smem, st>>>(qbar, kbar, Nb, scale, scores);
-  return SVA_OK;
+  return launch_dep(kern, dim3((Nb + TK - 1) / TK, (Nb + TQ - 1) / TQ, heads), 16 * TY, smem, st, qbar, kbar, Nb, scale, scores);
 }
 
 // Selection: one warp per query-block row, its Nb scores read straight from the score matrix (lane j owns
@@ -411,8 +411,9 @@ template <int ITEMS, bool MASS>
 __global__ void __launch_bounds__(SEL_WARPS * 32)
 select_rows_kernel(const float* __restrict__ scores, SelParams p, int32_t* __restrict__ row_ptr,
                    int32_t* __restrict__ col_idx, int32_t* __restrict__ tmp_idx, int32_t* __restrict__ counts, int R) {
+  grid_dep_launch();
   const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * SEL_WARPS + (threadIdx.x >> 5);
+  const int r = blockIdx.x * SEL_WARPS + (threadIdx.x >> 5) + grid_dep_wait();
   if (r >= R) return;
   const int Nb = p.Nb, bh = r / Nb, I = r % Nb;
   const float* srow = scores + (long long)r * Nb;
@@ -436,9 +437,10 @@ csr_kernel(const int32_t* __restrict__ tmp_idx, const int32_t* __restrict__ coun
   __shared__ int warp_sum[32];
   __shared__ int row_off[CSR_ROWS + 1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r0 = blockIdx.x * CSR_ROWS;
+  grid_dep_launch();
+  const int zero = grid_dep_wait(), r0 = blockIdx.x * CSR_ROWS + zero;
   int part = 0;
-  for (int i = threadIdx.x; i < r0; i += CSR_ROWS * 32) part += __ldg(counts + i);
+  for (int i = threadIdx.x + zero; i < r0; i += CSR_ROWS * 32) part += __ldg(counts + i);
 #pragma unroll
   for (int o = 16; o; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
   if (lane == 0) warp_sum[warp] = part;
@@ -498,6 +500,16 @@ size_t select_workspace_bytes(const Dims& m, const sva_select_t* s) {
 }
 
 template <int D>
+static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale,
+                         const float* k_scale, float* qbar, float* kbar, cudaStream_t st) {
+  const int run = pool_run(m);
+  const dim3 grid((m.Nb + run - 1) / run, m.B * m.H, 2);
+  return launch_dep(m.fp8 ? pool_kernel<D, 1> : pool_kernel<D, 2>, grid, POOL_THREADS, 0, st, (const uint8_t*)q, (const uint8_t*)k,
+                    make_strides(p->q_stride), make_strides(p->k_stride), m.fp8 ? q_scale : nullptr, m.fp8 ? k_scale : nullptr,
+                    m.H, m.N, m.block, m.Nb, run, qbar, kbar);
+}
+
+template <int D>
 static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_select_t* s,
                            const void* q, const void* k, const float* q_scale,
                            const float* k_scale, int32_t* row_ptr, int32_t* col_idx,
@@ -516,16 +528,8 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
     tmp_idx = reinterpret_cast<int32_t*>(w + 2 * pooled);
     counts = reinterpret_cast<int32_t*>(w + 2 * pooled + align256((size_t)m.R * cap * sizeof(int32_t)));
   }
-  const int run = pool_run(m);
-  dim3 pg((m.Nb + run - 1) / run, m.B * m.H, 2);
-  Strides sq = make_strides(p->q_stride), sk = make_strides(p->k_stride);
-  if (qbar_in) {
-  } else if (m.fp8)
-    pool_kernel<D, 1><<<pg, POOL_THREADS, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, q_scale,
-                                                   k_scale, m.H, m.N, m.block, m.Nb, run, qbar, kbar);
-  else
-    pool_kernel<D, 2><<<pg, POOL_THREADS, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, nullptr,
-                                                   nullptr, m.H, m.N, m.block, m.Nb, run, qbar, kbar);
+  int rc = SVA_OK;
+  if (!qbar_in && (rc = launch_pool_d<D>(m, p, q, k, q_scale, k_scale, qbar, kbar, st)) != SVA_OK) return rc;
   SelParams sp;
   sp.H = m.H; sp.Nb = m.Nb; sp.mode = s->mode; sp.k = s->k;
   sp.use_window = (s->win_t >= 0 && s->win_s >= 0 && s->blocks_per_frame > 0) ? 1 : 0;
@@ -542,27 +546,24 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
     // 64 x 64 tiles where they give most of the SMs a CTA, else 32 x 32: with few rows the time is one CTA's latency, and
     // that shrinks with its tile (16 heads of 64 blocks: 16 tiles of 64 x 64 take 6.8 us, 64 of 32 x 32 4.2 us).
     const int heads = m.B * m.H, nt = (m.Nb + 63) / 64;
-    const int rc = nt * nt * heads >= 96 ? launch_scores<D, 8, 4, 8>(qbar, kbar, m.Nb, heads, m.scale, scores, st)
+    rc = nt * nt * heads >= 96 ? launch_scores<D, 8, 4, 8>(qbar, kbar, m.Nb, heads, m.scale, scores, st)
                              : launch_scores<D, 2, 2, 16>(qbar, kbar, m.Nb, heads, m.scale, scores, st);
     if (rc != SVA_OK) return rc;
   }
   const int items = (m.Nb + 31) / 32;
   const int sg = (m.R + SEL_WARPS - 1) / SEL_WARPS;
-#define SVA_SEL_LAUNCH(IT)                                                                                                    \
-  do {                                                                                                                        \
-    if (s->mode == 1) select_rows_kernel<IT, true><<<sg, SEL_WARPS * 32, 0, st>>>(scores, sp, row_ptr, col_idx, tmp_idx, counts, m.R); \
-    else select_rows_kernel<IT, false><<<sg, SEL_WARPS * 32, 0, st>>>(scores, sp, row_ptr, col_idx, tmp_idx, counts, m.R);     \
-  } while (0)
-  if (items <= 4) SVA_SEL_LAUNCH(4);
-  else if (items <= 8) SVA_SEL_LAUNCH(8);
-  else if (items <= 12) SVA_SEL_LAUNCH(12);
-  else if (items <= 16) SVA_SEL_LAUNCH(16);
-  else SVA_SEL_LAUNCH(32);
-#undef SVA_SEL_LAUNCH
-  if (!fixed_n) {
-    csr_kernel<<<(m.R + CSR_ROWS - 1) / CSR_ROWS, CSR_ROWS * 32, 0, st>>>(tmp_idx, counts, cap, m.R, row_ptr, col_idx);
-  }
-  return cudaGetLastError() == cudaSuccess ? SVA_OK : SVA_ERR_CUDA;
+  auto select = [&](auto items_tag) {
+    constexpr int IT = decltype(items_tag)::value;
+    return launch_dep(s->mode == 1 ? select_rows_kernel<IT, true> : select_rows_kernel<IT, false>, sg, SEL_WARPS * 32, 0, st, scores, sp,
+                      row_ptr, col_idx, tmp_idx, counts, m.R);
+  };
+  if (items <= 4) rc = select(std::integral_constant<int, 4>{});
+  else if (items <= 8) rc = select(std::integral_constant<int, 8>{});
+  else if (items <= 12) rc = select(std::integral_constant<int, 12>{});
+  else if (items <= 16) rc = select(std::integral_constant<int, 16>{});
+  else rc = select(std::integral_constant<int, 32>{});
+  if (rc != SVA_OK || fixed_n) return rc;
+  return launch_dep(csr_kernel, (m.R + CSR_ROWS - 1) / CSR_ROWS, CSR_ROWS * 32, 0, st, tmp_idx, counts, cap, m.R, row_ptr, col_idx);
 }
 
 int launch_select(const Dims& m, const sva_problem_t* p, const sva_select_t* s, const void* q,
@@ -581,23 +582,9 @@ int launch_select(const Dims& m, const sva_problem_t* p, const sva_select_t* s, 
 // Pooling alone: block means of Q and K into the caller's arrays ([B,H,Nb,d] fp32 each).
 int launch_pool(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale,
                 const float* k_scale, float* qbar, float* kbar, cudaStream_t st) {
-  const int run = pool_run(m);
-  dim3 pg((m.Nb + run - 1) / run, m.B * m.H, 2);
-  Strides sq = make_strides(p->q_stride), sk = make_strides(p->k_stride);
-#define SVA_POOL_LAUNCH(DD)                                                                                        \
-  do {                                                                                                             \
-    if (m.fp8)                                                                                                     \
-      pool_kernel<DD, 1><<<pg, POOL_THREADS, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, q_scale, k_scale, \
-                                                      m.H, m.N, m.block, m.Nb, run, qbar, kbar);                       \
-    else                                                                                                           \
-      pool_kernel<DD, 2><<<pg, POOL_THREADS, 0, st>>>((const uint8_t*)q, (const uint8_t*)k, sq, sk, nullptr, nullptr, \
-                                                      m.H, m.N, m.block, m.Nb, run, qbar, kbar);                       \
-  } while (0)
-  if (m.d == 128) SVA_POOL_LAUNCH(128);
-  else if (m.d == 64) SVA_POOL_LAUNCH(64);
-  else return SVA_ERR_UNSUPPORTED;
-#undef SVA_POOL_LAUNCH
-  return cudaGetLastError() == cudaSuccess ? SVA_OK : SVA_ERR_CUDA;
+  if (m.d == 128) return launch_pool_d<128>(m, p, q, k, q_scale, k_scale, qbar, kbar, st);
+  if (m.d == 64) return launch_pool_d<64>(m, p, q, k, q_scale, k_scale, qbar, kbar, st);
+  return SVA_ERR_UNSUPPORTED;
 }
 
 // Routing from block means the caller already has (qbar, kbar: [B,H,Nb,d] fp32).
