@@ -126,11 +126,13 @@ def status_string(status: int) -> str:
 
 
 def _ptr(t):
-    return C.c_void_p(t.data_ptr()) if t is not None else None
+    return t.data_ptr() if t is not None else None              # (the functions' argument types make it a void*)
 
 
 def _stream():
-    return C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    """The current stream of the current device, as a pointer.  (torch.cuda.current_stream() builds a Stream object, 2 us of
+    the 14 us that the two calls of a small clip spend in Python.)"""
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
 
 
 def _strides(t):
