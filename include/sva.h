@@ -103,7 +103,9 @@ size_t sva_select_workspace_bytes(const sva_problem_t* p, const sva_select_t* s)
  * Routing (the paper's "score-based routing" of critical blocks).
  *   q, k          : Q and K as described by p (bf16, or e4m3 bytes + q_scale/k_scale)
  *   row_ptr       : out, [R+1] int32, row_ptr[R] = number of kept (row, block) pairs
- *   col_idx       : out, capacity sva_select_max_nnz entries; rows are packed back to back
+ *   col_idx       : out, capacity sva_select_max_nnz entries; rows are packed back to back, and every entry that
+ *                   row_ptr covers is written (a NaN score is never kept: a top-k row with fewer than k others is filled
+ *                   up with block 0)
  *   block_scores  : optional out, [B,H,Nb,Nb] fp32, the scaled pooled scores
  *   workspace     : >= sva_select_workspace_bytes, 256-byte aligned
  * Pooling is a mean over the VALID tokens of a block; score = softmax_scale*<qbar,kbar>;

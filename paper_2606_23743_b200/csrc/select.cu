@@ -306,6 +306,8 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
     if (sel) out[base + __popc(bal & ((1u << lane) - 1u))] = it * 32 + lane;
     base += __popc(bal);
   }
+  // (NaN scores are no candidates: a row of known length can come out short; what row_ptr covers is written all the same)
+  for (int t = base + lane; t < p.fixed_n; t += 32) out[t] = 0;
 }
 
 // Block scores of one head as a small fp32 GEMM: S[I][J] = scale * <qbar_I, kbar_J>.  A CTA computes a

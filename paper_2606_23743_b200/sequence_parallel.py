@@ -115,7 +115,7 @@ def sparse_attend(select, block: int = 128, status=None):
         p = B.make_problem(q, k, v, o, N, block)
         R = q.shape[0] * q.shape[1] * (-(-N // block))
         ws = torch.empty(max(B.select_workspace_bytes(p, select), 256), dtype=torch.uint8, device=q.device)
-        # (routing writes all of row_ptr and every entry of col_idx that row_ptr covers: nothing to clear first)
+        # (routing writes all of row_ptr and every entry of col_idx that row_ptr covers, with NaN scores too: nothing to clear first)
         row_ptr = torch.empty(R + 1, dtype=torch.int32, device=q.device)
         col_idx = torch.empty(max(B.select_max_nnz(p, select), 1), dtype=torch.int32, device=q.device)
         st = status if status is not None else torch.zeros(1, dtype=torch.int32, device=q.device)

@@ -185,3 +185,34 @@ def test_threshold_search_on_awkward_scores(nb, mode):
                 continue
             for r in (h * nb, h * nb + nb - 1):
                 assert ci[rp[r]:rp[r + 1]].tolist() == want, (h, k)
+
+
+@pytest.mark.parametrize("nb,k,window", [(16, 4, False), (16, 16, False), (40, 33, False), (129, 70, False), (16, 9, True)])
+def test_rows_of_a_known_length_are_written_whole(nb, k, window):
+    """A NaN score is never selected, so a row of top-k can find fewer than the k blocks its row_ptr covers: the entries left
+    over are block 0, whatever col_idx held before."""
+    d, n = 128, nb * 128
+    rng = np.random.default_rng(nb)
+    qbar, kbar = (rng.standard_normal((1, 3, nb, d)).astype(np.float32) for _ in range(2))
+    qbar[0, 0, [0, nb // 2, nb - 1]] = np.nan                    # head 0: rows without a candidate
+    kbar[0, 1, [1, nb - 1]] = np.nan                             # head 1: two blocks that no row can pick; head 2: as usual
+    t = torch.empty(1, 3, n, d, dtype=torch.bfloat16, device="cuda")
+    p = B.make_problem(t, t, None, None, n, 128)
+    s = B.make_select(0, k, 1.0, 1, 1, 4) if window else B.make_select(0, k)
+    ws = torch.empty(max(B.select_workspace_bytes(p, s), 256), dtype=torch.uint8, device="cuda")
+    got = []
+    for junk in (-7, 0x7fffffff):
+        rp = torch.full((3 * nb + 1,), junk, dtype=torch.int32, device="cuda")
+        ci = torch.full((B.select_max_nnz(p, s),), junk, dtype=torch.int32, device="cuda")
+        B.block_select_pooled(p, s, torch.tensor(qbar).cuda(), torch.tensor(kbar).cuda(), rp, ci, ws)
+        got.append((rp.cpu().numpy(), ci.cpu().numpy().reshape(3 * nb, k)))
+    rp, ci = got[0]
+    assert np.array_equal(rp, np.arange(3 * nb + 1) * k) and np.array_equal(rp, got[1][0]) and np.array_equal(ci, got[1][1])
+    scores = np.einsum("hid,hjd->hij", qbar[0], kbar[0]) / np.sqrt(np.float32(d))
+    for h in range(3):
+        for i in range(nb):
+            x = scores[h, i].astype(np.float64)
+            forced = [j for j in range(nb) if window and abs(i // 4 - j // 4) <= 1 and abs(i % 4 - j % 4) <= 1]
+            real = [j for j in range(nb) if not np.isnan(x[j]) and j not in forced]
+            kept = sorted(forced + sorted(real, key=lambda j: (-x[j], j))[:k - len(forced)])
+            assert ci[h * nb + i].tolist() == kept + [0] * (k - len(kept)), (h, i)

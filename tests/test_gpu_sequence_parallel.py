@@ -32,3 +32,27 @@ def test_one_rank_group_matches_the_direct_path_and_the_oracle():
         U.check_attn_vs_oracle(w, qb, kb, vb, rp, ci, o, None, U.sample_rows(w.R, w.Nb, 6))
     finally:
         dist.destroy_process_group()
+
+
+def test_attend_does_not_depend_on_what_its_buffers_held():
+    """A NaN token leaves its query block without scores, and its key block without candidates that k = Nb counts on: the output
+    is that of index arrays that were cleared, whatever the allocator hands out."""
+    w = shrink(WORKLOADS["medium"], H=2, T=1, k=8)                 # 8 blocks, all of them asked for
+    (q, k, v), _ = U.host_inputs(w)
+    qd, kd, vd = (U.dev(x)[:, :, :w.N].contiguous() for x in (q, k, v))
+    qd[0, 0, 300, 5] = float("nan")
+    kd[0, 1, 700, 9] = float("nan")
+    sel = B.make_select(0, w.k)
+    p = B.make_problem(qd, kd, vd, torch.empty_like(vd), w.N, w.block)
+    rp, ci = (torch.zeros(n, dtype=torch.int32, device="cuda") for n in (w.R + 1, B.select_max_nnz(p, sel)))
+    B.block_select(p, sel, qd, kd, rp, ci, torch.empty(B.select_workspace_bytes(p, sel), dtype=torch.uint8, device="cuda"))
+    want, _, st = U.gpu_attn(w, qd, kd, vd, rp, ci)
+    assert st == 0
+    attend = SP.sparse_attend(sel, w.block)
+    for junk in (3, 7):                                            # (valid indices: a stale list would go unnoticed)
+        for _ in range(2):                                         # what the caching allocator hands out next holds junk
+            held = [torch.full((n,), junk, dtype=torch.int32, device="cuda") for n in (ci.numel(), rp.numel()) for _ in range(4)]
+            del held
+            o = attend(qd, kd, vd)
+            assert int(attend.status.item()) == 0
+            assert torch.equal(o.view(torch.int16), want[:, :, :w.N].view(torch.int16))
