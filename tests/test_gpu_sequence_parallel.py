@@ -34,7 +34,7 @@ def test_one_rank_group_matches_the_direct_path_and_the_oracle():
         dist.destroy_process_group()
 
 
-def test_attend_does_not_depend_on_what_its_buffers_held():
+def test_attend_does_not_depend_on_what_its_buffers_held(monkeypatch):
     """A NaN token leaves its query block without scores, and its key block without candidates that k = Nb counts on: the output
     is that of index arrays that were cleared, whatever the allocator hands out."""
     w = shrink(WORKLOADS["medium"], H=2, T=1, k=8)                 # 8 blocks, all of them asked for
@@ -49,10 +49,13 @@ def test_attend_does_not_depend_on_what_its_buffers_held():
     want, _, st = U.gpu_attn(w, qd, kd, vd, rp, ci)
     assert st == 0
     attend = SP.sparse_attend(sel, w.block)
+    empty = torch.empty
     for junk in (3, 7):                                            # (valid indices: a stale list would go unnoticed)
-        for _ in range(2):                                         # what the caching allocator hands out next holds junk
-            held = [torch.full((n,), junk, dtype=torch.int32, device="cuda") for n in (ci.numel(), rp.numel()) for _ in range(4)]
-            del held
-            o = attend(qd, kd, vd)
-            assert int(attend.status.item()) == 0
-            assert torch.equal(o.view(torch.int16), want[:, :, :w.N].view(torch.int16))
+        def held(*size, dtype=None, **kw):                         # memory that an earlier call has used
+            x = empty(*size, dtype=dtype, **kw)
+            return x.fill_(junk) if dtype == torch.int32 else x
+        monkeypatch.setattr(torch, "empty", held)
+        o = attend(qd, kd, vd)
+        monkeypatch.setattr(torch, "empty", empty)
+        assert int(attend.status.item()) == 0
+        assert torch.equal(o.view(torch.int16), want[:, :, :w.N].view(torch.int16))
