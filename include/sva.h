@@ -301,6 +301,8 @@ int sva_quantize_qk_fp8(const sva_problem_t* p, const void* q_bf16, const void* 
  *   per element          code = e2m1(x / (value(sf) * g)), round-to-nearest-even, saturating at +-6
  *                        (e2m1 magnitudes 0, .5, 1, 1.5, 2, 3, 4, 6; code = sign << 3 | index; all 0 where sf = 0)
  *   x ~= value(code) * value(sf) * g
+ * A NaN element is left out of its scale block's amax, so that the other 15 keep a scale and codes of their own; its
+ * code has magnitude 6, and its (b,h) gets g = 1.
  * Outputs (device, 16-byte aligned), in the layout the block-scaled tensor-core MMA takes:
  *   q4, k4     : [B*H][Nb*128 tokens][64] bytes, two codes per byte (even element in the low nibble), rows >= N zero
  *   q_sf, k_sf : [B*H][Nb][2][32][4][4] bytes: for 128-token block I and half c of the head dimension, the scale of

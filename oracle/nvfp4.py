@@ -9,10 +9,10 @@ fixed bit for bit so that CPU and GPU bytes can be compared (all scalar steps ar
             max 448, subnormals down to 2^-9)
   tensor    one fp32 scale g per (b, h)
 
-  g    = amax(b,h) / (6 * 448)       over the tokens that exist; 1 if amax = 0
+  g    = amax(b,h) / (6 * 448)       over the tokens that exist; 1 if amax = 0 or an element is NaN
   sf   = e4m3( (amax(block) / 6) / g )                     round-to-nearest-even, saturating
   code = e2m1( x / (value(sf) * g) )                       round-to-nearest-even (even = mantissa bit 0), saturating
-         at +-6; a block whose sf is 0 has all codes 0
+         at +-6; a block whose sf is 0 has all codes 0.  A NaN does not count in amax(block); its magnitude is 6
   xhat = value(code) * value(sf) * g                        (the dequantised value, evaluated in fp64 here)
 
 Two codes per byte, the even element in the low nibble.  Only tests, the smoke check and the bench's CPU legs
@@ -81,7 +81,7 @@ def quantize(x_bf16: np.ndarray, N: int):
             gg = f32(amax / f32(6.0 * 448.0)) if amax > 0 else f32(1.0)
             g[b, h] = gg
             blk = v.reshape(N, d // BLOCK, BLOCK)
-            a = np.abs(blk).max(axis=2).astype(np.float32)
+            a = np.fmax.reduce(np.abs(blk), axis=2).astype(np.float32)      # (a NaN does not count)
             u = ((a / f32(6.0)).astype(np.float32) / gg).astype(np.float32)
             sf = e4m3_encode_pos(u)
             s = (tab[sf] * gg).astype(np.float32)                       # [N, d/16]

@@ -69,6 +69,14 @@ amax_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict
 
 __device__ __noinline__ float div_slow(float a, float b) { return __fdiv_rn(a, b); }
 
+// max |x| over a scale block, NaNs left out (rare, and kept out of the loop's way like the divisions)
+__device__ __noinline__ float amax_without_nan(const uint32_t* x) {
+  float a = 0.f;
+#pragma unroll 1
+  for (int e = 0; e < 8; ++e) a = fmaxf(a, fmaxf(fabsf(bf16lo(x[e])), fabsf(bf16hi(x[e]))));
+  return a;
+}
+
 // One CTA per (128-token block, head, tensor), in the reverse of the order in which amax_kernel read them, so that the tensors'
 // ends are still in the L2; a thread casts four 16-element scale blocks, whose loads are all in flight.  Issue-bound (75 % of
 // the issue slots at 105 us): the divisions are three FMA-pipe operations each, element pairs in packed ones, with true
@@ -110,7 +118,9 @@ quantize4_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     uint32_t mx = 0u;                                         // max |x| of the pairs (bf16 magnitudes order like integers)
 #pragma unroll
     for (int e = 0; e < 8; ++e) mx = __vmaxu2(mx, w[e] & 0x7fff7fffu);
-    const float a = __uint_as_float(max(mx << 16, mx & 0xffff0000u));
+    float a = __uint_as_float(max(mx << 16, mx & 0xffff0000u));
+    if (a != a)                                               // (a NaN orders above every number)
+      a = amax_without_nan(reinterpret_cast<const uint32_t*>(base + (long long)(lo + t) * s.n + kb * 16));
     const float u = g_fast && (a == 0.f || a >= 8.077935669463161e-28f)                       // 2^-90
                         ? div_fast(div_fast(a, 6.0f, 0.16666667163372039795f), g, g_rcp)
                         : div_slow(div_slow(a, 6.0f), g);

@@ -132,3 +132,31 @@ def test_quantiser_bytes_at_extreme_magnitudes(exponent):
         np.testing.assert_array_equal(gg.cpu().numpy().reshape(w.B, w.H), g)
         np.testing.assert_array_equal(untile_sf(gsf, w.Nb).reshape(w.B, w.H, w.Nb * 128, 8)[:, :, :w.N], sfs[:, :, :w.N])
         np.testing.assert_array_equal(g4.cpu().numpy().reshape(w.B, w.H, w.Nb * 128, 64)[:, :, :w.N], codes[:, :, :w.N])
+
+
+@pytest.mark.parametrize("magnitude", [1.0, 2.0 ** -100])
+def test_a_nan_costs_its_scale_block_nothing_but_its_own_code(magnitude):
+    """One NaN among 16 elements, in every position, of either sign: the others keep the scale and the codes that they have
+    without it (a head with a NaN has the tensor scale 1; tiny values then get scale and codes 0, by the slow divisions)."""
+    w = shrink(WORKLOADS["medium"], H=3, T=1, Hg=4, Wg=50)                           # N = 200
+    (q, k, _), _ = U.host_inputs(w)
+    q, k = ((x[:, :, :w.N].float() * magnitude).to(torch.bfloat16).contiguous() for x in (q, k))
+    nan_bits = torch.where(torch.arange(w.d) % 3 == 0, torch.tensor(0xFFC0 - 0x10000), torch.tensor(0x7FC1)).to(torch.int16)
+    where = {}
+    for x, h in ((q, 0), (k, 2)):
+        at = torch.zeros(x.shape, dtype=torch.bool)
+        for i in range(16):
+            at[0, h, 3 + 11 * i, 16 * (i % 8) + i] = True
+            at[0, h, w.N - 1 - i, 16 * ((i + 3) % 8) + i] = True
+        x.view(torch.int16).copy_(torch.where(at, nan_bits, x.view(torch.int16)))
+        where[h] = at.numpy()
+    q4, k4, qsf, ksf, qg, kg = gpu_quantize4(w, U.dev(q), U.dev(k))
+    for x, h, g4, gsf, gg in ((q, 0, q4, qsf, qg), (k, 2, k4, ksf, kg)):
+        codes, sfs, g = nvfp4.quantize(bf16_bits(x), w.N)
+        assert g[0, h] == 1.0 and (g[0, [i for i in range(3) if i != h]] != 1.0).all()
+        np.testing.assert_array_equal(gg.cpu().numpy().reshape(w.B, w.H), g)
+        np.testing.assert_array_equal(untile_sf(gsf, w.Nb).reshape(w.B, w.H, w.Nb * 128, 8)[:, :, :w.N], sfs[:, :, :w.N])
+        got = g4.cpu().numpy().reshape(w.B, w.H, w.Nb * 128, 64)[:, :, :w.N]
+        got, want = (np.stack((c & 15, c >> 4), axis=-1).reshape(w.B, w.H, w.N, w.d) for c in (got, codes[:, :, :w.N]))
+        assert (got[where[h]] & 7 == (7 if magnitude == 1.0 else 0)).all()
+        np.testing.assert_array_equal(np.where(where[h], 0, got), np.where(where[h], 0, want))
