@@ -191,3 +191,17 @@ def test_routing_limits_are_refused_on_the_host(lib):
                          (lib.sva_block_select_pooled, (fake, fake, fake, fake, None, fake, C.c_size_t(1 << 40), None)),
                          (lib.sva_block_select_noalloc, (fake, fake, None, None, fake, fake, None, None))):
             assert fn(C.byref(p), C.byref(sel), *args) == 2, fn
+
+
+def test_the_stream_comes_from_the_public_call_where_torch_lacks_the_short_one(monkeypatch):
+    import importlib.util
+    import types
+
+    import torch
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=0x1234))
+    spec = importlib.util.spec_from_file_location("binding_without_raw_stream", B.__file__)
+    m = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(m)
+    assert m._stream() == 0x1234
