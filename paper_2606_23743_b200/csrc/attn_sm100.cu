@@ -1543,7 +1543,7 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
     // block means of K ([Nbp rows][128], rows >= Nb zero) and of V (transposed tiles), then their maps
     __nv_bfloat16* kp = reinterpret_cast<__nv_bfloat16*>(wsb + L.kp_off);
     __nv_bfloat16* vtp = reinterpret_cast<__nv_bfloat16*>(wsb + L.vtp_off);
-    const int run = 2LL * m.R >= 4 * 148 * 4 ? 4 : 1;              // (a block per CTA while there are few)
+    const int run = blocks_per_cta(2LL * m.R);                     // (the padding blocks that the grid covers too are not read)
     if ((rc = launch_dep(pool_kv_kernel, dim3((L.Nbp + run - 1) / run, m.B * m.H, 2), 256, 0, st, (const __nv_bfloat16*)k,
                          (const __nv_bfloat16*)v, sk, make_strides(p->v_stride), m.H, m.N, m.block, m.Nb, L.Nbp, run, kp, vtp, vmn ? 1 : 0,
                          reinterpret_cast<int32_t*>(wsb + L.counter_off))) != SVA_OK)

@@ -92,6 +92,11 @@ inline int launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cu
   return SVA_ERR_CUDA;
 }
 
+// Consecutive token blocks per CTA of the kernels that stream a tensor's blocks (`blocks` of them over all heads and tensors) with
+// the next loads in flight while they reduce: runs of four once those still give each of the 148 SMs four CTAs; before that a block
+// each, since the time is then the longest CTA's latency.
+inline int blocks_per_cta(long long blocks) { return blocks >= 4LL * 4 * 148 ? 4 : 1; }
+
 // host-side argument checks shared by the entry points
 int validate_problem(const sva_problem_t* p);
 

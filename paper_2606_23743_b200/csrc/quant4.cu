@@ -170,7 +170,7 @@ int launch_quantize4(const Dims& m, const sva_problem_t* p, const void* q, const
   uint32_t* amax = static_cast<uint32_t*>(ws);
   if (cudaMemsetAsync(amax, 0, (size_t)2 * BH * sizeof(uint32_t), st) != cudaSuccess) return SVA_ERR_CUDA;
   const Strides sq = make_strides(p->q_stride), sk = make_strides(p->k_stride);
-  const int run = 2LL * m.R >= 4 * 148 * 4 ? 4 : 1;           // (a block per CTA while there are few)
+  const int run = blocks_per_cta(2LL * m.R);
   const int rc = launch_dep(amax_kernel, dim3((m.Nb + run - 1) / run, BH, 2), Q4_THREADS, 0, st, (const __nv_bfloat16*)q,
                             (const __nv_bfloat16*)k, sq, sk, m.H, m.N, BH, run, amax);
   if (rc != SVA_OK) return rc;

@@ -97,10 +97,6 @@ pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Stride
   }
 }
 
-// Blocks per CTA: runs of four once they still give every SM a few CTAs; before that a block each, since the time is then the
-// longest CTA's latency.
-static int pool_run(const Dims& m) { return 2LL * m.R >= 4 * 148 * 4 ? 4 : 1; }
-
 struct SelParams {
   int H, Nb, mode, k, use_window, win_t, win_s, bpf, cap, fixed_n;
   float scale, tau;
@@ -504,7 +500,7 @@ size_t select_workspace_bytes(const Dims& m, const sva_select_t* s) {
 template <int D>
 static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale,
                          const float* k_scale, float* qbar, float* kbar, cudaStream_t st) {
-  const int run = pool_run(m);
+  const int run = blocks_per_cta(2LL * m.R);
   const dim3 grid((m.Nb + run - 1) / run, m.B * m.H, 2);
   return launch_dep(m.fp8 ? pool_kernel<D, 1> : pool_kernel<D, 2>, grid, POOL_THREADS, 0, st, (const uint8_t*)q, (const uint8_t*)k,
                     make_strides(p->q_stride), make_strides(p->k_stride), m.fp8 ? q_scale : nullptr, m.fp8 ? k_scale : nullptr,
