@@ -269,7 +269,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int Nb = prm.Nt;             // row index arithmetic: rows per head
   constexpr int KB = B64 ? 64 : BS;  // tokens per key block
-  constexpr bool RMASK = REM && !B64; // remainder, 128-token blocks: kept-block bit masks (64-token blocks: the CSR look-up measured faster)
+  constexpr bool RMASK = REM && !B64; // remainder, 128-token blocks: the K producer leaves kept-block bit masks (64-token blocks: pair_lists_kernel does)
 
   // ---------------------------------------------------------------- set-up
   const long long t_cta0 = prm.prof ? clock64() : 0;

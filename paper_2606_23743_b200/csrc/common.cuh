@@ -65,10 +65,13 @@ __device__ __forceinline__ uint32_t e4m3x2(float lo, float hi) {
 // (programmatic stream serialisation), and starts with grid_dep_wait(), which returns when every earlier kernel of the
 // stream has completed and its writes are visible.  It returns 0, which the compiler does not know: added to the indices that a
 // kernel's first loads are made from, it keeps read-only loads from being moved in front of it.
-// grid_dep_launch() lets the next kernel be set up once every CTA has called it or ended.  Kernels of a wave or less call it at
-// their start; the streaming ones and the attention kernel do not, so that their successors come in when they end: called
+// grid_dep_launch() lets the next kernel be set up once every CTA has called it or ended -- whatever the size of the grid, none
+// of its CTAs can then be kept from an SM by one that waits for it.  The short kernels call it at their start (block scores,
+// selection, CSR, tile lists, mean key, remainder weights, row counters; none of them holds tensor memory); the streaming
+// ones, the tensor-core ones and the attention kernel do not, so that their successors come in when they end: called
 // there too, the successors' waiting CTAs made everything from a medium clip on 0.3 to 0.9 % slower than plain launches.  As
 // it is: a 5 580-token clip 95.3 -> 83.7 us for the whole call, 8 192 tokens x 16 heads 172 -> 166.5 us.
+// (The diagnostic CUDA-core attention kernel is launched plainly: it starts when everything before it has ended.)
 __device__ __forceinline__ int grid_dep_wait() {
   int zero;
   asm volatile("griddepcontrol.wait;\n\tmov.u32 %0, 0;" : "=r"(zero)::"memory");

@@ -3,12 +3,12 @@
 // window, CSR assembly.  (Paper: "score-based routing" of the critical blocks; block-wise
 // similarity metric of the sparse-attention section.)
 //
-// pool_kernel streams Q and K once from HBM: 128-bit loads, fp32 accumulation in a fixed order, one
-// CTA per (block, head, tensor).  block_scores_kernel computes a head's score matrix as a small fp32
-// GEMM (64 x 64 tiles from two shared-memory panels, fixed summation order).  select_rows_kernel is one
-// warp per query-block row: it reads the row's scores from that matrix (no shared memory), finds the
-// threshold of the rule by bisection on order-preserving integer keys and emits the kept blocks in
-// ascending order.  When the per-row count is known on the host (top-k with no window larger than k)
+// pool_kernel streams Q and K once from HBM: 128-bit loads, fp32 accumulation in a fixed order, a CTA per
+// run of one or four blocks of a head of a tensor.  block_scores_kernel computes a head's score matrix as a
+// small fp32 GEMM (64 x 64 or 32 x 32 tiles from two shared-memory panels, fixed summation order).
+// select_rows_kernel is one warp per query-block row: it reads the row's scores from that matrix (no shared
+// memory) as order-preserving integer keys, finds the threshold of the rule by narrowing an interval of scores
+// that holds it and emits the kept blocks in ascending order.  When the per-row count is known on the host (top-k with no window larger than k)
 // rows go straight into the CSR; otherwise they are staged and csr_kernel builds it in one launch.
 #include <mutex>
 #include <type_traits>
@@ -98,8 +98,8 @@ pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Stride
 }
 
 struct SelParams {
-  int H, Nb, mode, k, use_window, win_t, win_s, bpf, cap, fixed_n;
-  float scale, tau;
+  int Nb, k, use_window, win_t, win_s, bpf, cap, fixed_n;
+  float tau;
 };
 
 __device__ __forceinline__ bool in_window(int I, int J, const SelParams& p) {
@@ -529,10 +529,10 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
   int rc = SVA_OK;
   if (!qbar_in && (rc = launch_pool_d<D>(m, p, q, k, q_scale, k_scale, qbar, kbar, st)) != SVA_OK) return rc;
   SelParams sp;
-  sp.H = m.H; sp.Nb = m.Nb; sp.mode = s->mode; sp.k = s->k;
+  sp.Nb = m.Nb; sp.k = s->k;
   sp.use_window = (s->win_t >= 0 && s->win_s >= 0 && s->blocks_per_frame > 0) ? 1 : 0;
   sp.win_t = s->win_t; sp.win_s = s->win_s; sp.bpf = sp.use_window ? s->blocks_per_frame : 1;
-  sp.cap = cap; sp.fixed_n = fixed_n; sp.scale = m.scale; sp.tau = s->mass;
+  sp.cap = cap; sp.fixed_n = fixed_n; sp.tau = s->mass;
   // scores: into the caller's matrix if it wants one, else into the workspace (after the staging arrays)
   float* scores = block_scores;
   if (!scores) {
