@@ -69,12 +69,11 @@ amax_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict
 
 __device__ __noinline__ float div_slow(float a, float b) { return __fdiv_rn(a, b); }
 
-// max |x| over a scale block, NaNs left out (rare, and kept out of the loop's way like the divisions)
-__device__ __noinline__ float amax_without_nan(const uint32_t* x) {
-  float a = 0.f;
-#pragma unroll 1
-  for (int e = 0; e < 8; ++e) a = fmaxf(a, fmaxf(fabsf(bf16lo(x[e])), fabsf(bf16hi(x[e]))));
-  return a;
+// the larger of two bf16 pairs, lane by lane; a NaN loses against a number
+__device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("max.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
 }
 
 // One CTA per (128-token block, head, tensor), in the reverse of the order in which amax_kernel read them, so that the tensors'
@@ -115,12 +114,10 @@ quantize4_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
     const int i = threadIdx.x + r * Q4_THREADS;
     const int t = i >> 3, kb = i & 7;                         // token of the block, scale block of the token
     const uint32_t w[8] = {in[r][0].x, in[r][0].y, in[r][0].z, in[r][0].w, in[r][1].x, in[r][1].y, in[r][1].z, in[r][1].w};
-    uint32_t mx = 0u;                                         // max |x| of the pairs (bf16 magnitudes order like integers)
+    uint32_t mx = 0u;                                         // max |x| of the pairs, NaNs left out (an integer maximum would take them)
 #pragma unroll
-    for (int e = 0; e < 8; ++e) mx = __vmaxu2(mx, w[e] & 0x7fff7fffu);
-    float a = __uint_as_float(max(mx << 16, mx & 0xffff0000u));
-    if (a != a)                                               // (a NaN orders above every number)
-      a = amax_without_nan(reinterpret_cast<const uint32_t*>(base + (long long)(lo + t) * s.n + kb * 16));
+    for (int e = 0; e < 8; ++e) mx = max_bf16x2(mx, w[e] & 0x7fff7fffu);
+    const float a = __uint_as_float(max(mx << 16, mx & 0xffff0000u));
     const float u = g_fast && (a == 0.f || a >= 8.077935669463161e-28f)                       // 2^-90
                         ? div_fast(div_fast(a, 6.0f, 0.16666667163372039795f), g, g_rcp)
                         : div_slow(div_slow(a, 6.0f), g);
