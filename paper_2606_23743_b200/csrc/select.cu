@@ -289,6 +289,9 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
       row_ptr[r] = r * p.fixed_n;
       if (r == R - 1) row_ptr[R] = R * p.fixed_n;
     }
+    // (NaN scores are no candidates: the row can come out short; what row_ptr covers is written all the same)
+#pragma unroll 1
+    for (int t = n + lane; t < p.fixed_n; t += 32) out[t] = 0;
   } else {
     out = tmp_idx + (long long)r * p.cap;
     if (lane == 0) counts[r] = n;
@@ -302,8 +305,6 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
     if (sel) out[base + __popc(bal & ((1u << lane) - 1u))] = it * 32 + lane;
     base += __popc(bal);
   }
-  // (NaN scores are no candidates: a row of known length can come out short; what row_ptr covers is written all the same)
-  for (int t = base + lane; t < p.fixed_n; t += 32) out[t] = 0;
 }
 
 // Block scores of one head as a small fp32 GEMM: S[I][J] = scale * <qbar_I, kbar_J>.  A CTA computes a
