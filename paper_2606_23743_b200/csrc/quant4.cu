@@ -80,7 +80,8 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
 // ends are still in the L2; a thread casts four 16-element scale blocks, whose loads are all in flight.  Issue-bound (75 % of
 // the issue slots at 105 us): the divisions are three FMA-pipe operations each, element pairs in packed ones, with true
 // divisions out of line for magnitudes whose residuals could underflow; scales leave through shared memory.  Q and K of
-// 24 heads x 32 760 tokens (403 MB in, 113 MB out): 105 -> 85 us.
+// 24 heads x 32 760 tokens (403 MB in, 113 MB out): 105 -> 85 us alone
+// (in a call at the power cap 94).  Registers matter: with 72 of them, three CTAs per SM, the cast took 102 us.
 __global__ void __launch_bounds__(Q4_THREADS)
 quantize4_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, Strides sq, Strides sk, int H,
                  int N, int Nb, int BH, const uint32_t* __restrict__ amax, uint8_t* __restrict__ q4,
