@@ -104,8 +104,19 @@ class Call:
             self.reads = qkv + [rp, ci, scores]
             self.sets = sets(self.reads, route)
             self.run = lambda: remainder(int(name[-1]))
-        elif name == "step":                           # routing and attention with the remainder, nothing in between
+        elif name == "step_remainder":                 # whole steps: nothing but the library's kernels in between
             self.writes, self.run = [rp, ci, o, lse], lambda: (route(), remainder(1))
+        elif name == "step":
+            self.writes = [rp, ci, o, lse]
+            self.run = lambda: (route(), B.block_sparse_attn_fwd(p, q, k, v, rp, ci, o, lse, st, workspace=aws))
+        elif name == "step_e4m3":
+            self.writes = e4m3 + [rp, ci, o, lse]
+            self.run = lambda: (e4m3_cast(), B.block_select(p8, top, q8, k8, rp, ci, sws, qs, ks),
+                                B.block_sparse_attn_fwd(p8, q8, k8, v, rp, ci, o, lse, st, qs, ks, workspace=aws))
+        elif name == "step_4bit":
+            self.writes = f4 + [rp, ci, o, lse]
+            self.run = lambda: (route(), B.quantize_qk_fp4(p, q, k, *f4, f4_ws),
+                                B.block_sparse_attn_fwd_fp4(p, *f4, v, rp, ci, o, lse, st, aws))
         elif name == "quantize_e4m3":
             self.writes, self.run = e4m3, e4m3_cast
         elif name == "quantize_e4m3_smooth":
@@ -133,10 +144,11 @@ class Call:
 
 NAMES = ["block_select", "block_select_mass", "block_select_noalloc", "block_select_e4m3", "pool_qk", "block_select_pooled",
          "qk_norm_rope_pool", "attention", "attention_simt", "prepared", "dense", "attention_e4m3", "remainder0", "remainder1", "step",
-         "quantize_e4m3", "quantize_e4m3_smooth", "gather", "scatter"]
+         "step_remainder", "step_e4m3", "quantize_e4m3", "quantize_e4m3_smooth", "gather", "scatter"]
+CASES = [(n, b) for n in NAMES for b in (128, 64)] + [(n, 128) for n in ("quantize_4bit", "attention_4bit", "step_4bit")]
 
 
-@pytest.mark.parametrize("name,block", [(n, b) for n in NAMES for b in (128, 64)] + [("quantize_4bit", 128), ("attention_4bit", 128)])
+@pytest.mark.parametrize("name,block", CASES)
 def test_inputs_written_just_before_a_call(name, block):
     c = Call(name, W[block])
     want = []
