@@ -23,7 +23,6 @@ void sva_debug_set_prof_buffer(void* buf);
 
 /*
  * Kernel behaviour switches for the next attention launches (0 = normal operation).
- *   bit 0: skip the exponentials (tuning aid: timing only, results are wrong);
  *   bit 4: test aid: the K producer withholds a row's tiles after the first, so that a bounded pipeline wait
  *          runs out and the kernel takes its give-up path (SVA_DEV_TIMEOUT) -- nothing faults or hangs.
  *   bit 5: measurement aid: bf16 attention reads V where it lies (MN-major operand) instead of the transposed copy;

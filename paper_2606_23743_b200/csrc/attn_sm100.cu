@@ -1,18 +1,15 @@
 // Block-sparse / dense attention forward for sm_100a (tcgen05 / TMEM / TMA): every MMA of one form.
 // (Paper: critical blocks "computed exactly"; dense fallback.)
 //
-// The tensor pipe drains (~280 cycles, measured) whenever two consecutive MMAs differ in kind:
-// A operand from shared memory vs tensor memory, or another instruction descriptor.  Here both
-// S = Q K^T and O += P V have the same form -- A from TENSOR memory (Q resp. P, bf16 pairs), B
-// from shared memory, K-major, M = N = 128 -- so the pipe never drains:
+// S = Q K^T and O += P V both take A from TENSOR memory (Q resp. P, bf16 pairs) and B from shared memory, M = N = 128:
 //   * Q is written into TMEM once per row by the softmax threads (128-token blocks: by the group that finishes
 //     the row first, about a tile before the row ends, from a tile that TMA has put into the group's idle output
 //     staging panel; otherwise by both groups in the epilogue, straight from global memory);
 //   * V: in the two-step form it is consumed transposed (V^T tiles: d rows, keys contiguous) from a tiled transposed
-//     copy that a small kernel writes into the caller's workspace first, so that P V has the form of S.  The one-call
-//     entry points read V where it lies instead (template switch VMN: an MN-major B operand, a second instruction
-//     descriptor): the pipe is idle often enough for the switch to cost 1 % of the cycles, and the step is faster
-//     without the copy's pass over the HBM.
+//     copy that a small kernel writes into the caller's workspace first.  The one-call entry points read V where it lies
+//     instead (template switch VMN: an MN-major B operand, a second instruction descriptor), without the copy's pass over
+//     the HBM.  (MMAs of either kind, in any order, keep the pipe full: 8 + 8 of them take 1 024 cycles issued back to back,
+//     whether A comes from tensor or shared memory and B is K- or MN-major.)
 // The kernel is persistent: one CTA per SM takes rows (one row = one query block of one head, 128
 // query rows) from a device-wide counter until none is left.  All barriers keep running across rows
 // (every role derives the same phase counters from the same row sequence), so the producers run
@@ -20,8 +17,11 @@
 //   warps 0-3, 4-7  two softmax warpgroups; they take the kept key blocks alternately (even / odd
 //                   position in the row's list); thread <-> query row <-> TMEM lane
 //   warp  8         producer of the K tiles (TMA, one lane)
-//   warp  9         issues the Q K^T MMAs (one lane); owns the TMEM allocation
-//   warp  10        issues the P V MMAs (one lane)
+//   warp  9         issues the Q K^T MMAs; owns the TMEM allocation
+//   warp  10        issues the P V MMAs
+// The issuing warps run their loops with all lanes and let one elected lane execute the MMA: descriptors and addresses then stay in
+// uniform registers, and eight MMAs leave the warp in about 100 cycles; with a loop of one lane they took 400, and some 700 beside
+// busy softmax warps -- longer than the 512 cycles that they execute, in the P V -> P store -> P V chain.
 //   warp  11        producer of the V^T tiles (TMA, one lane)
 // TMEM columns: S of even blocks 0..127, S of odd blocks 128..255, O 256..383, Q 384..447 (bf16
 // pairs), P 448..511 (bf16 pairs).  Because P has columns of its own, an S buffer is free again as
@@ -30,12 +30,21 @@
 // completed, which also staggers the two warpgroups so that one group's exponentials overlap the
 // other group's maximum pass and stores.
 //
-// The two warpgroups share one O accumulator, so they share the reference exponent of every row:
-// the group working on block j takes the reference left by block j-1 (published through shared
-// memory right after that block's row-maximum pass), raises it only when the new row maximum
-// exceeds it by more than 2^LAZY_LOG2, and in that (rare) case rescales its row of O once P V(j-1)
-// has completed.  Row sums are kept per group and merged in the epilogue, where each group
-// normalises its half of O into a swizzled staging panel that one TMA tile store writes out.
+// The two warpgroups share one O accumulator, so they share the reference exponent m of every row (P = 2^(S*c - m)).  A row
+// starts with m = 0, and m is a whole number that changes only when a tile's maximum leaves it far behind (LAZY_LOG2; for the
+// row's first keys FRESH_LOG2): then -- rarely -- the group takes the maximum, rounded up.  A group starts a tile's exponentials
+// with the m that its own last tile ended with; the maximum is taken beside the first of them and looked at afterwards, and
+// the m that the other group ended tile j-1 with is compared when P V(j-1) has completed, just before P is handed over.  Where they
+// differ the larger one wins and P, or O, is scaled by a power of two.  Nothing that is common waits for a maximum or for the other
+// group's (exponentials after maximum and exchange: 1 610 cycles per tile of 128 x 128; this form: 1 480, 32 760 tokens x 24 heads).
+// Row sums are kept per group and merged in the epilogue, where each group normalises its half of O into a swizzled staging
+// panel that one TMA tile store writes out.
+//
+// What bounds the kernel is the softmax groups' instruction stream: 128 exponentials per thread and tile at about 10 cycles
+// each where one warp of a scheduler runs them alone, and instruction fetch -- a scheduler's two softmax warps walk through the
+// tile's straight-line code at different places.  Whatever is rare is therefore kept short or rolled (waits that do not find their
+// phase complete, the change of reference, the epilogue, the zero-fill of empty rows): with the same arithmetic but those
+// expanded in line, warps spent 11 to 20 % of their time waiting for instructions (now 5 %), and the kernel took 7 % longer.
 //
 // e4m3 Q/K (template switch): Q goes into TMEM as bytes (32 columns), a K tile is one 128 x 128-byte
 // panel, S takes four kind::f8f6f4 MMAs (A from TMEM like everything else), and the exponent's scale is
@@ -106,8 +115,7 @@ struct TsParams {
   float log2_block;           // log2(tokens per block): a block mean stands for that many keys
   float tail_bias;            // (log2(keys of the last block) - log2_block) / scale_log2: added to the last block's pooled logit
   long long* prof;            // tuning aid, normally null: entry 319 receives the longest CTA's cycle count
-  int debug;                  // bit0: skip the exponentials (tuning aid, wrong results);
-                              // bit4: starve the pipeline so that a wait runs out (test aid)
+  int debug;                  // bit4: starve the pipeline so that a wait runs out (test aid)
                               // (bit 7 acts in the launcher: the remainder looks kept blocks up in the CSR, without the mask)
 };
 
@@ -122,9 +130,9 @@ constexpr int OFF_K = 0;
 constexpr int OFF_V = OFF_K + KS * TILE;
 constexpr int OFF_O = OFF_V + VS * TILE;    // output staging: two [128 rows][128 B] panels (one per softmax group)
 constexpr int OFF_CTRL = OFF_O + TILE;      // 6 tiles = 192 KB
-constexpr int CTRL_BYTES = 256 + 2 * 128 * 4 + 4 * 128 * 4 + 256;   // barriers, reference exponents, row sums (two rows), row queue
-constexpr int OFF_Q4 = OFF_CTRL + 4096;     // 4-bit variant: the row's Q codes (8 KB) and their scale factors (1 KB)
-constexpr int OFF_QS = OFF_CTRL + 4096;     // bf16, 128-token blocks: staging of the second half (d 64..127) of a row's Q tile (16 KB)
+constexpr int CTRL_BYTES = 6144;            // barriers, row queue, reference exponents and row sums (two rows of each)
+constexpr int OFF_Q4 = OFF_CTRL + CTRL_BYTES;   // 4-bit variant: the row's Q codes (8 KB) and their scale factors (1 KB)
+constexpr int OFF_QS = OFF_CTRL + CTRL_BYTES;     // bf16, 128-token blocks: staging of the second half (d 64..127) of a row's Q tile (16 KB)
 #ifdef SVA_TIMELINE
 constexpr int OFF_KMASK = OFF_QS + 16384;   // remainder: kept-block bit masks, [8 rows in flight][32 words]
 constexpr int SMEM_BYTES = OFF_KMASK + 1024 + 1024 + 1400 * 8;
@@ -134,17 +142,21 @@ constexpr int SMEM_BYTES = OFF_KMASK + 1024 + 1024;          // + alignment slac
 #endif
 constexpr uint32_t COL_SFA = 384, COL_SFB = 392;              // 4-bit variant: scale factors in the Q columns (8 + 2 x 8)
 constexpr uint32_t COL_O = 256, COL_Q = 384, COL_P = 448;
-// The reference exponent of a row is raised only when a block's maximum exceeds it by more than this
-// many powers of two.  P then reaches at most 2^32 and a row sum 2^32 * N: far inside fp32 (and bf16
-// has fp32's exponent range), while raises -- each one a pass over the row's O accumulator -- become rare.
-constexpr float LAZY_LOG2 = 32.0f;
+// The reference exponent of a row is raised only when a block's maximum exceeds it by more than LAZY_LOG2 powers of two, and
+// set for the row's first keys only when their maximum is further than FRESH_LOG2 from the 0 that it starts with.  P then
+// reaches at most 2^48 and a row sum 2^48 * N: far inside fp32 (and bf16 has fp32's exponent range), and a change -- half a
+// tile's worth of cycles -- is rare: logits (in powers of two) of 32 760 tokens x 24 heads reach 21 and of sharper ones (Q and K
+// times 1.5) 49, with first maxima of 19 and 40.  (16 and 32 in their place: 10.0 instead of 9.7 M cycles on the latter.)
+constexpr float LAZY_LOG2 = 48.0f;
+constexpr float FRESH_LOG2 = 40.0f;
 }  // namespace ts
 
 // control block (bytes from OFF_CTRL):
-//   0 q_ready | 8 o_free | 16 s_full[2] | 32 p_full[2] | 48 pv_done[2] | 64 ref_ready[2] | 80 xch
+//   0 q_ready | 8 o_free | 16 s_full[2] | 32 p_full[2] | 48 pv_done[2] | 64 ref_first | 80 xch
 //   96 s_free[2] | 112 k_full[3] | 136 k_empty[3] | 160 v_full[3] | 184 v_empty[3]
-//   216 tmem_base | 220 abort | 224 o_staged[2] | 240 q_staged | 256 ref[2][128] floats | 1280 lx[2 rows][2][128] floats
-//   3328 row queue: QD entries {row, count, start, first entry, second entry, -, -, -} | 3456 rq_full[QD] | 3488 rq_empty[QD]
+//   216 tmem_base | 220 abort | 224 o_staged[2] | 240 q_staged | 256 rq_full[QD] | 288 rq_empty[QD]
+//   320 row queue: QD entries {row, count, start, first entry, second entry, tile of its head, head, batch item}
+//   512 ref[2 rows][2][128] floats | 2560 lx[2 rows][2][128] floats | 4608 lt[2 rows][128] floats
 
 // Work list of row r (a 128-query tile): count and start; returns false for a corrupt row_ptr pair.
 // 128-token blocks: the CSR row itself.  A pair that is not monotone, longer than Nb, negative or that
@@ -181,7 +193,7 @@ __device__ __forceinline__ bool entry_is_first_order(uint32_t e) {
 }
 // Entry j of a work list.  128-token blocks: the key block (an out-of-range entry is replaced by block 0;
 // the producer reports it).  64-token blocks: the tile descriptor.
-template <bool B64, bool REM = false>
+template <bool B64, bool REM = false, bool RAW = false>
 __device__ __forceinline__ uint32_t list_block(const TsParams& prm, int beg, int j, int n_own = 0) {
   if (REM && j >= n_own + prm.np) return (B64 ? 0xfffe0000u : 0x40000000u) | (uint32_t)(j - n_own - prm.np);
   if (REM && j >= n_own) return (B64 ? 0xffff0000u : 0x80000000u) | (uint32_t)(j - n_own);
@@ -194,7 +206,7 @@ __device__ __forceinline__ uint32_t list_block(const TsParams& prm, int beg, int
   }
   if (prm.row_ptr == nullptr) return (uint32_t)j;
   const int J = __ldg(prm.col_idx + beg + j);
-  return (J < 0 || J >= prm.Nb) ? 0u : (uint32_t)J;
+  return !RAW && (J < 0 || J >= prm.Nb) ? 0u : (uint32_t)J;
 }
 
 // -inf into the columns [from, to) of this warp's lanes; to is a multiple of 8.  Eight columns per store: with one per store
@@ -259,12 +271,13 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const uint32_t bar_q_ready = cb + 0, bar_o_free = cb + 8, bar_s_full = cb + 16, bar_p_full = cb + 32,
                  bar_pv_done = cb + 48, bar_ref = cb + 64, bar_xch = cb + 80, bar_s_free = cb + 96,
                  bar_k_full = cb + 112, bar_k_empty = cb + 136, bar_v_full = cb + 160, bar_v_empty = cb + 184,
-                 bar_ost = cb + 224, bar_qs = cb + 240, bar_rq_full = cb + 3456, bar_rq_empty = cb + 3488;
+                 bar_ost = cb + 224, bar_qs = cb + 240, bar_rq_full = cb + 256, bar_rq_empty = cb + 288;
   volatile uint32_t* tmem_base_p = reinterpret_cast<volatile uint32_t*>(ctrl + 216);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(ctrl + 220);
-  volatile float* ref = reinterpret_cast<volatile float*>(ctrl + 256);      // [2][128]
-  volatile float* lx = reinterpret_cast<volatile float*>(ctrl + 1280);      // [2][2][128]
-  volatile int* rowq = reinterpret_cast<volatile int*>(ctrl + 3328);        // [QD][8]
+  volatile int* rowq = reinterpret_cast<volatile int*>(ctrl + 320);         // [QD][8]
+  volatile float* ref = reinterpret_cast<volatile float*>(ctrl + 512);      // [2 rows][2][128]
+  volatile float* lx = reinterpret_cast<volatile float*>(ctrl + 2560);      // [2 rows][2][128]
+  volatile float* ltop = reinterpret_cast<volatile float*>(ctrl + 4608);    // [2 rows][128]: group 1's l_top
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int Nb = prm.Nt;             // row index arithmetic: rows per head
@@ -283,12 +296,12 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     mbar_init(bar_q_ready, (!F4 && !B64) ? 128 : 256);   // (128-token blocks, bf16 / e4m3 Q: one softmax group writes a row's Q)
     mbar_init(bar_o_free, 256);
     mbar_init(bar_xch, 256);
+    mbar_init(bar_ref, 128);
     mbar_init(bar_qs, 1);
     for (int w = 0; w < 2; ++w) {
       mbar_init(bar_s_full + 8 * w, 1);
       mbar_init(bar_p_full + 8 * w, 128);
       mbar_init(bar_pv_done + 8 * w, 1);
-      mbar_init(bar_ref + 8 * w, 128);
       mbar_init(bar_s_free + 8 * w, 128);
       mbar_init(bar_ost + 8 * w, 128);
     }
@@ -326,15 +339,20 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 
   // Entry i of the row sequence (the same for every role): false when a wait ran out.  r >= R ends the
   // sequence.  `arrive` tells whether this thread signs the entry off (one thread per consumer).
-  auto fetch_row = [&](uint32_t i, int& r, int& n, int& beg, uint32_t& e0, uint32_t& e1, bool arrive) -> bool {
+  // (the row's coordinates come with it: dividing r by the rows per head costs a softmax group some 300 cycles)
+  struct Row { int r, n, beg; uint32_t e0, e1; int I, hh, bb; };
+  auto fetch_row = [&](uint32_t i, Row& R, bool arrive) -> bool {
     const uint32_t slot = i % QD;
-    if (!mbar_wait(bar_rq_full + 8 * slot, (i / QD) & 1u, abort_flag, prm.status)) return false;
-    r = rowq[8 * slot];
-    n = rowq[8 * slot + 1];
-    beg = rowq[8 * slot + 2];
-    e0 = (uint32_t)rowq[8 * slot + 3];
-    e1 = (uint32_t)rowq[8 * slot + 4];
-    if (warp < 8) __syncwarp();                  // softmax warps: every lane has read the entry before lane 0 signs
+    if (!mbar_wait(bar_rq_full + 8 * slot, (i / QD) & 1u, abort_flag)) return false;
+    R.r = rowq[8 * slot];
+    R.n = rowq[8 * slot + 1];
+    R.beg = rowq[8 * slot + 2];
+    R.e0 = (uint32_t)rowq[8 * slot + 3];
+    R.e1 = (uint32_t)rowq[8 * slot + 4];
+    R.I = rowq[8 * slot + 5];
+    R.hh = rowq[8 * slot + 6];
+    R.bb = rowq[8 * slot + 7];
+    if (warp < 8 || warp == 9 || warp == 10) __syncwarp();   // whole warps: every lane has read the entry before lane 0 signs
     if (arrive) mbar_arrive(bar_rq_empty + 8 * slot);
     return true;
   };
@@ -351,7 +369,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         for (uint32_t i = 0; ok; ++i) {
           // ---- row scheduling: draw the next row with a non-empty list and publish it
           const uint32_t slot = i % QD;
-          if (i >= QD && !mbar_wait(bar_rq_empty + 8 * slot, (i / QD - 1u) & 1u, abort_flag, prm.status)) break;
+          if (i >= QD && !mbar_wait(bar_rq_empty + 8 * slot, (i / QD - 1u) & 1u, abort_flag)) break;
           int r, n = 0, beg = 0;
           for (;;) {
             r = atomicAdd(prm.next_row, 1);
@@ -360,15 +378,18 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             if (n > 0) break;
             // nothing kept (or a corrupt row_ptr pair): zeros and lse = -inf; rare, so this one lane does it
             const int I = r % Nb, bh0 = r / Nb;
+#pragma unroll 1
             for (int t = 0; t < BS; ++t) {
               const int qi = I * BS + t;
               if (qi >= prm.N) break;
               __nv_bfloat16* orow = prm.o + (long long)(bh0 / prm.H) * prm.so.b + (long long)(bh0 % prm.H) * prm.so.h +
                                     (long long)qi * prm.so.n;
+#pragma unroll 1
               for (int cc = 0; cc < prm.d; cc += 8) *reinterpret_cast<uint4*>(orow + cc) = make_uint4(0, 0, 0, 0);
               if (prm.lse) prm.lse[(long long)bh0 * prm.N + qi] = -INFINITY;
             }
           }
+          const int I = r % Nb, bh = r / Nb, hh = bh % prm.H, bb = bh / prm.H;
           uint32_t e0 = 0u, e1 = 0u;
           const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);        // entries of the row's own list
           if (r < prm.R) { e0 = list_block<B64, REM>(prm, beg, 0, n_own); if (n > 1) e1 = list_block<B64, REM>(prm, beg, 1, n_own); }
@@ -377,14 +398,13 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             // contiguous ([B,N,H,d], a packed projection) go as a tensor prefetch: with a plain one per token row this lane
             // spent about 9 000 cycles per row in which no K tile was on its way (32 760 tokens x 24 heads, 40 blocks kept:
             // 3.08 M cycles where [B,H,N,d] took 2.69 M; now the same).
-            const int I = r % Nb, bh0 = r / Nb;
             const uint32_t eb = F8 ? 1u : 2u, row_bytes = (uint32_t)prm.d * eb;
             if (prm.sq.n * (long long)eb == (long long)row_bytes) {
-              const long long q0 = (long long)(bh0 / prm.H) * prm.sq.b + (long long)(bh0 % prm.H) * prm.sq.h + (long long)I * BS * prm.sq.n;
+              const long long q0 = (long long)bb * prm.sq.b + (long long)hh * prm.sq.h + (long long)I * BS * prm.sq.n;
               bulk_prefetch_l2(reinterpret_cast<const uint8_t*>(prm.q) + q0 * eb, (uint32_t)min(BS, prm.N - I * BS) * row_bytes);
             } else {
-              tma_prefetch_4d(&tm_q, 0, I * BS, bh0 % prm.H, bh0 / prm.H);
-              if (!F8) tma_prefetch_4d(&tm_q, 64, I * BS, bh0 % prm.H, bh0 / prm.H);
+              tma_prefetch_4d(&tm_q, 0, I * BS, hh, bb);
+              if (!F8) tma_prefetch_4d(&tm_q, 64, I * BS, hh, bb);
             }
           }
           rowq[8 * slot] = r;
@@ -392,6 +412,9 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           rowq[8 * slot + 2] = beg;
           rowq[8 * slot + 3] = (int)e0;
           rowq[8 * slot + 4] = (int)e1;
+          rowq[8 * slot + 5] = I;
+          rowq[8 * slot + 6] = hh;
+          rowq[8 * slot + 7] = bb;
           mbar_arrive(bar_rq_full + 8 * slot);
           if (r >= prm.R) {
             // Every CTA ends by drawing one value >= R.  The last one to do so puts both counters back to 0,
@@ -403,7 +426,6 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             break;
           }
           // ---- K tiles of the row
-          const int bh = r / Nb, hh = bh % prm.H, bb = bh / prm.H;
           // Remainder (128-token blocks): while walking the row's list this lane leaves a bit mask of the kept blocks
           // for the softmax warps, which mask those columns of the block-mean tiles.  Eight masks in
           // rotation: this lane is at most four tiles (two K slots, two S buffers) -- so at most four rows -- ahead.
@@ -415,7 +437,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           }
           for (int j = 0; j < n; ++j) {
             if ((prm.debug & 16) && j >= 1) { ok = false; break; }   // test aid: starve the pipeline so that a wait runs out
-            if (!mbar_wait(bar_k_empty + 8 * s, ph ^ 1u, abort_flag, prm.status)) { ok = false; break; }
+            if (!mbar_wait(bar_k_empty + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
             const uint32_t dst = sbase + OFF_K + s * TILE;
             mbar_expect_tx(bar_k_full + 8 * s, F4 ? 8192 + 1024 : KTILE);
             if (F4) {
@@ -466,13 +488,12 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         uint32_t ph = 0;
         bool ok = true;
         for (uint32_t i = 0; ok; ++i) {
-          int r, n, beg;
-          uint32_t e0, e1;
-          if (!fetch_row(i, r, n, beg, e0, e1, true) || r >= prm.R) break;
-          const int bh = r / Nb, hh = bh % prm.H, bb = bh / prm.H;
+          Row cur;
+          if (!fetch_row(i, cur, true) || cur.r >= prm.R) break;
+          const int n = cur.n, beg = cur.beg, hh = cur.hh, bb = cur.bb;
           const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);
           for (int j = 0; j < n; ++j) {
-            if (!mbar_wait(bar_v_empty + 8 * s, ph ^ 1u, abort_flag, prm.status)) { ok = false; break; }
+            if (!mbar_wait(bar_v_empty + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
             const uint32_t e = list_block<B64, REM>(prm, beg, j, n_own);
             const uint32_t dst = sbase + OFF_V + s * TILE;
             mbar_expect_tx(bar_v_full + 8 * s, TILE);
@@ -486,7 +507,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
               } else {
                 // first-order tile: A^T (A when V is read keys-major) of the query block (64-token blocks: of the tile
                 // row's first / second one)
-                const int qb = B64 ? min(2 * (r % Nb) + (c - prm.np), prm.Nb - 1) : r % Nb;
+                const int qb = B64 ? min(2 * cur.I + (c - prm.np), prm.Nb - 1) : cur.I;
                 tma_load_4d(dst, &tm_at, bar_v_full + 8 * s, 0, qb * BS, hh, bb);
                 tma_load_4d(dst + TILE / 2, &tm_at, bar_v_full + 8 * s, 64, qb * BS, hh, bb);
               }
@@ -516,103 +537,95 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         }
       }
     } else if (warp == 9) {
-      // ---------------------------------------------------------- S issuer (one lane)
+      // ---------------------------------------------------------- S issuer
       // per row: S(0), S(1), then S(j) into the buffer of S(j-2) as soon as that block's softmax
       // has read it; the first S of a row also needs the row's Q in TMEM
-      if (lane == 0) {
-        const uint64_t kd0 = smem_desc(sbase + OFF_K, 16, 1024);
-        int s = 0;
-        uint32_t ph = 0;
-        uint32_t cs[2] = {0, 0};            // S tiles issued so far into buffer w
-        bool ok = true;
-        for (uint32_t i = 0; ok; ++i) {
-          int r, n, beg;
-          uint32_t e0, e1;
-          if (!fetch_row(i, r, n, beg, e0, e1, true) || r >= prm.R) break;
-          ok = mbar_wait(bar_q_ready, i & 1u, abort_flag, prm.status);
-          for (int j = 0; j < n && ok; ++j) {
-            const int w = j & 1;
-            if (cs[w] > 0) {
-              ok = mbar_wait(bar_s_free + 8 * w, (cs[w] - 1u) & 1u, abort_flag, prm.status);
-              if (!ok) break;
+      const uint32_t el = elect_one();
+      const uint64_t kd0 = smem_desc(sbase + OFF_K, 16, 1024);
+      int s = 0;
+      uint32_t ph = 0;
+      uint32_t cs[2] = {0, 0};            // S tiles issued so far into buffer w
+      for (uint32_t i = 0;; ++i) {
+        Row cur;
+        bool ok = fetch_row(i, cur, lane == 0) && cur.r < prm.R;
+        ok = ok && mbar_wait(bar_q_ready, i & 1u, abort_flag);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        const int n = __shfl_sync(0xffffffffu, cur.n, 0);
+        for (int j = 0; j < n; ++j) {
+          const int w = j & 1;
+          if (cs[w] > 0) mbar_wait(bar_s_free + 8 * w, (cs[w] - 1u) & 1u, abort_flag);
+          if (lane == 0) SVA_STAMP(2, i, j, 0);
+          mbar_wait(bar_k_full + 8 * s, ph, abort_flag);
+          if (lane == 0) SVA_STAMP(2, i, j, 1);
+          tc_fence_after();
+          const uint64_t kd = kd0 + (uint64_t)(s * (TILE >> 4));
+          if (F4) {
+            const uint32_t kslot = sbase + OFF_K + s * TILE;
+            if (j == 0) {                                    // the row's Q scale factors (q_ready: they are in shared memory)
+              tc_cp_sf(tmem_base + COL_SFA, smem_desc_plain(sbase + OFF_Q4 + 8192), el);
+              tc_cp_sf(tmem_base + COL_SFA + 4, smem_desc_plain(sbase + OFF_Q4 + 8192 + 512), el);
             }
-            SVA_STAMP(2, i, j, 0);
-            ok = mbar_wait(bar_k_full + 8 * s, ph, abort_flag, prm.status);
-            if (!ok) break;
-            SVA_STAMP(2, i, j, 1);
-            tc_fence_after();
-            const uint64_t kd = kd0 + (uint64_t)(s * (TILE >> 4));
-            if (F4) {
-              const uint32_t kslot = sbase + OFF_K + s * TILE;
-              if (j == 0) {                                    // the row's Q scale factors (q_ready: they are in shared memory)
-                tc_cp_sf(tmem_base + COL_SFA, smem_desc_plain(sbase + OFF_Q4 + 8192), 1u);
-                tc_cp_sf(tmem_base + COL_SFA + 4, smem_desc_plain(sbase + OFF_Q4 + 8192 + 512), 1u);
-              }
-              tc_cp_sf(tmem_base + COL_SFB + 8 * s, smem_desc_plain(kslot + 8192), 1u);
-              tc_cp_sf(tmem_base + COL_SFB + 8 * s + 4, smem_desc_plain(kslot + 8192 + 512), 1u);
-              const uint64_t qd4 = smem_desc_sw64(sbase + OFF_Q4), kd4 = smem_desc_sw64(kslot);
+            tc_cp_sf(tmem_base + COL_SFB + 8 * s, smem_desc_plain(kslot + 8192), el);
+            tc_cp_sf(tmem_base + COL_SFB + 8 * s + 4, smem_desc_plain(kslot + 8192 + 512), el);
+            const uint64_t qd4 = smem_desc_sw64(sbase + OFF_Q4), kd4 = smem_desc_sw64(kslot);
 #pragma unroll
-              for (int kk = 0; kk < 2; ++kk)                    // 64 elements (32 bytes) of d per instruction
-                tc_mma_bs4_ss(tmem_base + 128 * w, qd4 + (uint64_t)(kk * 2), kd4 + (uint64_t)(kk * 2), instr_desc_bs4(128, 128),
-                              tmem_base + COL_SFA + 4 * kk, tmem_base + COL_SFB + 8 * s + 4 * kk, kk > 0 ? 1u : 0u, 1u);
-            } else if (F8) {
+            for (int kk = 0; kk < 2; ++kk)                    // 64 elements (32 bytes) of d per instruction
+              tc_mma_bs4_ss(tmem_base + 128 * w, qd4 + (uint64_t)(kk * 2), kd4 + (uint64_t)(kk * 2), instr_desc_bs4(128, 128),
+                            tmem_base + COL_SFA + 4 * kk, tmem_base + COL_SFB + 8 * s + 4 * kk, kk > 0 ? 1u : 0u, el);
+          } else if (F8) {
 #pragma unroll
-              for (int kk = 0; kk < D / 32; ++kk)               // 32 e4m3 values (32 bytes, 8 TMEM columns) per step
-                tc_mma_ts<true>(tmem_base + 128 * w, tmem_base + COL_Q + 8 * kk, kd + (uint64_t)(kk * 2), IDESC_QK,
-                                kk > 0 ? 1u : 0u, 1u);
-            } else {
+            for (int kk = 0; kk < D / 32; ++kk)               // 32 e4m3 values (32 bytes, 8 TMEM columns) per step
+              tc_mma_ts<true>(tmem_base + 128 * w, tmem_base + COL_Q + 8 * kk, kd + (uint64_t)(kk * 2), IDESC_QK,
+                              kk > 0 ? 1u : 0u, el);
+          } else {
 #pragma unroll
-              for (int kk = 0; kk < D / 16; ++kk) {
-                const uint64_t off = (uint64_t)((kk / 4) * PANEL16 + (kk % 4) * 2);
-                tc_mma_ts(tmem_base + 128 * w, tmem_base + COL_Q + 8 * kk, kd + off, IDESC, kk > 0 ? 1u : 0u, 1u);
-              }
+            for (int kk = 0; kk < D / 16; ++kk) {
+              const uint64_t off = (uint64_t)((kk / 4) * PANEL16 + (kk % 4) * 2);
+              tc_mma_ts(tmem_base + 128 * w, tmem_base + COL_Q + 8 * kk, kd + off, IDESC, kk > 0 ? 1u : 0u, el);
             }
-            tc_commit(bar_k_empty + 8 * s, 1u);
-            SVA_STAMP(2, i, j, 2);
-            tc_commit(bar_s_full + 8 * w, 1u);
-            ++cs[w];
-            if (++s == KS) { s = 0; ph ^= 1u; }
           }
+          tc_commit(bar_k_empty + 8 * s, el);
+          if (lane == 0) SVA_STAMP(2, i, j, 2);
+          tc_commit(bar_s_full + 8 * w, el);
+          ++cs[w];
+          if (++s == KS) { s = 0; ph ^= 1u; }
         }
       }
     } else {
-      // ---------------------------------------------------------- P V issuer (one lane)
-      if (lane == 0) {
-        // (VMN: 64 d-values contiguous, the next 64 one panel = 16 KB on, 8 keys 1 KB apart)
-        const uint64_t vd0 = VMN ? smem_desc(sbase + OFF_V, TILE / 2, 1024) : smem_desc(sbase + OFF_V, 16, 1024);
-        constexpr uint32_t IDESC_PV = VMN ? instr_desc(128, 128, 1, true) : IDESC;
-        int s = 0;
-        uint32_t ph = 0;
-        uint32_t cp[2] = {0, 0};            // P V groups issued so far for parity w
-        bool ok = true;
-        for (uint32_t i = 0; ok; ++i) {
-          int r, n, beg;
-          uint32_t e0, e1;
-          if (!fetch_row(i, r, n, beg, e0, e1, true) || r >= prm.R) break;
-          // the first P V of a row overwrites O: the previous row's O must have been read
-          if (i > 0) ok = mbar_wait(bar_o_free, (i - 1u) & 1u, abort_flag, prm.status);
-          for (int j = 0; j < n && ok; ++j) {
-            const int w = j & 1;
-            const uint64_t vd = vd0 + (uint64_t)(s * (TILE >> 4));
-            ok = mbar_wait(bar_p_full + 8 * w, cp[w] & 1u, abort_flag, prm.status);
-            SVA_STAMP(3, i, j, 0);
-            ok = ok && mbar_wait(bar_v_full + 8 * s, ph, abort_flag, prm.status);
-            if (!ok) break;
-            SVA_STAMP(3, i, j, 1);
-            tc_fence_after();
+      // ---------------------------------------------------------- P V issuer
+      // (VMN: 64 d-values contiguous, the next 64 one panel = 16 KB on, 8 keys 1 KB apart)
+      const uint32_t el = elect_one();
+      const uint64_t vd0 = VMN ? smem_desc(sbase + OFF_V, TILE / 2, 1024) : smem_desc(sbase + OFF_V, 16, 1024);
+      constexpr uint32_t IDESC_PV = VMN ? instr_desc(128, 128, 1, true) : IDESC;
+      int s = 0;
+      uint32_t ph = 0;
+      uint32_t cp[2] = {0, 0};            // P V groups issued so far for parity w
+      for (uint32_t i = 0;; ++i) {
+        Row cur;
+        bool ok = fetch_row(i, cur, lane == 0) && cur.r < prm.R;
+        // the first P V of a row overwrites O: the previous row's O must have been read
+        if (i > 0) ok = ok && mbar_wait(bar_o_free, (i - 1u) & 1u, abort_flag);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        const int n = __shfl_sync(0xffffffffu, cur.n, 0);
+        for (int j = 0; j < n; ++j) {
+          const int w = j & 1;
+          const uint64_t vd = vd0 + (uint64_t)(s * (TILE >> 4));
+          mbar_wait(bar_v_full + 8 * s, ph, abort_flag);
+          if (lane == 0) SVA_STAMP(3, i, j, 0);
+          mbar_wait(bar_p_full + 8 * w, cp[w] & 1u, abort_flag);
+          if (lane == 0) SVA_STAMP(3, i, j, 1);
+          tc_fence_after();
 #pragma unroll
-            for (int kk = 0; kk < BS / 16; ++kk) {
-              const uint64_t off = VMN ? (uint64_t)(kk * 128)            // 16 keys = 16 rows of 128 bytes
-                                       : (uint64_t)((kk / 4) * PANEL16 + (kk % 4) * 2);
-              tc_mma_ts(tmem_base + COL_O, tmem_base + COL_P + 8 * kk, vd + off, IDESC_PV, (j > 0 || kk > 0) ? 1u : 0u, 1u);
-            }
-            SVA_STAMP(3, i, j, 2);
-            tc_commit(bar_v_empty + 8 * s, 1u);
-            tc_commit(bar_pv_done + 8 * w, 1u);
-            if (!ok) break;
-            ++cp[w];
-            if (++s == VS) { s = 0; ph ^= 1u; }
+          for (int kk = 0; kk < BS / 16; ++kk) {
+            const uint64_t off = VMN ? (uint64_t)(kk * 128)            // 16 keys = 16 rows of 128 bytes
+                                     : (uint64_t)((kk / 4) * PANEL16 + (kk % 4) * 2);
+            tc_mma_ts(tmem_base + COL_O, tmem_base + COL_P + 8 * kk, vd + off, IDESC_PV, (j > 0 || kk > 0) ? 1u : 0u, el);
           }
+          if (lane == 0) SVA_STAMP(3, i, j, 2);
+          tc_commit(bar_pv_done + 8 * w, el);
+          tc_commit(bar_v_empty + 8 * s, el);
+          ++cp[w];
+          if (++s == VS) { s = 0; ph ^= 1u; }
         }
       }
     }
@@ -636,13 +649,13 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     bool ok = true;
 
     // this group's half (d columns 64w..64w+63) of a row's Q: global -> registers -> TMEM
-    auto load_q = [&](int r, uint32_t* qv) {
+    auto load_q = [&](const Row& R, uint32_t* qv) {
 #pragma unroll
       for (int e = 0; e < 32; ++e) qv[e] = 0u;
-      if (F4 || r >= prm.R) return;                                     // (4-bit variant: the Q tile goes to shared memory by TMA)
-      const int bh = r / Nb, qi = (r % Nb) * BS + row;
+      if (F4 || R.r >= prm.R) return;                                   // (4-bit variant: the Q tile goes to shared memory by TMA)
+      const int qi = R.I * BS + row;
       if (qi >= prm.N || 64 * w >= prm.d) return;                      // (d = 64: the second group's half of Q is zero)
-      const long long eoff = (long long)(bh / prm.H) * prm.sq.b + (long long)(bh % prm.H) * prm.sq.h +
+      const long long eoff = (long long)R.bb * prm.sq.b + (long long)R.hh * prm.sq.h +
                              (long long)qi * prm.sq.n + 64 * w;           // in elements
       const uint4* src = F8 ? reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(prm.q) + eoff)
                             : reinterpret_cast<const uint4*>(prm.q + eoff);
@@ -652,15 +665,14 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         qv[4 * e] = u.x; qv[4 * e + 1] = u.y; qv[4 * e + 2] = u.z; qv[4 * e + 3] = u.w;
       }
     };
-    auto store_q = [&](const uint32_t* qv, int r) {
+    auto store_q = [&](const uint32_t* qv, const Row& R) {
       if (F4) {
         // one thread fetches the row's Q codes and scale factors; the barrier completes when every softmax thread
         // has arrived (none of them reads the previous row's Q any more) and the bytes have landed
         if (threadIdx.x == 0) {
-          const int bh = r / Nb, I = r % Nb;
           mbar_expect_tx_only(bar_q_ready, 8192 + 1024);
-          tma_load_4d(sbase + OFF_Q4, &tm_kp, bar_q_ready, 0, I * BS, bh % prm.H, bh / prm.H);
-          bulk_load(sbase + OFF_Q4 + 8192, prm.q_sf + ((long long)bh * prm.Nb + I) * 1024, 1024, bar_q_ready);
+          tma_load_4d(sbase + OFF_Q4, &tm_kp, bar_q_ready, 0, R.I * BS, R.hh, R.bb);
+          bulk_load(sbase + OFF_Q4 + 8192, prm.q_sf + ((long long)(R.bb * prm.H + R.hh) * prm.Nb + R.I) * 1024, 1024, bar_q_ready);
         }
         mbar_arrive(bar_q_ready);
         return;
@@ -681,15 +693,14 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // the control block, both loads in flight together; each thread then copies its row from shared memory into
     // tensor memory.  `use` counts these copies over the CTA's rows (the first row's is copy 0): the barrier's phase.
     constexpr bool EARLYQ = !F4 && !B64;
-    auto copy_q = [&](int r, uint32_t use) -> bool {
-      const int bh = r / Nb, I = r % Nb;
+    auto copy_q = [&](const Row& R, uint32_t use) -> bool {
       if ((threadIdx.x & 127) == 0) {
         bulk_wait_read0();                                                // my previous output store has read the panel
         mbar_expect_tx(bar_qs, F8 ? TILE / 2 : TILE);
-        tma_load_4d(sbase + OFF_O + w * (TILE / 2), &tm_q, bar_qs, 0, I * BS, bh % prm.H, bh / prm.H);
-        if (!F8) tma_load_4d(sbase + OFF_QS, &tm_q, bar_qs, 64, I * BS, bh % prm.H, bh / prm.H);
+        tma_load_4d(sbase + OFF_O + w * (TILE / 2), &tm_q, bar_qs, 0, R.I * BS, R.hh, R.bb);
+        if (!F8) tma_load_4d(sbase + OFF_QS, &tm_q, bar_qs, 64, R.I * BS, R.hh, R.bb);
       }
-      if (!mbar_wait(bar_qs, use & 1u, abort_flag, prm.status)) return false;
+      if (!mbar_wait(bar_qs, use & 1u, abort_flag)) return false;
       tc_fence_after();
 #pragma unroll
       for (int ps = 0; ps < (F8 ? 1 : 2); ++ps) {
@@ -713,27 +724,27 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // read in the epilogue (the producer has published it by then: it runs about two blocks ahead),
     // so the next row's Q and first list entries are at hand when the row changes.
     const bool signs = lane == 0;                             // one lane per warp signs queue entries off
-    int r_c = prm.R, n_c = 0, beg_c = 0;
-    uint32_t e0_c = 0u, e1_c = 0u;
-    if (!fetch_row(0, r_c, n_c, beg_c, e0_c, e1_c, signs)) ok = false;
+    Row nx = {prm.R, 0, 0, 0u, 0u, 0, 0, 0};
+    if (!fetch_row(0, nx, signs)) ok = false;
     if (EARLYQ) {
-      if (ok && r_c < prm.R && w == 1) ok = copy_q(r_c, 0u);
-    } else if (ok && r_c < prm.R) {
+      if (ok && nx.r < prm.R && w == 1) ok = copy_q(nx, 0u);
+    } else if (ok && nx.r < prm.R) {
       // first row: its Q goes in right away
       uint32_t qv[32];
-      load_q(r_c, qv);
-      store_q(qv, r_c);
+      load_q(nx, qv);
+      store_q(qv, nx);
     }
-    for (; ok && r_c < prm.R; ++rows_done) {
-      const int r = r_c, n = n_c, lbeg = beg_c;
-      uint32_t J = (w == 0) ? e0_c : e1_c;                           // my first list entry of the row
-      const int I = r % Nb, bh = r / Nb;
-      const int hh = bh % prm.H, bb = bh / prm.H;
+    for (; ok && nx.r < prm.R; ++rows_done) {
+      const int r = nx.r, n = nx.n, lbeg = nx.beg;
+      uint32_t J = (w == 0) ? nx.e0 : nx.e1;                         // my first list entry of the row
+      const int I = nx.I, hh = nx.hh, bb = nx.bb, bh = bb * prm.H + hh;
       const int qi = I * BS + row;
       const int wl = (n - 1) & 1;                                     // group that takes the row's last block
       const uint32_t last = cnt[wl] + (uint32_t)((n - 1) >> 1);       // phase index of that block
-      float m_mine = -INFINITY;      // reference exponent my partial row sum is relative to
+      float m_mine = -0.f;           // reference exponent my partial row sum is relative to (-0: my group has seen no key)
       float l = 0.f;                 // partial row sum over this group's blocks
+      float l_top = 0.f;             // what rounding to bf16 adds to the largest P of each of them
+      volatile float* refr = ref + (rows_done & 1u) * 256;
       float qs_row = 1.f, ks_next = 1.f, ks_next1 = 1.f;
       auto load_ks = [&](uint32_t e) {                                // scales of the key block(s) of list entry e
         const float* ks = prm.k_scale + (long long)bh * prm.Nb;
@@ -780,7 +791,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         }
         if (F8) { c = qs_row * ks_next; if (B64) c1 = qs_row * ks_next1; }
         if (j + 2 < n) {                                               // one entry ahead
-          J = list_block<B64, REM>(prm, lbeg, j + 2, n_own);
+          J = list_block<B64, REM, !F8>(prm, lbeg, j + 2, n_own);
           if (F8) load_ks(J);
         }
         uint4 kept = make_uint4(0u, 0u, 0u, 0u);
@@ -789,8 +800,12 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             kept = __ldg(prm.kept_mask + ((long long)r * 2 + qh) * 8 + pc);
           }
         }
+        if (j == 1) {                                                  // (the row's first reference is group 0's)
+          if (!mbar_wait(bar_ref, rows_done & 1u, abort_flag)) return false;
+          m_mine = refr[row];
+        }
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 0);
-        if (!mbar_wait(bar_s_full + 8 * w, mine & 1u, abort_flag, prm.status)) return false;
+        if (!mbar_wait(bar_s_full + 8 * w, mine & 1u, abort_flag)) return false;
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 1);
         tc_fence_after();
         if (B64 ? (v0 + v1 < BS) : (v0 < BS)) {
@@ -842,106 +857,92 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           }
           tc_wait_st();
         }
-        uint32_t sv[128];
-        tmem_ld32(s_tmem + 0, sv + 0);
-        tmem_ld32(s_tmem + 32, sv + 32);
-        tc_wait_ld();
-        tmem_ld32(s_tmem + 64, sv + 64);
-        tmem_ld32(s_tmem + 96, sv + 96);
-        float mxa = -INFINITY, mxb = -INFINITY, mxc = -INFINITY, mxd = -INFINITY;
-        float mx0, mx1;
-        if (!B64) {
-          // (the first half's maximum while the second half is still on its way from tensor memory)
-#pragma unroll
-          for (int e = 0; e < 64; e += 8) {
-            mxa = max3(mxa, __uint_as_float(sv[e + 0]), __uint_as_float(sv[e + 1]));
-            mxb = max3(mxb, __uint_as_float(sv[e + 2]), __uint_as_float(sv[e + 3]));
-            mxc = max3(mxc, __uint_as_float(sv[e + 4]), __uint_as_float(sv[e + 5]));
-            mxd = max3(mxd, __uint_as_float(sv[e + 6]), __uint_as_float(sv[e + 7]));
-          }
-        }
-        tc_wait_ld();
-        tc_fence_before();
-        mbar_arrive(bar_s_free + 8 * w);                     // the S issuer may refill this buffer
-        if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 2);
-        if (B64) {                                           // a, b: keys 0..63; c, d: keys 64..127
-#pragma unroll
-          for (int e = 0; e < 64; e += 4) {
-            mxa = max3(mxa, __uint_as_float(sv[e + 0]), __uint_as_float(sv[e + 1]));
-            mxb = max3(mxb, __uint_as_float(sv[e + 2]), __uint_as_float(sv[e + 3]));
-            mxc = max3(mxc, __uint_as_float(sv[e + 64]), __uint_as_float(sv[e + 65]));
-            mxd = max3(mxd, __uint_as_float(sv[e + 66]), __uint_as_float(sv[e + 67]));
-          }
-          mx0 = v0 > 0 ? fmaxf(mxa, mxb) : -INFINITY;        // a half this query block does not keep has no say
-          mx1 = v1 > 0 ? fmaxf(mxc, mxd) : -INFINITY;
-        } else {
-#pragma unroll
-          for (int e = 64; e < 128; e += 8) {
-            mxa = max3(mxa, __uint_as_float(sv[e + 0]), __uint_as_float(sv[e + 1]));
-            mxb = max3(mxb, __uint_as_float(sv[e + 2]), __uint_as_float(sv[e + 3]));
-            mxc = max3(mxc, __uint_as_float(sv[e + 4]), __uint_as_float(sv[e + 5]));
-            mxd = max3(mxd, __uint_as_float(sv[e + 6]), __uint_as_float(sv[e + 7]));
-          }
-          mx0 = fmaxf(mxa, mxb);
-          mx1 = fmaxf(mxc, mxd);
-        }
-        // (e4m3 with 64-token blocks: each half has its own scale; a half that is not kept stays -inf)
+        // P = 2^(S*c - m) with the reference m that this group's last tile ended with; the row maximum is taken beside the
+        // first 32 exponentials, in issue slots that they leave empty, and looked at after them: only when it has outgrown m
+        // (or m is still the 0 that a row starts with and the maximum lies far from it) are these 32 done again.
+        // (64-token blocks: -inf instead of -m for a half that is not kept makes those P exactly 0 at no cost)
         // (a pooled logit carries + log2(keys per block): a block mean stands for that many keys)
         const float bias = REM && pooled ? prm.log2_block : 0.f;
-        const float mx = (B64 && F8) ? fmaxf(v0 > 0 ? mx0 * c : -INFINITY, v1 > 0 ? mx1 * c1 : -INFINITY)
-                                     : REM ? fmaxf(mx0, mx1) * c + bias : fmaxf(mx0, mx1) * c;
-        // reference exponent left by block j-1 (other group)
-        float m_prev = -INFINITY;
-        if (j > 0) {
-          if (!mbar_wait(bar_ref + 8 * (w ^ 1), prev & 1u, abort_flag, prm.status)) return false;
-          m_prev = ref[(w ^ 1) * 128 + row];
+        const uint64_t c2 = pack2(c, c), c2h1 = (B64 && F8) ? pack2(c1, c1) : c2;
+        uint32_t sv[128], pv[64];
+        tmem_ld32(s_tmem + 0, sv + 0);
+        tmem_ld32(s_tmem + 32, sv + 32);
+        tc_wait_ld64(sv);
+        tmem_ld32(s_tmem + 64, sv + 64);
+        tmem_ld32(s_tmem + 96, sv + 96);
+        uint64_t nm2, nm2h1, sum2 = pack2(0.f, 0.f);
+        auto set_reference = [&](float m) {
+          float nm = REM ? bias - m : -m, nmh1 = nm;
+          if (B64) {
+            if (v0 == 0) nm = -INFINITY;
+            if (v1 == 0) nmh1 = -INFINITY;
+          }
+          nm2 = pack2(nm, nm);
+          nm2h1 = B64 ? pack2(nmh1, nmh1) : nm2;
+        };
+        auto two_exps = [&](int e) {
+          float x0, x1;
+          unpack2(fma2(pack2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])), e < 64 ? c2 : c2h1, e < 64 ? nm2 : nm2h1), x0, x1);
+          const float p0 = ex2(x0), p1 = ex2(x1);
+          sum2 = add2(sum2, pack2(p0, p1));
+          pv[e / 2] = pack_bf16(p0, p1);
+        };
+        float m_try = m_mine;
+        set_reference(m_try);
+        float mx, top, mx0 = -INFINITY;
+        {
+          float mxa = -INFINITY, mxb = -INFINITY, mxc = -INFINITY, mxd = -INFINITY;
+#pragma unroll
+          for (int e = 0; e < 32; e += 2) {
+            if (e == 16) {
+              if (B64) {
+                mx0 = v0 > 0 ? fmaxf(fmaxf(mxa, mxb), fmaxf(mxc, mxd)) : -INFINITY;     // (a half that is not kept has no say)
+                mxa = mxb = mxc = mxd = -INFINITY;
+              }
+              tc_wait_ld64(sv + 64);
+              tc_fence_before();
+              mbar_arrive(bar_s_free + 8 * w);                       // the S issuer may refill this buffer
+              if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 2);
+            }
+            two_exps(e);
+            const int k = 4 * e;                                       // eight logits' part in the maximum
+            mxa = max3(mxa, __uint_as_float(sv[k + 0]), __uint_as_float(sv[k + 1]));
+            mxb = max3(mxb, __uint_as_float(sv[k + 2]), __uint_as_float(sv[k + 3]));
+            mxc = max3(mxc, __uint_as_float(sv[k + 4]), __uint_as_float(sv[k + 5]));
+            mxd = max3(mxd, __uint_as_float(sv[k + 6]), __uint_as_float(sv[k + 7]));
+          }
+          float mx1 = fmaxf(fmaxf(mxa, mxb), fmaxf(mxc, mxd));
+          if (B64 && v1 == 0) mx1 = -INFINITY;
+          // (e4m3 with 64-token blocks: each half has its own scale; a half that is not kept stays -inf)
+          top = (B64 && F8) ? fmaxf(v0 > 0 ? mx0 * c : -INFINITY, v1 > 0 ? mx1 * c1 : -INFINITY) : fmaxf(mx0, mx1);
+          mx = (B64 && F8) ? top : REM ? top * c + bias : top * c;
+        }
+        const bool fresh = __float_as_uint(m_try) == 0x80000000u;
+        if (__builtin_expect(__any_sync(0xffffffffu, fresh ? fabsf(mx) > FRESH_LOG2 && mx > -INFINITY : mx > m_try + LAZY_LOG2), 0)) {
+          if (fresh ? fabsf(mx) > 8.f && mx > -INFINITY : mx > m_try + 8.f) {
+            const float m_up = ceilf(mx);
+            if (l != 0.f) { const float f = ex2(m_try - m_up); l *= f; l_top *= f; }
+            m_try = m_up;
+          }
+          set_reference(m_try);
+          sum2 = pack2(0.f, 0.f);
+#pragma unroll
+          for (int e = 0; e < 32; e += 2) two_exps(e);
+        }
+        if (mx > -INFINITY) m_try += 0.f;                              // (-0 becomes +0: a key has been seen)
+        // P V sums P rounded to bf16.  Its normaliser takes the largest P of every tile as rounded too, so that a row that is all
+        // but one key comes out as that key's V (as it does where the reference is the row maximum and that P exactly 1).
+        {
+          const float p = ex2((B64 && F8) ? top - m_try : fmaf(top, c, REM ? bias - m_try : -m_try));
+          if (p < INFINITY) l_top += __uint_as_float(pack_bf16(0.f, p) & 0xffff0000u) - p;
+        }
+        if (j == 0) {
+          refr[row] = m_try;
+          mbar_arrive(bar_ref);
         }
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 3);
-        // lazy rule: raise the reference only when the row maximum outgrows it by more than 2^LAZY_LOG2
-        const float m_new = (mx > m_prev + LAZY_LOG2) ? mx : m_prev;
-        ref[w * 128 + row] = m_new;
-        mbar_arrive(bar_ref + 8 * w);
-        if (m_new != m_mine) { l *= ex2(m_mine - m_new); m_mine = m_new; }      // first block: 0 * 2^-inf
-        bool pv_waited = false;
-        if (j > 0 && __any_sync(0xffffffffu, m_new != m_prev)) {
-          // rescale this row of O once P V(j-1) has completed (O is then quiescent: P V(j) waits for us)
-          if (!mbar_wait(bar_pv_done + 8 * (w ^ 1), prev & 1u, abort_flag, prm.status)) return false;
-          pv_waited = true;
-          tc_fence_after();
-          const float alpha = ex2(m_prev - m_new);
-#pragma unroll 1
-          for (int cc = 0; cc < D; cc += 16) {
-            uint32_t ov[16];
-            tmem_ld16(o_tmem + cc, ov);
-            tc_wait_ld();
 #pragma unroll
-            for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * alpha);
-            tmem_st16(o_tmem + cc, ov);
-          }
-          tc_wait_st();
-        }
-        // P = 2^(S*c - m); the packed bf16 pairs overwrite sv[0..63]
-        // (64-token blocks: -inf instead of -m for a half that is not kept, or while the row has seen no
-        // kept key yet, makes those P exactly 0 at no cost)
-        float nm = -m_new, nmh1 = -m_new;
-        if (REM) { nm += bias; nmh1 = nm; }
-        if (B64) {
-          if (m_new == -INFINITY || v0 == 0) nm = -INFINITY;
-          if (m_new == -INFINITY || v1 == 0) nmh1 = -INFINITY;
-        }
-        const uint64_t c2 = pack2(c, c), nm2 = pack2(nm, nm), nm2h1 = B64 ? pack2(nmh1, nmh1) : nm2;
-        const uint64_t c2h1 = (B64 && F8) ? pack2(c1, c1) : c2;
-        uint64_t sum2 = pack2(0.f, 0.f);
-        if (!(prm.debug & 1)) {
-#pragma unroll
-          for (int e = 0; e < 128; e += 2) {
-            float x0, x1;
-            unpack2(fma2(pack2(__uint_as_float(sv[e]), __uint_as_float(sv[e + 1])), e < 64 ? c2 : c2h1, e < 64 ? nm2 : nm2h1), x0, x1);
-            const float p0 = ex2(x0), p1 = ex2(x1);
-            sum2 = add2(sum2, pack2(p0, p1));
-            sv[e / 2] = pack_bf16(p0, p1);
-          }
-        }
+        for (int e = 32; e < 128; e += 2) two_exps(e);
         {
           float sum_a, sum_b;
           unpack2(sum2, sum_a, sum_b);
@@ -950,12 +951,46 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 4);
         // the P columns are free once P V(j-1) has completed (block 0: the previous row's last P V
         // was waited for in that row's epilogue)
-        if (j > 0 && !pv_waited &&
-            !mbar_wait(bar_pv_done + 8 * (w ^ 1), prev & 1u, abort_flag, prm.status)) return false;
-        if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 5);
+        if (j > 0 && !mbar_wait(bar_pv_done + 8 * (w ^ 1), prev & 1u, abort_flag)) return false;
         tc_fence_after();
-        tmem_st32(p_tmem, sv);
-        tmem_st32(p_tmem + 32, sv + 32);
+        tmem_st32(p_tmem, pv);
+        tmem_st32(p_tmem + 32, pv + 32);
+        // The reference that O is relative to: what the other group's tile j-1 ended with.  (Its threads wrote it before they
+        // arrived on p_full, without which P V(j-1) would not have been issued.)
+        const float m_prev = j > 0 ? refr[(w ^ 1) * 128 + row] : m_try;
+        float m_new = __uint_as_float(__float_as_uint(m_prev) & __float_as_uint(m_try));       // (equal, or zeros: -0 only if both are)
+        if (__builtin_expect(__any_sync(0xffffffffu, m_prev != m_try), 0)) {
+          // The larger one wins; O, or P and the row sum, follow (O is quiescent: P V(j) waits for us; P scales exactly,
+          // references being whole numbers).  A reference that no key has confirmed (-0) gives way.
+          const bool seen_o = __float_as_uint(m_prev) != 0x80000000u, seen_p = __float_as_uint(m_try) != 0x80000000u;
+          if (m_prev != m_try) m_new = !seen_o ? m_try : !seen_p ? m_prev : fmaxf(m_prev, m_try);
+          const float fo = !seen_o || m_prev == m_new ? 1.f : ex2(m_prev - m_new);
+          const float fp = !seen_p || m_try == m_new ? 1.f : ex2(m_try - m_new);
+          l *= fp;
+          l_top *= fp;
+          tc_wait_st();
+#pragma unroll 1
+          for (int cc = 0; cc < D / 2; cc += 16) {
+            uint32_t ov[16];
+            tmem_ld16(p_tmem + cc, ov);
+            tc_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) ov[e] = pack_bf16(bf16lo(ov[e]) * fp, bf16hi(ov[e]) * fp);
+            tmem_st16(p_tmem + cc, ov);
+          }
+#pragma unroll 1
+          for (int cc = 0; cc < D && j > 0; cc += 16) {
+            uint32_t ov[16];
+            tmem_ld16(o_tmem + cc, ov);
+            tc_wait_ld();
+#pragma unroll
+            for (int e = 0; e < 16; ++e) ov[e] = __float_as_uint(__uint_as_float(ov[e]) * fo);
+            tmem_st16(o_tmem + cc, ov);
+          }
+        }
+        m_mine = m_new;
+        refr[w * 128 + row] = m_new;
+        if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 5);
         tc_wait_st();
         tc_fence_before();
         mbar_arrive(bar_p_full + 8 * w);
@@ -969,20 +1004,20 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const uint32_t mine = cnt[w] + (uint32_t)(j >> 1), prev = cnt[w ^ 1] + (uint32_t)((j - 1) >> 1);
         const uint32_t J_now = J;
         if (j + 2 < n) J = list_block<B64, REM>(prm, lbeg, j + 2, n_own);
-        if (!mbar_wait(bar_s_full + 8 * w, mine & 1u, abort_flag, prm.status)) return false;
+        if (!mbar_wait(bar_s_full + 8 * w, mine & 1u, abort_flag)) return false;
         mbar_arrive(bar_s_free + 8 * w);
-        if (!mbar_wait(bar_ref + 8 * (w ^ 1), prev & 1u, abort_flag, prm.status)) return false;
-        const float m_now = ref[(w ^ 1) * 128 + row];                 // (j > 0: the row has at least one tile of block means)
-        ref[w * 128 + row] = m_now;
-        mbar_arrive(bar_ref + 8 * w);
-        if (m_now != m_mine) { l *= ex2(m_mine - m_now); m_mine = m_now; }
+        if (!mbar_wait(bar_pv_done + 8 * (w ^ 1), prev & 1u, abort_flag)) return false;
+        tc_fence_after();
+        if (!mbar_wait(bar_p_full + 8 * (w ^ 1), prev & 1u, abort_flag)) return false;
+        const float m_now = refr[(w ^ 1) * 128 + row];                // (j > 0: the row has at least one tile of block means)
+        refr[w * 128 + row] = m_now;
+        if (l != 0.f) { const float f = ex2(m_mine - m_now); l *= f; l_top *= f; }
+        m_mine = m_now;
         const int qb = B64 ? min(2 * I + qh, prm.Nb - 1) : I;
-        const bool mine_rows = (qi < prm.N) && (!B64 || qh == (int)(J_now & 1u)) && m_now != -INFINITY;
+        const bool mine_rows = (qi < prm.N) && (!B64 || qh == (int)(J_now & 1u));
         const float f = mine_rows ? prm.scale_log2 * 0.6931471805599453f *
                                         ex2(__ldg(prm.mu + (long long)bh * prm.Nb + qb) * 1.4426950408889634f - m_now)
                                   : 0.f;
-        if (!mbar_wait(bar_pv_done + 8 * (w ^ 1), prev & 1u, abort_flag, prm.status)) return false;
-        tc_fence_after();
 #pragma unroll 1
         for (int cc = 0; cc < D / 2; cc += 16) {
           uint32_t qv[16];
@@ -1010,70 +1045,80 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       }
       if (!ok) break;
       if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 7);
-      if (EARLYQ && !fetch_row(rows_done + 1u, r_c, n_c, beg_c, e0_c, e1_c, signs)) { ok = false; break; }   // the row after this one, or the end mark
       // ---- epilogue: merge the two groups' row sums, hand the next row's Q to the S issuer,
       // normalise and store (each group half of d)
-      if (!EARLYQ && !fetch_row(rows_done + 1u, r_c, n_c, beg_c, e0_c, e1_c, signs)) { ok = false; break; }   // the row after this one, or the end mark
-      const int r_next = r_c;                                         // (the queue holds non-empty rows only)
+      if (!fetch_row(rows_done + 1u, nx, signs)) { ok = false; break; }   // the row after this one (never an empty one), or the end mark
       uint32_t qn[32];
-      if (!EARLYQ) load_q(r_next, qn);                                // in flight during the waits below
-      if (!mbar_wait(bar_ref + 8 * wl, last & 1u, abort_flag, prm.status)) { ok = false; break; }
-      const float m_fin = ref[wl * 128 + row];
-      if (m_mine != m_fin) { l *= ex2(m_mine - m_fin); m_mine = m_fin; }        // l = 0 for a group without blocks
+      if (!EARLYQ) load_q(nx, qn);                                // in flight during the waits below
       volatile float* lxr = lx + (rows_done & 1u) * 256;
-      lxr[w * 128 + row] = l;
+      lxr[w * 128 + row] = l + l_top;
+      if (w == 1) ltop[(rows_done & 1u) * 128 + row] = l_top;
       if ((threadIdx.x & 127) == 0) bulk_wait_read0();                // the previous row's store has read the staging panel
       mbar_arrive(bar_xch);
       if (EARLYQ && w != wl) {
         // (after this group's row sums are out, so that the other group's epilogue does not wait for the copy)
         // The row's last S tile (the other group's) has been computed, and with it every S of the row: Q is free.
         // (Its barrier's previous phase completed before the S tile this group has just worked on, or in an earlier row.)
-        if (!mbar_wait(bar_s_full + 8 * wl, last & 1u, abort_flag, prm.status)) { ok = false; break; }
+        if (!mbar_wait(bar_s_full + 8 * wl, last & 1u, abort_flag)) { ok = false; break; }
         // (... and a last tile of first order has read it.  Its barrier's previous phase completed before P V of the tile two
         // before it, which this group has waited for.)
-        if (REM && prm.n1 > 0 && !mbar_wait(bar_p_full + 8 * wl, last & 1u, abort_flag, prm.status)) { ok = false; break; }
-        if (r_next < prm.R && !copy_q(r_next, rows_done + 1u)) { ok = false; break; }
+        if (REM && prm.n1 > 0 && !mbar_wait(bar_p_full + 8 * wl, last & 1u, abort_flag)) { ok = false; break; }
+        if (nx.r < prm.R && !copy_q(nx, rows_done + 1u)) { ok = false; break; }
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 8);
       }
-      if (!mbar_wait(bar_xch, rows_done & 1u, abort_flag, prm.status)) { ok = false; break; }
+      if (!mbar_wait(bar_xch, rows_done & 1u, abort_flag)) { ok = false; break; }
       // both groups have seen all their S tiles: no MMA reads Q any more
-      if (!EARLYQ && r_next < prm.R) store_q(qn, r_next);
+      if (!EARLYQ && nx.r < prm.R) store_q(qn, nx);
       if (!EARLYQ && (threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 8);
-      if (!mbar_wait(bar_pv_done + 8 * wl, last & 1u, abort_flag, prm.status)) { ok = false; break; }
+      if (!mbar_wait(bar_pv_done + 8 * wl, last & 1u, abort_flag)) { ok = false; break; }
       if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 9);
       tc_fence_after();
-      const float lt = l + lxr[(w ^ 1) * 128 + row];
+      // The row's final reference is the one its last tile ended with; the other group's sums may be relative to an earlier, lower
+      // one (0 stays 0: a group without keys has no reference).
+      const float m_fin = refr[wl * 128 + row];
+      float f_early = 1.f;
+      {
+        const float m_other = refr[(wl ^ 1) * 128 + row];
+        if (lxr[(wl ^ 1) * 128 + row] != 0.f && m_other != m_fin) f_early = ex2(m_other - m_fin);
+      }
+      const float f0 = wl == 0 ? 1.f : f_early, f1 = wl == 0 ? f_early : 1.f;
+      const float lt = lxr[row] * f0 + lxr[128 + row] * f1;
       // (64-token blocks: a query block with an empty list beside one with work has lt = 0 -> zeros, lse = -inf)
       const float inv = (!B64 || lt > 0.f) ? 1.0f / lt : 0.f;
       {
-        uint32_t ov[64];
-        tmem_ld32(o_tmem + (D / 2) * w, ov);
-        tmem_ld32(o_tmem + (D / 2) * w + 32, ov + 32);
-        tc_wait_ld();
-        tc_fence_before();
-        mbar_arrive(bar_o_free);                                      // the next row may overwrite O
         // normalised bf16 row -> this group's staging panel (128-byte swizzle), then one tile store;
         // rows beyond N are clipped by the tensor map
         uint8_t* stg = smem + OFF_O + w * (TILE / 2) + row * 128;
+#pragma unroll 1
+        for (int cc = 0; cc < D / 2; cc += 16) {
+          uint32_t ov[16];
+          tmem_ld16(o_tmem + (D / 2) * w + cc, ov);
+          tc_wait_ld();
 #pragma unroll
-        for (int e = 0; e < 64; e += 8) {
-          uint4 v4;
-          v4.x = pack_bf16(__uint_as_float(ov[e + 0]) * inv, __uint_as_float(ov[e + 1]) * inv);
-          v4.y = pack_bf16(__uint_as_float(ov[e + 2]) * inv, __uint_as_float(ov[e + 3]) * inv);
-          v4.z = pack_bf16(__uint_as_float(ov[e + 4]) * inv, __uint_as_float(ov[e + 5]) * inv);
-          v4.w = pack_bf16(__uint_as_float(ov[e + 6]) * inv, __uint_as_float(ov[e + 7]) * inv);
-          *reinterpret_cast<uint4*>(stg + (((e >> 3) ^ (row & 7)) << 4)) = v4;
+          for (int e = 0; e < 16; e += 8) {
+            uint4 v4;
+            v4.x = pack_bf16(__uint_as_float(ov[e + 0]) * inv, __uint_as_float(ov[e + 1]) * inv);
+            v4.y = pack_bf16(__uint_as_float(ov[e + 2]) * inv, __uint_as_float(ov[e + 3]) * inv);
+            v4.z = pack_bf16(__uint_as_float(ov[e + 4]) * inv, __uint_as_float(ov[e + 5]) * inv);
+            v4.w = pack_bf16(__uint_as_float(ov[e + 6]) * inv, __uint_as_float(ov[e + 7]) * inv);
+            *reinterpret_cast<uint4*>(stg + ((((cc + e) >> 3) ^ (row & 7)) << 4)) = v4;
+          }
         }
+        tc_fence_before();
+        mbar_arrive(bar_o_free);                                      // the next row may overwrite O
         fence_async_smem();
         mbar_arrive(bar_ost + 8 * w);
         if ((threadIdx.x & 127) == 0) {
           // (a wait that runs out has raised the abort flag; the other threads leave at their next wait)
-          if (mbar_wait(bar_ost + 8 * w, rows_done & 1u, abort_flag, prm.status) && (D / 2) * w < prm.d) {
+          if (mbar_wait(bar_ost + 8 * w, rows_done & 1u, abort_flag) && (D / 2) * w < prm.d) {
             tma_store_4d(&tm_o, sbase + OFF_O + w * (TILE / 2), (D / 2) * w, I * BS, hh, bb);
             bulk_commit();
           }
         }
-        if (qi < prm.N && prm.lse && w == 0) prm.lse[(long long)bh * prm.N + qi] = (m_fin + log2f(lt)) * 0.6931471805599453f;
+        if (qi < prm.N && prm.lse && w == 0) {
+          const float ls = l * f0 + (lxr[128 + row] - ltop[(rows_done & 1u) * 128 + row]) * f1;     // (the sum itself)
+          prm.lse[(long long)bh * prm.N + qi] = B64 || ls != 0.f ? (m_fin + log2f(ls)) * 0.6931471805599453f : NAN;
+        }
       }
       if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 10);
       cnt[0] += (uint32_t)((n + 1) >> 1);
@@ -1096,6 +1141,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   }
   tc_fence_before();
   __syncthreads();
+  if (threadIdx.x == 0 && *abort_flag && prm.status) atomicOr(prm.status, SVA_DEV_TIMEOUT);
   if (warp == 9) {
     tc_fence_after();
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
@@ -1664,8 +1710,8 @@ int launch_attn_ts_fp4(const Dims& m, const sva_problem_t* p, const void* q4, co
 void ts_set_prof_buffer(void* p) { g_prof_ts = (long long*)p; }
 void ts_set_debug_mode(int v) { g_debug_ts = v; }
 int ts_set_wait_limit(long long cycles) {
-  if (cycles <= 0) cycles = WAIT_LIMIT_CYCLES;
-  return cudaMemcpyToSymbol(g_wait_limit, &cycles, sizeof(cycles)) == cudaSuccess ? 0 : 1;
+  const uint32_t limit = cycles <= 0 ? WAIT_LIMIT_CYCLES : (uint32_t)(cycles < 4000000000LL ? cycles : 4000000000LL);
+  return cudaMemcpyToSymbol(g_wait_limit, &limit, sizeof(limit)) == cudaSuccess ? 0 : 1;
 }
 
 }  // namespace sva

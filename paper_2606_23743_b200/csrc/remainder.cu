@@ -14,6 +14,12 @@
 
 namespace sva {
 
+static __device__ __forceinline__ bool wait_or_report(uint32_t bar, uint32_t parity, volatile int* abort_flag, int32_t* status) {
+  if (mbar_wait(bar, parity, abort_flag)) return true;
+  if (status) atomicOr(status, SVA_DEV_TIMEOUT);
+  return false;
+}
+
 namespace rem {
 constexpr int D = 128;
 constexpr int TILE = BS * D * 2;                  // 32 KB: 128 rows x 256 bytes as two 128-byte panels
@@ -61,7 +67,7 @@ cov_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUt
     tma_load_4d(sbase + TILE, &tm_v, bar_full, 0, J * block, hh, bb);
     tma_load_4d(sbase + TILE + panel, &tm_v, bar_full, 64, J * block, hh, bb);
   }
-  bool ok = mbar_wait(bar_full, 0u, abort_flag, status);
+  bool ok = wait_or_report(bar_full, 0u, abort_flag, status);
   if (ok) {
     // column means of the two tiles: thread c owns column c (rows beyond N arrive as zeros)
     const int c = threadIdx.x;
@@ -87,7 +93,7 @@ cov_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUt
     }
   }
   __syncthreads();
-  ok = ok && mbar_wait(bar_mma, 0u, abort_flag, status);
+  ok = ok && wait_or_report(bar_mma, 0u, abort_flag, status);
   if (ok) {
     tc_fence_after();
     const int e = threadIdx.x;                                // TMEM lane = row e of C_J^T
@@ -192,20 +198,20 @@ aggregate_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
     const uint64_t ad = smem_desc(sbase, 16, 1024), bd = smem_desc(sbase + A_BYTES, B_PANEL, 1024);
     const int chunks = Nbw / 64;
     for (int ch = 0; ch < chunks && ok; ++ch) {
-      if (ch > 0) ok = mbar_wait(bar_mma, (uint32_t)(ch - 1) & 1u, abort_flag, status);     // the tiles are free again
+      if (ch > 0) ok = wait_or_report(bar_mma, (uint32_t)(ch - 1) & 1u, abort_flag, status);     // the tiles are free again
       if (!ok) break;
       mbar_expect_tx(bar_full, A_BYTES + 2 * B_PANEL);
       tma_load_3d(sbase, &tm_w, bar_full, ch * 64, it * 128, bh);
       tma_load_3d(sbase + A_BYTES, &tm_c, bar_full, nt * 128, ch * 64, bh);
       tma_load_3d(sbase + A_BYTES + B_PANEL, &tm_c, bar_full, nt * 128 + 64, ch * 64, bh);
-      ok = mbar_wait(bar_full, (uint32_t)ch & 1u, abort_flag, status);
+      ok = wait_or_report(bar_full, (uint32_t)ch & 1u, abort_flag, status);
       if (!ok) break;
       tc_fence_after();
       for (int kk = 0; kk < 4; ++kk)                                       // 16 J per instruction
         tc_mma_ss_bf16(tmem_base, ad + (uint64_t)(kk * 2), bd + (uint64_t)(kk * 128), idesc, (ch > 0 || kk > 0) ? 1u : 0u);
       tc_commit(bar_mma, 1u);
     }
-    if (ok) ok = mbar_wait(bar_mma, (uint32_t)(chunks - 1) & 1u, abort_flag, status);
+    if (ok) ok = wait_or_report(bar_mma, (uint32_t)(chunks - 1) & 1u, abort_flag, status);
     if (!ok) abort_s = 1;
   }
   __syncthreads();

@@ -8,9 +8,9 @@
 namespace sva {
 
 static constexpr int BS = 128;                 // rows per tile (queries and keys)
-static constexpr long long WAIT_LIMIT_CYCLES = 3000000000LL;
+static constexpr uint32_t WAIT_LIMIT_CYCLES = 3000000000u;
 // cycles a wait may last before the CTA gives up (read only on the slow path of a wait)
-static __device__ long long g_wait_limit = WAIT_LIMIT_CYCLES;   // one copy per translation unit
+static __device__ uint32_t g_wait_limit = WAIT_LIMIT_CYCLES;   // one copy per translation unit
 
 // ------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -37,28 +37,17 @@ __device__ __forceinline__ uint32_t mbar_try_wait(uint32_t bar, uint32_t parity)
       : "=r"(ok) : "r"(bar), "r"(parity), "r"(SVA_SUSPEND_HINT_NS) : "memory");
   return ok;
 }
-// Bounded wait.  Returns false when the CTA is aborting.  SLEEP_NS > 0 backs off between polls
-// (for roles whose wake-up latency is not on the critical path).  The first poll is marked as the
-// likely exit so that the polling loop is laid out away from the hot instruction stream
-// (instruction fetch is a measurable cost in these kernels).
-template <int SLEEP_NS = 0>
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag,
-                                          int32_t* status) {
+// Bounded wait.  Returns false when the CTA is aborting, or when the limit has run out, after setting the CTA's abort flag (which
+// the kernel reports when it ends).  Short on purpose: the attention kernel has some thirty of these and is bound by its
+// instruction stream.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag) {
   if (__builtin_expect(mbar_try_wait(bar, parity) != 0u, 1)) return true;
-  const long long t0 = clock64();
-  uint32_t spins = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if (SLEEP_NS > 0) __nanosleep(SLEEP_NS);
-    if ((++spins & 63u) == 0u) {
-      if (*abort_flag) return false;
-      if (clock64() - t0 > g_wait_limit) {
-        *abort_flag = 1;
-        if (status) atomicOr(status, SVA_DEV_TIMEOUT);
-        return false;
-      }
-    }
-  }
-  return true;
+  const uint32_t t0 = (uint32_t)clock();
+  do {
+    if (mbar_try_wait(bar, parity)) return true;
+  } while (!*abort_flag && (uint32_t)clock() - t0 <= g_wait_limit);
+  *abort_flag = 1;
+  return false;
 }
 
 __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map, uint32_t bar, int c0,
@@ -98,8 +87,21 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tc_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+// The same, with 64 registers that loads in flight fill: what reads them stays behind the wait.
+#define SVA_T8(v, i) "+r"(v[i]), "+r"(v[i + 1]), "+r"(v[i + 2]), "+r"(v[i + 3]), "+r"(v[i + 4]), "+r"(v[i + 5]), "+r"(v[i + 6]), "+r"(v[i + 7])
+__device__ __forceinline__ void tc_wait_ld64(uint32_t* v) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : SVA_T8(v, 0), SVA_T8(v, 8), SVA_T8(v, 16), SVA_T8(v, 24), SVA_T8(v, 32), SVA_T8(v, 40), SVA_T8(v, 48), SVA_T8(v, 56)
+               ::"memory");
+}
+#undef SVA_T8
 // The MMA warp runs its loop with all lanes (so addresses and descriptors stay warp-uniform)
 // and only the elected lane executes the tcgen05 instruction itself.
+__device__ __forceinline__ uint32_t elect_one() {
+  uint32_t e;
+  asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+  return e;
+}
 __device__ __forceinline__ void tc_commit(uint32_t bar, uint32_t elected) {
   asm volatile("{\n.reg .pred q;\nsetp.ne.b32 q, %1, 0;\n"
                "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}"
