@@ -16,13 +16,13 @@
 // ahead into the next row while the softmax groups finish the current one.
 //   warps 0-3, 4-7  two softmax warpgroups; they take the kept key blocks alternately (even / odd
 //                   position in the row's list); thread <-> query row <-> TMEM lane
-//   warp  8         producer of the K tiles (TMA, one lane)
+//   warp  8         producer of the K tiles (TMA)
 //   warp  9         issues the Q K^T MMAs; owns the TMEM allocation
 //   warp  10        issues the P V MMAs
 // The issuing warps run their loops with all lanes and let one elected lane execute the MMA: descriptors and addresses then stay in
 // uniform registers, and eight MMAs leave the warp in about 100 cycles; with a loop of one lane they took 400, and some 700 beside
 // busy softmax warps -- longer than the 512 cycles that they execute, in the P V -> P store -> P V chain.
-//   warp  11        producer of the V^T tiles (TMA, one lane)
+//   warp  11        producer of the V^T tiles (TMA)
 // TMEM columns: S of even blocks 0..127, S of odd blocks 128..255, O 256..383, Q 384..447 (bf16
 // pairs), P 448..511 (bf16 pairs).  Because P has columns of its own, an S buffer is free again as
 // soon as its warpgroup has read it into registers: the MMA warp computes S(j+2) while the softmax
@@ -352,7 +352,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     R.I = rowq[8 * slot + 5];
     R.hh = rowq[8 * slot + 6];
     R.bb = rowq[8 * slot + 7];
-    if (warp < 8 || warp == 9 || warp == 10) __syncwarp();   // whole warps: every lane has read the entry before lane 0 signs
+    __syncwarp();                                // every lane has read the entry before lane 0 signs
     if (arrive) mbar_arrive(bar_rq_empty + 8 * slot);
     return true;
   };
@@ -360,27 +360,29 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   if (warp >= 8) {
     asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
     if (warp == 8) {
-      // ---------------------------------------------------------- K producer (one lane)
-      if (lane == 0) {
+      // ---------------------------------------------------------- K producer (its rows are drawn by one lane)
+      {
+        const uint32_t el = elect_one();
         int s = 0;
         uint32_t ph = 0;
-        bool ok = true;
         const int nnz_bound = (!B64 && prm.row_ptr) ? __ldg(prm.row_ptr + prm.R + zero) : 0;
-        for (uint32_t i = 0; ok; ++i) {
+        for (uint32_t i = 0;; ++i) {
           // ---- row scheduling: draw the next row with a non-empty list and publish it
           const uint32_t slot = i % QD;
-          if (i >= QD && !mbar_wait(bar_rq_empty + 8 * slot, (i / QD - 1u) & 1u, abort_flag)) break;
-          int r, n = 0, beg = 0;
+          bool ok = i < QD || mbar_wait(bar_rq_empty + 8 * slot, (i / QD - 1u) & 1u, abort_flag);
+          if (!__all_sync(0xffffffffu, ok)) break;
+          int r, n = 0, beg = 0, I = 0, hh = 0, bb = 0;
+          if (lane == 0) {
           for (;;) {
             r = atomicAdd(prm.next_row, 1);
             if (r >= prm.R) break;
             if (!row_list<B64, REM>(prm, r, nnz_bound, n, beg) && prm.status) atomicOr(prm.status, SVA_DEV_BAD_INDEX);
             if (n > 0) break;
             // nothing kept (or a corrupt row_ptr pair): zeros and lse = -inf; rare, so this one lane does it
-            const int I = r % Nb, bh0 = r / Nb;
+            const int I0 = r % Nb, bh0 = r / Nb;
 #pragma unroll 1
             for (int t = 0; t < BS; ++t) {
-              const int qi = I * BS + t;
+              const int qi = I0 * BS + t;
               if (qi >= prm.N) break;
               __nv_bfloat16* orow = prm.o + (long long)(bh0 / prm.H) * prm.so.b + (long long)(bh0 % prm.H) * prm.so.h +
                                     (long long)qi * prm.so.n;
@@ -389,7 +391,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
               if (prm.lse) prm.lse[(long long)bh0 * prm.N + qi] = -INFINITY;
             }
           }
-          const int I = r % Nb, bh = r / Nb, hh = bh % prm.H, bb = bh / prm.H;
+          I = r % Nb; hh = r / Nb % prm.H; bb = r / Nb / prm.H;
           uint32_t e0 = 0u, e1 = 0u;
           const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);        // entries of the row's own list
           if (r < prm.R) { e0 = list_block<B64, REM>(prm, beg, 0, n_own); if (n > 1) e1 = list_block<B64, REM>(prm, beg, 1, n_own); }
@@ -423,8 +425,16 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
               prm.next_row[1] = 0;
               prm.next_row[0] = 0;
             }
-            break;
           }
+          }
+          r = __shfl_sync(0xffffffffu, r, 0);
+          if (r >= prm.R) break;
+          n = __shfl_sync(0xffffffffu, n, 0);
+          beg = __shfl_sync(0xffffffffu, beg, 0);
+          I = __shfl_sync(0xffffffffu, I, 0);
+          hh = __shfl_sync(0xffffffffu, hh, 0);
+          bb = __shfl_sync(0xffffffffu, bb, 0);
+          const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);
           // ---- K tiles of the row
           // Remainder (128-token blocks): while walking the row's list this lane leaves a bit mask of the kept blocks
           // for the softmax warps, which mask those columns of the block-mean tiles.  Eight masks in
@@ -433,28 +443,30 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           // softmax warps' read (expect_tx arrive -> k_full -> S MMA -> s_full).
           volatile uint32_t* kmask = reinterpret_cast<volatile uint32_t*>(smem + OFF_KMASK) + (i & 7u) * 32;
           if (RMASK && prm.rem_mask) {
-            for (int t = 0; t < 32; ++t) kmask[t] = 0u;
+            kmask[lane] = 0u;
+            __syncwarp();
           }
           for (int j = 0; j < n; ++j) {
             if ((prm.debug & 16) && j >= 1) { ok = false; break; }   // test aid: starve the pipeline so that a wait runs out
-            if (!mbar_wait(bar_k_empty + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
-            const uint32_t dst = sbase + OFF_K + s * TILE;
-            mbar_expect_tx(bar_k_full + 8 * s, F4 ? 8192 + 1024 : KTILE);
+            ok = __all_sync(0xffffffffu, mbar_wait(bar_k_empty + 8 * s, ph ^ 1u, abort_flag));
+            if (!ok) break;
+            const uint32_t dst = sbase + OFF_K + s * TILE, bar = bar_k_full + 8 * s;
+            mbar_expect_tx_if(bar, F4 ? 8192 + 1024 : KTILE, el);
             if (F4) {
               // packed codes of the key block (128 rows x 64 bytes, 64-byte swizzle) and its 1 KB of scale factors
               int J = j;
               if (prm.row_ptr) {
                 J = __ldg(prm.col_idx + beg + j);
-                if (J < 0 || J >= prm.Nb) { J = 0; if (prm.status) atomicOr(prm.status, SVA_DEV_BAD_INDEX); }
+                if (J < 0 || J >= prm.Nb) { J = 0; if (prm.status && lane == 0) atomicOr(prm.status, SVA_DEV_BAD_INDEX); }
               }
-              tma_load_4d(dst, &tm_k, bar_k_full + 8 * s, 0, J * BS, hh, bb);
-              bulk_load(dst + 8192, prm.k_sf + ((long long)bh * prm.Nb + J) * 1024, 1024, bar_k_full + 8 * s);
+              tma_load_4d_if(dst, &tm_k, bar, 0, J * BS, hh, bb, el);
+              if (el) bulk_load(dst + 8192, prm.k_sf + ((long long)(bb * prm.H + hh) * prm.Nb + J) * 1024, 1024, bar);
             } else if (REM && j >= n_own) {
               // pooled tile: 128 block means of K (rows beyond Nb are zero in the pooled tensor)
               // (a first-order tile has no logits of its own: its S is computed from pooled tile 0 and ignored)
               const int c = j - n_own < prm.np ? j - n_own : 0;
-              tma_load_4d(dst, &tm_kp, bar_k_full + 8 * s, 0, c * BS, hh, bb);
-              tma_load_4d(dst + TILE / 2, &tm_kp, bar_k_full + 8 * s, 64, c * BS, hh, bb);
+              tma_load_4d_if(dst, &tm_kp, bar, 0, c * BS, hh, bb, el);
+              tma_load_4d_if(dst + TILE / 2, &tm_kp, bar, 64, c * BS, hh, bb, el);
             } else if (B64) {
               // two 64-key blocks side by side: rows 0..63 and 64..127 of both d-panels
               // (e4m3: one 128-byte panel, so one load per key block)
@@ -463,53 +475,57 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
               for (int h = 0; h < 2; ++h) {
                 const int J = (int)((dsc >> (16 * h)) & 0x3fffu);
 
-                tma_load_4d(dst + h * (TILE / 4), &tm_k, bar_k_full + 8 * s, 0, J * KB, hh, bb);
-                if (!F8) tma_load_4d(dst + TILE / 2 + h * (TILE / 4), &tm_k, bar_k_full + 8 * s, 64, J * KB, hh, bb);
+                tma_load_4d_if(dst + h * (TILE / 4), &tm_k, bar, 0, J * KB, hh, bb, el);
+                if (!F8) tma_load_4d_if(dst + TILE / 2 + h * (TILE / 4), &tm_k, bar, 64, J * KB, hh, bb, el);
               }
             } else {
               int J = j;
               if (prm.row_ptr) {
                 J = __ldg(prm.col_idx + beg + j);
-                if (J < 0 || J >= prm.Nb) { J = 0; if (prm.status) atomicOr(prm.status, SVA_DEV_BAD_INDEX); }
-                if (RMASK && prm.rem_mask) kmask[J >> 5] |= 1u << (J & 31);
+                if (J < 0 || J >= prm.Nb) { J = 0; if (prm.status && lane == 0) atomicOr(prm.status, SVA_DEV_BAD_INDEX); }
+                if (RMASK && prm.rem_mask && el) kmask[J >> 5] |= 1u << (J & 31);
               }
-              tma_load_4d(dst, &tm_k, bar_k_full + 8 * s, 0, J * BS, hh, bb);      // e4m3: the whole tile (128 x 128 bytes)
-              if (!F8) tma_load_4d(dst + TILE / 2, &tm_k, bar_k_full + 8 * s, 64, J * BS, hh, bb);
+              tma_load_4d_if(dst, &tm_k, bar, 0, J * BS, hh, bb, el);      // e4m3: the whole tile (128 x 128 bytes)
+              if (!F8) tma_load_4d_if(dst + TILE / 2, &tm_k, bar, 64, J * BS, hh, bb, el);
             }
             if (++s == KS) { s = 0; ph ^= 1u; }
           }
+          if (!ok) break;
         }
       }
     } else if (warp == 11) {
-      // ---------------------------------------------------------- V^T producer (one lane)
+      // ---------------------------------------------------------- V^T producer
       // tile J of head (b,h): 128 d-rows x 128 keys, contiguous 32 KB, two 64-key panels
-      if (lane == 0) {
+      {
+        const uint32_t el = elect_one();
         int s = 0;
         uint32_t ph = 0;
-        bool ok = true;
-        for (uint32_t i = 0; ok; ++i) {
+        for (uint32_t i = 0;; ++i) {
           Row cur;
-          if (!fetch_row(i, cur, true) || cur.r >= prm.R) break;
-          const int n = cur.n, beg = cur.beg, hh = cur.hh, bb = cur.bb;
+          bool ok = fetch_row(i, cur, lane == 0) && cur.r < prm.R;
+          if (!__all_sync(0xffffffffu, ok)) break;
+          const int n = __shfl_sync(0xffffffffu, cur.n, 0), beg = __shfl_sync(0xffffffffu, cur.beg, 0);
+          const int hh = __shfl_sync(0xffffffffu, cur.hh, 0), bb = __shfl_sync(0xffffffffu, cur.bb, 0);
           const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);
           for (int j = 0; j < n; ++j) {
-            if (!mbar_wait(bar_v_empty + 8 * s, ph ^ 1u, abort_flag)) { ok = false; break; }
+            ok = __all_sync(0xffffffffu, mbar_wait(bar_v_empty + 8 * s, ph ^ 1u, abort_flag));
+            if (!ok) break;
             const uint32_t e = list_block<B64, REM>(prm, beg, j, n_own);
             const uint32_t dst = sbase + OFF_V + s * TILE;
-            mbar_expect_tx(bar_v_full + 8 * s, TILE);
+            mbar_expect_tx_if(bar_v_full + 8 * s, TILE, el);
             if (REM && j >= n_own) {
               // pooled tile: the block means of V ([128 d rows][128 blocks], or [128 blocks][128 d] when V itself is
               // read keys-major; blocks beyond Nb zero)
               const int c = j - n_own;
               if (c < prm.np) {
-                tma_load_4d(dst, &tm_vtp, bar_v_full + 8 * s, 0, c * BS, hh, bb);
-                tma_load_4d(dst + TILE / 2, &tm_vtp, bar_v_full + 8 * s, 64, c * BS, hh, bb);
+                tma_load_4d_if(dst, &tm_vtp, bar_v_full + 8 * s, 0, c * BS, hh, bb, el);
+                tma_load_4d_if(dst + TILE / 2, &tm_vtp, bar_v_full + 8 * s, 64, c * BS, hh, bb, el);
               } else {
                 // first-order tile: A^T (A when V is read keys-major) of the query block (64-token blocks: of the tile
                 // row's first / second one)
                 const int qb = B64 ? min(2 * cur.I + (c - prm.np), prm.Nb - 1) : cur.I;
-                tma_load_4d(dst, &tm_at, bar_v_full + 8 * s, 0, qb * BS, hh, bb);
-                tma_load_4d(dst + TILE / 2, &tm_at, bar_v_full + 8 * s, 64, qb * BS, hh, bb);
+                tma_load_4d_if(dst, &tm_at, bar_v_full + 8 * s, 0, qb * BS, hh, bb, el);
+                tma_load_4d_if(dst + TILE / 2, &tm_at, bar_v_full + 8 * s, 64, qb * BS, hh, bb, el);
               }
             } else if (VMN) {
               // V itself: two d-panels of [128 keys][64 d] (64-token blocks: each panel's two halves from two key blocks)
@@ -517,23 +533,24 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                   const int Jh = (int)((e >> (16 * h)) & 0x3fffu);
-                  tma_load_4d(dst + h * (TILE / 4), &tm_vt, bar_v_full + 8 * s, 0, Jh * KB, hh, bb);
-                  tma_load_4d(dst + TILE / 2 + h * (TILE / 4), &tm_vt, bar_v_full + 8 * s, 64, Jh * KB, hh, bb);
+                  tma_load_4d_if(dst + h * (TILE / 4), &tm_vt, bar_v_full + 8 * s, 0, Jh * KB, hh, bb, el);
+                  tma_load_4d_if(dst + TILE / 2 + h * (TILE / 4), &tm_vt, bar_v_full + 8 * s, 64, Jh * KB, hh, bb, el);
                 }
               } else {
-                tma_load_4d(dst, &tm_vt, bar_v_full + 8 * s, 0, (int)e * BS, hh, bb);
-                tma_load_4d(dst + TILE / 2, &tm_vt, bar_v_full + 8 * s, 64, (int)e * BS, hh, bb);
+                tma_load_4d_if(dst, &tm_vt, bar_v_full + 8 * s, 0, (int)e * BS, hh, bb, el);
+                tma_load_4d_if(dst + TILE / 2, &tm_vt, bar_v_full + 8 * s, 64, (int)e * BS, hh, bb, el);
               }
             } else if (B64) {
               // each 64-key panel of the tile is one key block's transposed V: [128 d rows][64 keys]
-              tma_load_4d(dst, &tm_vt, bar_v_full + 8 * s, 0, (int)(e & 0x3fffu) * D, hh, bb);
-              tma_load_4d(dst + TILE / 2, &tm_vt, bar_v_full + 8 * s, 0, (int)((e >> 16) & 0x3fffu) * D, hh, bb);
+              tma_load_4d_if(dst, &tm_vt, bar_v_full + 8 * s, 0, (int)(e & 0x3fffu) * D, hh, bb, el);
+              tma_load_4d_if(dst + TILE / 2, &tm_vt, bar_v_full + 8 * s, 0, (int)((e >> 16) & 0x3fffu) * D, hh, bb, el);
             } else {
-              tma_load_4d(dst, &tm_vt, bar_v_full + 8 * s, 0, (int)e * BS, hh, bb);
-              tma_load_4d(dst + TILE / 2, &tm_vt, bar_v_full + 8 * s, 64, (int)e * BS, hh, bb);
+              tma_load_4d_if(dst, &tm_vt, bar_v_full + 8 * s, 0, (int)e * BS, hh, bb, el);
+              tma_load_4d_if(dst + TILE / 2, &tm_vt, bar_v_full + 8 * s, 64, (int)e * BS, hh, bb, el);
             }
             if (++s == VS) { s = 0; ph ^= 1u; }
           }
+          if (!ok) break;
         }
       }
     } else if (warp == 9) {

@@ -325,3 +325,51 @@ def test_b64_more_than_1024_key_blocks():
     rows = [r for r in [0, 1, 3] + list(range(4, nb, 41)) + [nb - 1] if len(lists[r])]
     U.check_attn_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, rows)
     assert (o[0, 0, 128:192] == 0).all()                       # the empty list's rows
+
+
+# Row logits (powers of two) per key block: within the reference's range, far below and above it from the first block on, and
+# leaving it later, upwards and by steps; 0 for all the others.
+REFERENCE_LOGITS = {"low": [-300.0] * 4, "high_then_low": [300.0, -300.0], "low_then_high": [-300.0, -60.0, 5.0, 60.0, 300.0],
+                    "steps": [30.0, 70.0, 110.0, 160.0, 211.0], "at_the_line": [39.0, 41.0, -39.0, -41.0, 47.0, 49.0]}
+
+
+@pytest.mark.parametrize("block", [128, 64])
+@pytest.mark.parametrize("name", list(REFERENCE_LOGITS))
+def test_reference_exponent_follows_the_logits(name, block):
+    """P = 2^(logit - m): m starts at 0 and changes only for logits far from it.  Query blocks keep different lists (64-token blocks:
+    a tile's two query blocks share only some of their key blocks), odd and even list lengths."""
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=8, Wg=block + 5, block=block, k=4)       # 9 blocks, ragged tail
+    gen = torch.Generator().manual_seed(len(name))
+    lev = REFERENCE_LOGITS[name]
+    lev = torch.tensor([lev[j] if j < len(lev) else 0.0 for j in range(w.Nb)]).repeat_interleave(block)[:w.N]
+    q = torch.ones(1, 1, w.n_alloc, w.d) + 0.05 * torch.randn(1, 1, w.n_alloc, w.d, generator=gen)
+    k = torch.zeros(1, 1, w.n_alloc, w.d)
+    k[0, 0, :w.N] = (lev / (w.scale * 1.4426950408889634 * w.d))[:, None] + 0.3 * torch.randn(w.N, w.d, generator=gen)
+    v = 2.0 * torch.rand(1, 1, w.n_alloc, w.d, generator=gen) - 1.0
+    q[:, :, w.N:] = 0.0
+    v[:, :, w.N:] = 0.0
+    q, k, v = q.bfloat16(), k.bfloat16(), v.bfloat16()
+    from paper_2606_23743_b200.workloads import bf16_bits
+    bits = (bf16_bits(q), bf16_bits(k), bf16_bits(v))
+    lists = [list(range(w.Nb)), [0], [1, 2, 3, 4], [0, 4, 5, 8], list(range(1, w.Nb, 2)), list(range(0, w.Nb, 2)), [8], [2, 3], [5, 6, 7]]
+    rp = torch.zeros(w.R + 1, dtype=torch.int32)
+    rp[1:] = torch.cumsum(torch.tensor([len(x) for x in lists]), 0)
+    ci = torch.tensor([j for x in lists for j in x], dtype=torch.int32)
+    o, lse, st = U.gpu_attn(w, U.dev(q), U.dev(k), U.dev(v), rp.cuda(), ci.cuda())
+    assert st == 0
+    U.check_attn_vs_oracle(w, *bits, rp.cuda(), ci.cuda(), o, lse, list(range(w.R)))
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("-inf"), float("nan")])
+def test_logits_that_are_not_finite_stay_in_their_rows(bad):
+    """An infinite or NaN query element makes its own row NaN (or, where every logit is finite, not) and no other."""
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=4, Wg=150, k=3)
+    (q, k, v), (qb, kb, vb) = U.host_inputs(w)
+    rp, ci, _ = U.gpu_select(w, U.dev(q), U.dev(k))
+    clean, _, _ = U.gpu_attn(w, U.dev(q), U.dev(k), U.dev(v), rp, ci)
+    q = q.clone()
+    q[0, 0, 201, 5] = bad
+    o, lse, st = U.gpu_attn(w, U.dev(q), U.dev(k), U.dev(v), rp, ci)
+    rows = [r for r in range(w.N) if r != 201]
+    assert st == 0 and torch.equal(o[0, 0, rows], clean[0, 0, rows])
+    assert torch.isnan(o[0, 0, 201]).all() and torch.isnan(lse[0, 0, 201])
