@@ -258,3 +258,22 @@ def test_ragged_tile_of_block_means(nb, block):
     o, lse, st = gpu_remainder(w, qd, kd, vd, rp, ci)
     assert st == 0
     check_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, [0, 1, nb // 2, nb - 2, nb - 1])
+
+
+@pytest.mark.parametrize("block,nb,tail", [(64, 1, 64), (64, 2, 1), (64, 32, 63), (64, 33, 1), (64, 63, 64), (64, 64, 9), (64, 65, 64), (128, 65, 1), (64, 129, 63),
+                                           (64, 193, 64)])
+def test_first_order_statistics_at_the_edges(block, nb, tail):
+    """Block statistics and weights at the edges: one block, last blocks of 1, 9 and 63 keys, key blocks around the 64 that a step of the
+    sum over A_I takes and around the 32 of a word of the kept-block mask."""
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=1, Wg=(nb - 1) * block + tail, block=block, k=max(1, nb // 5))
+    (q, k, v), (qb, kb, vb) = U.host_inputs(w)
+    qd, kd, vd = U.dev(q), U.dev(k), U.dev(v)
+    rp, ci, scores = U.gpu_select(w, qd, kd, want_scores=True)
+    o, lse, st = gpu_remainder(w, qd, kd, vd, rp, ci, 1, scores=scores)
+    assert st == 0
+    rows = sorted({0, w.R - 1, *U.sample_rows_per_head(1, w.Nb, min(4, w.Nb), seed=3)})
+    o_ref, l_ref = oracle.attn_remainder_rows(qb, kb, vb, w.N, w.block, w.scale, rp.cpu().numpy(), ci.cpu().numpy(), rows, order=1,
+                                              stats="bf16")
+    max_abs, rel, lse_err = U.attn_errors(o, lse, o_ref, l_ref, rows, w.N, w.block, 1)
+    # (the correction is not bounded by V: one bf16 unit of the largest output)
+    assert max_abs <= max(U.BF16_MAX_ABS, 2.0 ** -7 * float(np.nanmax(np.abs(o_ref)))) and rel <= U.BF16_REL_L2 and lse_err <= 2e-3
