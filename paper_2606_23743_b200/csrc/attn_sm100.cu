@@ -2,9 +2,8 @@
 // (Paper: critical blocks "computed exactly"; dense fallback.)
 //
 // S = Q K^T and O += P V both take A from TENSOR memory (Q resp. P, bf16 pairs) and B from shared memory, M = N = 128:
-//   * Q is written into TMEM once per row by the softmax threads (128-token blocks: by the group that finishes
-//     the row first, about a tile before the row ends, from a tile that TMA has put into the group's idle output
-//     staging panel; otherwise by both groups in the epilogue, straight from global memory);
+//   * Q is written into TMEM once per row by the softmax group that finishes the row first, about a tile before the row
+//     ends, from a tile that TMA has put into the group's idle output staging panel;
 //   * V: in the two-step form it is consumed transposed (V^T tiles: d rows, keys contiguous) from a tiled transposed
 //     copy that a small kernel writes into the caller's workspace first.  The one-call entry points read V where it lies
 //     instead (template switch VMN: an MN-major B operand, a second instruction descriptor), without the copy's pass over
@@ -86,6 +85,7 @@ namespace sva {
 struct TsParams {
   const __nv_bfloat16* q;     // e4m3 variant: bytes (strides in elements either way)
   Strides sq;
+  int q_each_h, q_each_b;     // 0: all heads / batch items have the same Q (the map of Q then has one)
   const float* q_scale;       // e4m3 variant: one scale per (b, h, block) for Q and for K; 4-bit variant: one per (b, h)
   const float* k_scale;
   const uint8_t* q_sf;        // 4-bit variant: e4m3 scale factors, 1024 bytes per (b, h, 128-token block), tile order
@@ -132,7 +132,7 @@ constexpr int OFF_O = OFF_V + VS * TILE;    // output staging: two [128 rows][12
 constexpr int OFF_CTRL = OFF_O + TILE;      // 6 tiles = 192 KB
 constexpr int CTRL_BYTES = 6144;            // barriers, row queue, reference exponents and row sums (two rows of each)
 constexpr int OFF_Q4 = OFF_CTRL + CTRL_BYTES;   // 4-bit variant: the row's Q codes (8 KB) and their scale factors (1 KB)
-constexpr int OFF_QS = OFF_CTRL + CTRL_BYTES;     // bf16, 128-token blocks: staging of the second half (d 64..127) of a row's Q tile (16 KB)
+constexpr int OFF_QS = OFF_CTRL + CTRL_BYTES;     // bf16: staging of the second half (d 64..127) of a row's Q tile (16 KB)
 #ifdef SVA_TIMELINE
 constexpr int OFF_KMASK = OFF_QS + 16384;   // remainder: kept-block bit masks, [8 rows in flight][32 words]
 constexpr int SMEM_BYTES = OFF_KMASK + 1024 + 1024 + 1400 * 8;
@@ -293,7 +293,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   __syncthreads();
 #endif
   if (threadIdx.x == 0) {
-    mbar_init(bar_q_ready, (!F4 && !B64) ? 128 : 256);   // (128-token blocks, bf16 / e4m3 Q: one softmax group writes a row's Q)
+    mbar_init(bar_q_ready, F4 ? 256 : 128);             // (bf16 / e4m3 Q: one softmax group writes a row's Q)
     mbar_init(bar_o_free, 256);
     mbar_init(bar_xch, 256);
     mbar_init(bar_ref, 128);
@@ -321,7 +321,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   }
   if (warp == 8 && lane == 0) { prefetch_tmap(&tm_k); if (REM) prefetch_tmap(&tm_kp); }
   if (warp == 11 && lane == 0) { prefetch_tmap(&tm_vt); if (REM) { prefetch_tmap(&tm_vtp); prefetch_tmap(&tm_at); } }
-  if (warp == 0 && lane == 0) { prefetch_tmap(&tm_o); if (!F4 && !B64) prefetch_tmap(&tm_q); }
+  if (warp == 0 && lane == 0) { prefetch_tmap(&tm_o); if (!F4) prefetch_tmap(&tm_q); }
   if (warp == 9) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                  ::"r"(cb + 216), "r"(512u) : "memory");
@@ -395,7 +395,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           uint32_t e0 = 0u, e1 = 0u;
           const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);        // entries of the row's own list
           if (r < prm.R) { e0 = list_block<B64, REM>(prm, beg, 0, n_own); if (n > 1) e1 = list_block<B64, REM>(prm, beg, 1, n_own); }
-          if (!F4 && !B64 && r < prm.R) {
+          if (!F4 && r < prm.R) {
             // the row's Q tile will be fetched about a row from now: start it on its way into the L2.  Token rows that are not
             // contiguous ([B,N,H,d], a packed projection) go as a tensor prefetch: with a plain one per token row this lane
             // spent about 9 000 cycles per row in which no K tile was on its way (32 760 tokens x 24 heads, 40 blocks kept:
@@ -405,8 +405,8 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
               const long long q0 = (long long)bb * prm.sq.b + (long long)hh * prm.sq.h + (long long)I * BS * prm.sq.n;
               bulk_prefetch_l2(reinterpret_cast<const uint8_t*>(prm.q) + q0 * eb, (uint32_t)min(BS, prm.N - I * BS) * row_bytes);
             } else {
-              tma_prefetch_4d(&tm_q, 0, I * BS, hh, bb);
-              if (!F8) tma_prefetch_4d(&tm_q, 64, I * BS, hh, bb);
+              tma_prefetch_4d(&tm_q, 0, I * BS, hh * prm.q_each_h, bb * prm.q_each_b);
+              if (!F8) tma_prefetch_4d(&tm_q, 64, I * BS, hh * prm.q_each_h, bb * prm.q_each_b);
             }
           }
           rowq[8 * slot] = r;
@@ -655,7 +655,6 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     const uint32_t s_tmem = tmem_base + lane_addr + 128 * w;
     const uint32_t o_tmem = tmem_base + lane_addr + COL_O;
     const uint32_t p_tmem = tmem_base + lane_addr + COL_P;
-    const uint32_t q_tmem = tmem_base + lane_addr + COL_Q + (F8 ? 16 : 32) * w;
     const int tail_keys = prm.N - (prm.Nb - 1) * KB;         // valid keys of the last key block
     const int nnz_total = (REM && prm.row_ptr) ? __ldg(prm.row_ptr + (prm.R / prm.Nt) * prm.Nb + zero) : 0;   // row_ptr[R of the CSR]
     const int qh = row >> 6;                                 // 64-token blocks: which query block of the tile I am in
@@ -665,43 +664,18 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     uint32_t rows_done = 0;        // non-empty rows finished
     bool ok = true;
 
-    // this group's half (d columns 64w..64w+63) of a row's Q: global -> registers -> TMEM
-    auto load_q = [&](const Row& R, uint32_t* qv) {
-#pragma unroll
-      for (int e = 0; e < 32; ++e) qv[e] = 0u;
-      if (F4 || R.r >= prm.R) return;                                   // (4-bit variant: the Q tile goes to shared memory by TMA)
-      const int qi = R.I * BS + row;
-      if (qi >= prm.N || 64 * w >= prm.d) return;                      // (d = 64: the second group's half of Q is zero)
-      const long long eoff = (long long)R.bb * prm.sq.b + (long long)R.hh * prm.sq.h +
-                             (long long)qi * prm.sq.n + 64 * w;           // in elements
-      const uint4* src = F8 ? reinterpret_cast<const uint4*>(reinterpret_cast<const uint8_t*>(prm.q) + eoff)
-                            : reinterpret_cast<const uint4*>(prm.q + eoff);
-#pragma unroll
-      for (int e = 0; e < (F8 ? 4 : 8); ++e) {                            // 64 elements: 64 or 128 bytes
-        const uint4 u = __ldg(src + e);
-        qv[4 * e] = u.x; qv[4 * e + 1] = u.y; qv[4 * e + 2] = u.z; qv[4 * e + 3] = u.w;
+    // 4-bit variant: one thread fetches a row's Q codes and scale factors into shared memory; the barrier completes when every softmax
+    // thread has arrived (none of them reads the previous row's Q any more) and the bytes have landed
+    auto fetch_q4 = [&](const Row& R) {
+      if (threadIdx.x == 0) {
+        mbar_expect_tx_only(bar_q_ready, 8192 + 1024);
+        tma_load_4d(sbase + OFF_Q4, &tm_kp, bar_q_ready, 0, R.I * BS, R.hh, R.bb);
+        bulk_load(sbase + OFF_Q4 + 8192, prm.q_sf + ((long long)(R.bb * prm.H + R.hh) * prm.Nb + R.I) * 1024, 1024, bar_q_ready);
       }
-    };
-    auto store_q = [&](const uint32_t* qv, const Row& R) {
-      if (F4) {
-        // one thread fetches the row's Q codes and scale factors; the barrier completes when every softmax thread
-        // has arrived (none of them reads the previous row's Q any more) and the bytes have landed
-        if (threadIdx.x == 0) {
-          mbar_expect_tx_only(bar_q_ready, 8192 + 1024);
-          tma_load_4d(sbase + OFF_Q4, &tm_kp, bar_q_ready, 0, R.I * BS, R.hh, R.bb);
-          bulk_load(sbase + OFF_Q4 + 8192, prm.q_sf + ((long long)(R.bb * prm.H + R.hh) * prm.Nb + R.I) * 1024, 1024, bar_q_ready);
-        }
-        mbar_arrive(bar_q_ready);
-        return;
-      }
-      tc_fence_after();
-      if (F8) tmem_st16(q_tmem, qv); else tmem_st32(q_tmem, qv);
-      tc_wait_st();
-      tc_fence_before();
       mbar_arrive(bar_q_ready);
     };
 
-    // 128-token blocks (bf16 / e4m3 Q): ONE group writes the whole Q of the next row -- the group that does not take
+    // bf16 / e4m3 Q: ONE group writes the whole Q of the next row -- the group that does not take
     // the current row's last tile, as soon as that last S has been computed, about a tile before the row ends -- so
     // that the S issuer starts on the next row while this one is still finishing.  The Q tile comes by TMA (a
     // thread-per-row read of Q from global memory costs 32 cache lines per load instruction, and that
@@ -709,13 +683,15 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     // the group's own output staging panel (idle between two epilogues), the other 64 into a 16 KB buffer behind
     // the control block, both loads in flight together; each thread then copies its row from shared memory into
     // tensor memory.  `use` counts these copies over the CTA's rows (the first row's is copy 0): the barrier's phase.
-    constexpr bool EARLYQ = !F4 && !B64;
+    // (64-token blocks, 32 760 tokens x 24 heads, 51 of 512 blocks kept: 2.10 M cycles with both groups reading Q from global memory
+    // in the epilogue, 2.01 this way; with the remainder 2.63 and 2.56; 16 380 of the tokens 0.65 and 0.61.)
+    constexpr bool EARLYQ = !F4;
     auto copy_q = [&](const Row& R, uint32_t use) -> bool {
       if ((threadIdx.x & 127) == 0) {
         bulk_wait_read0();                                                // my previous output store has read the panel
         mbar_expect_tx(bar_qs, F8 ? TILE / 2 : TILE);
-        tma_load_4d(sbase + OFF_O + w * (TILE / 2), &tm_q, bar_qs, 0, R.I * BS, R.hh, R.bb);
-        if (!F8) tma_load_4d(sbase + OFF_QS, &tm_q, bar_qs, 64, R.I * BS, R.hh, R.bb);
+        tma_load_4d(sbase + OFF_O + w * (TILE / 2), &tm_q, bar_qs, 0, R.I * BS, R.hh * prm.q_each_h, R.bb * prm.q_each_b);
+        if (!F8) tma_load_4d(sbase + OFF_QS, &tm_q, bar_qs, 64, R.I * BS, R.hh * prm.q_each_h, R.bb * prm.q_each_b);
       }
       if (!mbar_wait(bar_qs, use & 1u, abort_flag)) return false;
       tc_fence_after();
@@ -746,10 +722,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     if (EARLYQ) {
       if (ok && nx.r < prm.R && w == 1) ok = copy_q(nx, 0u);
     } else if (ok && nx.r < prm.R) {
-      // first row: its Q goes in right away
-      uint32_t qv[32];
-      load_q(nx, qv);
-      store_q(qv, nx);
+      fetch_q4(nx);                                                     // first row: right away
     }
     for (; ok && nx.r < prm.R; ++rows_done) {
       const int r = nx.r, n = nx.n, lbeg = nx.beg;
@@ -762,6 +735,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       float l = 0.f;                 // partial row sum over this group's blocks
       float l_top = 0.f;             // what rounding to bf16 adds to the largest P of each of them
       volatile float* refr = ref + (rows_done & 1u) * 256;
+      uint32_t J2 = 0u;              // e4m3, 128-token blocks: the list entry after J
       float qs_row = 1.f, ks_next = 1.f, ks_next1 = 1.f;
       auto load_ks = [&](uint32_t e) {                                // scales of the key block(s) of list entry e
         const float* ks = prm.k_scale + (long long)bh * prm.Nb;
@@ -777,6 +751,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const int qb = B64 ? min(2 * I + qh, prm.Nb - 1) : I;         // my query block
         qs_row = __ldg(prm.q_scale + (long long)bh * prm.Nb + qb) * prm.scale_log2;
         if (w < n) load_ks(J);
+        if (!B64 && w + 2 < n) J2 = list_block<B64, REM, true>(prm, lbeg, w + 2);
       }
       const int n_own = n - ((REM && prm.row_ptr) ? prm.np + prm.n1 : 0);      // entries of the row's own list
       // One tile of the row: a kept key block, or (REM) a tile of block means.  128-token blocks: one copy of the body per kind
@@ -808,8 +783,16 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         }
         if (F8) { c = qs_row * ks_next; if (B64) c1 = qs_row * ks_next1; }
         if (j + 2 < n) {                                               // one entry ahead
-          J = list_block<B64, REM, !F8>(prm, lbeg, j + 2, n_own);
-          if (F8) load_ks(J);
+          if (F8 && !B64) {
+            // (the entry was sent for a tile ago: the address of its scale does not wait for it; 32 760 tokens x 24 heads 2.58 ->
+            // 2.53 M cycles.  With 64-token blocks it gains nothing)
+            J = prm.row_ptr == nullptr || J2 < (uint32_t)prm.Nb ? J2 : 0u;
+            load_ks(J);
+            if (j + 4 < n) J2 = list_block<B64, REM, true>(prm, lbeg, j + 4, n_own);
+          } else {
+            J = list_block<B64, REM, true>(prm, lbeg, j + 2, n_own);
+            if (F8) load_ks(J);
+          }
         }
         uint4 kept = make_uint4(0u, 0u, 0u, 0u);
         if (REM && pooled && prm.rem_mask) {                          // four words for this tile's 128 blocks
@@ -1065,8 +1048,6 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       // ---- epilogue: merge the two groups' row sums, hand the next row's Q to the S issuer,
       // normalise and store (each group half of d)
       if (!fetch_row(rows_done + 1u, nx, signs)) { ok = false; break; }   // the row after this one (never an empty one), or the end mark
-      uint32_t qn[32];
-      if (!EARLYQ) load_q(nx, qn);                                // in flight during the waits below
       volatile float* lxr = lx + (rows_done & 1u) * 256;
       lxr[w * 128 + row] = l + l_top;
       if (w == 1) ltop[(rows_done & 1u) * 128 + row] = l_top;
@@ -1085,7 +1066,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
       }
       if (!mbar_wait(bar_xch, rows_done & 1u, abort_flag)) { ok = false; break; }
       // both groups have seen all their S tiles: no MMA reads Q any more
-      if (!EARLYQ && nx.r < prm.R) store_q(qn, nx);
+      if (!EARLYQ && nx.r < prm.R) fetch_q4(nx);
       if (!EARLYQ && (threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 8);
       if (!mbar_wait(bar_pv_done + 8 * wl, last & 1u, abort_flag)) { ok = false; break; }
       if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 9);
@@ -1134,7 +1115,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         }
         if (qi < prm.N && prm.lse && w == 0) {
           const float ls = l * f0 + (lxr[128 + row] - ltop[(rows_done & 1u) * 128 + row]) * f1;     // (the sum itself)
-          prm.lse[(long long)bh * prm.N + qi] = B64 || ls != 0.f ? (m_fin + log2f(ls)) * 0.6931471805599453f : NAN;
+          prm.lse[(long long)bh * prm.N + qi] = B64 || __float_as_uint(m_fin) != 0x80000000u ? (m_fin + log2f(ls)) * 0.6931471805599453f : NAN;
         }
       }
       if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 10);
@@ -1585,12 +1566,16 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
   }
   if (rc != SVA_OK) return rc;
   tkp = tk; tvp = tv; tat = tv;  // (placeholders when there is no remainder: the kernel never touches them)
-  // Q as 128-row tiles, like K (128-token blocks: a row's Q reaches the kernel by TMA; otherwise unused)
-  CUtensorMap tq = tk;
-  if (!b64) {
+  // Q as 128-row tiles (a row's Q reaches the kernel by TMA)
+  CUtensorMap tq;
+  int q_each_h, q_each_b;
+  {
     const Strides sq = make_strides(p->q_stride);
-    if ((rc = make_map_ts(&tq, q, m.d, m.N, m.H, m.B, (cuuint64_t)sq.n * eb, (cuuint64_t)sq.h * eb, (cuuint64_t)sq.b * eb,
-                          m.block, eb)) != SVA_OK)
+    // (64-token blocks also take a Q that heads or batch items share -- stride 0, which a tensor map does not)
+    const int hq = b64 && sq.h == 0 ? 1 : m.H, bq = b64 && sq.b == 0 ? 1 : m.B;
+    q_each_h = hq == m.H ? 1 : 0;
+    q_each_b = bq == m.B ? 1 : 0;
+    if ((rc = make_map_ts(&tq, q, m.d, m.N, hq, bq, (cuuint64_t)sq.n * eb, (cuuint64_t)sq.h * eb, (cuuint64_t)sq.b * eb, BS, eb)) != SVA_OK)
       return rc;
   }
   if (rem && remainder_order == 1) {
@@ -1635,6 +1620,7 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
   }
   TsParams prm;
   prm.q = (const __nv_bfloat16*)q; prm.sq = make_strides(p->q_stride);
+  prm.q_each_h = q_each_h; prm.q_each_b = q_each_b;
   prm.q_scale = q_scale; prm.k_scale = k_scale;
   prm.q_sf = nullptr; prm.k_sf = nullptr;
   prm.row_ptr = row_ptr; prm.col_idx = col_idx;

@@ -373,3 +373,17 @@ def test_logits_that_are_not_finite_stay_in_their_rows(bad):
     rows = [r for r in range(w.N) if r != 201]
     assert st == 0 and torch.equal(o[0, 0, rows], clean[0, 0, rows])
     assert torch.isnan(o[0, 0, 201]).all() and torch.isnan(lse[0, 0, 201])
+
+
+@pytest.mark.parametrize("shared", ["heads", "items"])
+def test_a_q_that_heads_or_items_share(shared):
+    """64-token blocks: Q with a stride of 0 over heads or batch items gives what a copy of it gives."""
+    w = shrink(WORKLOADS["medium"], B=2, H=3, T=1, Hg=8, Wg=66, block=64, k=4)
+    (q, k, v), _ = U.host_inputs(w)
+    q, k, v = U.dev(q), U.dev(k), U.dev(v)
+    part = q[:, :1] if shared == "heads" else q[:1]
+    qx, qc = part.expand(q.shape), part.expand(q.shape).contiguous()
+    rp, ci, _ = U.gpu_select(w, qc, k)
+    o, lse, st = U.gpu_attn(w, qc, k, v, rp, ci)
+    ox, lx, sx = U.gpu_attn(w, qx, k, v, rp, ci)
+    assert st == 0 and sx == 0 and torch.equal(ox, o) and torch.equal(lx, lse)

@@ -238,3 +238,23 @@ def test_fp8_two_step_form_matches_the_one_call_form():
         torch.cuda.synchronize()
         assert int(status.item()) == 0
         assert torch.equal(o2[:, :, :w.N], o1[:, :, :w.N]) and torch.equal(l2, l1)
+
+
+@pytest.mark.parametrize("block", [128, 64])
+def test_fp8_lists_of_every_short_length(block):
+    """The scales of a list entry are fetched two entries ahead: lists of 1 to 9 entries with gaps, blocks of very different scale."""
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=8, Wg=2 * block - 3, block=block, k=4)      # 16 blocks, ragged tail
+    (q, k, v), _ = U.host_inputs(w)
+    gain = (2.0 ** ((torch.arange(w.n_alloc) // block) % 5 - 2).float())[None, None, :, None]
+    q, k = (q.float() * gain).bfloat16(), (k.float() / gain).bfloat16()
+    from paper_2606_23743_b200.workloads import bf16_bits
+    qb, kb, vb = bf16_bits(q), bf16_bits(k), bf16_bits(v)
+    q8, k8, qs, ks = _quantize(w, U.dev(q), U.dev(k))
+    qh, kh = U.oracle_fp8_inputs(w, qb, kb, q8, k8, qs, ks)
+    lists = [sorted({(3 * r + 5 * i) % w.Nb for i in range(1 + r % 9)}) for r in range(w.R)]
+    rp = torch.zeros(w.R + 1, dtype=torch.int32)
+    rp[1:] = torch.cumsum(torch.tensor([len(x) for x in lists]), 0)
+    rp, ci = rp.cuda(), torch.tensor([j for x in lists for j in x], dtype=torch.int32).cuda()
+    o, lse, st = U.gpu_attn(w, q8, k8, U.dev(v), rp, ci, q_scale=qs, k_scale=ks, fp8=True)
+    assert st == 0
+    U.check_attn_vs_oracle(w, qh, kh, vb, rp, ci, o, lse, list(range(w.R)), rel_tol=U.FP8_REL_L2, abs_tol=5e-2)
