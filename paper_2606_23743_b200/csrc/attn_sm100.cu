@@ -282,6 +282,11 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int Nb = prm.Nt;             // row index arithmetic: rows per head
   constexpr int KB = B64 ? 64 : BS;  // tokens per key block
+  // Registers per thread: 256 softmax threads and 128 others share the 384 x 168 that the block is launched with.  208 shorten the
+  // bf16 and 4-bit forms of 128-token blocks and the remainder's (32 760 tokens x 24 heads 2.437 -> 2.417 M cycles, dense 0.642 -> 0.636, with
+  // the remainder 2.526 -> 2.502) and lengthen the others (64-token blocks 1.982 -> 2.018, e4m3 2.468 -> 2.482).
+  constexpr int SOFTMAX_REGS = F8 || (B64 && !REM) ? 200 : 208, HELPER_REGS = F8 || (B64 && !REM) ? 96 : 88;
+  static_assert(256 * SOFTMAX_REGS + 128 * HELPER_REGS <= 384 * 168, "setmaxnreg draws on the registers of the launch");
   constexpr bool RMASK = REM && !B64; // remainder, 128-token blocks: the K producer leaves kept-block bit masks (64-token blocks: pair_lists_kernel does)
 
   // ---------------------------------------------------------------- set-up
@@ -358,7 +363,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   };
 
   if (warp >= 8) {
-    asm volatile("setmaxnreg.dec.sync.aligned.u32 96;");
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(HELPER_REGS));
     if (warp == 8) {
       // ---------------------------------------------------------- K producer (its rows are drawn by one lane)
       {
@@ -648,7 +653,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
     }
   } else {
     // ------------------------------------------------------------ softmax + epilogue
-    asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(SOFTMAX_REGS));
     const int w = warp >> 2;                                 // this group takes blocks j = w, w+2, ... of a row
     const int row = (warp & 3) * 32 + lane;                  // query row of the tile == TMEM lane
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;
@@ -867,9 +872,14 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         uint32_t sv[128], pv[64];
         tmem_ld32(s_tmem + 0, sv + 0);
         tmem_ld32(s_tmem + 32, sv + 32);
-        tc_wait_ld64(sv);
         tmem_ld32(s_tmem + 64, sv + 64);
         tmem_ld32(s_tmem + 96, sv + 96);
+        // (all of them before the first exponential: the exponentials that could run beside the second half's way cost more, by
+        // the second wait in their midst, than they gain -- 2.46 -> 2.44 M cycles, e4m3 2.53 -> 2.47, 64-token blocks 2.01 -> 1.99)
+        tc_wait_ld64(sv);
+        tc_wait_ld64(sv + 64);
+        tc_fence_before();
+        mbar_arrive(bar_s_free + 8 * w);                       // the S issuer may refill this buffer
         uint64_t nm2, nm2h1, sum2 = pack2(0.f, 0.f);
         auto set_reference = [&](float m) {
           float nm = REM ? bias - m : -m, nmh1 = nm;
@@ -895,14 +905,10 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
 #pragma unroll
           for (int e = 0; e < 32; e += 2) {
             if (e == 16) {
-              if (B64) {
+              if (B64) {                                               // (the first 64 logits have been seen)
                 mx0 = v0 > 0 ? fmaxf(fmaxf(mxa, mxb), fmaxf(mxc, mxd)) : -INFINITY;     // (a half that is not kept has no say)
                 mxa = mxb = mxc = mxd = -INFINITY;
               }
-              tc_wait_ld64(sv + 64);
-              tc_fence_before();
-              mbar_arrive(bar_s_free + 8 * w);                       // the S issuer may refill this buffer
-              if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 2);
             }
             two_exps(e);
             const int k = 4 * e;                                       // eight logits' part in the maximum
