@@ -27,7 +27,7 @@
 // soon as its warpgroup has read it into registers: the MMA warp computes S(j+2) while the softmax
 // of block j is still running.  P is single-buffered: block j's P is stored once P V(j-1) has
 // completed, which also staggers the two warpgroups so that one group's exponentials overlap the
-// other group's maximum pass and stores.
+// other group's loads and stores.
 //
 // The two warpgroups share one O accumulator, so they share the reference exponent m of every row (P = 2^(S*c - m)).  A row
 // starts with m = 0, and m is a whole number that changes only when a tile's maximum leaves it far behind (LAZY_LOG2; for the
@@ -35,7 +35,7 @@
 // with the m that its own last tile ended with; the maximum is taken beside the first of them and looked at afterwards, and
 // the m that the other group ended tile j-1 with is compared when P V(j-1) has completed, just before P is handed over.  Where they
 // differ the larger one wins and P, or O, is scaled by a power of two.  Nothing that is common waits for a maximum or for the other
-// group's (exponentials after maximum and exchange: 1 610 cycles per tile of 128 x 128; this form: 1 480, 32 760 tokens x 24 heads).
+// group's (exponentials after maximum and exchange: 1 610 cycles per tile of 128 x 128; this form: 1 457, 32 760 tokens x 24 heads).
 // Row sums are kept per group and merged in the epilogue, where each group normalises its half of O into a swizzled staging
 // panel that one TMA tile store writes out.
 //
@@ -146,7 +146,8 @@ constexpr uint32_t COL_O = 256, COL_Q = 384, COL_P = 448;
 // set for the row's first keys only when their maximum is further than FRESH_LOG2 from the 0 that it starts with.  P then
 // reaches at most 2^48 and a row sum 2^48 * N: far inside fp32 (and bf16 has fp32's exponent range), and a change -- half a
 // tile's worth of cycles -- is rare: logits (in powers of two) of 32 760 tokens x 24 heads reach 21 and of sharper ones (Q and K
-// times 1.5) 49, with first maxima of 19 and 40.  (16 and 32 in their place: 10.0 instead of 9.7 M cycles on the latter.)
+// times 1.5) 49, with first maxima of 19 and 40.  (With 32 for both, and each group setting a row's first reference for itself, the
+// latter took 12.7 M cycles, a third more than with the maximum first.)
 constexpr float LAZY_LOG2 = 48.0f;
 constexpr float FRESH_LOG2 = 40.0f;
 }  // namespace ts
@@ -252,9 +253,8 @@ __device__ __noinline__ void mask_pooled_from_csr(const int32_t* row_ptr, const 
 // block-scaled 4-bit MMA whose operands both come from shared memory (the Q tile is fetched by TMA once per row
 // instead of being written to tensor memory; tm_kp is the map of the Q codes), with the scale factors copied
 // into the tensor-memory columns the bf16 Q would have used.  128-token blocks, d = 128 only.
-// VMN: V is read where it lies ([keys][d], d contiguous) and enters P V as an MN-major B operand -- another
-// instruction descriptor than S, which costs a tensor-pipe drain per switch (hidden in the pipe's idle time: +1 % of
-// the cycles), but no transposed copy of V and no workspace for it.  Every one-call entry point uses it; tm_vt is then
+// VMN: V is read where it lies ([keys][d], d contiguous) and enters P V as an MN-major B operand: no transposed copy of V and no
+// workspace for it.  Every one-call entry point uses it; tm_vt is then
 // the map of V (and, with REM, tm_vtp the block means of V as rows and tm_at the matrices A_I rather than their transposes).
 template <bool B64, bool F8, bool REM, bool F4 = false, bool VMN = false>
 __global__ void __launch_bounds__(384, 1)
