@@ -575,9 +575,12 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const int n = __shfl_sync(0xffffffffu, cur.n, 0);
         for (int j = 0; j < n; ++j) {
           const int w = j & 1;
-          if (cs[w] > 0) mbar_wait(bar_s_free + 8 * w, (cs[w] - 1u) & 1u, abort_flag);
+          // (a wait that has run out ends the loop, for all lanes: nothing more is issued, and nothing committed that others wait for)
+          ok = cs[w] == 0 || mbar_wait(bar_s_free + 8 * w, (cs[w] - 1u) & 1u, abort_flag);
           if (lane == 0) SVA_STAMP(2, i, j, 0);
-          mbar_wait(bar_k_full + 8 * s, ph, abort_flag);
+          ok = ok && mbar_wait(bar_k_full + 8 * s, ph, abort_flag);
+          ok = __all_sync(0xffffffffu, ok);
+          if (!ok) break;
           if (lane == 0) SVA_STAMP(2, i, j, 1);
           tc_fence_after();
           const uint64_t kd = kd0 + (uint64_t)(s * (TILE >> 4));
@@ -612,6 +615,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           ++cs[w];
           if (++s == KS) { s = 0; ph ^= 1u; }
         }
+        if (!ok) break;
       }
     } else {
       // ---------------------------------------------------------- P V issuer
@@ -632,9 +636,11 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         for (int j = 0; j < n; ++j) {
           const int w = j & 1;
           const uint64_t vd = vd0 + (uint64_t)(s * (TILE >> 4));
-          mbar_wait(bar_v_full + 8 * s, ph, abort_flag);
+          ok = mbar_wait(bar_v_full + 8 * s, ph, abort_flag);
           if (lane == 0) SVA_STAMP(3, i, j, 0);
-          mbar_wait(bar_p_full + 8 * w, cp[w] & 1u, abort_flag);
+          ok = ok && mbar_wait(bar_p_full + 8 * w, cp[w] & 1u, abort_flag);
+          ok = __all_sync(0xffffffffu, ok);                           // (as in the S issuer)
+          if (!ok) break;
           if (lane == 0) SVA_STAMP(3, i, j, 1);
           tc_fence_after();
 #pragma unroll
@@ -649,6 +655,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           ++cp[w];
           if (++s == VS) { s = 0; ph ^= 1u; }
         }
+        if (!ok) break;
       }
     }
   } else {
