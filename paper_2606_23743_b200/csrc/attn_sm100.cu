@@ -348,7 +348,8 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
   struct Row { int r, n, beg; uint32_t e0, e1; int I, hh, bb; };
   auto fetch_row = [&](uint32_t i, Row& R, bool arrive) -> bool {
     const uint32_t slot = i % QD;
-    if (!mbar_wait(bar_rq_full + 8 * slot, (i / QD) & 1u, abort_flag)) return false;
+    // (one answer for the warp: where a wait has run out, no lane may be left in the warp barrier below)
+    if (!__all_sync(0xffffffffu, mbar_wait(bar_rq_full + 8 * slot, (i / QD) & 1u, abort_flag))) return false;
     R.r = rowq[8 * slot];
     R.n = rowq[8 * slot + 1];
     R.beg = rowq[8 * slot + 2];
