@@ -198,7 +198,8 @@ weights_kernel(const float* __restrict__ scores, const int32_t* __restrict__ row
     }
     __syncwarp();
   }
-  if (lane == 0) mu[r] = none ? 0.f : mx;
+  // (nothing dropped: -inf, so that the first-order tile's factor exp(mu - m) is 0 for every reference m, also one far below 0)
+  if (lane == 0) mu[r] = mx;
 }
 
 // ------------------------------------------------------------------ A_I^T = sum_J W[I][J] C_J^T

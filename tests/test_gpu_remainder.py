@@ -277,3 +277,25 @@ def test_first_order_statistics_at_the_edges(block, nb, tail):
     max_abs, rel, lse_err = U.attn_errors(o, lse, o_ref, l_ref, rows, w.N, w.block, 1)
     # (the correction is not bounded by V: one bf16 unit of the largest output)
     assert max_abs <= max(U.BF16_MAX_ABS, 2.0 ** -7 * float(np.nanmax(np.abs(o_ref)))) and rel <= U.BF16_REL_L2 and lse_err <= 2e-3
+
+
+@pytest.mark.parametrize("block", [128, 64])
+def test_rows_that_drop_nothing_with_logits_far_below_zero(block):
+    """First-order term, all logits near -300 (powers of two): a row that keeps every block has no dropped block to weigh (its A_I is
+    zero) and stays the exact result, beside rows that drop some."""
+    from paper_2606_23743_b200.workloads import bf16_bits
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=8, Wg=block + 5, block=block, k=4)       # 9 blocks, ragged tail
+    gen = torch.Generator().manual_seed(11)
+    q = 1.0 + 0.05 * torch.randn(1, 1, w.n_alloc, w.d, generator=gen)
+    k = -300.0 / (w.scale * 1.4426950408889634 * w.d) + 0.3 * torch.randn(1, 1, w.n_alloc, w.d, generator=gen)
+    v = 2.0 * torch.rand(1, 1, w.n_alloc, w.d, generator=gen) - 1.0
+    q, k, v = (x.bfloat16() for x in (q, k, v))
+    qb, kb, vb = bf16_bits(q), bf16_bits(k), bf16_bits(v)
+    _, _, scores = U.gpu_select(w, U.dev(q), U.dev(k), want_scores=True)
+    lists = [list(range(w.Nb)), [0, 3], list(range(w.Nb)), list(range(w.Nb)), [1], [2, 5, 8], list(range(8)), [4], list(range(w.Nb))]
+    rp = torch.zeros(w.R + 1, dtype=torch.int32)
+    rp[1:] = torch.cumsum(torch.tensor([len(x) for x in lists]), 0)
+    rp, ci = rp.cuda(), torch.tensor([j for x in lists for j in x], dtype=torch.int32).cuda()
+    o, lse, st = gpu_remainder(w, U.dev(q), U.dev(k), U.dev(v), rp, ci, 1, scores=scores)
+    assert st == 0 and torch.isfinite(o[:, :, :w.N]).all() and torch.isfinite(lse).all()
+    check_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, [r for r in range(w.R) if len(lists[r]) == w.Nb], 1)
