@@ -147,9 +147,12 @@ constexpr uint32_t COL_O = 256, COL_Q = 384, COL_P = 448;
 // reaches at most 2^48 and a row sum 2^48 * N: far inside fp32 (and bf16 has fp32's exponent range), and a change -- half a
 // tile's worth of cycles -- is rare: logits (in powers of two) of 32 760 tokens x 24 heads reach 21 and of sharper ones (Q and K
 // times 1.5) 49, with first maxima of 19 and 40.  (With 32 for both, and each group setting a row's first reference for itself, the
-// latter took 12.7 M cycles, a third more than with the maximum first.)
+// latter took 12.7 M cycles, a third more than with the maximum first.)  Rows of a warp that change at different tiles each cost the warp
+// a pass, so FRESH_LOG2 lies where sharp rows set theirs at their first tile, together.  With 8 / 16 / 24 / 32 / 40 there, M cycles: 32 760 x 24
+// 2.43 / 2.42 / 2.42 / 2.42 / 2.42, its Q and K times 2 0.57 / 0.57 / 0.58 / 0.69 / 0.78 (0.78 with the maximum first), 64-token blocks 2.02 / 1.97 / 1.98 / 1.97 /
+// 1.98, their Q and K times 2 2.02 / 2.03 / 2.15 / 2.35 / 2.68.
 constexpr float LAZY_LOG2 = 48.0f;
-constexpr float FRESH_LOG2 = 40.0f;
+constexpr float FRESH_LOG2 = 16.0f;
 }  // namespace ts
 
 // control block (bytes from OFF_CTRL):
@@ -931,9 +934,11 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           top = (B64 && F8) ? fmaxf(v0 > 0 ? mx0 * c : -INFINITY, v1 > 0 ? mx1 * c1 : -INFINITY) : fmaxf(mx0, mx1);
           mx = (B64 && F8) ? top : REM ? top * c + bias : top * c;
         }
+        // (each row decides by itself: its bits do not depend on the rows beside it)
         const bool fresh = __float_as_uint(m_try) == 0x80000000u;
-        if (__builtin_expect(__any_sync(0xffffffffu, fresh ? fabsf(mx) > FRESH_LOG2 && mx > -INFINITY : mx > m_try + LAZY_LOG2), 0)) {
-          if (fresh ? fabsf(mx) > 8.f && mx > -INFINITY : mx > m_try + 8.f) {
+        const bool far_off = fresh ? fabsf(mx) > FRESH_LOG2 && mx > -INFINITY : mx > m_try + LAZY_LOG2;
+        if (__builtin_expect(__any_sync(0xffffffffu, far_off), 0)) {
+          if (far_off) {
             const float m_up = ceilf(mx);
             if (l != 0.f) { const float f = ex2(m_try - m_up); l *= f; l_top *= f; }
             m_try = m_up;
@@ -983,8 +988,12 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           l *= fp;
           l_top *= fp;
           tc_wait_st();
+          // (64-token blocks leave out a pass in which no row of the warp changes: Q and K times 3, 2.52 -> 2.37 M cycles.  The others do not gain.)
+          constexpr bool CHOOSE = B64 && !REM;
+          const int p_end = !CHOOSE || __any_sync(0xffffffffu, fp != 1.f) ? D / 2 : 0;
+          const int o_end = j > 0 && (!CHOOSE || __any_sync(0xffffffffu, fo != 1.f)) ? D : 0;
 #pragma unroll 1
-          for (int cc = 0; cc < D / 2; cc += 16) {
+          for (int cc = 0; cc < p_end; cc += 16) {
             uint32_t ov[16];
             tmem_ld16(p_tmem + cc, ov);
             tc_wait_ld();
@@ -993,7 +1002,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
             tmem_st16(p_tmem + cc, ov);
           }
 #pragma unroll 1
-          for (int cc = 0; cc < D && j > 0; cc += 16) {
+          for (int cc = 0; cc < o_end; cc += 16) {
             uint32_t ov[16];
             tmem_ld16(o_tmem + cc, ov);
             tc_wait_ld();

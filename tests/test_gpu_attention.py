@@ -387,3 +387,21 @@ def test_a_q_that_heads_or_items_share(shared):
     o, lse, st = U.gpu_attn(w, qc, k, v, rp, ci)
     ox, lx, sx = U.gpu_attn(w, qx, k, v, rp, ci)
     assert st == 0 and sx == 0 and torch.equal(ox, o) and torch.equal(lx, lse)
+
+
+@pytest.mark.parametrize("block", [128, 64])
+def test_a_row_does_not_depend_on_the_rows_beside_it(block):
+    """A row whose logits move its reference leaves the bits of the other rows of its warp as they are."""
+    w = shrink(WORKLOADS["medium"], H=2, T=2, block=block, k=7, qk_mult=1.5)              # largest logits about 8 to 40 powers of two
+    (q, k, v), _ = U.host_inputs(w)
+    k, v = U.dev(k), U.dev(v)
+    rp, ci, _ = U.gpu_select(w, U.dev(q), k)
+    o, lse, st = U.gpu_attn(w, U.dev(q), k, v, rp, ci)
+    sharp = torch.arange(w.n_alloc) % 32 == 7                                             # one row in every warp
+    q = q.clone()
+    q[:, :, sharp] = (q[:, :, sharp].float() * 30.0).bfloat16()
+    o2, lse2, st2 = U.gpu_attn(w, U.dev(q), k, v, rp, ci)
+    assert st == 0 and st2 == 0
+    same = ~sharp[:w.N].cuda()
+    assert torch.equal(o2[:, :, :w.N][:, :, same], o[:, :, :w.N][:, :, same]) and torch.equal(lse2[:, :, same], lse[:, :, same])
+    assert not torch.equal(o2, o)
