@@ -195,6 +195,8 @@ int sva_block_select_noalloc(const sva_problem_t* p, const sva_select_t* s, cons
  *   o_i = sum_j softmax_j(scale*<q_i,k_j>) v_j,  j over the valid keys of the kept blocks
  *   lse_i = log sum_j exp(scale*<q_i,k_j>)       (optional, [B,H,N] fp32 contiguous)
  * O is bf16.  A row with an empty list writes zeros and lse = -inf.
+ * P V is summed in fp32 with probabilities that are not normalised yet (a row's largest lies between 2^-32 and 2^32): |V| may reach 2^80; below
+ * 2^-94 products sink into denormals.
  * q, k, v, o must be 16-byte aligned and every stride a multiple of 8 elements
  * (16 for e4m3 Q/K).  One tensor-core kernel (bf16 x bf16 or e4m3 x e4m3 MMA for Q K^T, bf16 for P V,
  * fp32 accumulate) serves every supported shape: d = 128 or 64 (64 is computed as 128 with a zero upper

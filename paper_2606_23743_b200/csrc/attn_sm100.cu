@@ -29,7 +29,7 @@
 // completed, which also staggers the two warpgroups so that one group's exponentials overlap the
 // other group's loads and stores.
 //
-// The two warpgroups share one O accumulator, so they share the reference exponent m of every row (P = 2^(S*c - m)).  A row
+// The two warpgroups share one O accumulator, so they share the reference exponent m of every row (P = 2^(S*c - m - 16)).  A row
 // starts with m = 0, and m is a whole number that changes only when a tile's maximum leaves it far behind (LAZY_LOG2; for the
 // row's first keys FRESH_LOG2): then -- rarely -- the group takes the maximum, rounded up.  A group starts a tile's exponentials
 // with the m that its own last tile ended with; the maximum is taken beside the first of them and looked at afterwards, and
@@ -143,16 +143,18 @@ constexpr int SMEM_BYTES = OFF_KMASK + 1024 + 1024;          // + alignment slac
 constexpr uint32_t COL_SFA = 384, COL_SFB = 392;              // 4-bit variant: scale factors in the Q columns (8 + 2 x 8)
 constexpr uint32_t COL_O = 256, COL_Q = 384, COL_P = 448;
 // The reference exponent of a row is raised only when a block's maximum exceeds it by more than LAZY_LOG2 powers of two, and
-// set for the row's first keys only when their maximum is further than FRESH_LOG2 from the 0 that it starts with.  P then
-// reaches at most 2^48 and a row sum 2^48 * N: far inside fp32 (and bf16 has fp32's exponent range), and a change -- half a
-// tile's worth of cycles -- is rare: logits (in powers of two) of 32 760 tokens x 24 heads reach 21 and of sharper ones (Q and K
-// times 1.5) 49, with first maxima of 19 and 40.  (With 32 for both, and each group setting a row's first reference for itself, the
-// latter took 12.7 M cycles, a third more than with the maximum first.)  Rows of a warp that change at different tiles each cost the warp
+// set for the row's first keys only when their maximum is further than FRESH_LOG2 from the 0 that it starts with: a change costs half a
+// tile's worth of cycles.  P = 2^(logit - m - P_SHIFT): a row's largest P then lies between 2^-32 and 2^32, its sum below 2^32 * N, and P V
+// neither overflows for |V| up to 2^80 nor sinks into denormals for |V| above 2^-94 (without the shift, and 40 for FRESH_LOG2, 2^64 and 2^-86).
+// A smaller line and shift would raise references often: logits (in powers of two) of 32 760 tokens x 24 heads reach 21 and of sharper ones (Q and K
+// times 1.5) 49, with first maxima of 19 and 40.  (47 616 tokens x 32 x 2, Q and K times 1.5: 8.64 M cycles with 48 and 16, 8.73 with 40 and
+// 8, 9.53 with 32 and 0.)  Rows of a warp that change at different tiles each cost the warp
 // a pass, so FRESH_LOG2 lies where sharp rows set theirs at their first tile, together.  With 8 / 16 / 24 / 32 / 40 there, M cycles: 32 760 x 24
 // 2.43 / 2.42 / 2.42 / 2.42 / 2.42, its Q and K times 2 0.57 / 0.57 / 0.58 / 0.69 / 0.78 (0.78 with the maximum first), 64-token blocks 2.02 / 1.97 / 1.98 / 1.97 /
 // 1.98, their Q and K times 2 2.02 / 2.03 / 2.15 / 2.35 / 2.68.
 constexpr float LAZY_LOG2 = 48.0f;
 constexpr float FRESH_LOG2 = 16.0f;
+constexpr float P_SHIFT = 16.0f;
 }  // namespace ts
 
 // control block (bytes from OFF_CTRL):
@@ -873,7 +875,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
           }
           tc_wait_st();
         }
-        // P = 2^(S*c - m) with the reference m that this group's last tile ended with; the row maximum is taken beside the
+        // P = 2^(S*c - m - 16) with the reference m that this group's last tile ended with; the row maximum is taken beside the
         // first 32 exponentials, in issue slots that they leave empty, and looked at after them: only when it has outgrown m
         // (or m is still the 0 that a row starts with and the maximum lies far from it) are these 32 done again.
         // (64-token blocks: -inf instead of -m for a half that is not kept makes those P exactly 0 at no cost)
@@ -893,7 +895,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         mbar_arrive(bar_s_free + 8 * w);                       // the S issuer may refill this buffer
         uint64_t nm2, nm2h1, sum2 = pack2(0.f, 0.f);
         auto set_reference = [&](float m) {
-          float nm = REM ? bias - m : -m, nmh1 = nm;
+          float nm = REM ? bias - P_SHIFT - m : -P_SHIFT - m, nmh1 = nm;
           if (B64) {
             if (v0 == 0) nm = -INFINITY;
             if (v1 == 0) nmh1 = -INFINITY;
@@ -952,7 +954,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         // P V sums P rounded to bf16.  Its normaliser takes the largest P of every tile as rounded too, so that a row that is all
         // but one key comes out as that key's V (as it does where the reference is the row maximum and that P exactly 1).
         {
-          const float p = ex2((B64 && F8) ? top - m_try : fmaf(top, c, REM ? bias - m_try : -m_try));
+          const float p = ex2((B64 && F8) ? top - P_SHIFT - m_try : fmaf(top, c, REM ? bias - P_SHIFT - m_try : -P_SHIFT - m_try));
           if (p < INFINITY) l_top += __uint_as_float(pack_bf16(0.f, p) & 0xffff0000u) - p;
         }
         if (j == 0) {
@@ -1039,7 +1041,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         const int qb = B64 ? min(2 * I + qh, prm.Nb - 1) : I;
         const bool mine_rows = (qi < prm.N) && (!B64 || qh == (int)(J_now & 1u));
         const float f = mine_rows ? prm.scale_log2 * 0.6931471805599453f *
-                                        ex2(__ldg(prm.mu + (long long)bh * prm.Nb + qb) * 1.4426950408889634f - m_now)
+                                        ex2(__ldg(prm.mu + (long long)bh * prm.Nb + qb) * 1.4426950408889634f - P_SHIFT - m_now)
                                   : 0.f;
 #pragma unroll 1
         for (int cc = 0; cc < D / 2; cc += 16) {
@@ -1138,7 +1140,7 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         }
         if (qi < prm.N && prm.lse && w == 0) {
           const float ls = l * f0 + (lxr[128 + row] - ltop[(rows_done & 1u) * 128 + row]) * f1;     // (the sum itself)
-          prm.lse[(long long)bh * prm.N + qi] = B64 || __float_as_uint(m_fin) != 0x80000000u ? (m_fin + log2f(ls)) * 0.6931471805599453f : NAN;
+          prm.lse[(long long)bh * prm.N + qi] = B64 || __float_as_uint(m_fin) != 0x80000000u ? (m_fin + P_SHIFT + log2f(ls)) * 0.6931471805599453f : NAN;
         }
       }
       if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, 255, 10);

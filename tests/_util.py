@@ -161,3 +161,23 @@ def oracle_fp8_inputs(w: Workload, qb, kb, q8, k8, qs, ks):
         assert np.array_equal(g8.cpu().numpy()[:, :, :w.N], codes[:, :, :w.N])
         out.append(oracle.dequantize_e4m3(codes, scales, w.N, w.block))
     return out
+
+
+def level_inputs(levels, block, seed=0):
+    """Inputs of one head and 9 key blocks whose logits lie near `levels` (powers of two, a level per key block; 0 for the rest), and lists
+    of odd and even lengths that differ between the query blocks of a tile: (workload, (q, k, v), (row_ptr, col_idx) on the GPU)."""
+    from paper_2606_23743_b200.workloads import WORKLOADS, shrink
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=8, Wg=block + 5, block=block, k=4)       # ragged tail
+    gen = torch.Generator().manual_seed(seed)
+    lev = torch.tensor([levels[j] if j < len(levels) else 0.0 for j in range(w.Nb)]).repeat_interleave(block)[:w.N]
+    q = torch.ones(1, 1, w.n_alloc, w.d) + 0.05 * torch.randn(1, 1, w.n_alloc, w.d, generator=gen)
+    k = torch.zeros(1, 1, w.n_alloc, w.d)
+    k[0, 0, :w.N] = (lev / (w.scale * 1.4426950408889634 * w.d))[:, None] + 0.3 * torch.randn(w.N, w.d, generator=gen)
+    v = 2.0 * torch.rand(1, 1, w.n_alloc, w.d, generator=gen) - 1.0
+    q[:, :, w.N:] = 0.0
+    v[:, :, w.N:] = 0.0
+    lists = [list(range(w.Nb)), [0], [1, 2, 3, 4], [0, 4, 5, 8], list(range(1, w.Nb, 2)), list(range(0, w.Nb, 2)), [8], [2, 3], [5, 6, 7]]
+    rp = torch.zeros(w.R + 1, dtype=torch.int32)
+    rp[1:] = torch.cumsum(torch.tensor([len(x) for x in lists]), 0)
+    ci = torch.tensor([j for x in lists for j in x], dtype=torch.int32)
+    return w, (q.bfloat16(), k.bfloat16(), v.bfloat16()), (rp.cuda(), ci.cuda())

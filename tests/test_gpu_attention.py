@@ -405,3 +405,22 @@ def test_a_row_does_not_depend_on_the_rows_beside_it(block):
     same = ~sharp[:w.N].cuda()
     assert torch.equal(o2[:, :, :w.N][:, :, same], o[:, :, :w.N][:, :, same]) and torch.equal(lse2[:, :, same], lse[:, :, same])
     assert not torch.equal(o2, o)
+
+
+@pytest.mark.parametrize("block", [128, 64])
+@pytest.mark.parametrize("levels,power", [([5.0, 45.0, 30.0], 80), ([30.0, 70.0, 99.0], 80), ([-39.0], -104), ([-14.0], -90)])
+def test_v_far_from_unit_size(levels, power, block):
+    """A row's largest P stays within 2^-32 and 2^32: V times a power of two gives the output times it, for |V| up to 2^80 and down to about
+    2^-94, whichever way the logits (one level per key block) lie to the reference."""
+    w, (q, k, v), (rp, ci) = U.level_inputs(levels, block)
+    q, k, v = U.dev(q), U.dev(k), U.dev(v)
+    o, lse, st = U.gpu_attn(w, q, k, v, rp, ci)
+    o2, lse2, st2 = U.gpu_attn(w, q, k, (v.double() * 2.0 ** power).bfloat16(), rp, ci)
+    assert st == 0 and st2 == 0 and torch.equal(lse2, lse)
+    back, want = o2[:, :, :w.N].double() * 2.0 ** -power, o[:, :, :w.N].double()
+    if power > 0:
+        assert torch.equal(back, want)
+    else:
+        # V of unit size times 2^power times P (about 2^-16, 2^-30) is 2^-120 here: products below 2^-126 may be flushed, those of the
+        # elements of V below 2^-6
+        assert float((back - want).norm() / want.norm()) <= 2e-3
