@@ -33,7 +33,7 @@
 // starts with m = 0, and m is a whole number that changes only when a tile's maximum leaves it far behind (LAZY_LOG2; for the
 // row's first keys FRESH_LOG2): then -- rarely -- the group takes the maximum, rounded up.  A group starts a tile's exponentials
 // with the m that its own last tile ended with; the maximum is taken beside the first of them and looked at afterwards, and
-// the m that the other group ended tile j-1 with is compared when P V(j-1) has completed, just before P is handed over.  Where they
+// the m that the other group ended tile j-1 with is read once that group has handed P over and compared when P V(j-1) has completed.  Where they
 // differ the larger one wins and P, or O, is scaled by a power of two.  Nothing that is common waits for a maximum or for the other
 // group's (exponentials after maximum and exchange: 1 610 cycles per tile of 128 x 128; this form: 1 457, 32 760 tokens x 24 heads).
 // Row sums are kept per group and merged in the epilogue, where each group normalises its half of O into a swizzled staging
@@ -972,13 +972,17 @@ attn_ts_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__
         if ((threadIdx.x & 127) == 0) SVA_STAMP(w, rows_done, j, 4);
         // the P columns are free once P V(j-1) has completed (block 0: the previous row's last P V
         // was waited for in that row's epilogue)
+        // (... and the reference that O is relative to is what the other group's tile j-1 ended with: its threads wrote it before they arrived
+        // on p_full.  That phase ends well before P V(j-1) does, and its successor waits for this tile.)
+        float m_prev = m_try;
+        if (j > 0) {
+          if (!mbar_wait(bar_p_full + 8 * (w ^ 1), prev & 1u, abort_flag)) return false;
+          m_prev = refr[(w ^ 1) * 128 + row];
+        }
         if (j > 0 && !mbar_wait(bar_pv_done + 8 * (w ^ 1), prev & 1u, abort_flag)) return false;
         tc_fence_after();
         tmem_st32(p_tmem, pv);
         tmem_st32(p_tmem + 32, pv + 32);
-        // The reference that O is relative to: what the other group's tile j-1 ended with.  (Its threads wrote it before they
-        // arrived on p_full, without which P V(j-1) would not have been issued.)
-        const float m_prev = j > 0 ? refr[(w ^ 1) * 128 + row] : m_try;
         float m_new = __uint_as_float(__float_as_uint(m_prev) & __float_as_uint(m_try));       // (equal, or zeros: -0 only if both are)
         if (__builtin_expect(__any_sync(0xffffffffu, m_prev != m_try), 0)) {
           // The larger one wins; O, or P and the row sum, follow (O is quiescent: P V(j) waits for us; P scales exactly,
