@@ -7,6 +7,7 @@ import _util as U
 from oracle import nvfp4
 from paper_2606_23743_b200 import binding as B
 from paper_2606_23743_b200.workloads import WORKLOADS, bf16_bits, shrink
+from test_gpu_attention import REFERENCE_LOGITS
 
 pytestmark = pytest.mark.gpu
 
@@ -160,3 +161,14 @@ def test_a_nan_costs_its_scale_block_nothing_but_its_own_code(magnitude):
         got, want = (np.stack((c & 15, c >> 4), axis=-1).reshape(w.B, w.H, w.N, w.d) for c in (got, codes[:, :, :w.N]))
         assert (got[where[h]] & 7 == (7 if magnitude == 1.0 else 0)).all()
         np.testing.assert_array_equal(np.where(where[h], 0, got), np.where(where[h], 0, want))
+
+
+@pytest.mark.parametrize("name", list(REFERENCE_LOGITS))
+def test_fp4_reference_exponent_follows_the_logits(name):
+    """Logits below, above and at the lines where a row's reference changes, with 4-bit Q/K."""
+    w, (q, k, v), (rp, ci) = U.level_inputs(REFERENCE_LOGITS[name], 128, seed=len(name))
+    quant = gpu_quantize4(w, U.dev(q), U.dev(k))
+    qh, kh = oracle_dequantised(w, bf16_bits(q), bf16_bits(k))
+    o, lse, st = gpu_attn_fp4(w, quant, U.dev(v), rp, ci)
+    assert st == 0
+    U.check_attn_vs_oracle(w, qh, kh, bf16_bits(v), rp, ci, o, lse, list(range(w.R)), rel_tol=FP4_REL_L2, abs_tol=FP4_MAX_ABS)

@@ -8,6 +8,7 @@ import oracle
 import _util as U
 from paper_2606_23743_b200 import binding as B
 from paper_2606_23743_b200.workloads import WORKLOADS, shrink
+from test_gpu_attention import REFERENCE_LOGITS
 
 pytestmark = pytest.mark.gpu
 
@@ -258,3 +259,16 @@ def test_fp8_lists_of_every_short_length(block):
     o, lse, st = U.gpu_attn(w, q8, k8, U.dev(v), rp, ci, q_scale=qs, k_scale=ks, fp8=True)
     assert st == 0
     U.check_attn_vs_oracle(w, qh, kh, vb, rp, ci, o, lse, list(range(w.R)), rel_tol=U.FP8_REL_L2, abs_tol=5e-2)
+
+
+@pytest.mark.parametrize("block", [128, 64])
+@pytest.mark.parametrize("name", list(REFERENCE_LOGITS))
+def test_fp8_reference_exponent_follows_the_logits(name, block):
+    """Logits below, above and at the lines where a row's reference changes, with e4m3 Q/K (a scale per key block)."""
+    from paper_2606_23743_b200.workloads import bf16_bits
+    w, (q, k, v), (rp, ci) = U.level_inputs(REFERENCE_LOGITS[name], block, seed=len(name))
+    q8, k8, qs, ks = _quantize(w, U.dev(q), U.dev(k))
+    qh, kh = U.oracle_fp8_inputs(w, bf16_bits(q), bf16_bits(k), q8, k8, qs, ks)
+    o, lse, st = U.gpu_attn(w, q8, k8, U.dev(v), rp, ci, q_scale=qs, k_scale=ks, fp8=True)
+    assert st == 0
+    U.check_attn_vs_oracle(w, qh, kh, bf16_bits(v), rp, ci, o, lse, list(range(w.R)), rel_tol=U.FP8_REL_L2, abs_tol=5e-2)

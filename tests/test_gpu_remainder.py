@@ -6,8 +6,10 @@ import torch
 
 import oracle
 import _util as U
+from oracle import remainder
 from paper_2606_23743_b200 import binding as B
 from paper_2606_23743_b200.workloads import WORKLOADS, shrink
+from test_gpu_attention import REFERENCE_LOGITS
 
 pytestmark = pytest.mark.gpu
 
@@ -299,3 +301,56 @@ def test_rows_that_drop_nothing_with_logits_far_below_zero(block):
     o, lse, st = gpu_remainder(w, U.dev(q), U.dev(k), U.dev(v), rp, ci, 1, scores=scores)
     assert st == 0 and torch.isfinite(o[:, :, :w.N]).all() and torch.isfinite(lse).all()
     check_vs_oracle(w, qb, kb, vb, rp, ci, o, lse, [r for r in range(w.R) if len(lists[r]) == w.Nb], 1)
+
+
+@pytest.mark.parametrize("order", [0, 1])
+@pytest.mark.parametrize("block", [128, 64])
+@pytest.mark.parametrize("name", list(REFERENCE_LOGITS))
+def test_reference_exponent_follows_the_logits_of_block_means(name, block, order):
+    """Logits below, above and at the lines where a row's reference changes, in kept blocks and in the means of dropped ones."""
+    from paper_2606_23743_b200.workloads import bf16_bits
+    w, (q, k, v), (rp, ci) = U.level_inputs(REFERENCE_LOGITS[name], block, seed=len(name))
+    qb, kb, vb = bf16_bits(q), bf16_bits(k), bf16_bits(v)
+    _, _, scores = U.gpu_select(w, U.dev(q), U.dev(k), want_scores=True)
+    o, lse, st = gpu_remainder(w, U.dev(q), U.dev(k), U.dev(v), rp, ci, order, scores=scores)
+    assert st == 0
+    rows = list(range(w.R))
+    o_ref, l_ref = oracle.attn_remainder_rows(qb, kb, vb, w.N, w.block, w.scale, rp.cpu().numpy(), ci.cpu().numpy(), rows, order=order,
+                                              stats="bf16")
+    max_abs, rel, lse_err = U.attn_errors(o, lse, o_ref, l_ref, rows, w.N, w.block, 1)
+    abs_tol, rel_tol = U.BF16_MAX_ABS, U.BF16_REL_L2
+    if order == 1:
+        # The oracle weighs the first-order terms by block means rounded to bf16, the kernel by the routing's fp32 scores: keys of size
+        # |k| = |logit| / (scale * log2(e) * d) move a score by up to scale * sqrt(d) * 2^-9 |k| (independent roundings), the weight of a block
+        # against another by twice that, and the term, which is not bounded by V, by that share (an oracle with weights from unrounded
+        # means differs from this one by 0.096 and 2.6e-2 on low_then_high with 64-token blocks).
+        delta = 2.0 * w.scale * w.d ** 0.5 * 2.0 ** -9 * max(map(abs, REFERENCE_LOGITS[name])) / (w.scale * 1.4426950408889634 * w.d)
+        mag = float(np.nanmax(np.abs(o_ref)))
+        abs_tol, rel_tol = max(abs_tol, (2.0 ** -7 + delta) * mag), rel_tol + delta
+    assert max_abs <= abs_tol and rel <= rel_tol and lse_err <= 2e-3, (max_abs, rel, lse_err)
+
+
+@pytest.mark.parametrize("order", [0, 1])
+def test_more_than_1024_key_blocks(order):
+    """64-token blocks, 1 031 of them, lists of the caller's own: the weights mark kept blocks 1 024 at a time, and the kernel looks them up
+    in the lists (its bit masks hold 1 024)."""
+    from paper_2606_23743_b200.workloads import bf16_bits
+    nb = 1031
+    w = shrink(WORKLOADS["medium"], H=1, T=1, Hg=nb, Wg=64, block=64, k=6)
+    (q, k, v), (qb, kb, _) = U.host_inputs(w)
+    v = (v.float() + 4.0 * k.float()).to(torch.bfloat16)                     # (the first-order term is large: see above)
+    vb = bf16_bits(v)
+    rng = np.random.default_rng(6)
+    lists = [np.sort(rng.choice(nb, rng.integers(1, 9), replace=False)) for _ in range(nb)]
+    lists[0], lists[1], lists[2], lists[3] = np.array([1023, 1024, 1030]), np.array([0, 1024]), np.arange(nb), np.array([1030])
+    rp = torch.tensor(np.concatenate([[0], np.cumsum([len(x) for x in lists])]), dtype=torch.int32).cuda()
+    ci = torch.tensor(np.concatenate(lists), dtype=torch.int32).cuda()
+    kbar, qbar = (remainder.block_stats(x, x, w.N, 64, want_cov=False)[1] for x in (kb, qb))
+    scores = torch.tensor(w.scale * qbar[0, 0] @ kbar[0, 0].T, dtype=torch.float32).reshape(1, 1, nb, nb).cuda()
+    o, lse, st = gpu_remainder(w, U.dev(q), U.dev(k), U.dev(v), rp, ci, order, scores=scores)
+    assert st == 0
+    rows = [0, 1, 2, 3, 500, nb - 2, nb - 1]
+    o_ref, l_ref = oracle.attn_remainder_rows(qb, kb, vb, w.N, w.block, w.scale, rp.cpu().numpy(), ci.cpu().numpy(), rows, order=order,
+                                              stats="bf16")
+    max_abs, rel, lse_err = U.attn_errors(o, lse, o_ref, l_ref, rows, w.N, w.block, 1)
+    assert max_abs <= max(U.BF16_MAX_ABS, 2.0 ** -7 * float(np.nanmax(np.abs(o_ref)))) and rel <= U.BF16_REL_L2 and lse_err <= 2e-3
