@@ -25,7 +25,8 @@ void sva_debug_set_prof_buffer(void* buf);
  * Kernel behaviour switches for the next attention launches (0 = normal operation).
  *   bit 4: test aid: the K producer withholds a row's tiles after the first, so that a bounded pipeline wait
  *          runs out and the kernel takes its give-up path (SVA_DEV_TIMEOUT) -- nothing faults or hangs.
- *   bit 5: measurement aid: bf16 attention reads V where it lies (MN-major operand) instead of the transposed copy;
+ *   bit 5: measurement aid: the one-call forms (but the 4-bit one) read a transposed copy of V that they make first, as the two-step form
+ *          does, instead of V where it lies; they then need sva_attn_workspace_bytes() (the remainder: its own query, asked meanwhile);
  *   bit 7: test aid: the remainder call masks the kept blocks of a block-mean tile by looking them up in the CSR
  *          (the form that serves more than 1024 key blocks) even where the kept-block bit masks would serve.
  */

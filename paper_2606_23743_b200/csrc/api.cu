@@ -387,8 +387,8 @@ const char* sva_status_string(int status) {
 /* tuning aid (not part of the public header): device buffer of 320 int64; entry 319 receives the longest
    CTA's cycle count of the next attention launches; NULL = off */
 void sva_debug_set_prof_buffer(void* p) { ts_set_prof_buffer(p); }
-/* bit 0 skips the exponentials (tuning aid: results are wrong); bit 4 (test aid) withholds a row's K
-   tiles after the first so that a bounded wait runs out */
+/* bit 4 (test aid) withholds a row's K tiles after the first so that a bounded wait runs out; bit 5 (measurement aid) has the one-call
+   forms read a transposed copy of V; bit 7 (test aid) has the remainder look kept blocks up in the CSR */
 void sva_debug_set_mode(int v) { ts_set_debug_mode(v); }
 /* test aid: cycles a device-side wait may last before the CTA gives up (<= 0 restores the default) */
 int sva_debug_set_wait_limit(long long cycles) { return ts_set_wait_limit(cycles); }

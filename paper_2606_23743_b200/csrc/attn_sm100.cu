@@ -1571,7 +1571,7 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
   const bool b64 = m.block == 64;
   // With V at hand it is read where it lies (an MN-major B operand): no transposed copy, no workspace for it, and
   // under the power cap the step is faster without the copy's HBM traffic although the kernel needs 1 % more cycles.
-  // (The two-step form keeps the copy, and so does the remainder; bit 5 of the debug mode forces it here, to measure.)
+  // (The two-step form keeps the copy; bit 5 of the debug mode forces it here, to measure.)
   const bool vmn = v != nullptr && !(g_debug_ts & 32);
   const TsLayout L = ts_layout(m, vmn);
   uint8_t* wsb = static_cast<uint8_t*>(ws);
