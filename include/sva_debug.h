@@ -33,8 +33,8 @@ void sva_debug_set_prof_buffer(void* buf);
 void sva_debug_set_mode(int bits);
 
 /*
- * Test aid: the number of SM cycles a device-side wait may last before its CTA gives up (default 3e9;
- * cycles <= 0 restores the default).  Synchronous (a small host-to-device copy on the current device).
+ * Test aid: the number of SM cycles a device-side wait may last before its CTA gives up (default 3e9, at most 4e9: larger
+ * values count as that; cycles <= 0 restores the default).  Synchronous (a small host-to-device copy on the current device).
  * Returns 0 on success.
  */
 int sva_debug_set_wait_limit(long long cycles);
