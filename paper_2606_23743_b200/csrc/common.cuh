@@ -78,21 +78,30 @@ __device__ __forceinline__ int grid_dep_wait() {
   return zero;
 }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// (cluster: CTAs per thread-block cluster; the grid is then a multiple of it in x)
 template <typename... P, typename... A>
-inline int launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
-  cudaLaunchAttribute attr[1];
+inline int launch_dep_cluster(int cluster, void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim.x = (unsigned)cluster;
+  attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
   cfg.dynamicSmemBytes = smem;
   cfg.stream = st;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = cluster > 1 ? 2 : 1;
   if (cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...) == cudaSuccess) return SVA_OK;
   (void)cudaGetLastError();                    // (reported by the status; not left behind for the caller's next check)
   return SVA_ERR_CUDA;
+}
+
+template <typename... P, typename... A>
+inline int launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
+  return launch_dep_cluster(1, kern, grid, block, smem, st, static_cast<A&&>(args)...);
 }
 
 // Consecutive token blocks per CTA of the kernels that stream a tensor's blocks (`blocks` of them over all heads and tensors) with

@@ -5,7 +5,8 @@
 //
 // pool_kernel streams Q and K once from HBM: 128-bit loads, fp32 accumulation in a fixed order, a CTA per
 // run of one or four blocks of a head of a tensor.  block_scores_kernel computes a head's score matrix as a
-// small fp32 GEMM (64 x 64 or 32 x 32 tiles from two shared-memory panels, fixed summation order).
+// small fp32 GEMM (64 x 64 or 32 x 32 tiles from two shared-memory panels, fixed summation order).  Small problems take one
+// kernel for all three (route_cluster_kernel).
 // select_rows_kernel is one warp per query-block row: it reads the row's scores from that matrix (no shared
 // memory) as order-preserving integer keys, finds the threshold of the rule by narrowing an interval of scores
 // that holds it and emits the kept blocks in ascending order.  When the per-row count is known on the host (top-k with no window larger than k)
@@ -18,6 +19,22 @@
 namespace sva {
 
 static constexpr int POOL_THREADS = 256;
+
+// acc += the elements of a 16-byte vector (eight bf16 or sixteen e4m3 codes), in pairs
+template <int ELEM_BYTES>
+__device__ __forceinline__ void add_vector(const uint4& u, uint64_t (&acc)[8 / ELEM_BYTES]) {
+  const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    if constexpr (ELEM_BYTES == 2) {
+      acc[e] = add2(acc[e], pack2(bf16lo(w[e]), bf16hi(w[e])));
+    } else {
+      const float2 lo2 = e4m3x2_to_float2(w[e] & 0xffffu), hi2 = e4m3x2_to_float2(w[e] >> 16);
+      acc[2 * e] = add2(acc[2 * e], pack2(lo2.x, lo2.y));
+      acc[2 * e + 1] = add2(acc[2 * e + 1], pack2(hi2.x, hi2.y));
+    }
+  }
+}
 
 // Block means of one head of one tensor (blockIdx.z: 0 = Q, 1 = K); a CTA pools `run` consecutive blocks.
 // ELEM_BYTES = 2: bf16 input.  ELEM_BYTES = 1: e4m3 codes, multiplied by the block's scale.
@@ -35,7 +52,7 @@ pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Stride
   constexpr int VPR = D / EPV;                  // vectors per token row
   constexpr int GROUPS = POOL_THREADS / VPR;    // token rows read concurrently
   constexpr int STEP = GROUPS * 4;              // token rows per step
-  __shared__ float part[GROUPS][D + 1];
+  __shared__ float part[EPV][POOL_THREADS + (EPV == 8 ? 4 : 2)];    // (a warp's writes and its reads touch every bank once)
 
   const int bh = blockIdx.y + grid_dep_wait(), which = blockIdx.z;
   const int b = bh / H, h = bh % H;
@@ -56,9 +73,9 @@ pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Stride
       if (t < cnt) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(lo + t) * s.n * ELEM_BYTES) + vec);
     }
   };
-  float acc[EPV];
+  uint64_t acc[EPV / 2];
 #pragma unroll
-  for (int e = 0; e < EPV; ++e) acc[e] = 0.f;
+  for (int e = 0; e < EPV / 2; ++e) acc[e] = 0ull;
   load(0);
   for (int step = 0; step < steps; ++step) {
     uint4 c[4];
@@ -66,28 +83,19 @@ pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Stride
     for (int j = 0; j < 4; ++j) c[j] = u[j];
     load(step + 1);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const uint32_t w[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
-      if constexpr (ELEM_BYTES == 2) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) { acc[2 * e] += bf16lo(w[e]); acc[2 * e + 1] += bf16hi(w[e]); }
-      } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-          const float2 lo2 = e4m3x2_to_float2(w[e] & 0xffffu), hi2 = e4m3x2_to_float2(w[e] >> 16);
-          acc[4 * e] += lo2.x; acc[4 * e + 1] += lo2.y; acc[4 * e + 2] += hi2.x; acc[4 * e + 3] += hi2.y;
-        }
-      }
-    }
+    for (int j = 0; j < 4; ++j) add_vector<ELEM_BYTES>(c[j], acc);
     if ((step + 1) % per_block == 0) {                            // the block's rows are in: reduce over the groups
       const int I = I0 + step / per_block;
 #pragma unroll
-      for (int e = 0; e < EPV; ++e) { part[grp][vec * EPV + e] = acc[e]; acc[e] = 0.f; }
+      for (int e = 0; e < EPV / 2; ++e) {
+        unpack2(acc[e], part[2 * e][grp * VPR + vec], part[2 * e + 1][grp * VPR + vec]);
+        acc[e] = 0ull;
+      }
       __syncthreads();
       if (threadIdx.x < D) {
         float sum = 0.f;
 #pragma unroll 8
-        for (int g = 0; g < GROUPS; ++g) sum += part[g][threadIdx.x];   // fixed order
+        for (int g = 0; g < GROUPS; ++g) sum += part[threadIdx.x % EPV][g * VPR + threadIdx.x / EPV];   // fixed order
         float mean = sum / (float)min(block, N - I * block);
         if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
         (which ? kbar : qbar)[((long long)bh * Nb + I) * D + threadIdx.x] = mean;
@@ -116,6 +124,60 @@ __device__ __forceinline__ uint32_t score_key(float v) {
 }
 __device__ __forceinline__ float key_score(uint32_t key) {
   return __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
+}
+
+// Mass rule: the softmax weights of a row's candidates, in units of 2^-31 (0 where there is none).
+template <int ITEMS>
+__device__ __forceinline__ void mass_weights(const uint32_t (&key)[ITEMS], uint32_t (&wgt)[ITEMS]) {
+      uint32_t km = 0u;
+  #pragma unroll
+      for (int it = 0; it < ITEMS; ++it) km = max(km, key[it]);
+      km = __reduce_max_sync(0xffffffffu, km);
+      const float mx = key_score(km);
+      float z = 0.f, ew[ITEMS];
+  #pragma unroll
+      for (int it = 0; it < ITEMS; ++it) {
+        ew[it] = 0.f;
+        if (key[it]) { ew[it] = expf(key_score(key[it]) - mx); z += ew[it]; }
+      }
+  #pragma unroll
+      for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+      const float inv_z = 1.0f / z;
+  #pragma unroll
+      for (int it = 0; it < ITEMS; ++it) wgt[it] = __float2uint_rn(ew[it] * inv_z * 2147483648.f);
+}
+
+// A row's kept blocks (bit it of `mask`: block it*32 + lane; n of them) in ascending order: straight into the CSR where every row has
+// the same count, else staged with its count.
+template <int ITEMS>
+__device__ __forceinline__ void emit_row(const uint32_t mask, const int n, const int I, const int bh, const int lane, const SelParams& p,
+                                         int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx, int32_t* __restrict__ tmp_idx,
+                                         int32_t* __restrict__ counts, const int R) {
+  const int Nb = p.Nb;
+  const int r = bh * Nb + I;
+  int32_t* out;
+  if (p.fixed_n) {
+    out = col_idx + (long long)r * p.fixed_n;
+    if (lane == 0) {
+      row_ptr[r] = r * p.fixed_n;
+      if (r == R - 1) row_ptr[R] = R * p.fixed_n;
+    }
+    // (NaN scores are no candidates: the row can come out short; what row_ptr covers is written all the same)
+#pragma unroll 1
+    for (int t = n + lane; t < p.fixed_n; t += 32) out[t] = 0;
+  } else {
+    out = tmp_idx + (long long)r * p.cap;
+    if (lane == 0) counts[r] = n;
+  }
+  int base = 0;
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    if (it * 32 >= Nb) break;
+    bool sel = mask >> it & 1u;
+    uint32_t bal = __ballot_sync(0xffffffffu, sel);
+    if (sel) out[base + __popc(bal & ((1u << lane) - 1u))] = it * 32 + lane;
+    base += __popc(bal);
+  }
 }
 
 // Selection and emission of one query-block row by one warp.  Lane j owns the key blocks
@@ -148,27 +210,11 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
   int n = 0;
   uint32_t cum = 0u;            // kept mass so far, units of 2^-31
   const uint32_t tau_q = __float2uint_rn(fminf(fmaxf(p.tau, 0.f), 1.f) * 2147483648.f);
-  float mx = 0.f, inv_z = 0.f;
   uint32_t wgt[ITEMS];          // mode 1: softmax weight of every candidate, units of 2^-31
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) wgt[it] = 0u;
   if (MASS) {
-    uint32_t km = 0u;
-#pragma unroll
-    for (int it = 0; it < ITEMS; ++it) km = max(km, key[it]);
-    km = __reduce_max_sync(0xffffffffu, km);
-    mx = key_score(km);
-    float z = 0.f, ew[ITEMS];
-#pragma unroll
-    for (int it = 0; it < ITEMS; ++it) {
-      ew[it] = 0.f;
-      if (key[it]) { ew[it] = expf(key_score(key[it]) - mx); z += ew[it]; }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-    inv_z = 1.0f / z;
-#pragma unroll
-    for (int it = 0; it < ITEMS; ++it) wgt[it] = __float2uint_rn(ew[it] * inv_z * 2147483648.f);
+    mass_weights<ITEMS>(key, wgt);
   }
   if (p.use_window) {
     uint32_t fm = 0u;
@@ -280,31 +326,75 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
     n = have;
   }
 
-  // ---- emit ascending
-  const int r = bh * Nb + I;
-  int32_t* out;
-  if (p.fixed_n) {
-    out = col_idx + (long long)r * p.fixed_n;
-    if (lane == 0) {
-      row_ptr[r] = r * p.fixed_n;
-      if (r == R - 1) row_ptr[R] = R * p.fixed_n;
+  emit_row<ITEMS>(mask, n, I, bh, lane, p, row_ptr, col_idx, tmp_idx, counts, R);
+}
+
+// The same rule for short rows: each candidate counts the candidates in front of it (larger score, or equal and a lower index) and, for the
+// mass rule, adds up their mass; it is kept if the sequential rule would still run when its turn comes.  No search, so a row is Nb steps of
+// two or three independent instructions: 64 scores in about 600 cycles where narrowing the threshold takes 3 500 (a warp alone on its scheduler).
+// sk, sw: the row's keys and weights in shared memory (32 * ITEMS words each).
+template <int ITEMS, bool MASS>
+__device__ __forceinline__ void rank_and_emit(uint32_t (&key)[ITEMS], uint32_t* sk, uint32_t* sw, const int I, const int bh,
+                                              const int lane, const SelParams& p, int32_t* __restrict__ row_ptr,
+                                              int32_t* __restrict__ col_idx, int32_t* __restrict__ tmp_idx,
+                                              int32_t* __restrict__ counts, const int R) {
+  const int Nb = p.Nb;
+  const uint32_t tau_q = __float2uint_rn(fminf(fmaxf(p.tau, 0.f), 1.f) * 2147483648.f);
+  uint32_t mask = 0u, cum = 0u, wgt[ITEMS], ahead[ITEMS], before[ITEMS];
+  int n = 0;
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) wgt[it] = ahead[it] = before[it] = 0u;
+  if (MASS) mass_weights<ITEMS>(key, wgt);
+  if (p.use_window) {
+    uint32_t fm = 0u;
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) {
+      const int J = it * 32 + lane;
+      if (J < Nb && in_window(I, J, p)) {
+        mask |= 1u << it;
+        fm += wgt[it];
+        key[it] = wgt[it] = 0u;              // no longer a candidate
+      }
     }
-    // (NaN scores are no candidates: the row can come out short; what row_ptr covers is written all the same)
-#pragma unroll 1
-    for (int t = n + lane; t < p.fixed_n; t += 32) out[t] = 0;
-  } else {
-    out = tmp_idx + (long long)r * p.cap;
-    if (lane == 0) counts[r] = n;
+    n = (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(mask));
+    if (MASS) cum = __reduce_add_sync(0xffffffffu, fm);
   }
-  int base = 0;
 #pragma unroll
   for (int it = 0; it < ITEMS; ++it) {
-    if (it * 32 >= Nb) break;
-    bool sel = mask >> it & 1u;
-    uint32_t bal = __ballot_sync(0xffffffffu, sel);
-    if (sel) out[base + __popc(bal & ((1u << lane) - 1u))] = it * 32 + lane;
-    base += __popc(bal);
+    sk[it * 32 + lane] = key[it];
+    if (MASS) sw[it * 32 + lane] = wgt[it];
   }
+  __syncwarp();
+#pragma unroll
+  for (int jb = 0; jb < ITEMS; ++jb) {
+    const int j1 = min(32, Nb - jb * 32);                          // (what lies beyond Nb has key 0: in front of nothing)
+#pragma unroll 2
+    for (int j = 0; j < j1; j += 4) {
+      const uint4 k4 = *reinterpret_cast<const uint4*>(sk + jb * 32 + j);
+      uint4 w4 = make_uint4(0u, 0u, 0u, 0u);
+      if (MASS) w4 = *reinterpret_cast<const uint4*>(sw + jb * 32 + j);
+      const uint32_t kj[4] = {k4.x, k4.y, k4.z, k4.w}, wj[4] = {w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+          // (equal scores: the lower index goes first; a block that is no candidate, key 0, is behind everything or irrelevant)
+          const bool precedes = jb < it ? kj[e] >= key[it] : kj[e] > (jb == it && j + e < lane ? key[it] - 1u : key[it]);
+          if (precedes) ++ahead[it];
+          if (MASS && precedes) before[it] += wj[e];
+        }
+    }
+  }
+  const uint32_t kk = (uint32_t)min(p.k, Nb);
+  uint32_t kept = 0u;
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    const uint32_t at = (uint32_t)n + ahead[it];                   // blocks kept when this one's turn comes
+    if (key[it] != 0u && at < kk && !(MASS && at >= 1u && cum + before[it] >= tau_q)) kept |= 1u << it;
+  }
+  mask |= kept;
+  n += (int)__reduce_add_sync(0xffffffffu, (unsigned)__popc(kept));
+  emit_row<ITEMS>(mask, n, I, bh, lane, p, row_ptr, col_idx, tmp_idx, counts, R);
 }
 
 // Block scores of one head as a small fp32 GEMM: S[I][J] = scale * <qbar_I, kbar_J>.  A CTA computes a
@@ -383,22 +473,30 @@ block_scores_kernel(const float* __restrict__ qbar, const float* __restrict__ kb
   }
 }
 
+// Function attributes of a kernel, set once per device and instantiation instead of per call.
+struct DeviceOnce {
+  std::mutex mutex;
+  bool done[64] = {false};
+  template <typename F>
+  int run(F set) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SVA_ERR_CUDA;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (!done[dev]) {
+      if (!set()) return SVA_ERR_CUDA;
+      done[dev] = true;
+    }
+    return SVA_OK;
+  }
+};
+
 template <int D, int PQ, int PK, int TY>
 static int launch_scores(const float* qbar, const float* kbar, int Nb, int heads, float scale, float* scores, cudaStream_t st) {
   auto kern = block_scores_kernel<D, PQ, PK, TY>;
   constexpr int TQ = PQ * TY, TK = PK * 16, smem = (TQ + TK) * (D + 4) * (int)sizeof(float);
-  // (the shared-memory attribute is set once per device and instantiation, not per call)
-  static std::mutex attr_mutex;
-  static bool attr_set[64] = {false};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SVA_ERR_CUDA;
-  {
-    std::lock_guard<std::mutex> lock(attr_mutex);
-    if (!attr_set[dev]) {
-      if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return SVA_ERR_CUDA;
-      attr_set[dev] = true;
-    }
-  }
+  static DeviceOnce once;
+  const int rc = once.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess; });
+  if (rc != SVA_OK) return rc;
   return launch_dep(kern, dim3((Nb + TK - 1) / TK, (Nb + TQ - 1) / TQ, heads), 16 * TY, smem, st, qbar, kbar, Nb, scale, scores);
 }
 
@@ -423,6 +521,154 @@ select_rows_kernel(const float* __restrict__ scores, SelParams p, int32_t* __res
     key[it] = J < Nb ? score_key(__ldg(srow + J)) : 0u;
   }
   select_and_emit<ITEMS, MASS>(key, I, bh, lane, p, row_ptr, col_idx, tmp_idx, counts, R);
+}
+
+// Small problems: pooling, scores and selection of one head by one cluster of eight CTAs, one launch instead of three.  Each CTA pools
+// its share of the head's blocks of Q and K (a team of 256 threads per block), writes a key mean into the shared memory of all eight,
+// and then scores and selects its own query blocks.  Sums run in the orders of pool_kernel and block_scores_kernel, so lists and
+// scores are the same bytes.
+// Bound by latency: launches, the cluster's barriers, a pooling round of 32 KB (about 1 100 cycles of loads, sums and reduction), and a
+// score and selection phase of a few warps.  Microseconds of a routing call, three kernels -> this one (top-k / mass rule with csr_kernel):
+// 2 heads x 16 blocks of 64 x 64 8.8 -> 5.3, 12 heads x 44 blocks of 128 x 128 15.0 -> 12.1 / 17.9 -> 14.7, 32 x 64 38.3 -> 27.4 / 41.7 -> 32.6.
+static constexpr int RC_CTAS = 8, RC_TEAM = 256, RC_ITEMS = 2, RC_MAX_NB = 32 * RC_ITEMS;
+static constexpr int RC_ROWS = RC_MAX_NB / RC_CTAS;                         // query blocks per CTA at most (a multiple of 4)
+__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+// a float into the shared memory of CTA `rank` of the cluster, at this CTA's address `addr`
+__device__ __forceinline__ void store_cluster(uint32_t addr, int rank, float v) {
+  asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, %1;\nst.shared::cluster.f32 [a], %2;\n}" ::"r"(addr), "r"(rank), "f"(v) : "memory");
+}
+template <int D, int ELEM_BYTES, int TEAMS>
+struct RcSmem {
+  static constexpr int VPR = D * ELEM_BYTES / 16, GROUPS = RC_TEAM / VPR, EPV = 16 / ELEM_BYTES, LD = D + 4;
+  // partial sums [element of the vector][group][vector]: both the writes (a lane per vector) and the reads (a lane per column) of a
+  // warp touch every bank once
+  static constexpr int PART = GROUPS * VPR + (EPV == 8 ? 4 : 2);
+  float part[TEAMS][EPV * PART];
+};
+// TEAMS: blocks pooled at a time.  Four while a CTA has an SM to itself, two (so that two CTAs fit on an SM) beyond that.
+template <int D, int ELEM_BYTES, int TEAMS, bool MASS>
+__global__ void __launch_bounds__(TEAMS * RC_TEAM, 4 / TEAMS)
+route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Strides sq, Strides sk,
+                     const float* __restrict__ q_scale, const float* __restrict__ k_scale, int H, int N, int block, float scale,
+                     SelParams p, float* __restrict__ scores, int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx,
+                     int32_t* __restrict__ tmp_idx, int32_t* __restrict__ counts, int R) {
+  using Sm = RcSmem<D, ELEM_BYTES, TEAMS>;
+  constexpr int VPR = Sm::VPR, GROUPS = Sm::GROUPS, EPV = Sm::EPV, LD = Sm::LD, NV = 128 / GROUPS;     // NV: vectors per thread and block
+  constexpr int ITEMS = RC_ITEMS;
+  extern __shared__ __align__(16) uint8_t rc_smem[];
+  Sm& sm = *reinterpret_cast<Sm*>(rc_smem);
+  float* ks = reinterpret_cast<float*>(rc_smem + sizeof(Sm));          // [32 * ITEMS][LD] key means of the head
+  float* qm = ks + 32 * ITEMS * LD;                                    // [rows][LD] means of my query blocks
+  uint32_t* keys = reinterpret_cast<uint32_t*>(qm + RC_ROWS * LD);      // [rows][32 * ITEMS] scores as keys
+  uint32_t* wgts = keys + RC_ROWS * 32 * ITEMS;                 // ... and their weights
+  const int Nb = p.Nb, per = (Nb + RC_CTAS - 1) / RC_CTAS;
+  cluster_arrive();                        // (the CTAs of the cluster have started: they may be written to)
+  const int rank = blockIdx.x % RC_CTAS, bh = blockIdx.x / RC_CTAS + grid_dep_wait();
+  const int b = bh / H, h = bh % H, I0 = rank * per, mine = max(0, min(per, Nb - I0));
+  const int team = threadIdx.x / RC_TEAM, tt = threadIdx.x % RC_TEAM, vec = tt % VPR, grp = tt / VPR;
+
+  // ---- pooling: items 0 .. mine-1 are blocks of Q, the rest blocks of K; the next item's loads are in flight behind a reduction
+  uint4 u[NV];
+  auto load = [&](int item) {
+    const int which = item >= mine, I = I0 + (which ? item - mine : item);
+    const Strides s = which ? sk : sq;
+    const int lo = I * block, cnt = item < 2 * mine ? min(block, N - lo) : 0;
+    const uint8_t* base = (which ? k : q) + ((long long)b * s.b + (long long)h * s.h + (long long)(lo + grp) * s.n) * ELEM_BYTES;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      u[j] = make_uint4(0, 0, 0, 0);
+      if (grp + j * GROUPS < cnt) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(j * GROUPS) * s.n * ELEM_BYTES) + vec);
+    }
+  };
+  load(team);
+  cluster_wait();
+  for (int item = team; item < 2 * mine; item += TEAMS) {
+    const int which = item >= mine, li = which ? item - mine : item, I = I0 + li;
+    uint64_t acc[EPV / 2];
+#pragma unroll
+    for (int e = 0; e < EPV / 2; ++e) acc[e] = 0ull;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) add_vector<ELEM_BYTES>(u[j], acc);
+    load(item + TEAMS);
+    float* part = sm.part[team];
+#pragma unroll
+    for (int e = 0; e < EPV / 2; ++e)
+      unpack2(acc[e], part[2 * e * Sm::PART + grp * VPR + vec], part[(2 * e + 1) * Sm::PART + grp * VPR + vec]);
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(RC_TEAM) : "memory");
+    if (tt < D) {
+      float sum = 0.f;
+#pragma unroll 8
+      for (int g = 0; g < GROUPS; ++g) sum += part[(tt % EPV) * Sm::PART + g * VPR + tt / EPV];       // fixed order
+      float mean = sum / (float)min(block, N - I * block);
+      if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
+      if (which) {
+        const uint32_t dst = smem_addr(ks + I * LD + tt);
+#pragma unroll
+        for (int r = 0; r < RC_CTAS; ++r) store_cluster(dst, r, mean);
+      } else {
+        qm[li * LD + tt] = mean;
+      }
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(RC_TEAM) : "memory");
+  }
+  grid_dep_launch();
+  cluster_arrive();
+  cluster_wait();
+
+  // ---- scores of my query blocks as keys: a thread per four query blocks and ITEMS key blocks, sums as in block_scores_kernel
+  constexpr int RQ = 4;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (warp * RQ < mine) {
+    uint64_t acc[RQ][ITEMS];
+#pragma unroll
+    for (int i = 0; i < RQ; ++i)
+#pragma unroll
+      for (int it = 0; it < ITEMS; ++it) acc[i][it] = pack2(0.f, 0.f);
+    const float* qrow = qm + warp * RQ * LD;
+    const float* krow = ks + lane * LD;
+#pragma unroll 2
+    for (int c = 0; c < D; c += 4) {
+      ulonglong2 kv[ITEMS];
+#pragma unroll
+      for (int it = 0; it < ITEMS; ++it) kv[it] = *reinterpret_cast<const ulonglong2*>(krow + it * 32 * LD + c);
+#pragma unroll
+      for (int i = 0; i < RQ; ++i) {
+        const ulonglong2 qv = *reinterpret_cast<const ulonglong2*>(qrow + i * LD + c);
+#pragma unroll
+        for (int it = 0; it < ITEMS; ++it) {
+          acc[i][it] = fma2(qv.x, kv[it].x, acc[i][it]);
+          acc[i][it] = fma2(qv.y, kv[it].y, acc[i][it]);
+        }
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < RQ; ++i) {
+      const int li = warp * RQ + i;
+      if (li >= mine) break;
+#pragma unroll
+      for (int it = 0; it < ITEMS; ++it) {
+        const int J = it * 32 + lane;
+        float s0, s1;
+        unpack2(acc[i][it], s0, s1);
+        const float v = (s0 + s1) * scale;
+        keys[li * 32 * ITEMS + J] = J < Nb ? score_key(v) : 0u;
+        if (scores && J < Nb) scores[((long long)bh * Nb + I0 + li) * Nb + J] = v;
+      }
+    }
+  }
+  __syncthreads();
+
+  // ---- selection: a warp per row
+  const int li = warp;
+  if (li < mine) {
+    uint32_t* sk = keys + li * 32 * ITEMS;
+    uint32_t key[ITEMS];
+#pragma unroll
+    for (int it = 0; it < ITEMS; ++it) key[it] = sk[it * 32 + lane];
+    rank_and_emit<ITEMS, MASS>(key, sk, wgts + li * 32 * ITEMS, I0 + li, bh, lane, p, row_ptr, col_idx, tmp_idx, counts, R);
+  }
 }
 
 // CSR assembly for rows of varying length, one launch: a CTA owns 32 consecutive rows (one warp each).  It
@@ -508,6 +754,35 @@ static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, c
                     m.H, m.N, m.block, m.Nb, run, qbar, kbar);
 }
 
+// Where the cluster kernel routes: blocks pooled at a time per CTA, or 0 for the three kernels (us, three kernels / this one).
+// Up to 14 heads each CTA has an SM to itself (15 or more clusters of eight SMs do not fit: 16 heads x 64 blocks 22.0 / 27.5): 14 x 64
+// 21.3 / 15.4, and no form of up to 64 blocks is slower except where few heads leave most SMs without a block to pool (2 x 64 9.8 / 12.8,
+// 4 x 64 11.4 / 15.6, but 8 x 44 12.3 / 11.4).
+// With two CTAs per SM more heads fit, at half the pooling rate each: with 16 blocks a head, 32 x 16 14.1 / 10.7, or where pooling is bound by the
+// HBM anyway, blocks of 32 KB: 24 x 32 18.4 / 13.9, 18 x 64 24.2 / 22.8, 32 x 64 38.3 / 27.4 (16 KB: 18 x 44 14.1 / 17.0; 36 x 64 39.7 / 41.8).
+// Beyond 64 blocks the exchanged means cost an SM its second CTA (24 x 96: 43.6 / 56.9).
+static int route_teams(const Dims& m) {
+  const int heads = m.B * m.H;
+  if (m.Nb > RC_MAX_NB || heads > 32) return 0;
+  if (heads <= 14) return m.Nb <= 32 || heads * m.Nb >= 8 * 44 ? 4 : 0;
+  const bool big_blocks = m.block * m.d * (m.fp8 ? 1 : 2) == 32768;
+  return m.Nb <= 16 || (big_blocks && (m.Nb <= 32 ? heads <= 24 : heads >= 18)) ? 2 : 0;
+}
+template <int D, int ELEM_BYTES, int TEAMS, bool MASS>
+static int launch_route(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale, const float* k_scale,
+                        const SelParams& sp, float* scores, int32_t* row_ptr, int32_t* col_idx, int32_t* tmp_idx, int32_t* counts,
+                        cudaStream_t st) {
+  auto kern = route_cluster_kernel<D, ELEM_BYTES, TEAMS, MASS>;
+  using Sm = RcSmem<D, ELEM_BYTES, TEAMS>;
+  constexpr int smem = (int)sizeof(Sm) + 4 * ((RC_MAX_NB + RC_ROWS) * Sm::LD + 2 * RC_ROWS * RC_MAX_NB);
+  static DeviceOnce once;
+  const int rc = once.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess; });
+  if (rc != SVA_OK) return rc;
+  return launch_dep_cluster(RC_CTAS, kern, m.B * m.H * RC_CTAS, TEAMS * RC_TEAM, smem, st, (const uint8_t*)q, (const uint8_t*)k,
+                            make_strides(p->q_stride), make_strides(p->k_stride), q_scale, k_scale, m.H, m.N, m.block, m.scale, sp,
+                            scores, row_ptr, col_idx, tmp_idx, counts, m.R);
+}
+
 template <int D>
 static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_select_t* s,
                            const void* q, const void* k, const float* q_scale,
@@ -528,12 +803,30 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
     counts = reinterpret_cast<int32_t*>(w + 2 * pooled + align256((size_t)m.R * cap * sizeof(int32_t)));
   }
   int rc = SVA_OK;
-  if (!qbar_in && (rc = launch_pool_d<D>(m, p, q, k, q_scale, k_scale, qbar, kbar, st)) != SVA_OK) return rc;
   SelParams sp;
   sp.Nb = m.Nb; sp.k = s->k;
   sp.use_window = (s->win_t >= 0 && s->win_s >= 0 && s->blocks_per_frame > 0) ? 1 : 0;
   sp.win_t = s->win_t; sp.win_s = s->win_s; sp.bpf = sp.use_window ? s->blocks_per_frame : 1;
   sp.cap = cap; sp.fixed_n = fixed_n; sp.tau = s->mass;
+  auto csr = [&]() {
+    if (fixed_n) return (int)SVA_OK;
+    return launch_dep(csr_kernel, (m.R + CSR_ROWS - 1) / CSR_ROWS, CSR_ROWS * 32, 0, st, tmp_idx, counts, cap, m.R, row_ptr, col_idx);
+  };
+  if (const int teams = qbar_in ? 0 : route_teams(m)) {
+    auto route = [&](auto elem_tag, auto teams_tag, auto mass_tag) {
+      return launch_route<D, decltype(elem_tag)::value, decltype(teams_tag)::value, decltype(mass_tag)::value>(
+          m, p, q, k, m.fp8 ? q_scale : nullptr, m.fp8 ? k_scale : nullptr, sp, block_scores, row_ptr, col_idx, tmp_idx, counts, st);
+    };
+    auto by_mass = [&](auto elem_tag, auto teams_tag) {
+      return s->mode == 1 ? route(elem_tag, teams_tag, std::true_type{}) : route(elem_tag, teams_tag, std::false_type{});
+    };
+    auto by_teams = [&](auto elem_tag) {
+      return teams == 4 ? by_mass(elem_tag, std::integral_constant<int, 4>{}) : by_mass(elem_tag, std::integral_constant<int, 2>{});
+    };
+    rc = m.fp8 ? by_teams(std::integral_constant<int, 1>{}) : by_teams(std::integral_constant<int, 2>{});
+    return rc != SVA_OK ? rc : csr();
+  }
+  if (!qbar_in && (rc = launch_pool_d<D>(m, p, q, k, q_scale, k_scale, qbar, kbar, st)) != SVA_OK) return rc;
   // scores: into the caller's matrix if it wants one, else into the workspace (after the staging arrays)
   float* scores = block_scores;
   if (!scores) {
@@ -561,8 +854,7 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
   else if (items <= 12) rc = select(std::integral_constant<int, 12>{});
   else if (items <= 16) rc = select(std::integral_constant<int, 16>{});
   else rc = select(std::integral_constant<int, 32>{});
-  if (rc != SVA_OK || fixed_n) return rc;
-  return launch_dep(csr_kernel, (m.R + CSR_ROWS - 1) / CSR_ROWS, CSR_ROWS * 32, 0, st, tmp_idx, counts, cap, m.R, row_ptr, col_idx);
+  return rc != SVA_OK ? rc : csr();
 }
 
 int launch_select(const Dims& m, const sva_problem_t* p, const sva_select_t* s, const void* q,

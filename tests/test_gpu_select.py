@@ -216,3 +216,58 @@ def test_rows_of_a_known_length_are_written_whole(nb, k, window):
             real = [j for j in range(nb) if not np.isnan(x[j]) and j not in forced]
             kept = sorted(forced + sorted(real, key=lambda j: (-x[j], j))[:k - len(forced)])
             assert ci[h * nb + i].tolist() == kept + [0] * (k - len(kept)), (h, i)
+
+
+@pytest.mark.parametrize("B_,H,Nb,block,d,fp8,mode,k,window,layout,values", [
+    (1, 1, 1, 128, 128, False, 0, 1, False, "heads", "normal"),           # one block, ragged
+    (1, 3, 9, 128, 128, False, 1, 4, False, "tokens", "normal"),          # CTAs of the cluster without a block
+    (2, 7, 64, 64, 128, False, 0, 11, False, "packed", "normal"),         # 14 heads, the most blocks
+    (1, 12, 44, 128, 64, False, 1, 12, True, "heads", "normal"),          # forced window and mass
+    (1, 8, 44, 64, 64, False, 0, 3, True, "tokens", "ties"),              # window larger than k, equal scores
+    (1, 2, 31, 128, 128, False, 1, 40, False, "heads", "zero"),           # every score equal, k beyond Nb
+    (1, 4, 20, 64, 128, False, 0, 7, False, "heads", "nan"),              # rows of NaN scores come out short
+    (1, 9, 33, 64, 128, True, 1, 6, False, "tokens", "normal"),           # e4m3 codes, 3 rows in a CTA's last quad
+    (1, 16, 16, 64, 64, True, 0, 5, False, "heads", "normal"),            # two CTAs per SM
+    (2, 9, 64, 128, 128, False, 1, 9, False, "packed", "normal"),
+    (1, 24, 17, 128, 128, False, 0, 2, False, "heads", "ties"),
+])
+def test_routing_in_one_launch_is_routing_in_three(B_, H, Nb, block, d, fp8, mode, k, window, layout, values):
+    """Small problems are routed by one kernel; the split calls (means, then routing from means) take the general ones: the same bytes."""
+    N = Nb * block - (37 if Nb % 2 else 0)
+    g = torch.Generator(device="cuda").manual_seed(Nb)
+    shape = {"heads": (2, B_, H, N, d), "tokens": (2, B_, N, H, d), "packed": (B_, N, 2, H, d)}[layout]
+    x = torch.randn(shape, generator=g, device="cuda")
+    qk = x.transpose(2, 3) if layout == "tokens" else x.permute(2, 0, 3, 1, 4) if layout == "packed" else x       # [2, B, H, N, d] views
+    if values == "ties":
+        qk[:, :, :, block:] = qk[:, :, :, : N - block].clone() if Nb < 3 else qk[:, :, :, :1]      # all blocks but the first alike
+    elif values == "zero":
+        qk.zero_()
+    elif values == "nan":
+        qk[1, :, 1, : 3 * block] = float("nan")                           # keys of three blocks: no candidates
+        qk[0, :, 2, :5] = float("nan")                                    # a query block without a score
+        qk[1, :, 3, 7] = float("inf")
+    scales = [None, None]
+    if fp8:
+        qk = qk.to(torch.float8_e4m3fn).view(torch.uint8)
+        scales = [torch.rand(B_, H, Nb, generator=g, device="cuda") + 0.5 for _ in range(2)]
+    else:
+        qk = qk.to(torch.bfloat16)
+    q, kk = qk[0], qk[1]
+    p = B.make_problem(q, kk, None, None, N, block, 0.0, True) if fp8 else B.make_problem(q, kk, None, None, N, block)
+    s = B.make_select(mode, k, 0.7, *((1, 1, 4) if window else (-1, -1, 0)))
+    got = []
+    for split in (False, True):
+        ws = torch.full((B.select_workspace_bytes(p, s),), 255, dtype=torch.uint8, device="cuda")
+        rp = torch.full((B_ * H * Nb + 1,), -7, dtype=torch.int32, device="cuda")
+        ci = torch.full((B.select_max_nnz(p, s),), -7, dtype=torch.int32, device="cuda")
+        sc = torch.full((B_, H, Nb, Nb), -7.0, device="cuda")
+        if split:
+            qm, km = (torch.zeros(B_, H, Nb, d, device="cuda") for _ in range(2))
+            B.pool_qk(p, q, kk, qm, km, *scales)
+            B.block_select_pooled(p, s, qm, km, rp, ci, ws, sc)
+        else:
+            B.block_select(p, s, q, kk, rp, ci, ws, *scales, sc)
+        torch.cuda.synchronize()
+        got.append((rp, ci, sc.view(torch.int32)))
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
