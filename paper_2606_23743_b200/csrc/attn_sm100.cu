@@ -1485,7 +1485,8 @@ bool attn_ts_remainder_serves(const Dims& m) { return attn_ts_serves(m) && m.d =
 size_t remainder1_bytes(const Dims& m);
 int launch_remainder1(const Dims& m, const sva_problem_t* p, const void* k, const void* v, const float* scores,
                       const int32_t* row_ptr, const int32_t* col_idx, void* buf, const __nv_bfloat16** at_out,
-                      const float** mu_out, int32_t* status, cudaStream_t st, bool natural);
+                      const float** mu_out, int32_t* status, cudaStream_t st, bool natural, __nv_bfloat16* k_mean, __nv_bfloat16* v_mean,
+                      int Nbp, int32_t* row_counter);
 // (order 1 adds the buffers of the first-order term behind those of order 0; 64-token blocks: then the tile rows' kept-block
 // masks, for which a smaller workspace is accepted too -- the kernel then looks the kept blocks up in the CSR)
 static size_t remainder_base_bytes(const Dims& m, int order) {
@@ -1607,23 +1608,26 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
     if ((rc = make_map_ts(&tq, q, m.d, m.N, hq, bq, (cuuint64_t)sq.n * eb, (cuuint64_t)sq.h * eb, (cuuint64_t)sq.b * eb, BS, eb)) != SVA_OK)
       return rc;
   }
-  if (rem && remainder_order == 1) {
-    // first-order term: C_J, weights, A_I (remainder.cu) into the buffers behind those of order 0
-    const __nv_bfloat16* at = nullptr;
-    if ((rc = launch_remainder1(m, p, k, v, block_scores, row_ptr, col_idx, wsb + L.total_rem, &at, &mu_dev, status, st, vmn)) != SVA_OK)
-      return rc;
-    const cuuint64_t arow = (cuuint64_t)m.Nb * BS;               // per head: Nb matrices of 128 rows x 128 bf16
-    if ((rc = make_map_ts(&tat, at, BS, arow, m.H, m.B, (cuuint64_t)BS * 2, arow * BS * 2, arow * BS * 2 * m.H, BS)) != SVA_OK)
-      return rc;
-  }
   if (rem) {
-    // block means of K ([Nbp rows][128], rows >= Nb zero) and of V (transposed tiles), then their maps
     __nv_bfloat16* kp = reinterpret_cast<__nv_bfloat16*>(wsb + L.kp_off);
     __nv_bfloat16* vtp = reinterpret_cast<__nv_bfloat16*>(wsb + L.vtp_off);
+    int32_t* counter = reinterpret_cast<int32_t*>(wsb + L.counter_off);
+    const bool with_cov = remainder_order == 1 && vmn;                   // the covariance kernel leaves the block means too
+    if (remainder_order == 1) {
+      // first-order term: C_J, weights, A_I (remainder.cu) into the buffers behind those of order 0
+      const __nv_bfloat16* at = nullptr;
+      if ((rc = launch_remainder1(m, p, k, v, block_scores, row_ptr, col_idx, wsb + L.total_rem, &at, &mu_dev, status, st, vmn,
+                                  with_cov ? kp : nullptr, with_cov ? vtp : nullptr, L.Nbp, counter)) != SVA_OK)
+        return rc;
+      const cuuint64_t arow = (cuuint64_t)m.Nb * BS;               // per head: Nb matrices of 128 rows x 128 bf16
+      if ((rc = make_map_ts(&tat, at, BS, arow, m.H, m.B, (cuuint64_t)BS * 2, arow * BS * 2, arow * BS * 2 * m.H, BS)) != SVA_OK)
+        return rc;
+    }
+    // block means of K ([Nbp rows][128], rows >= Nb zero) and of V (transposed tiles), then their maps
     const int run = blocks_per_cta(2LL * m.R);                     // (the padding blocks that the grid covers too are not read)
-    if ((rc = launch_dep(pool_kv_kernel, dim3((L.Nbp + run - 1) / run, m.B * m.H, 2), 256, 0, st, (const __nv_bfloat16*)k,
+    if (!with_cov && (rc = launch_dep(pool_kv_kernel, dim3((L.Nbp + run - 1) / run, m.B * m.H, 2), 256, 0, st, (const __nv_bfloat16*)k,
                          (const __nv_bfloat16*)v, sk, make_strides(p->v_stride), m.H, m.N, m.block, m.Nb, L.Nbp, run, kp, vtp, vmn ? 1 : 0,
-                         reinterpret_cast<int32_t*>(wsb + L.counter_off))) != SVA_OK)
+                         counter)) != SVA_OK)
       return rc;
     const cuuint64_t prow = (cuuint64_t)L.Nbp;
     if ((rc = make_map_ts(&tkp, kp, ts::D, prow, m.H, m.B, (cuuint64_t)ts::D * 2, prow * ts::D * 2,

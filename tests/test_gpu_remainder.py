@@ -354,3 +354,22 @@ def test_more_than_1024_key_blocks(order):
                                               stats="bf16")
     max_abs, rel, lse_err = U.attn_errors(o, lse, o_ref, l_ref, rows, w.N, w.block, 1)
     assert max_abs <= max(U.BF16_MAX_ABS, 2.0 ** -7 * float(np.nanmax(np.abs(o_ref)))) and rel <= U.BF16_REL_L2 and lse_err <= 2e-3
+
+
+@pytest.mark.parametrize("block,nb", [(128, 64), (64, 128), (64, 129), (64, 256), (64, 257), (64, 512), (64, 513)])
+def test_first_order_aggregation_at_the_edges_of_its_forms(block, nb):
+    """The sums over A_I keep the weights of one I-tile up to 128 key blocks, of two up to 256, of one up to 512 and of none beyond that."""
+    from paper_2606_23743_b200.workloads import bf16_bits
+    w = shrink(WORKLOADS["medium"], H=2, T=1, Hg=nb, Wg=block, block=block, k=max(1, nb // 16))
+    (q, k, v), (qb, kb, _) = U.host_inputs(w)
+    v = (v.float() + 4.0 * k.float()).to(torch.bfloat16)                     # (the first-order term is large: see above)
+    vb = bf16_bits(v)
+    qd, kd, vd = U.dev(q), U.dev(k), U.dev(v)
+    rp, ci, scores = U.gpu_select(w, qd, kd, want_scores=True)
+    o, lse, st = gpu_remainder(w, qd, kd, vd, rp, ci, 1, scores=scores)
+    assert st == 0
+    rows = [0, min(127, nb - 1), nb - 1, nb, nb + nb // 2, 2 * nb - 1]       # (of both heads)
+    o_ref, l_ref = oracle.attn_remainder_rows(qb, kb, vb, w.N, w.block, w.scale, rp.cpu().numpy(), ci.cpu().numpy(), rows, order=1,
+                                              stats="bf16")
+    max_abs, rel, lse_err = U.attn_errors(o, lse, o_ref, l_ref, rows, w.N, w.block, 2)
+    assert max_abs <= max(U.BF16_MAX_ABS, 2.0 ** -7 * float(np.nanmax(np.abs(o_ref)))) and rel <= U.BF16_REL_L2 and lse_err <= 2e-3
