@@ -1307,19 +1307,20 @@ pair_lists_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict
 // The mean over the existing tokens of a block, fp32 accumulation in a fixed order, rounded to bf16.  K means go to kp
 // [B*H][Nbp][128] (rows >= Nb zero), V means likewise (v_rows) or transposed to vtp [B*H][np][128 d][128 blocks], the
 // layout of a V^T tile.  HBM-bound; a CTA takes `run` consecutive blocks of one head of K or V, the next loads in flight while
-// it reduces (as the routing's pooling does; 24 heads x 32 760 tokens in 64-token blocks: 79 -> 72 us).
+// it reduces (as the routing's pooling does; 24 heads x 32 760 tokens in 64-token blocks: 79 -> 72 us).  From the end of K, which the
+// routing's pooling read last: 91 -> 87 us in the pass.
 __global__ void __launch_bounds__(256)
 pool_kv_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, Strides sk, Strides sv,
                int H, int N, int block, int Nb, int Nbp, int run, __nv_bfloat16* __restrict__ kp,
                __nv_bfloat16* __restrict__ vtp, int v_rows, int32_t* __restrict__ row_counter) {
   __shared__ float part[16][ts::D + 1];
-  const int zero = grid_dep_wait(), bh = blockIdx.y + zero, which = blockIdx.z;
+  const int zero = grid_dep_wait(), bh = gridDim.y - 1 - blockIdx.y + zero, which = blockIdx.z;
   // the attention kernel that follows draws its rows from this counter
   if (blockIdx.x == 0 && blockIdx.y == 0 && which == 0 && threadIdx.x < 2) row_counter[threadIdx.x] = 0;
   const int b = bh / H, h = bh % H;
   const Strides s = which ? sv : sk;
   const __nv_bfloat16* base = (which ? v : k) + (long long)b * s.b + (long long)h * s.h;
-  const int J0 = blockIdx.x * run, J1 = min(J0 + run, Nbp);
+  const int J0 = (gridDim.x - 1 - blockIdx.x) * run, J1 = min(J0 + run, Nbp);
   const int vec = threadIdx.x & 15, grp = threadIdx.x >> 4;          // 16 vectors of 8 elements per row, 16 rows at a time
   const int per_block = block / 64, steps = (J1 - J0) * per_block;   // 64 rows per step
   uint4 u[4];

@@ -19,16 +19,17 @@ namespace sva {
 static constexpr int Q4_THREADS = 256;
 
 // amax[tensor * BH + bh] (as fp32 bits; the launcher zeroes it) = max |x| over the existing tokens
+// From the end of the tensors, which a kernel that has just written them (the prologue) leaves in the L2.
 // A CTA reads `run` consecutive 128-token blocks, the next half block's loads in flight behind the current one's maxima, and
 // does one atomicMax: with a block per CTA and an atomic per warp (98 304 of them on 48 words) the pass took 100 us for
 // 403 MB, now 70 us (5.7 TB/s).
 __global__ void __launch_bounds__(Q4_THREADS)
 amax_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, Strides sq, Strides sk, int H, int N,
             int BH, int run, uint32_t* __restrict__ amax) {
-  const int bh = blockIdx.y + grid_dep_wait(), which = blockIdx.z;
+  const int bh = gridDim.y - 1 - blockIdx.y + grid_dep_wait(), which = 1 - blockIdx.z;
   const Strides s = which ? sk : sq;
   const __nv_bfloat16* base = (which ? k : q) + (long long)(bh / H) * s.b + (long long)(bh % H) * s.h;
-  const int lo = blockIdx.x * run * 128, hi = min(lo + run * 128, N);
+  const int lo = (gridDim.x - 1 - blockIdx.x) * run * 128, hi = min(lo + run * 128, N);
   const int row = threadIdx.x >> 4, vec = threadIdx.x & 15;   // 16 vectors of 8 elements per token, 16 tokens at a time
   uint4 u[4];
   auto load = [&](int t0) {
@@ -77,7 +78,7 @@ __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
 }
 
 // One CTA per (128-token block, head, tensor), in the reverse of the order in which amax_kernel read them, so that the tensors'
-// ends are still in the L2; a thread casts four 16-element scale blocks, whose loads are all in flight.  Issue-bound (75 % of
+// beginnings are still in the L2; a thread casts four 16-element scale blocks, whose loads are all in flight.  Issue-bound (75 % of
 // the issue slots at 105 us): the divisions are three FMA-pipe operations each, element pairs in packed ones, with true
 // divisions out of line for magnitudes whose residuals could underflow; scales leave through shared memory.  Q and K of
 // 24 heads x 32 760 tokens (403 MB in, 113 MB out): 105 -> 85 us alone
@@ -87,7 +88,7 @@ quantize4_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __res
                  int N, int Nb, int BH, const uint32_t* __restrict__ amax, uint8_t* __restrict__ q4,
                  uint8_t* __restrict__ k4, uint8_t* __restrict__ q_sf, uint8_t* __restrict__ k_sf, float* __restrict__ q_g,
                  float* __restrict__ k_g) {
-  const int I = gridDim.x - 1 - blockIdx.x, bh = gridDim.y - 1 - blockIdx.y + grid_dep_wait(), which = 1 - blockIdx.z;
+  const int I = blockIdx.x, bh = blockIdx.y + grid_dep_wait(), which = blockIdx.z;
   const Strides s = which ? sk : sq;
   const __nv_bfloat16* base = (which ? k : q) + (long long)(bh / H) * s.b + (long long)(bh % H) * s.h;
   uint8_t* codes = (which ? k4 : q4) + ((long long)bh * Nb + I) * 128 * 64;

@@ -42,7 +42,8 @@ __device__ __forceinline__ void add_vector(const uint4& u, uint64_t (&acc)[8 / E
 // the blocks of its run, so the reduction at the end of a block (two barriers) happens with the next block's loads in
 // flight; with a CTA per block nothing was in flight while it reduced.  Q and K of 24 heads
 // x 32 760 tokens, d = 128 (403 MB): 75.8 -> 71.8 us (5.6 TB/s) with 128-token blocks, 81 -> 72.7 us with 64-token
-// ones; e4m3 codes (201 MB, converted in pairs): 66.5 -> 58.6 us.
+// ones.  e4m3 codes (201 MB, converted in pairs) are bound by the sums and the reduction, which half the bytes do not hide: 66.5 -> 58.6 us with the
+// run, 52.6 -> 46.4 (on a faster box) with pairs added in one instruction and partial sums laid out so that no two lanes of a warp meet in a bank.
 template <int D, int ELEM_BYTES>
 __global__ void __launch_bounds__(POOL_THREADS)
 pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Strides sq, Strides sk,
@@ -54,11 +55,13 @@ pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Stride
   constexpr int STEP = GROUPS * 4;              // token rows per step
   __shared__ float part[EPV][POOL_THREADS + (EPV == 8 ? 4 : 2)];    // (a warp's writes and its reads touch every bank once)
 
-  const int bh = blockIdx.y + grid_dep_wait(), which = blockIdx.z;
+  // (e4m3 codes: from the end, which the quantiser has just written and the L2 still holds)
+  constexpr bool BACK = ELEM_BYTES == 1;
+  const int zero = grid_dep_wait(), bh = (BACK ? gridDim.y - 1 - blockIdx.y : blockIdx.y) + zero, which = BACK ? 1 - blockIdx.z : blockIdx.z;
   const int b = bh / H, h = bh % H;
   const Strides s = which ? sk : sq;
   const uint8_t* base = (which ? k : q) + ((long long)b * s.b + (long long)h * s.h) * ELEM_BYTES;
-  const int I0 = blockIdx.x * run, I1 = min(I0 + run, Nb);
+  const int I0 = (BACK ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * run, I1 = min(I0 + run, Nb);
   const int vec = threadIdx.x % VPR, grp = threadIdx.x / VPR;
   const int per_block = (block + STEP - 1) / STEP, steps = (I1 - I0) * per_block;
 
