@@ -1309,6 +1309,7 @@ pair_lists_kernel(const int32_t* __restrict__ row_ptr, const int32_t* __restrict
 // layout of a V^T tile.  HBM-bound; a CTA takes `run` consecutive blocks of one head of K or V, the next loads in flight while
 // it reduces (as the routing's pooling does; 24 heads x 32 760 tokens in 64-token blocks: 79 -> 72 us).  From the end of K, which the
 // routing's pooling read last: 91 -> 87 us in the pass.
+template <int VECS>                              // 16-byte vectors of a block per thread: 4 (64 tokens) or 8 (128)
 __global__ void __launch_bounds__(256)
 pool_kv_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restrict__ v, Strides sk, Strides sv,
                int H, int N, int block, int Nb, int Nbp, int run, __nv_bfloat16* __restrict__ kp,
@@ -1322,36 +1323,32 @@ pool_kv_kernel(const __nv_bfloat16* __restrict__ k, const __nv_bfloat16* __restr
   const __nv_bfloat16* base = (which ? v : k) + (long long)b * s.b + (long long)h * s.h;
   const int J0 = (gridDim.x - 1 - blockIdx.x) * run, J1 = min(J0 + run, Nbp);
   const int vec = threadIdx.x & 15, grp = threadIdx.x >> 4;          // 16 vectors of 8 elements per row, 16 rows at a time
-  const int per_block = block / 64, steps = (J1 - J0) * per_block;   // 64 rows per step
-  uint4 u[4];
-  auto load = [&](int step) {
-    const int lo = (J0 + step / per_block) * block + (step % per_block) * 64;
+  uint4 u[VECS];
+  auto load = [&](int J) {
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int t = lo + 16 * j + grp;
+    for (int j = 0; j < VECS; ++j) {
+      const int t = J * block + 16 * j + grp;
       u[j] = make_uint4(0u, 0u, 0u, 0u);
-      if (step < steps && t < N) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)t * s.n) + vec);
+      if (J < J1 && t < N) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)t * s.n) + vec);
     }
   };
-  float acc[8];
+  load(J0);
+  for (int J = J0; J < J1; ++J) {
+    float acc[8];
 #pragma unroll
-  for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-  load(0);
-  for (int step = 0; step < steps; ++step) {
-    uint4 c[4];
+    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+    uint4 c[VECS];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) c[j] = u[j];
-    load(step + 1);
+    for (int j = 0; j < VECS; ++j) c[j] = u[j];
+    load(J + 1);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for (int j = 0; j < VECS; ++j) {
       const uint32_t wd[4] = {c[j].x, c[j].y, c[j].z, c[j].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) { acc[2 * e] += bf16lo(wd[e]); acc[2 * e + 1] += bf16hi(wd[e]); }
     }
-    if ((step + 1) % per_block != 0) continue;
-    const int J = J0 + step / per_block;
 #pragma unroll
-    for (int e = 0; e < 8; ++e) { part[grp][vec * 8 + e] = acc[e]; acc[e] = 0.f; }
+    for (int e = 0; e < 8; ++e) part[grp][vec * 8 + e] = acc[e];
     __syncthreads();
     if (threadIdx.x < ts::D) {
       float sum = 0.f;
@@ -1625,8 +1622,8 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
         return rc;
     }
     // block means of K ([Nbp rows][128], rows >= Nb zero) and of V (transposed tiles), then their maps
-    const int run = blocks_per_cta(2LL * m.R);                     // (the padding blocks that the grid covers too are not read)
-    if (!with_cov && (rc = launch_dep(pool_kv_kernel, dim3((L.Nbp + run - 1) / run, m.B * m.H, 2), 256, 0, st, (const __nv_bfloat16*)k,
+    const int run = blocks_per_cta(2LL * m.R, m.block * ts::D * 2);            // (the padding blocks that the grid covers too are not read)
+    if (!with_cov && (rc = launch_dep(m.block == 64 ? pool_kv_kernel<4> : pool_kv_kernel<8>, dim3((L.Nbp + run - 1) / run, m.B * m.H, 2), 256, 0, st, (const __nv_bfloat16*)k,
                          (const __nv_bfloat16*)v, sk, make_strides(p->v_stride), m.H, m.N, m.block, m.Nb, L.Nbp, run, kp, vtp, vmn ? 1 : 0,
                          counter)) != SVA_OK)
       return rc;

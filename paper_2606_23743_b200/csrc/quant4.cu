@@ -20,7 +20,7 @@ static constexpr int Q4_THREADS = 256;
 
 // amax[tensor * BH + bh] (as fp32 bits; the launcher zeroes it) = max |x| over the existing tokens
 // From the end of the tensors, which a kernel that has just written them (the prologue) leaves in the L2.
-// A CTA reads `run` consecutive 128-token blocks, the next half block's loads in flight behind the current one's maxima, and
+// A CTA reads `run` consecutive 128-token blocks, the next block's loads in flight behind the current one's maxima, and
 // does one atomicMax: with a block per CTA and an atomic per warp (98 304 of them on 48 words) the pass took 100 us for
 // 403 MB, now 70 us (5.7 TB/s).
 __global__ void __launch_bounds__(Q4_THREADS)
@@ -31,10 +31,10 @@ amax_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict
   const __nv_bfloat16* base = (which ? k : q) + (long long)(bh / H) * s.b + (long long)(bh % H) * s.h;
   const int lo = (gridDim.x - 1 - blockIdx.x) * run * 128, hi = min(lo + run * 128, N);
   const int row = threadIdx.x >> 4, vec = threadIdx.x & 15;   // 16 vectors of 8 elements per token, 16 tokens at a time
-  uint4 u[4];
+  uint4 u[8];
   auto load = [&](int t0) {
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < 8; ++r) {
       const int t = t0 + 16 * r + row;
       u[r] = make_uint4(0u, 0u, 0u, 0u);
       if (t < hi) u[r] = __ldg(reinterpret_cast<const uint4*>(base + (long long)t * s.n) + vec);
@@ -42,13 +42,13 @@ amax_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict
   };
   uint32_t m = 0u;                                            // max of the |x| bit patterns (bf16 in the upper half)
   load(lo);
-  for (int t0 = lo; t0 < hi; t0 += 64) {
-    uint4 c[4];
+  for (int t0 = lo; t0 < hi; t0 += 128) {
+    uint4 c[8];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) c[r] = u[r];
-    load(t0 + 64);
+    for (int r = 0; r < 8; ++r) c[r] = u[r];
+    load(t0 + 128);
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
+    for (int r = 0; r < 8; ++r) {
       const uint32_t w[4] = {c[r].x, c[r].y, c[r].z, c[r].w};
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
@@ -169,7 +169,7 @@ int launch_quantize4(const Dims& m, const sva_problem_t* p, const void* q, const
   uint32_t* amax = static_cast<uint32_t*>(ws);
   if (cudaMemsetAsync(amax, 0, (size_t)2 * BH * sizeof(uint32_t), st) != cudaSuccess) return SVA_ERR_CUDA;
   const Strides sq = make_strides(p->q_stride), sk = make_strides(p->k_stride);
-  const int run = blocks_per_cta(2LL * m.R);
+  const int run = blocks_per_cta(2LL * m.R, 32 << 10);
   const int rc = launch_dep(amax_kernel, dim3((m.Nb + run - 1) / run, BH, 2), Q4_THREADS, 0, st, (const __nv_bfloat16*)q,
                             (const __nv_bfloat16*)k, sq, sk, m.H, m.N, BH, run, amax);
   if (rc != SVA_OK) return rc;

@@ -4,7 +4,7 @@
 // similarity metric of the sparse-attention section.)
 //
 // pool_kernel streams Q and K once from HBM: 128-bit loads, fp32 accumulation in a fixed order, a CTA per
-// run of one or four blocks of a head of a tensor.  block_scores_kernel computes a head's score matrix as a
+// run of blocks of a head of a tensor.  block_scores_kernel computes a head's score matrix as a
 // small fp32 GEMM (64 x 64 or 32 x 32 tiles from two shared-memory panels, fixed summation order).  Small problems take one
 // kernel for all three (route_cluster_kernel).
 // select_rows_kernel is one warp per query-block row: it reads the row's scores from that matrix (no shared
@@ -38,21 +38,23 @@ __device__ __forceinline__ void add_vector(const uint4& u, uint64_t (&acc)[8 / E
 
 // Block means of one head of one tensor (blockIdx.z: 0 = Q, 1 = K); a CTA pools `run` consecutive blocks.
 // ELEM_BYTES = 2: bf16 input.  ELEM_BYTES = 1: e4m3 codes, multiplied by the block's scale.
-// Bound by the HBM: one pass over Q and K.  A CTA's loads run one step (four vectors per thread) ahead of its sums, across
-// the blocks of its run, so the reduction at the end of a block (two barriers) happens with the next block's loads in
-// flight; with a CTA per block nothing was in flight while it reduced.  Q and K of 24 heads
-// x 32 760 tokens, d = 128 (403 MB): 75.8 -> 71.8 us (5.6 TB/s) with 128-token blocks, 81 -> 72.7 us with 64-token
-// ones.  e4m3 codes (201 MB, converted in pairs) are bound by the sums and the reduction, which half the bytes do not hide: 66.5 -> 58.6 us with the
-// run, 52.6 -> 46.4 (on a faster box) with pairs added in one instruction and partial sums laid out so that no two lanes of a warp meet in a bank.
-template <int D, int ELEM_BYTES>
+// Bound by the HBM: one pass over Q and K.  A CTA's loads run one block ahead of its sums, across the reduction (two barriers); with a
+// CTA per block nothing was in flight while it reduced.  VECS: 16-byte vectors of a block per thread, so that a step is a whole block
+// whatever its size (with four per step a 128-token block took two steps, and 64-token blocks of e4m3 codes or of d = 64 masked half of the loads).
+// Q and K of 24 heads x 32 760 tokens, d = 128 (403 MB): 75.8 us with a CTA per block, 70.8 with runs of four, two steps a block, 69.1 so (5.8 TB/s);
+// another box, four vectors and runs of four -> a block at a time and runs of up to 128 KB: 24 x 32 760 66.9 -> 61.8 (6.5 TB/s), in 64-token blocks
+// 68.6 -> 65.0, 16 heads x 8 192 14.6 -> 12.3, 20 x 17 550 33.6 -> 30.9, 64 x 47 616 236.5 -> 223.4; d = 64 in 64-token blocks, 16 x 8 192, 11.7 -> 8.0.
+// e4m3 codes (201 MB, converted in pairs) are bound by the sums and the reduction, which half the bytes do not hide: 66.5 -> 58.6 us with the
+// run, 52.6 -> 46.4 (on a faster box) with pairs added in one instruction and partial sums laid out so that no two lanes of a warp meet in a
+// bank, 41.2 with runs of eight; in 64-token blocks 87.4 -> 47.4.
+template <int D, int ELEM_BYTES, int VECS>
 __global__ void __launch_bounds__(POOL_THREADS)
 pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Strides sq, Strides sk,
             const float* __restrict__ q_scale, const float* __restrict__ k_scale, int H, int N,
             int block, int Nb, int run, float* __restrict__ qbar, float* __restrict__ kbar) {
   constexpr int EPV = 16 / ELEM_BYTES;          // elements per 16-byte vector
   constexpr int VPR = D / EPV;                  // vectors per token row
-  constexpr int GROUPS = POOL_THREADS / VPR;    // token rows read concurrently
-  constexpr int STEP = GROUPS * 4;              // token rows per step
+  constexpr int GROUPS = POOL_THREADS / VPR;    // token rows read concurrently; VECS * GROUPS = block
   __shared__ float part[EPV][POOL_THREADS + (EPV == 8 ? 4 : 2)];    // (a warp's writes and its reads touch every bank once)
 
   // (e4m3 codes: from the end, which the quantiser has just written and the L2 still holds)
@@ -63,48 +65,40 @@ pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Stride
   const uint8_t* base = (which ? k : q) + ((long long)b * s.b + (long long)h * s.h) * ELEM_BYTES;
   const int I0 = (BACK ? gridDim.x - 1 - blockIdx.x : blockIdx.x) * run, I1 = min(I0 + run, Nb);
   const int vec = threadIdx.x % VPR, grp = threadIdx.x / VPR;
-  const int per_block = (block + STEP - 1) / STEP, steps = (I1 - I0) * per_block;
 
-  uint4 u[4];
-  auto load = [&](int step) {
-    const int I = I0 + step / per_block, t0 = (step % per_block) * STEP + grp;
-    const int lo = I * block, cnt = step < steps ? min(block, N - lo) : 0;
+  uint4 u[VECS];
+  auto load = [&](int I) {
+    const int lo = I * block, cnt = I < I1 ? min(block, N - lo) : 0;
 #pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      const int t = t0 + j * GROUPS;
+    for (int j = 0; j < VECS; ++j) {
+      const int t = grp + j * GROUPS;
       u[j] = make_uint4(0, 0, 0, 0);
       if (t < cnt) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(lo + t) * s.n * ELEM_BYTES) + vec);
     }
   };
-  uint64_t acc[EPV / 2];
+  load(I0);
+  for (int I = I0; I < I1; ++I) {
+    uint64_t acc[EPV / 2];
 #pragma unroll
-  for (int e = 0; e < EPV / 2; ++e) acc[e] = 0ull;
-  load(0);
-  for (int step = 0; step < steps; ++step) {
-    uint4 c[4];
+    for (int e = 0; e < EPV / 2; ++e) acc[e] = 0ull;
+    uint4 c[VECS];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) c[j] = u[j];
-    load(step + 1);
+    for (int j = 0; j < VECS; ++j) c[j] = u[j];
+    load(I + 1);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) add_vector<ELEM_BYTES>(c[j], acc);
-    if ((step + 1) % per_block == 0) {                            // the block's rows are in: reduce over the groups
-      const int I = I0 + step / per_block;
+    for (int j = 0; j < VECS; ++j) add_vector<ELEM_BYTES>(c[j], acc);
 #pragma unroll
-      for (int e = 0; e < EPV / 2; ++e) {
-        unpack2(acc[e], part[2 * e][grp * VPR + vec], part[2 * e + 1][grp * VPR + vec]);
-        acc[e] = 0ull;
-      }
-      __syncthreads();
-      if (threadIdx.x < D) {
-        float sum = 0.f;
+    for (int e = 0; e < EPV / 2; ++e) unpack2(acc[e], part[2 * e][grp * VPR + vec], part[2 * e + 1][grp * VPR + vec]);
+    __syncthreads();
+    if (threadIdx.x < D) {
+      float sum = 0.f;
 #pragma unroll 8
-        for (int g = 0; g < GROUPS; ++g) sum += part[threadIdx.x % EPV][g * VPR + threadIdx.x / EPV];   // fixed order
-        float mean = sum / (float)min(block, N - I * block);
-        if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
-        (which ? kbar : qbar)[((long long)bh * Nb + I) * D + threadIdx.x] = mean;
-      }
-      __syncthreads();
+      for (int g = 0; g < GROUPS; ++g) sum += part[threadIdx.x % EPV][g * VPR + threadIdx.x / EPV];   // fixed order
+      float mean = sum / (float)min(block, N - I * block);
+      if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
+      (which ? kbar : qbar)[((long long)bh * Nb + I) * D + threadIdx.x] = mean;
     }
+    __syncthreads();
   }
 }
 
@@ -750,9 +744,13 @@ size_t select_workspace_bytes(const Dims& m, const sva_select_t* s) {
 template <int D>
 static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale,
                          const float* k_scale, float* qbar, float* kbar, cudaStream_t st) {
-  const int run = blocks_per_cta(2LL * m.R);
+  const int eb = m.fp8 ? 1 : 2, run = blocks_per_cta(2LL * m.R, m.block * D * eb);
   const dim3 grid((m.Nb + run - 1) / run, m.B * m.H, 2);
-  return launch_dep(m.fp8 ? pool_kernel<D, 1> : pool_kernel<D, 2>, grid, POOL_THREADS, 0, st, (const uint8_t*)q, (const uint8_t*)k,
+  // (blocks of 64 or 128 tokens: block * D * eb bytes over 256 threads of 16)
+  constexpr int V2 = D / 32, V1 = D / 64;                         // vectors per thread of a 64-token block, bf16 and e4m3
+  auto kern = m.block == 64 ? (m.fp8 ? pool_kernel<D, 1, V1> : pool_kernel<D, 2, V2>)
+                            : (m.fp8 ? pool_kernel<D, 1, 2 * V1> : pool_kernel<D, 2, 2 * V2>);
+  return launch_dep(kern, grid, POOL_THREADS, 0, st, (const uint8_t*)q, (const uint8_t*)k,
                     make_strides(p->q_stride), make_strides(p->k_stride), m.fp8 ? q_scale : nullptr, m.fp8 ? k_scale : nullptr,
                     m.H, m.N, m.block, m.Nb, run, qbar, kbar);
 }
