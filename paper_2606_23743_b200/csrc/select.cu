@@ -5,8 +5,8 @@
 //
 // pool_kernel streams Q and K once from HBM: 128-bit loads, fp32 accumulation in a fixed order, a CTA per
 // run of blocks of a head of a tensor.  block_scores_kernel computes a head's score matrix as a
-// small fp32 GEMM (64 x 64 or 32 x 32 tiles from two shared-memory panels, fixed summation order).  Small problems take one
-// kernel for all three (route_cluster_kernel).
+// small fp32 GEMM (64 x 64 or 32 x 32 tiles from two shared-memory panels, fixed summation order).  Up to 64 blocks per head one kernel
+// scores and selects (route_means_kernel); the smallest problems take one for all three (route_cluster_kernel).
 // select_rows_kernel is one warp per query-block row: it reads the row's scores from that matrix (no shared
 // memory) as order-preserving integer keys, finds the threshold of the rule by narrowing an interval of scores
 // that holds it and emits the kept blocks in ascending order.  When the per-row count is known on the host (top-k with no window larger than k)
@@ -520,14 +520,14 @@ select_rows_kernel(const float* __restrict__ scores, SelParams p, int32_t* __res
   select_and_emit<ITEMS, MASS>(key, I, bh, lane, p, row_ptr, col_idx, tmp_idx, counts, R);
 }
 
-// Small problems: pooling, scores and selection of one head by one cluster of eight CTAs, one launch instead of three.  Each CTA pools
+// The smallest problems: pooling, scores and selection of one head by one cluster of eight CTAs, one launch.  Each CTA pools
 // its share of the head's blocks of Q and K (a team of 256 threads per block), writes a key mean into the shared memory of all eight,
 // and then scores and selects its own query blocks.  Sums run in the orders of pool_kernel and block_scores_kernel, so lists and
 // scores are the same bytes.
-// Bound by latency: launches, the cluster's barriers, a pooling round of 32 KB (about 1 100 cycles of loads, sums and reduction), and a
-// score and selection phase of a few warps.  Microseconds of a routing call, three kernels -> this one (top-k / mass rule with csr_kernel):
-// 2 heads x 16 blocks of 64 x 64 8.8 -> 5.3, 12 heads x 44 blocks of 128 x 128 15.0 -> 12.1 / 17.9 -> 14.7, 32 x 64 38.3 -> 27.4 / 41.7 -> 32.6.
-static constexpr int RC_CTAS = 8, RC_TEAM = 256, RC_ITEMS = 2, RC_MAX_NB = 32 * RC_ITEMS;
+// Bound by latency: the launch, the cluster's barriers (about 0.5 us each), a pooling round of a block per team (about 1 100 cycles of loads, sums
+// and reduction), and the score and selection phase of a warp per row.  Microseconds of a routing call (top-k), pool_kernel and
+// route_means_kernel / this one: 2 heads x 16 blocks of 64 x 64 7.3 / 5.3, of 128 x 128 7.35 / 6.3; 1 x 8 7.3 / 5.5.
+static constexpr int RC_CTAS = 8, RC_TEAMS = 4, RC_TEAM = 256, RC_ITEMS = 1, RC_MAX_NB = 32 * RC_ITEMS;
 static constexpr int RC_ROWS = RC_MAX_NB / RC_CTAS;                         // query blocks per CTA at most (a multiple of 4)
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
@@ -536,86 +536,24 @@ __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.w
 __device__ __forceinline__ void store_cluster(uint32_t addr, int rank, float v) {
   asm volatile("{\n.reg .b32 a;\nmapa.shared::cluster.u32 a, %0, %1;\nst.shared::cluster.f32 [a], %2;\n}" ::"r"(addr), "r"(rank), "f"(v) : "memory");
 }
-template <int D, int ELEM_BYTES, int TEAMS>
+template <int D, int ELEM_BYTES>
 struct RcSmem {
   static constexpr int VPR = D * ELEM_BYTES / 16, GROUPS = RC_TEAM / VPR, EPV = 16 / ELEM_BYTES, LD = D + 4;
   // partial sums [element of the vector][group][vector]: both the writes (a lane per vector) and the reads (a lane per column) of a
   // warp touch every bank once
   static constexpr int PART = GROUPS * VPR + (EPV == 8 ? 4 : 2);
-  float part[TEAMS][EPV * PART];
+  float part[RC_TEAMS][EPV * PART];
 };
-// TEAMS: blocks pooled at a time.  Four while a CTA has an SM to itself, two (so that two CTAs fit on an SM) beyond that.
-template <int D, int ELEM_BYTES, int TEAMS, bool MASS>
-__global__ void __launch_bounds__(TEAMS * RC_TEAM, 4 / TEAMS)
-route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Strides sq, Strides sk,
-                     const float* __restrict__ q_scale, const float* __restrict__ k_scale, int H, int N, int block, float scale,
-                     SelParams p, float* __restrict__ scores, int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx,
-                     int32_t* __restrict__ tmp_idx, int32_t* __restrict__ counts, int R) {
-  using Sm = RcSmem<D, ELEM_BYTES, TEAMS>;
-  constexpr int VPR = Sm::VPR, GROUPS = Sm::GROUPS, EPV = Sm::EPV, LD = Sm::LD, NV = 128 / GROUPS;     // NV: vectors per thread and block
-  constexpr int ITEMS = RC_ITEMS;
-  extern __shared__ __align__(16) uint8_t rc_smem[];
-  Sm& sm = *reinterpret_cast<Sm*>(rc_smem);
-  float* ks = reinterpret_cast<float*>(rc_smem + sizeof(Sm));          // [32 * ITEMS][LD] key means of the head
-  float* qm = ks + 32 * ITEMS * LD;                                    // [rows][LD] means of my query blocks
-  uint32_t* keys = reinterpret_cast<uint32_t*>(qm + RC_ROWS * LD);      // [rows][32 * ITEMS] scores as keys
-  uint32_t* wgts = keys + RC_ROWS * 32 * ITEMS;                 // ... and their weights
-  const int Nb = p.Nb, per = (Nb + RC_CTAS - 1) / RC_CTAS;
-  cluster_arrive();                        // (the CTAs of the cluster have started: they may be written to)
-  const int rank = blockIdx.x % RC_CTAS, bh = blockIdx.x / RC_CTAS + grid_dep_wait();
-  const int b = bh / H, h = bh % H, I0 = rank * per, mine = max(0, min(per, Nb - I0));
-  const int team = threadIdx.x / RC_TEAM, tt = threadIdx.x % RC_TEAM, vec = tt % VPR, grp = tt / VPR;
-
-  // ---- pooling: items 0 .. mine-1 are blocks of Q, the rest blocks of K; the next item's loads are in flight behind a reduction
-  uint4 u[NV];
-  auto load = [&](int item) {
-    const int which = item >= mine, I = I0 + (which ? item - mine : item);
-    const Strides s = which ? sk : sq;
-    const int lo = I * block, cnt = item < 2 * mine ? min(block, N - lo) : 0;
-    const uint8_t* base = (which ? k : q) + ((long long)b * s.b + (long long)h * s.h + (long long)(lo + grp) * s.n) * ELEM_BYTES;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      u[j] = make_uint4(0, 0, 0, 0);
-      if (grp + j * GROUPS < cnt) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(j * GROUPS) * s.n * ELEM_BYTES) + vec);
-    }
-  };
-  load(team);
-  cluster_wait();
-  for (int item = team; item < 2 * mine; item += TEAMS) {
-    const int which = item >= mine, li = which ? item - mine : item, I = I0 + li;
-    uint64_t acc[EPV / 2];
-#pragma unroll
-    for (int e = 0; e < EPV / 2; ++e) acc[e] = 0ull;
-#pragma unroll
-    for (int j = 0; j < NV; ++j) add_vector<ELEM_BYTES>(u[j], acc);
-    load(item + TEAMS);
-    float* part = sm.part[team];
-#pragma unroll
-    for (int e = 0; e < EPV / 2; ++e)
-      unpack2(acc[e], part[2 * e * Sm::PART + grp * VPR + vec], part[(2 * e + 1) * Sm::PART + grp * VPR + vec]);
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(RC_TEAM) : "memory");
-    if (tt < D) {
-      float sum = 0.f;
-#pragma unroll 8
-      for (int g = 0; g < GROUPS; ++g) sum += part[(tt % EPV) * Sm::PART + g * VPR + tt / EPV];       // fixed order
-      float mean = sum / (float)min(block, N - I * block);
-      if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
-      if (which) {
-        const uint32_t dst = smem_addr(ks + I * LD + tt);
-#pragma unroll
-        for (int r = 0; r < RC_CTAS; ++r) store_cluster(dst, r, mean);
-      } else {
-        qm[li * LD + tt] = mean;
-      }
-    }
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(RC_TEAM) : "memory");
-  }
-  grid_dep_launch();
-  cluster_arrive();
-  cluster_wait();
-
-  // ---- scores of my query blocks as keys: a thread per four query blocks and ITEMS key blocks, sums as in block_scores_kernel
-  constexpr int RQ = 4;
+// Scores and selection of `mine` consecutive query blocks of a head, from I0 on, by a whole CTA (a warp per row at least): ks, qm are the
+// head's key means and the blocks' means in shared memory ([..][D + 4]), keys and wgts room for 32 * ITEMS words per row.
+template <int D, int RQ, int ITEMS, bool MASS>
+__device__ __forceinline__ void score_and_select(const float* ks, const float* qm, uint32_t* keys, uint32_t* wgts, const int mine, const int I0,
+                                                 const int bh, const float scale, const SelParams& p, float* __restrict__ scores,
+                                                 int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx,
+                                                 int32_t* __restrict__ tmp_idx, int32_t* __restrict__ counts, const int R) {
+  constexpr int LD = D + 4;
+  const int Nb = p.Nb;
+  // ---- scores as keys: a thread per RQ query blocks and ITEMS key blocks, sums as in block_scores_kernel
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp * RQ < mine) {
     uint64_t acc[RQ][ITEMS];
@@ -666,6 +604,115 @@ route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ 
     for (int it = 0; it < ITEMS; ++it) key[it] = sk[it * 32 + lane];
     rank_and_emit<ITEMS, MASS>(key, sk, wgts + li * 32 * ITEMS, I0 + li, bh, lane, p, row_ptr, col_idx, tmp_idx, counts, R);
   }
+}
+template <int D, int ELEM_BYTES, bool MASS>
+__global__ void __launch_bounds__(RC_TEAMS * RC_TEAM)
+route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Strides sq, Strides sk,
+                     const float* __restrict__ q_scale, const float* __restrict__ k_scale, int H, int N, int block, float scale,
+                     SelParams p, float* __restrict__ scores, int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx,
+                     int32_t* __restrict__ tmp_idx, int32_t* __restrict__ counts, int R) {
+  using Sm = RcSmem<D, ELEM_BYTES>;
+  constexpr int VPR = Sm::VPR, GROUPS = Sm::GROUPS, EPV = Sm::EPV, LD = Sm::LD, NV = 128 / GROUPS;     // NV: vectors per thread and block
+  constexpr int ITEMS = RC_ITEMS;
+  extern __shared__ __align__(16) uint8_t rc_smem[];
+  Sm& sm = *reinterpret_cast<Sm*>(rc_smem);
+  float* ks = reinterpret_cast<float*>(rc_smem + sizeof(Sm));          // [32 * ITEMS][LD] key means of the head
+  float* qm = ks + 32 * ITEMS * LD;                                    // [rows][LD] means of my query blocks
+  uint32_t* keys = reinterpret_cast<uint32_t*>(qm + RC_ROWS * LD);      // [rows][32 * ITEMS] scores as keys
+  uint32_t* wgts = keys + RC_ROWS * 32 * ITEMS;                 // ... and their weights
+  const int Nb = p.Nb, per = (Nb + RC_CTAS - 1) / RC_CTAS;
+  cluster_arrive();                        // (the CTAs of the cluster have started: they may be written to)
+  const int rank = blockIdx.x % RC_CTAS, bh = blockIdx.x / RC_CTAS + grid_dep_wait();
+  const int b = bh / H, h = bh % H, I0 = rank * per, mine = max(0, min(per, Nb - I0));
+  const int team = threadIdx.x / RC_TEAM, tt = threadIdx.x % RC_TEAM, vec = tt % VPR, grp = tt / VPR;
+
+  // ---- pooling: items 0 .. mine-1 are blocks of Q, the rest blocks of K; the next item's loads are in flight behind a reduction
+  uint4 u[NV];
+  auto load = [&](int item) {
+    const int which = item >= mine, I = I0 + (which ? item - mine : item);
+    const Strides s = which ? sk : sq;
+    const int lo = I * block, cnt = item < 2 * mine ? min(block, N - lo) : 0;
+    const uint8_t* base = (which ? k : q) + ((long long)b * s.b + (long long)h * s.h + (long long)(lo + grp) * s.n) * ELEM_BYTES;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) {
+      u[j] = make_uint4(0, 0, 0, 0);
+      if (grp + j * GROUPS < cnt) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(j * GROUPS) * s.n * ELEM_BYTES) + vec);
+    }
+  };
+  load(team);
+  cluster_wait();
+  for (int item = team; item < 2 * mine; item += RC_TEAMS) {
+    const int which = item >= mine, li = which ? item - mine : item, I = I0 + li;
+    uint64_t acc[EPV / 2];
+#pragma unroll
+    for (int e = 0; e < EPV / 2; ++e) acc[e] = 0ull;
+#pragma unroll
+    for (int j = 0; j < NV; ++j) add_vector<ELEM_BYTES>(u[j], acc);
+    load(item + RC_TEAMS);
+    float* part = sm.part[team];
+#pragma unroll
+    for (int e = 0; e < EPV / 2; ++e)
+      unpack2(acc[e], part[2 * e * Sm::PART + grp * VPR + vec], part[(2 * e + 1) * Sm::PART + grp * VPR + vec]);
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(RC_TEAM) : "memory");
+    if (tt < D) {
+      float sum = 0.f;
+#pragma unroll 8
+      for (int g = 0; g < GROUPS; ++g) sum += part[(tt % EPV) * Sm::PART + g * VPR + tt / EPV];       // fixed order
+      float mean = sum / (float)min(block, N - I * block);
+      if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
+      if (which) {
+        const uint32_t dst = smem_addr(ks + I * LD + tt);
+#pragma unroll
+        for (int r = 0; r < RC_CTAS; ++r) store_cluster(dst, r, mean);
+      } else {
+        qm[li * LD + tt] = mean;
+      }
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(RC_TEAM) : "memory");
+  }
+  grid_dep_launch();
+  cluster_arrive();
+  cluster_wait();
+
+  score_and_select<D, 2, ITEMS, MASS>(ks, qm, keys, wgts, mine, I0, bh, scale, p, scores, row_ptr, col_idx, tmp_idx, counts, R);
+}
+
+// The same tail for block means that are at hand (a pooling or prologue kernel has written them): scores and selection of eight query
+// blocks of a head per CTA, one launch instead of two.  Up to 64 blocks per head, where the key means fit beside one another and a row's rank is
+// counted.  Bound by latency: the means' way from the L2, then as above.  Routing from means, scores and selection kernels -> this one (us, top-k / mass rule with csr_kernel):
+// 16 heads x 64 blocks 8.0 -> 4.9 / 15.2 -> 6.9, 24 x 64 12.3 -> 8.6 / 20.5 -> 11.2, 128 x 64 22.3 -> 15.0 / 27.8 -> 20.8, 2 x 16 6.3 -> 4.9 / 8.4 -> 6.9; nothing up to 64
+// blocks is slower.
+static constexpr int RT_ROWS = 8, RT_ITEMS = 2, RT_MAX_NB = 32 * RT_ITEMS;
+template <int D, bool MASS>
+__global__ void __launch_bounds__(RT_ROWS * 32)
+route_means_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar, float scale, SelParams p, float* __restrict__ scores,
+                   int32_t* __restrict__ row_ptr, int32_t* __restrict__ col_idx, int32_t* __restrict__ tmp_idx,
+                   int32_t* __restrict__ counts, int R) {
+  constexpr int LD = D + 4, V = D / 4;
+  extern __shared__ __align__(16) uint8_t rc_smem[];
+  float* ks = reinterpret_cast<float*>(rc_smem);                       // [64][LD]
+  float* qm = ks + RT_MAX_NB * LD;                                     // [8][LD]
+  uint32_t* keys = reinterpret_cast<uint32_t*>(qm + RT_ROWS * LD);
+  uint32_t* wgts = keys + RT_ROWS * RT_MAX_NB;
+  grid_dep_launch();
+  const int bh = blockIdx.y + grid_dep_wait(), I0 = blockIdx.x * RT_ROWS, mine = min(RT_ROWS, p.Nb - I0);
+  const float4* ksrc = reinterpret_cast<const float4*>(kbar + (long long)bh * p.Nb * D);
+  const float4* qsrc = reinterpret_cast<const float4*>(qbar + ((long long)bh * p.Nb + I0) * D);
+  constexpr int PER = RT_MAX_NB * V / (RT_ROWS * 32);                  // 16-byte vectors per thread, all in flight
+  float4 a[PER];
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const int x = threadIdx.x + u * RT_ROWS * 32;
+    a[u] = x < p.Nb * V ? __ldg(ksrc + x) : make_float4(0.f, 0.f, 0.f, 0.f);
+  }
+  for (int x = threadIdx.x; x < mine * V; x += RT_ROWS * 32) *reinterpret_cast<float4*>(qm + x / V * LD + 4 * (x % V)) = __ldg(qsrc + x);
+#pragma unroll
+  for (int u = 0; u < PER; ++u) {
+    const int x = threadIdx.x + u * RT_ROWS * 32;
+    *reinterpret_cast<float4*>(ks + x / V * LD + 4 * (x % V)) = a[u];
+  }
+  __syncthreads();
+  score_and_select<D, 2, RT_ITEMS, MASS>(ks, qm, keys, wgts, mine, I0, bh, scale, p, scores, row_ptr, col_idx, tmp_idx, counts, R);
 }
 
 // CSR assembly for rows of varying length, one launch: a CTA owns 32 consecutive rows (one warp each).  It
@@ -755,31 +802,21 @@ static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, c
                     m.H, m.N, m.block, m.Nb, run, qbar, kbar);
 }
 
-// Where the cluster kernel routes: blocks pooled at a time per CTA, or 0 for the three kernels (us, three kernels / this one).
-// Up to 14 heads each CTA has an SM to itself (15 or more clusters of eight SMs do not fit: 16 heads x 64 blocks 22.0 / 27.5): 14 x 64
-// 21.3 / 15.4, and no form of up to 64 blocks is slower except where few heads leave most SMs without a block to pool (2 x 64 9.8 / 12.8,
-// 4 x 64 11.4 / 15.6, but 8 x 44 12.3 / 11.4).
-// With two CTAs per SM more heads fit, at half the pooling rate each: with 16 blocks a head, 32 x 16 14.1 / 10.7, or where pooling is bound by the
-// HBM anyway, blocks of 32 KB: 24 x 32 18.4 / 13.9, 18 x 64 24.2 / 22.8, 32 x 64 38.3 / 27.4 (16 KB: 18 x 44 14.1 / 17.0; 36 x 64 39.7 / 41.8).
-// Beyond 64 blocks the exchanged means cost an SM its second CTA (24 x 96: 43.6 / 56.9).
-static int route_teams(const Dims& m) {
-  const int heads = m.B * m.H;
-  if (m.Nb > RC_MAX_NB || heads > 32) return 0;
-  if (heads <= 14) return m.Nb <= 32 || heads * m.Nb >= 8 * 44 ? 4 : 0;
-  const bool big_blocks = m.block * m.d * (m.fp8 ? 1 : 2) == 32768;
-  return m.Nb <= 16 || (big_blocks && (m.Nb <= 32 ? heads <= 24 : heads >= 18)) ? 2 : 0;
-}
-template <int D, int ELEM_BYTES, int TEAMS, bool MASS>
+// Where the cluster kernel routes.  Up to 14 heads each of its CTAs has an SM to itself (15 or more clusters of eight SMs do not fit: 16 heads x 64 blocks 22.0 /
+// 27.5 when both ended in three launches' tail), and up to 16 blocks a CTA pools in one round.  Beyond that pooling over all SMs and
+// route_means_kernel are faster: 12 heads x 20 blocks of 128 x 128 7.3 / 7.9, 12 x 44 9.8 / 12.2, 16 x 16 7.2 / 8.0 (two CTAs per SM).
+static bool route_in_cluster(const Dims& m) { return m.Nb <= 16 && m.B * m.H <= 14; }
+template <int D, int ELEM_BYTES, bool MASS>
 static int launch_route(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale, const float* k_scale,
                         const SelParams& sp, float* scores, int32_t* row_ptr, int32_t* col_idx, int32_t* tmp_idx, int32_t* counts,
                         cudaStream_t st) {
-  auto kern = route_cluster_kernel<D, ELEM_BYTES, TEAMS, MASS>;
-  using Sm = RcSmem<D, ELEM_BYTES, TEAMS>;
+  auto kern = route_cluster_kernel<D, ELEM_BYTES, MASS>;
+  using Sm = RcSmem<D, ELEM_BYTES>;
   constexpr int smem = (int)sizeof(Sm) + 4 * ((RC_MAX_NB + RC_ROWS) * Sm::LD + 2 * RC_ROWS * RC_MAX_NB);
   static DeviceOnce once;
   const int rc = once.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess; });
   if (rc != SVA_OK) return rc;
-  return launch_dep_cluster(RC_CTAS, kern, m.B * m.H * RC_CTAS, TEAMS * RC_TEAM, smem, st, (const uint8_t*)q, (const uint8_t*)k,
+  return launch_dep_cluster(RC_CTAS, kern, m.B * m.H * RC_CTAS, RC_TEAMS * RC_TEAM, smem, st, (const uint8_t*)q, (const uint8_t*)k,
                             make_strides(p->q_stride), make_strides(p->k_stride), q_scale, k_scale, m.H, m.N, m.block, m.scale, sp,
                             scores, row_ptr, col_idx, tmp_idx, counts, m.R);
 }
@@ -813,21 +850,23 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
     if (fixed_n) return (int)SVA_OK;
     return launch_dep(csr_kernel, (m.R + CSR_ROWS - 1) / CSR_ROWS, CSR_ROWS * 32, 0, st, tmp_idx, counts, cap, m.R, row_ptr, col_idx);
   };
-  if (const int teams = qbar_in ? 0 : route_teams(m)) {
-    auto route = [&](auto elem_tag, auto teams_tag, auto mass_tag) {
-      return launch_route<D, decltype(elem_tag)::value, decltype(teams_tag)::value, decltype(mass_tag)::value>(
+  if (!qbar_in && route_in_cluster(m)) {
+    auto route = [&](auto elem_tag, auto mass_tag) {
+      return launch_route<D, decltype(elem_tag)::value, decltype(mass_tag)::value>(
           m, p, q, k, m.fp8 ? q_scale : nullptr, m.fp8 ? k_scale : nullptr, sp, block_scores, row_ptr, col_idx, tmp_idx, counts, st);
     };
-    auto by_mass = [&](auto elem_tag, auto teams_tag) {
-      return s->mode == 1 ? route(elem_tag, teams_tag, std::true_type{}) : route(elem_tag, teams_tag, std::false_type{});
-    };
-    auto by_teams = [&](auto elem_tag) {
-      return teams == 4 ? by_mass(elem_tag, std::integral_constant<int, 4>{}) : by_mass(elem_tag, std::integral_constant<int, 2>{});
-    };
-    rc = m.fp8 ? by_teams(std::integral_constant<int, 1>{}) : by_teams(std::integral_constant<int, 2>{});
+    auto by_mass = [&](auto elem_tag) { return s->mode == 1 ? route(elem_tag, std::true_type{}) : route(elem_tag, std::false_type{}); };
+    rc = m.fp8 ? by_mass(std::integral_constant<int, 1>{}) : by_mass(std::integral_constant<int, 2>{});
     return rc != SVA_OK ? rc : csr();
   }
   if (!qbar_in && (rc = launch_pool_d<D>(m, p, q, k, q_scale, k_scale, qbar, kbar, st)) != SVA_OK) return rc;
+  if (m.Nb <= RT_MAX_NB) {
+    constexpr int smem = 4 * ((RT_MAX_NB + RT_ROWS) * (D + 4) + 2 * RT_ROWS * RT_MAX_NB);      // (below the 48 KB that need no attribute)
+    static_assert(smem <= 48 * 1024, "");
+    rc = launch_dep(s->mode == 1 ? route_means_kernel<D, true> : route_means_kernel<D, false>, dim3((m.Nb + RT_ROWS - 1) / RT_ROWS, m.B * m.H),
+                    RT_ROWS * 32, smem, st, (const float*)qbar, (const float*)kbar, m.scale, sp, block_scores, row_ptr, col_idx, tmp_idx, counts, m.R);
+    return rc != SVA_OK ? rc : csr();
+  }
   // scores: into the caller's matrix if it wants one, else into the workspace (after the staging arrays)
   float* scores = block_scores;
   if (!scores) {

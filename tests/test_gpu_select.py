@@ -219,27 +219,32 @@ def test_rows_of_a_known_length_are_written_whole(nb, k, window):
 
 
 @pytest.mark.parametrize("B_,H,Nb,block,d,fp8,mode,k,window,layout,values", [
-    (1, 1, 1, 128, 128, False, 0, 1, False, "heads", "normal"),           # one block, ragged
-    (1, 3, 9, 128, 128, False, 1, 4, False, "tokens", "normal"),          # CTAs of the cluster without a block
-    (2, 7, 64, 64, 128, False, 0, 11, False, "packed", "normal"),         # 14 heads, the most blocks
-    (1, 12, 44, 128, 64, False, 1, 12, True, "heads", "normal"),          # forced window and mass
-    (1, 8, 44, 64, 64, False, 0, 3, True, "tokens", "ties"),              # window larger than k, equal scores
-    (1, 2, 31, 128, 128, False, 1, 40, False, "heads", "zero"),           # every score equal, k beyond Nb
-    (1, 4, 20, 64, 128, False, 0, 7, False, "heads", "nan"),              # rows of NaN scores come out short
-    (1, 9, 33, 64, 128, True, 1, 6, False, "tokens", "normal"),           # e4m3 codes, 3 rows in a CTA's last quad
-    (1, 16, 16, 64, 64, True, 0, 5, False, "heads", "normal"),            # two CTAs per SM
+    (1, 1, 1, 128, 128, False, 0, 1, False, "heads", "normal"),           # one launch: one block, ragged
+    (1, 3, 9, 128, 128, False, 1, 4, False, "tokens", "normal"),          # ... CTAs of the cluster without a block
+    (2, 7, 16, 64, 64, True, 0, 5, True, "heads", "normal"),              # ... 14 heads, the most blocks, e4m3, forced window
+    (1, 4, 12, 64, 128, False, 0, 9, False, "heads", "nan"),              # ... rows of NaN scores come out short
+    (1, 2, 13, 128, 64, True, 1, 40, False, "packed8", "zero"),           # ... every score equal, k beyond Nb
+    (1, 15, 16, 64, 64, False, 0, 5, False, "heads", "normal"),           # means, then scores and selection: one head too many
+    (2, 7, 64, 64, 128, False, 0, 11, False, "packed", "normal"),         # ... the most blocks
+    (1, 12, 44, 128, 64, False, 1, 12, True, "heads", "normal"),          # ... forced window and mass
+    (1, 8, 44, 64, 64, False, 0, 3, True, "tokens", "ties"),              # ... window larger than k, equal scores
+    (1, 2, 31, 128, 128, False, 1, 40, False, "heads", "zero"),
+    (1, 4, 20, 64, 128, False, 0, 7, False, "heads", "nan"),
+    (1, 9, 33, 64, 128, True, 1, 6, False, "tokens", "normal"),           # ... e4m3 codes, a row in a CTA of its own
     (2, 9, 64, 128, 128, False, 1, 9, False, "packed", "normal"),
     (1, 24, 17, 128, 128, False, 0, 2, False, "heads", "ties"),
+    (1, 5, 65, 64, 64, False, 1, 9, False, "heads", "normal"),            # the general kernels, one block more
 ])
-def test_routing_in_one_launch_is_routing_in_three(B_, H, Nb, block, d, fp8, mode, k, window, layout, values):
-    """Small problems are routed by one kernel; the split calls (means, then routing from means) take the general ones: the same bytes."""
+def test_routing_of_small_problems(B_, H, Nb, block, d, fp8, mode, k, window, layout, values):
+    """Few blocks per head take kernels of their own, which rank a row's candidates instead of searching a threshold: the lists are what the sequential
+    rule takes from the kernel's own scores, and routing in one call is routing from means that another call has made, byte for byte."""
     N = Nb * block - (37 if Nb % 2 else 0)
     g = torch.Generator(device="cuda").manual_seed(Nb)
-    shape = {"heads": (2, B_, H, N, d), "tokens": (2, B_, N, H, d), "packed": (B_, N, 2, H, d)}[layout]
+    shape = {"heads": (2, B_, H, N, d), "tokens": (2, B_, N, H, d)}.get(layout, (B_, N, 2, H, d))
     x = torch.randn(shape, generator=g, device="cuda")
-    qk = x.transpose(2, 3) if layout == "tokens" else x.permute(2, 0, 3, 1, 4) if layout == "packed" else x       # [2, B, H, N, d] views
+    qk = x.transpose(2, 3) if layout == "tokens" else x if layout == "heads" else x.permute(2, 0, 3, 1, 4)       # [2, B, H, N, d] views
     if values == "ties":
-        qk[:, :, :, block:] = qk[:, :, :, : N - block].clone() if Nb < 3 else qk[:, :, :, :1]      # all blocks but the first alike
+        qk[:, :, :, block:] = qk[:, :, :, :1]                             # all blocks but the first alike
     elif values == "zero":
         qk.zero_()
     elif values == "nan":
@@ -253,8 +258,9 @@ def test_routing_in_one_launch_is_routing_in_three(B_, H, Nb, block, d, fp8, mod
     else:
         qk = qk.to(torch.bfloat16)
     q, kk = qk[0], qk[1]
+    tau, bpf = 0.7, 4
     p = B.make_problem(q, kk, None, None, N, block, 0.0, True) if fp8 else B.make_problem(q, kk, None, None, N, block)
-    s = B.make_select(mode, k, 0.7, *((1, 1, 4) if window else (-1, -1, 0)))
+    s = B.make_select(mode, k, tau, *((1, 1, bpf) if window else (-1, -1, 0)))
     got = []
     for split in (False, True):
         ws = torch.full((B.select_workspace_bytes(p, s),), 255, dtype=torch.uint8, device="cuda")
@@ -271,3 +277,27 @@ def test_routing_in_one_launch_is_routing_in_three(B_, H, Nb, block, d, fp8, mod
         got.append((rp, ci, sc.view(torch.int32)))
     for a, b in zip(*got):
         assert torch.equal(a, b)
+    rp, ci, sc = got[0][0].cpu().numpy(), got[0][1].cpu().numpy(), got[0][2].view(torch.float32).cpu().numpy().reshape(-1, Nb)
+    for r in range(B_ * H * Nb):
+        v, I = sc[r].astype(np.float64), r % Nb
+        kept = [J for J in range(Nb) if window and abs(I // bpf - J // bpf) <= 1 and abs(I % bpf - J % bpf) <= 1]
+        cand = np.flatnonzero(~np.isnan(v))
+        w = np.zeros(Nb)
+        if cand.size:
+            with np.errstate(invalid="ignore"):
+                w[cand] = np.exp(v[cand] - v[cand].max())
+            w /= w.sum()
+        near = False                                                      # (the mass comes within summation noise of tau: either is right)
+        for J in sorted((c for c in cand if c not in kept), key=lambda c: (-v[c], c)):
+            mass = w[kept].sum()
+            near = near or (mode == 1 and kept and abs(mass - tau) < 1e-5)
+            if len(kept) >= min(k, Nb) or (mode == 1 and kept and mass >= tau):
+                break
+            kept.append(J)
+        want = sorted(kept)
+        if mode == 0 and not window:
+            want += [0] * (min(k, Nb) - len(want))                        # (a short row is filled up)
+        have = ci[rp[r]:rp[r + 1]].tolist()
+        if values == "nan":
+            have, want = sorted(have), sorted(want)
+        assert near or have == want, (r, have, want)
