@@ -802,9 +802,9 @@ static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, c
                     m.H, m.N, m.block, m.Nb, run, qbar, kbar);
 }
 
-// Where the cluster kernel routes.  Up to 14 heads each of its CTAs has an SM to itself (15 or more clusters of eight SMs do not fit: 16 heads x 64 blocks 22.0 /
-// 27.5 when both ended in three launches' tail), and up to 16 blocks a CTA pools in one round.  Beyond that pooling over all SMs and
-// route_means_kernel are faster: 12 heads x 20 blocks of 128 x 128 7.3 / 7.9, 12 x 44 9.8 / 12.2, 16 x 16 7.2 / 8.0 (two CTAs per SM).
+// Where the cluster kernel routes.  Up to 14 heads each of its CTAs has an SM to itself (15 or more clusters of eight SMs do not fit at once), and up to
+// 16 blocks a CTA pools in one round.  Beyond that pooling over all SMs and route_means_kernel are faster (us, them / a cluster): 12 heads x 20 blocks
+// of 128 x 128 7.3 / 7.9, 12 x 44 9.8 / 12.2, 16 x 16 7.2 / 8.0 (with two CTAs per SM), 6 x 64 8.5 / 13.4.
 static bool route_in_cluster(const Dims& m) { return m.Nb <= 16 && m.B * m.H <= 14; }
 template <int D, int ELEM_BYTES, bool MASS>
 static int launch_route(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale, const float* k_scale,
