@@ -5,7 +5,7 @@
 //
 // pool_kernel streams Q and K once from HBM: 128-bit loads, fp32 accumulation in a fixed order, a CTA per
 // run of blocks of a head of a tensor.  block_scores_kernel computes a head's score matrix as a
-// small fp32 GEMM (64 x 64 or 32 x 32 tiles from two shared-memory panels, fixed summation order).  Up to 64 blocks per head one kernel
+// small fp32 GEMM (64 x 64 or 32 x 32 tiles from two shared-memory panels, fixed summation order).  With few blocks per head one kernel
 // scores and selects (route_means_kernel); the smallest problems take one for all three (route_cluster_kernel).
 // select_rows_kernel is one warp per query-block row: it reads the row's scores from that matrix (no shared
 // memory) as order-preserving integer keys, finds the threshold of the rule by narrowing an interval of scores
@@ -681,9 +681,15 @@ route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ 
 // The same tail for block means that are at hand (a pooling or prologue kernel has written them): scores and selection of eight query
 // blocks of a head per CTA, one launch instead of two.  Up to 64 blocks per head, where the key means fit beside one another and a row's rank is
 // counted.  Bound by latency: the means' way from the L2, then as above.  Routing from means, scores and selection kernels -> this one (us, top-k / mass rule with csr_kernel):
-// 16 heads x 64 blocks 8.0 -> 4.9 / 15.2 -> 6.9, 24 x 64 12.3 -> 8.6 / 20.5 -> 11.2, 128 x 64 22.3 -> 15.0 / 27.8 -> 20.8, 2 x 16 6.3 -> 4.9 / 8.4 -> 6.9; nothing up to 64
-// blocks is slower.
+// 16 heads x 64 blocks 8.0 -> 4.9 / 15.2 -> 6.9, 24 x 64 12.3 -> 8.6 / 20.5 -> 11.2, 128 x 64 22.3 -> 15.0 / 27.8 -> 20.8, 2 x 16 6.3 -> 4.9 / 8.4 -> 6.9.
 static constexpr int RT_ROWS = 8, RT_ITEMS = 2, RT_MAX_NB = 32 * RT_ITEMS;
+// Counting ranks is Nb steps per row where the threshold search takes about log2(Nb) + 2, so with long rows it pays only while the two launches that it
+// saves weigh more than the counting: up to 40 blocks always, beyond that up to a work (CTAs x steps) that 160 heads of 64 blocks come to (187 with the
+// mass rule, whose search carries the masses along).  From means, d = 128, us, scores and selection kernels / this one: top-k, 128 heads x 64 blocks 22.3 / 15.0,
+// 160 x 64 19.4 / 18.3, 200 x 64 20.8 / 22.0, 1 024 x 64 76.6 / 99.2, 220 x 52 19.6 / 19.6, 1 200 x 52 78 / 89, 1 200 x 40 67 / 63; mass rule, 200 x 64 32.9 / 31.0, 300 x 64 40.6 / 44.5.
+static bool route_by_rank(const Dims& m, int mode) {
+  return m.Nb <= 40 || (m.Nb <= RT_MAX_NB && (long long)m.B * m.H * ((m.Nb + RT_ROWS - 1) / RT_ROWS) * m.Nb <= (mode == 1 ? 96000 : 82000));
+}
 template <int D, bool MASS>
 __global__ void __launch_bounds__(RT_ROWS * 32)
 route_means_kernel(const float* __restrict__ qbar, const float* __restrict__ kbar, float scale, SelParams p, float* __restrict__ scores,
@@ -861,7 +867,7 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
     return rc != SVA_OK ? rc : csr();
   }
   if (!qbar_in && (rc = launch_pool_d<D>(m, p, q, k, q_scale, k_scale, qbar, kbar, st)) != SVA_OK) return rc;
-  if (m.Nb <= RT_MAX_NB) {
+  if (route_by_rank(m, s->mode)) {
     constexpr int smem = 4 * ((RT_MAX_NB + RT_ROWS) * (D + 4) + 2 * RT_ROWS * RT_MAX_NB);      // (below the 48 KB that need no attribute)
     static_assert(smem <= 48 * 1024, "");
     rc = launch_dep(s->mode == 1 ? route_means_kernel<D, true> : route_means_kernel<D, false>, dim3((m.Nb + RT_ROWS - 1) / RT_ROWS, m.B * m.H),

@@ -301,3 +301,34 @@ def test_routing_of_small_problems(B_, H, Nb, block, d, fp8, mode, k, window, la
         if values == "nan":
             have, want = sorted(have), sorted(want)
         assert near or have == want, (r, have, want)
+
+
+@pytest.mark.parametrize("mode,k,window,H,Nb,by_rank", [
+    (mode, k, window, H, Nb, by_rank) for mode, k, window, lines in [
+        (0, 9, False, ((160, 64), (310, 44))), (0, 5, True, ((160, 64), (310, 44))),
+        (1, 12, False, ((187, 64), (363, 44))), (1, 30, True, ((187, 64), (363, 44)))]
+    for H, Nb, by_rank in [(lines[0][0], 64, True), (lines[0][0] + 1, 64, False), (500, 64, False),
+                           (lines[1][0], 44, True), (lines[1][0] + 1, 44, False), (900, 40, True)]])
+def test_heads_at_the_end_of_counting_ranks(mode, k, window, H, Nb, by_rank):
+    """Many heads of 41 to 64 blocks search a threshold in a kernel of its own (which leaves the scores in the workspace), fewer count
+    ranks: on either side of the line a call returns what calls on a few of its heads return."""
+    g = torch.Generator(device="cuda").manual_seed(Nb)
+    qm, km = (torch.randn(1, H, Nb, 64, generator=g, device="cuda") for _ in range(2))
+    s = B.make_select(mode, k, 0.8, *((1, 1, 4) if window else (-1, -1, 0)))
+
+    def route(h0, h1):
+        t = torch.empty(1, h1 - h0, Nb * 64, 64, dtype=torch.bfloat16, device="cuda")
+        p = B.make_problem(t, t, None, None, Nb * 64, 64)
+        ws = torch.full((B.select_workspace_bytes(p, s),), 255, dtype=torch.uint8, device="cuda")
+        rp = torch.full(((h1 - h0) * Nb + 1,), -7, dtype=torch.int32, device="cuda")
+        ci = torch.full((B.select_max_nnz(p, s),), -7, dtype=torch.int32, device="cuda")
+        B.block_select_pooled(p, s, qm[:, h0:h1].contiguous(), km[:, h0:h1].contiguous(), rp, ci, ws)
+        torch.cuda.synchronize()
+        scores = ws[ws.numel() - (4 * (h1 - h0) * Nb * Nb + 255) // 256 * 256:]
+        return rp[1:] - rp[:-1], ci[:int(rp[-1])], bool((scores == 255).all())
+
+    counts, blocks, untouched = route(0, H)
+    assert untouched == by_rank
+    parts = [route(h, min(h + 100, H)) for h in range(0, H, 100)]
+    assert all(p[2] for p in parts)
+    assert torch.equal(counts, torch.cat([p[0] for p in parts])) and torch.equal(blocks, torch.cat([p[1] for p in parts]))
