@@ -20,17 +20,17 @@ static constexpr int Q4_THREADS = 256;
 
 // amax[tensor * BH + bh] (as fp32 bits; the launcher zeroes it) = max |x| over the existing tokens
 // From the end of the tensors, which a kernel that has just written them (the prologue) leaves in the L2.
-// A CTA reads `run` consecutive 128-token blocks, the next half block's loads in flight behind the current one's maxima (a whole block's: 73.1 us in the
-// pass against 70.6), and
-// does one atomicMax: with a block per CTA and an atomic per warp (98 304 of them on 48 words) the pass took 100 us for
-// 403 MB, now 70 us (5.7 TB/s).
+// A CTA per 128-token block, its second half's loads in flight behind the first half's maxima, and one atomicMax.  (An atomic per warp, 98 304 of
+// them on 48 words, took 100 us for 403 MB.  Runs of blocks per CTA, as pooling has them, are slower: there is no reduction per block to hide.
+// The whole quantiser, us, inputs not in the L2, runs of four / a block per CTA: 24 heads x 32 760 tokens 155.9 / 153.5, 16 x 16 384 61.2 / 56.1, 16 x 8 192
+// 33.3 / 32.8, 8 x 4 096 16.4 / 13.4; inputs in the L2, 16 x 8 192 30.4 / 28.7.)
 __global__ void __launch_bounds__(Q4_THREADS)
 amax_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, Strides sq, Strides sk, int H, int N,
-            int BH, int run, uint32_t* __restrict__ amax) {
+            int BH, uint32_t* __restrict__ amax) {
   const int bh = gridDim.y - 1 - blockIdx.y + grid_dep_wait(), which = 1 - blockIdx.z;
   const Strides s = which ? sk : sq;
   const __nv_bfloat16* base = (which ? k : q) + (long long)(bh / H) * s.b + (long long)(bh % H) * s.h;
-  const int lo = (gridDim.x - 1 - blockIdx.x) * run * 128, hi = min(lo + run * 128, N);
+  const int lo = (gridDim.x - 1 - blockIdx.x) * 128, hi = min(lo + 128, N);
   const int row = threadIdx.x >> 4, vec = threadIdx.x & 15;   // 16 vectors of 8 elements per token, 16 tokens at a time
   uint4 u[4];
   auto load = [&](int t0) {
@@ -170,9 +170,8 @@ int launch_quantize4(const Dims& m, const sva_problem_t* p, const void* q, const
   uint32_t* amax = static_cast<uint32_t*>(ws);
   if (cudaMemsetAsync(amax, 0, (size_t)2 * BH * sizeof(uint32_t), st) != cudaSuccess) return SVA_ERR_CUDA;
   const Strides sq = make_strides(p->q_stride), sk = make_strides(p->k_stride);
-  const int run = blocks_per_cta(2LL * m.R, 32 << 10);
-  const int rc = launch_dep(amax_kernel, dim3((m.Nb + run - 1) / run, BH, 2), Q4_THREADS, 0, st, (const __nv_bfloat16*)q,
-                            (const __nv_bfloat16*)k, sq, sk, m.H, m.N, BH, run, amax);
+  const int rc = launch_dep(amax_kernel, dim3(m.Nb, BH, 2), Q4_THREADS, 0, st, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, sq, sk, m.H,
+                            m.N, BH, amax);
   if (rc != SVA_OK) return rc;
   return launch_dep(quantize4_kernel, dim3(m.Nb, BH, 2), Q4_THREADS, 0, st, (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, sq, sk,
                     m.H, m.N, m.Nb, BH, amax, (uint8_t*)q4, (uint8_t*)k4, (uint8_t*)q_sf, (uint8_t*)k_sf, q_g, k_g);
