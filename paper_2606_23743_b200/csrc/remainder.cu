@@ -247,10 +247,12 @@ inline Plan plan(int Nb, int chunks) {
   p.smem = 1024 + w + p.stages * stage + OUT_STAGE;
   return p;
 }
-// Runs of n-tiles per group of I-tiles: the number that gives the shortest longest SM (a run costs about two n-tiles to begin).
+// Runs of n-tiles per group of I-tiles: the number that gives the shortest longest SM of the B200's 148 (a run costs about two n-tiles to begin), up to
+// an n-tile each: one or two groups -- a call of one or two heads -- would leave most SMs idle otherwise.  The whole call, us, at most 32 runs / so: 1 head x
+// 4 blocks of 128 24.3 / 22.4, x 64 28.0 / 25.6, x 129 42.2 / 37.1, x 256 77.9 / 70.0, 2 heads x 64 29.7 / 28.3, 3 x 64 38.9 / 38.2.
 inline int runs(int groups) {
   int best = 1, cost = 1 << 30;
-  for (int r = 1; r <= 32; ++r) {
+  for (int r = 1; r <= rem::D; ++r) {
     const int c = (groups * r + 147) / 148 * ((rem::D + r - 1) / r + 2);
     if (c < cost) { cost = c; best = r; }
   }
