@@ -1,8 +1,8 @@
 /*
  * sva_debug.h -- test and tuning aids exported by libsva.so next to the public calls of sva.h.
  *
- * Unlike everything in sva.h these three calls keep PROCESS-GLOBAL state (two host variables and one device
- * variable per loaded library): a setting stays in force for every later attention launch of the process
+ * Unlike everything in sva.h these three calls keep PROCESS-GLOBAL state (host variables and one device
+ * variable per loaded library): a setting stays in force for every later launch of the process
  * until it is set back.  They are meant for single-threaded test and bench programs.  The paper has no
  * counterpart.
  */
@@ -22,11 +22,13 @@ extern "C" {
 void sva_debug_set_prof_buffer(void* buf);
 
 /*
- * Kernel behaviour switches for the next attention launches (0 = normal operation).
+ * Kernel behaviour switches for the next launches (0 = normal operation).
  *   bit 4: test aid: the K producer withholds a row's tiles after the first, so that a bounded pipeline wait
  *          runs out and the kernel takes its give-up path (SVA_DEV_TIMEOUT) -- nothing faults or hangs.
  *   bit 5: measurement aid: the one-call forms (but the 4-bit one) read a transposed copy of V that they make first, as the two-step form
  *          does, instead of V where it lies; they then need sva_attn_workspace_bytes() (the remainder: its own query, asked meanwhile);
+ *   bit 6: test aid: the one-launch routing of small problems asks for clusters of 32 CTAs, which no device holds, so that the
+ *          call goes the way it goes in a partition of the device that is too small for its clusters;
  *   bit 7: test aid: the remainder call masks the kept blocks of a block-mean tile by looking them up in the CSR
  *          (the form that serves more than 1024 key blocks) even where the kept-block bit masks would serve.
  */

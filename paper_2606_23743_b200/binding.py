@@ -318,7 +318,7 @@ def debug_set_prof_buffer(buf) -> None:
 
 
 def debug_set_mode(bits: int) -> None:
-    """Kernel behaviour switches of later attention launches (include/sva_debug.h); 0 = normal."""
+    """Kernel behaviour switches of later launches (include/sva_debug.h); 0 = normal."""
     lib().sva_debug_set_mode(int(bits))
 
 

@@ -5,6 +5,7 @@ namespace sva {
 
 void ts_set_prof_buffer(void* p);
 void ts_set_debug_mode(int v);
+void route_set_debug_mode(int v);
 int ts_set_wait_limit(long long cycles);
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
@@ -388,8 +389,12 @@ const char* sva_status_string(int status) {
    CTA's cycle count of the next attention launches; NULL = off */
 void sva_debug_set_prof_buffer(void* p) { ts_set_prof_buffer(p); }
 /* bit 4 (test aid) withholds a row's K tiles after the first so that a bounded wait runs out; bit 5 (measurement aid) has the one-call
-   forms read a transposed copy of V; bit 7 (test aid) has the remainder look kept blocks up in the CSR */
-void sva_debug_set_mode(int v) { ts_set_debug_mode(v); }
+   forms read a transposed copy of V; bit 6 (test aid) has routing ask for clusters that no device holds; bit 7 (test aid) has the
+   remainder look kept blocks up in the CSR */
+void sva_debug_set_mode(int v) {
+  ts_set_debug_mode(v);
+  route_set_debug_mode(v);
+}
 /* test aid: cycles a device-side wait may last before the CTA gives up (<= 0 restores the default) */
 int sva_debug_set_wait_limit(long long cycles) { return ts_set_wait_limit(cycles); }
 

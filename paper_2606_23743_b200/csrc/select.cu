@@ -812,6 +812,9 @@ static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, c
 // Where the cluster kernel routes.  Up to 14 heads each of its CTAs has an SM to itself (15 or more clusters of eight SMs do not fit at once), and up to
 // 16 blocks a CTA pools in one round.  Beyond that pooling over all SMs and route_means_kernel are faster (us, them / a cluster): 12 heads x 20 blocks
 // of 128 x 128 7.3 / 7.9, 12 x 44 9.8 / 12.2, 16 x 16 7.2 / 8.0 (with two CTAs per SM), 6 x 64 8.5 / 13.4.
+// Where the device cannot hold such a cluster -- the largest cluster shrinks in a partition of too few SMs -- those two serve these sizes too.
+static int g_debug_route = 0;
+void route_set_debug_mode(int v) { g_debug_route = v; }
 static bool route_in_cluster(const Dims& m) { return m.Nb <= 16 && m.B * m.H <= 14; }
 template <int D, int ELEM_BYTES, bool MASS>
 static int launch_route(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale, const float* k_scale,
@@ -820,8 +823,26 @@ static int launch_route(const Dims& m, const sva_problem_t* p, const void* q, co
   auto kern = route_cluster_kernel<D, ELEM_BYTES, MASS>;
   using Sm = RcSmem<D, ELEM_BYTES>;
   constexpr int smem = (int)sizeof(Sm) + 4 * ((RC_MAX_NB + RC_ROWS) * Sm::LD + 2 * RC_ROWS * RC_MAX_NB);
+  const int ctas = g_debug_route & 64 ? 32 : RC_CTAS;                  // (test aid: more CTAs than any device takes)
+  auto fits = [&] {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = (unsigned)ctas;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(ctas);
+    cfg.blockDim = dim3(RC_TEAMS * RC_TEAM);
+    cfg.dynamicSmemBytes = smem;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    int n = 0;
+    const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
+                    cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0;
+    if (!ok) (void)cudaGetLastError();
+    return ok;
+  };
   static DeviceOnce once;
-  const int rc = once.run([&] { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess; });
+  const int rc = ctas == RC_CTAS ? once.run(fits) : fits() ? (int)SVA_OK : (int)SVA_ERR_CUDA;
   if (rc != SVA_OK) return rc;
   return launch_dep_cluster(RC_CTAS, kern, m.B * m.H * RC_CTAS, RC_TEAMS * RC_TEAM, smem, st, (const uint8_t*)q, (const uint8_t*)k,
                             make_strides(p->q_stride), make_strides(p->k_stride), q_scale, k_scale, m.H, m.N, m.block, m.scale, sp,
@@ -864,7 +885,7 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
     };
     auto by_mass = [&](auto elem_tag) { return s->mode == 1 ? route(elem_tag, std::true_type{}) : route(elem_tag, std::false_type{}); };
     rc = m.fp8 ? by_mass(std::integral_constant<int, 1>{}) : by_mass(std::integral_constant<int, 2>{});
-    return rc != SVA_OK ? rc : csr();
+    if (rc == SVA_OK) return csr();                              // (else: no room for a cluster, nothing was launched)
   }
   if (!qbar_in && (rc = launch_pool_d<D>(m, p, q, k, q_scale, k_scale, qbar, kbar, st)) != SVA_OK) return rc;
   if (route_by_rank(m, s->mode)) {

@@ -332,3 +332,36 @@ def test_heads_at_the_end_of_counting_ranks(mode, k, window, H, Nb, by_rank):
     parts = [route(h, min(h + 100, H)) for h in range(0, H, 100)]
     assert all(p[2] for p in parts)
     assert torch.equal(counts, torch.cat([p[0] for p in parts])) and torch.equal(blocks, torch.cat([p[1] for p in parts]))
+
+
+@pytest.mark.parametrize("H,Nb,block,d,fp8", [(2, 16, 64, 64, False), (14, 16, 128, 128, False), (1, 1, 128, 128, False), (3, 9, 64, 128, True)])
+@pytest.mark.parametrize("mode", [0, 1])
+def test_small_problems_where_no_cluster_fits(H, Nb, block, d, fp8, mode):
+    """A partition of the device can be too small for the clusters of the one-launch routing (the test switch asks for larger ones than
+    exist): the call then takes other kernels and returns the same."""
+    N = Nb * block - 5
+    g = torch.Generator(device="cuda").manual_seed(Nb)
+    q, k = torch.randn(2, 1, H, N, d, generator=g, device="cuda").to(torch.bfloat16)
+    scales = [None, None]
+    if fp8:
+        q, k = (x.to(torch.float8_e4m3fn).view(torch.uint8) for x in (q, k))
+        scales = [torch.rand(1, H, Nb, generator=g, device="cuda") + 0.5 for _ in range(2)]
+    p, s = B.make_problem(q, k, None, None, N, block, 0.0, fp8), B.make_select(mode, max(1, Nb // 3), 0.6)
+
+    def route(entry):
+        rp = torch.full((H * Nb + 1,), -7, dtype=torch.int32, device="cuda")
+        ci = torch.full((B.select_max_nnz(p, s),), -7, dtype=torch.int32, device="cuda")
+        sc = torch.full((1, H, Nb, Nb), -7.0, device="cuda")
+        ws = torch.full((B.select_workspace_bytes(p, s),), 255, dtype=torch.uint8, device="cuda")
+        entry(p, s, q, k, rp, ci, *((ws,) if entry is B.block_select else ()), *scales, sc)
+        torch.cuda.synchronize()
+        return rp, ci, sc
+
+    want = route(B.block_select)
+    try:
+        B.debug_set_mode(64)
+        got = [route(B.block_select), route(B.block_select_noalloc)]
+    finally:
+        B.debug_set_mode(0)
+    for x in got + [route(B.block_select)]:
+        assert all(torch.equal(a, b) for a, b in zip(want, x))
