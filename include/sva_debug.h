@@ -1,8 +1,8 @@
 /*
  * sva_debug.h -- test and tuning aids exported by libsva.so next to the public calls of sva.h.
  *
- * Unlike everything in sva.h these three calls keep PROCESS-GLOBAL state (host variables and one device
- * variable per loaded library): a setting stays in force for every later launch of the process
+ * Unlike everything in sva.h these three calls keep PROCESS-GLOBAL state (host variables and two device
+ * variables per loaded library): a setting stays in force for every later launch of the process
  * until it is set back.  They are meant for single-threaded test and bench programs.  The paper has no
  * counterpart.
  */
@@ -30,13 +30,15 @@ void sva_debug_set_prof_buffer(void* buf);
  *   bit 6: test aid: the one-launch routing of small problems asks for clusters of 32 CTAs, which no device holds, so that the
  *          call goes the way it goes in a partition of the device that is too small for its clusters;
  *   bit 7: test aid: the remainder call masks the kept blocks of a block-mean tile by looking them up in the CSR
- *          (the form that serves more than 1024 key blocks) even where the kept-block bit masks would serve.
+ *          (the form that serves more than 1024 key blocks) even where the kept-block bit masks would serve;
+ *   bit 8: test aid: the kernel of the first-order term's block covariances withholds a part of its V tile, and
+ *   bit 9: the one that adds them up withholds every column tile of a CTA after its first, so that bounded waits run out.
  */
 void sva_debug_set_mode(int bits);
 
 /*
  * Test aid: the number of SM cycles a device-side wait may last before its CTA gives up (default 3e9, at most 4e9: larger
- * values count as that; cycles <= 0 restores the default).  Synchronous (a small host-to-device copy on the current device).
+ * values count as that; cycles <= 0 restores the default).  Synchronous (two small host-to-device copies on the current device).
  * Returns 0 on success.
  */
 int sva_debug_set_wait_limit(long long cycles);

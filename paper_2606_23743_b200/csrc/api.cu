@@ -6,7 +6,9 @@ namespace sva {
 void ts_set_prof_buffer(void* p);
 void ts_set_debug_mode(int v);
 void route_set_debug_mode(int v);
+void rem_set_debug_mode(int v);
 int ts_set_wait_limit(long long cycles);
+int rem_set_wait_limit(long long cycles);
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
@@ -390,12 +392,13 @@ const char* sva_status_string(int status) {
 void sva_debug_set_prof_buffer(void* p) { ts_set_prof_buffer(p); }
 /* bit 4 (test aid) withholds a row's K tiles after the first so that a bounded wait runs out; bit 5 (measurement aid) has the one-call
    forms read a transposed copy of V; bit 6 (test aid) has routing ask for clusters that no device holds; bit 7 (test aid) has the
-   remainder look kept blocks up in the CSR */
+   remainder look kept blocks up in the CSR; bits 8 and 9 (test aids) withhold loads of the first-order term's kernels */
 void sva_debug_set_mode(int v) {
   ts_set_debug_mode(v);
   route_set_debug_mode(v);
+  rem_set_debug_mode(v);
 }
 /* test aid: cycles a device-side wait may last before the CTA gives up (<= 0 restores the default) */
-int sva_debug_set_wait_limit(long long cycles) { return ts_set_wait_limit(cycles); }
+int sva_debug_set_wait_limit(long long cycles) { return ts_set_wait_limit(cycles) | rem_set_wait_limit(cycles); }
 
 }  // extern "C"

@@ -1743,9 +1743,6 @@ int launch_attn_ts_fp4(const Dims& m, const sva_problem_t* p, const void* q4, co
 
 void ts_set_prof_buffer(void* p) { g_prof_ts = (long long*)p; }
 void ts_set_debug_mode(int v) { g_debug_ts = v; }
-int ts_set_wait_limit(long long cycles) {
-  const uint32_t limit = cycles <= 0 ? WAIT_LIMIT_CYCLES : (uint32_t)(cycles < 4000000000LL ? cycles : 4000000000LL);
-  return cudaMemcpyToSymbol(g_wait_limit, &limit, sizeof(limit)) == cudaSuccess ? 0 : 1;
-}
+int ts_set_wait_limit(long long cycles) { return set_wait_limit(cycles); }
 
 }  // namespace sva

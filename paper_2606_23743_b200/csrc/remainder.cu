@@ -52,7 +52,7 @@ static __device__ __forceinline__ void stage_row(uint8_t* tile, int row, int c0,
 __global__ void __launch_bounds__(128)
 cov_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ct,
            int H, int N, int block, int Nb, __nv_bfloat16* __restrict__ mean_k, __nv_bfloat16* __restrict__ mean_v, int Nbp,
-           int32_t* __restrict__ row_counter, int32_t* __restrict__ status) {
+           int32_t* __restrict__ row_counter, int debug, int32_t* __restrict__ status) {
   using namespace rem;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -94,7 +94,7 @@ cov_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUt
     tma_load_4d(sbase, &tm_k, bar_full, 0, J * block, hh, bb);
     tma_load_4d(sbase + panel, &tm_k, bar_full, 64, J * block, hh, bb);
     tma_load_4d(sbase + TILE, &tm_v, bar_full, 0, J * block, hh, bb);
-    tma_load_4d(sbase + TILE + panel, &tm_v, bar_full, 64, J * block, hh, bb);
+    if (!(debug & 256)) tma_load_4d(sbase + TILE + panel, &tm_v, bar_full, 64, J * block, hh, bb);      // (test aid: the wait runs out)
   }
   bool ok = wait_or_report(bar_full, 0u, abort_flag, status);
   ok = __syncthreads_and(ok);                                   // (every thread or none goes on: there are barriers below)
@@ -268,7 +268,7 @@ static __device__ __forceinline__ bool epilogue_all(bool ok) {
 }
 __global__ void __launch_bounds__(192, 1)
 aggregate_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_c, const __grid_constant__ CUtensorMap tm_at,
-                 int Nb, int chunks, int tiles_per_cta, int resident, int stages, int32_t* __restrict__ status) {
+                 int Nb, int chunks, int tiles_per_cta, int resident, int stages, int debug, int32_t* __restrict__ status) {
   using namespace rem;
   using namespace agg;
   extern __shared__ uint8_t smem_raw[];
@@ -313,7 +313,8 @@ aggregate_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
       }
       int st = 0;
       uint32_t ph = 0;
-      for (int nt = nt0; nt < nt1 && ok; ++nt)
+      for (int nt = nt0; nt < nt1 && ok; ++nt) {
+        if ((debug & 512) && nt > nt0) break;                              // test aid: starve the ring so that waits run out
         for (int ch = 0; ch < chunks; ++ch) {
           ok = wait_or_report(bar_empty + 8 * st, ph ^ 1u, abort_flag, status);
           if (!ok) break;
@@ -324,6 +325,7 @@ aggregate_kernel(const __grid_constant__ CUtensorMap tm_w, const __grid_constant
           if (!resident) tma_load_3d(dst + 2 * B_PANEL, &tm_w, bar, ch * 64, it0 * 128, bh);
           if (++st == stages) { st = 0; ph ^= 1u; }
         }
+      }
     }
   } else if (warp == 5) {
     if (lane == 0) {
@@ -438,6 +440,10 @@ size_t remainder1_bytes(const Dims& m) {
   return 2 * mats + al256((size_t)m.R * Nbw * 2) + al256((size_t)m.R * 4);
 }
 
+static int g_debug_rem = 0;
+void rem_set_debug_mode(int v) { g_debug_rem = v; }
+int rem_set_wait_limit(long long cycles) { return set_wait_limit(cycles); }
+
 // Fills `buf` (remainder1_bytes) from K, V, the routing's score matrix and the CSR.  *at_out / *mu_out: where the
 // attention kernel finds A_I^T ([R][128 e][128 c] bf16) and mu_I.
 // natural: A_I itself ([R][128 c][128 e]) instead of its transpose -- for an attention kernel that takes its "V" tiles
@@ -486,12 +492,12 @@ int launch_remainder1(const Dims& m, const sva_problem_t* p, const void* k, cons
       cudaFuncSetAttribute(aggregate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess)
     return SVA_ERR_CUDA;
   if ((rc = launch_dep(cov_kernel, dim3(m.Nb, m.B * m.H), 128, smem_cov, st, natural ? tv : tk, natural ? tk : tv, tco, m.H, m.N, m.block,
-                       m.Nb, natural ? v_mean : k_mean, natural ? k_mean : v_mean, Nbp, row_counter, status)) != SVA_OK)
+                       m.Nb, natural ? v_mean : k_mean, natural ? k_mean : v_mean, Nbp, row_counter, g_debug_rem, status)) != SVA_OK)
     return rc;
   if ((rc = launch_dep(weights_kernel, (m.R + 7) / 8, 256, 0, st, scores, row_ptr, col_idx, m.R, m.Nb, Nbw, w, mu)) != SVA_OK) return rc;
   const int groups = ((m.Nb + 127) / 128 + ap.tiles - 1) / ap.tiles;
   if ((rc = launch_dep(aggregate_kernel, dim3(agg::runs(groups * m.B * m.H), groups, m.B * m.H), 192, ap.smem, st, tw, tc, ta, m.Nb, chunks, ap.tiles,
-                       ap.resident, ap.stages, status)) != SVA_OK)
+                       ap.resident, ap.stages, g_debug_rem, status)) != SVA_OK)
     return rc;
   *at_out = at;
   *mu_out = mu;

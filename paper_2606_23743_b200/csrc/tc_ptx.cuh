@@ -10,7 +10,11 @@ namespace sva {
 static constexpr int BS = 128;                 // rows per tile (queries and keys)
 static constexpr uint32_t WAIT_LIMIT_CYCLES = 3000000000u;
 // cycles a wait may last before the CTA gives up (read only on the slow path of a wait)
-static __device__ uint32_t g_wait_limit = WAIT_LIMIT_CYCLES;   // one copy per translation unit
+static __device__ uint32_t g_wait_limit = WAIT_LIMIT_CYCLES;   // one copy per translation unit, each of which has a setter
+static inline int set_wait_limit(long long cycles) {
+  const uint32_t limit = cycles <= 0 ? WAIT_LIMIT_CYCLES : (uint32_t)(cycles < 4000000000LL ? cycles : 4000000000LL);
+  return cudaMemcpyToSymbol(g_wait_limit, &limit, sizeof(limit)) == cudaSuccess ? 0 : 1;
+}
 
 // ------------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }

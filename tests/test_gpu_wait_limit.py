@@ -1,5 +1,7 @@
-"""The give-up path of the attention kernel in each of its forms: a row's K tiles after the first are withheld (test switch), the
-bounded waits run out, and every role leaves.  Nothing faults or hangs."""
+"""The give-up paths: in each form of the attention kernel a row's K tiles after the first are withheld (test switch), in the kernels of the
+remainder's first-order term some of their loads; the bounded waits run out, and every role leaves.  Nothing faults or hangs."""
+import time
+
 import pytest
 import torch
 
@@ -49,4 +51,29 @@ def test_a_starved_row_is_reported_and_not_stored(form, block):
     assert st == B.SVA_DEV_TIMEOUT
     assert (o == 7.0).all() and (lse == 7.0).all()                            # (as the caller left them)
     o, lse, st = call()                                                       # the context and the next call are intact
+    assert st == 0 and torch.equal(o, want) and torch.equal(lse, want_lse)
+
+
+@pytest.mark.parametrize("block", [128, 64])
+@pytest.mark.parametrize("switch", [256, 512], ids=["covariances", "aggregation"])
+def test_starved_first_order_kernels_give_up(switch, block):
+    """A CTA of either kernel whose load never arrives reports it and leaves, with stores of its first tiles under way, in the time that the
+    limit allows (the default limit is thirty times that)."""
+    w = shrink(WORKLOADS["medium"], H=4, T=2, block=block, k=6)               # (four heads: several column tiles per CTA)
+    (q, k, v), _ = U.host_inputs(w)
+    q, k, v = U.dev(q), U.dev(k), U.dev(v)
+    rp, ci, scores = U.gpu_select(w, q, k, want_scores=True)
+    want, want_lse, st = gpu_remainder(w, q, k, v, rp, ci, 1, scores=scores)
+    assert st == 0
+    try:
+        B.debug_set_wait_limit(100_000_000)                                   # about 50 ms
+        B.debug_set_mode(switch)
+        t0 = time.monotonic()
+        _, _, st = gpu_remainder(w, q, k, v, rp, ci, 1, scores=scores)
+        took = time.monotonic() - t0
+    finally:
+        B.debug_set_mode(0)
+        B.debug_set_wait_limit(0)
+    assert st == B.SVA_DEV_TIMEOUT and 0.04 < took < 1.0, took
+    o, lse, st = gpu_remainder(w, q, k, v, rp, ci, 1, scores=scores)
     assert st == 0 and torch.equal(o, want) and torch.equal(lse, want_lse)
