@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <mutex>
+
 #include "../../include/sva.h"
 
 namespace sva {
@@ -103,6 +105,23 @@ template <typename... P, typename... A>
 inline int launch_dep(void (*kern)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, A&&... args) {
   return launch_dep_cluster(1, kern, grid, block, smem, st, static_cast<A&&>(args)...);
 }
+
+// Function attributes of a kernel, set once per device and instantiation instead of per call.
+struct DeviceOnce {
+  std::mutex mutex;
+  bool done[64] = {false};
+  template <typename F>
+  int run(F set) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SVA_ERR_CUDA;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (!done[dev]) {
+      if (!set()) return SVA_ERR_CUDA;
+      done[dev] = true;
+    }
+    return SVA_OK;
+  }
+};
 
 // Consecutive token blocks per CTA of the kernels that stream a tensor's blocks (`blocks` of them over all heads and tensors, of
 // block_bytes) with the next block's loads in flight while they reduce: runs of up to 128 KB, as long as the CTAs' first loads together still

@@ -488,9 +488,12 @@ int launch_remainder1(const Dims& m, const sva_problem_t* p, const void* k, cons
   }
   const int smem_cov = 2 * rem::TILE + 1024, chunks = Nbw / 64;
   const agg::Plan ap = agg::plan(m.Nb, chunks);
-  if (cudaFuncSetAttribute(cov_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_cov) != cudaSuccess ||
-      cudaFuncSetAttribute(aggregate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) != cudaSuccess)
-    return SVA_ERR_CUDA;
+  static DeviceOnce once;
+  if ((rc = once.run([&] {
+         return cudaFuncSetAttribute(cov_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_cov) == cudaSuccess &&
+                cudaFuncSetAttribute(aggregate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 226 * 1024) == cudaSuccess;
+       })) != SVA_OK)
+    return rc;
   if ((rc = launch_dep(cov_kernel, dim3(m.Nb, m.B * m.H), 128, smem_cov, st, natural ? tv : tk, natural ? tk : tv, tco, m.H, m.N, m.block,
                        m.Nb, natural ? v_mean : k_mean, natural ? k_mean : v_mean, Nbp, row_counter, g_debug_rem, status)) != SVA_OK)
     return rc;

@@ -471,23 +471,6 @@ block_scores_kernel(const float* __restrict__ qbar, const float* __restrict__ kb
   }
 }
 
-// Function attributes of a kernel, set once per device and instantiation instead of per call.
-struct DeviceOnce {
-  std::mutex mutex;
-  bool done[64] = {false};
-  template <typename F>
-  int run(F set) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return SVA_ERR_CUDA;
-    std::lock_guard<std::mutex> lock(mutex);
-    if (!done[dev]) {
-      if (!set()) return SVA_ERR_CUDA;
-      done[dev] = true;
-    }
-    return SVA_OK;
-  }
-};
-
 template <int D, int PQ, int PK, int TY>
 static int launch_scores(const float* qbar, const float* kbar, int Nb, int heads, float scale, float* scores, cudaStream_t st) {
   auto kern = block_scores_kernel<D, PQ, PK, TY>;
