@@ -508,11 +508,13 @@ select_rows_kernel(const float* __restrict__ scores, SelParams p, int32_t* __res
 // its share of the head's blocks of Q and K (a team of 256 threads per block), writes a key mean into the shared memory of all eight,
 // and then scores and selects its own query blocks.  Sums run in the orders of pool_kernel and block_scores_kernel, so lists and
 // scores are the same bytes.
-// Bound by latency: the launch, the cluster's barriers (about 0.5 us each), a pooling round of a block per team (about 1 100 cycles of loads, sums
+// Bound by latency: the launch, the cluster's barriers (about 0.5 us each), the pooling of a block per team (about 1 100 cycles of loads, sums
 // and reduction), and the score and selection phase of a warp per row.  Microseconds of a routing call (top-k), pool_kernel and
 // route_means_kernel / this one: 2 heads x 16 blocks of 64 x 64 7.3 / 5.3, of 128 x 128 7.35 / 6.3; 1 x 8 7.3 / 5.5.
-static constexpr int RC_CTAS = 8, RC_TEAMS = 4, RC_TEAM = 256, RC_ITEMS = 1, RC_MAX_NB = 32 * RC_ITEMS;
-static constexpr int RC_ROWS = RC_MAX_NB / RC_CTAS;                         // query blocks per CTA at most (a multiple of 4)
+static constexpr int RC_CTAS = 8, RC_TEAMS = 4, RC_TEAM = 256, RC_MAX_NB = 16;
+static constexpr int RC_ROWS = RC_MAX_NB / RC_CTAS;                         // query blocks per CTA at most
+static constexpr int RC_KEYS = 32;                                          // rows of the panel of key means, one per lane
+static_assert(2 * RC_ROWS <= RC_TEAMS && RC_MAX_NB <= RC_KEYS, "a team per block of Q and K");
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
@@ -597,42 +599,39 @@ route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ 
                      int32_t* __restrict__ tmp_idx, int32_t* __restrict__ counts, int R) {
   using Sm = RcSmem<D, ELEM_BYTES>;
   constexpr int VPR = Sm::VPR, GROUPS = Sm::GROUPS, EPV = Sm::EPV, LD = Sm::LD, NV = 128 / GROUPS;     // NV: vectors per thread and block
-  constexpr int ITEMS = RC_ITEMS;
   extern __shared__ __align__(16) uint8_t rc_smem[];
   Sm& sm = *reinterpret_cast<Sm*>(rc_smem);
-  float* ks = reinterpret_cast<float*>(rc_smem + sizeof(Sm));          // [32 * ITEMS][LD] key means of the head
-  float* qm = ks + 32 * ITEMS * LD;                                    // [rows][LD] means of my query blocks
-  uint32_t* keys = reinterpret_cast<uint32_t*>(qm + RC_ROWS * LD);      // [rows][32 * ITEMS] scores as keys
-  uint32_t* wgts = keys + RC_ROWS * 32 * ITEMS;                 // ... and their weights
+  float* ks = reinterpret_cast<float*>(rc_smem + sizeof(Sm));          // [32][LD] key means of the head
+  float* qm = ks + RC_KEYS * LD;                                       // [rows][LD] means of my query blocks
+  uint32_t* keys = reinterpret_cast<uint32_t*>(qm + RC_ROWS * LD);      // [rows][32] scores as keys
+  uint32_t* wgts = keys + RC_ROWS * RC_KEYS;                            // ... and their weights
   const int Nb = p.Nb, per = (Nb + RC_CTAS - 1) / RC_CTAS;
   cluster_arrive();                        // (the CTAs of the cluster have started: they may be written to)
   const int rank = blockIdx.x % RC_CTAS, bh = blockIdx.x / RC_CTAS + grid_dep_wait();
   const int b = bh / H, h = bh % H, I0 = rank * per, mine = max(0, min(per, Nb - I0));
   const int team = threadIdx.x / RC_TEAM, tt = threadIdx.x % RC_TEAM, vec = tt % VPR, grp = tt / VPR;
 
-  // ---- pooling: items 0 .. mine-1 are blocks of Q, the rest blocks of K; the next item's loads are in flight behind a reduction
+  // ---- pooling: teams 0 .. mine-1 take a block of Q each, the next ones a block of K
+  const bool pools = team < 2 * mine;
+  const int which = team >= mine, li = which ? team - mine : team, I = I0 + li;
+  const int lo = I * block, cnt = pools ? min(block, N - lo) : 0;
   uint4 u[NV];
-  auto load = [&](int item) {
-    const int which = item >= mine, I = I0 + (which ? item - mine : item);
+  {
     const Strides s = which ? sk : sq;
-    const int lo = I * block, cnt = item < 2 * mine ? min(block, N - lo) : 0;
     const uint8_t* base = (which ? k : q) + ((long long)b * s.b + (long long)h * s.h + (long long)(lo + grp) * s.n) * ELEM_BYTES;
 #pragma unroll
     for (int j = 0; j < NV; ++j) {
       u[j] = make_uint4(0, 0, 0, 0);
       if (grp + j * GROUPS < cnt) u[j] = __ldg(reinterpret_cast<const uint4*>(base + (long long)(j * GROUPS) * s.n * ELEM_BYTES) + vec);
     }
-  };
-  load(team);
+  }
   cluster_wait();
-  for (int item = team; item < 2 * mine; item += RC_TEAMS) {
-    const int which = item >= mine, li = which ? item - mine : item, I = I0 + li;
+  if (pools) {
     uint64_t acc[EPV / 2];
 #pragma unroll
     for (int e = 0; e < EPV / 2; ++e) acc[e] = 0ull;
 #pragma unroll
     for (int j = 0; j < NV; ++j) add_vector<ELEM_BYTES>(u[j], acc);
-    load(item + RC_TEAMS);
     float* part = sm.part[team];
 #pragma unroll
     for (int e = 0; e < EPV / 2; ++e)
@@ -642,7 +641,7 @@ route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ 
       float sum = 0.f;
 #pragma unroll 8
       for (int g = 0; g < GROUPS; ++g) sum += part[(tt % EPV) * Sm::PART + g * VPR + tt / EPV];       // fixed order
-      float mean = sum / (float)min(block, N - I * block);
+      float mean = sum / (float)cnt;
       if (ELEM_BYTES == 1) mean *= (which ? k_scale : q_scale)[(long long)bh * Nb + I];
       if (which) {
         const uint32_t dst = smem_addr(ks + I * LD + tt);
@@ -652,13 +651,12 @@ route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ 
         qm[li * LD + tt] = mean;
       }
     }
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(RC_TEAM) : "memory");
   }
   grid_dep_launch();
   cluster_arrive();
   cluster_wait();
 
-  score_and_select<D, 2, ITEMS, MASS>(ks, qm, keys, wgts, mine, I0, bh, scale, p, scores, row_ptr, col_idx, tmp_idx, counts, R);
+  score_and_select<D, RC_ROWS, 1, MASS>(ks, qm, keys, wgts, mine, I0, bh, scale, p, scores, row_ptr, col_idx, tmp_idx, counts, R);
 }
 
 // The same tail for block means that are at hand (a pooling or prologue kernel has written them): scores and selection of eight query
@@ -793,19 +791,19 @@ static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, c
 }
 
 // Where the cluster kernel routes.  Up to 14 heads each of its CTAs has an SM to itself (15 or more clusters of eight SMs do not fit at once), and up to
-// 16 blocks a CTA pools in one round.  Beyond that pooling over all SMs and route_means_kernel are faster (us, them / a cluster): 12 heads x 20 blocks
+// 16 blocks (RC_MAX_NB) a CTA pools in one round.  Beyond that pooling over all SMs and route_means_kernel are faster (us, them / a cluster): 12 heads x 20 blocks
 // of 128 x 128 7.3 / 7.9, 12 x 44 9.8 / 12.2, 16 x 16 7.2 / 8.0 (with two CTAs per SM), 6 x 64 8.5 / 13.4.
 // Where the device cannot hold such a cluster -- the largest cluster shrinks in a partition of too few SMs -- those two serve these sizes too.
 static int g_debug_route = 0;
 void route_set_debug_mode(int v) { g_debug_route = v; }
-static bool route_in_cluster(const Dims& m) { return m.Nb <= 16 && m.B * m.H <= 14; }
+static bool route_in_cluster(const Dims& m) { return m.Nb <= RC_MAX_NB && m.B * m.H <= 14; }
 template <int D, int ELEM_BYTES, bool MASS>
 static int launch_route(const Dims& m, const sva_problem_t* p, const void* q, const void* k, const float* q_scale, const float* k_scale,
                         const SelParams& sp, float* scores, int32_t* row_ptr, int32_t* col_idx, int32_t* tmp_idx, int32_t* counts,
                         cudaStream_t st) {
   auto kern = route_cluster_kernel<D, ELEM_BYTES, MASS>;
   using Sm = RcSmem<D, ELEM_BYTES>;
-  constexpr int smem = (int)sizeof(Sm) + 4 * ((RC_MAX_NB + RC_ROWS) * Sm::LD + 2 * RC_ROWS * RC_MAX_NB);
+  constexpr int smem = (int)sizeof(Sm) + 4 * ((RC_KEYS + RC_ROWS) * Sm::LD + 2 * RC_ROWS * RC_KEYS);
   const int ctas = g_debug_route & 64 ? 32 : RC_CTAS;                  // (test aid: more CTAs than any device takes)
   auto fits = [&] {
     cudaLaunchAttribute attr;
