@@ -359,8 +359,18 @@ def test_more_than_1024_key_blocks(order):
 @pytest.mark.parametrize("block,nb", [(128, 64), (64, 128), (64, 129), (64, 256), (64, 257), (64, 512), (64, 513)])
 def test_first_order_aggregation_at_the_edges_of_its_forms(block, nb):
     """The sums over A_I keep the weights of one I-tile up to 128 key blocks, of two up to 256, of one up to 512 and of none beyond that."""
+    _check_first_order(block, nb, 2)
+
+
+@pytest.mark.parametrize("H,nb", [(1, 3), (1, 64), (1, 129), (1, 300), (3, 64), (3, 129), (5, 30)])
+def test_first_order_aggregation_of_few_heads(H, nb):
+    """Few heads spread their 128 column tiles over more CTAs, down to a tile each; 128 need not be a multiple of the runs."""
+    _check_first_order(64, nb, H)
+
+
+def _check_first_order(block, nb, H):
     from paper_2606_23743_b200.workloads import bf16_bits
-    w = shrink(WORKLOADS["medium"], H=2, T=1, Hg=nb, Wg=block, block=block, k=max(1, nb // 16))
+    w = shrink(WORKLOADS["medium"], H=H, T=1, Hg=nb, Wg=block, block=block, k=max(1, nb // 16))
     (q, k, v), (qb, kb, _) = U.host_inputs(w)
     v = (v.float() + 4.0 * k.float()).to(torch.bfloat16)                     # (the first-order term is large: see above)
     vb = bf16_bits(v)
@@ -368,8 +378,8 @@ def test_first_order_aggregation_at_the_edges_of_its_forms(block, nb):
     rp, ci, scores = U.gpu_select(w, qd, kd, want_scores=True)
     o, lse, st = gpu_remainder(w, qd, kd, vd, rp, ci, 1, scores=scores)
     assert st == 0
-    rows = [0, min(127, nb - 1), nb - 1, nb, nb + nb // 2, 2 * nb - 1]       # (of both heads)
+    rows = sorted({0, min(127, nb - 1), nb - 1, (H - 1) * nb, (H - 1) * nb + nb // 2, H * nb - 1})      # (of the first head and the last)
     o_ref, l_ref = oracle.attn_remainder_rows(qb, kb, vb, w.N, w.block, w.scale, rp.cpu().numpy(), ci.cpu().numpy(), rows, order=1,
                                               stats="bf16")
-    max_abs, rel, lse_err = U.attn_errors(o, lse, o_ref, l_ref, rows, w.N, w.block, 2)
+    max_abs, rel, lse_err = U.attn_errors(o, lse, o_ref, l_ref, rows, w.N, w.block, H)
     assert max_abs <= max(U.BF16_MAX_ABS, 2.0 ** -7 * float(np.nanmax(np.abs(o_ref)))) and rel <= U.BF16_REL_L2 and lse_err <= 2e-3
