@@ -13,6 +13,10 @@ pytestmark = pytest.mark.gpu
 W = {128: shrink(WORKLOADS["medium"], H=3, T=2, Hg=30, Wg=31, k=5),                    # N = 1860: 15 blocks, the last ragged
      64: shrink(WORKLOADS["medium"], H=3, T=2, Hg=30, Wg=31, k=9, block=64)}
 
+# more than 64 blocks, the last ragged: scores and selection are kernels of their own
+LONG = {128: shrink(WORKLOADS["medium"], H=3, T=9, Hg=30, Wg=31, k=9),                 # N = 8370: 66 blocks
+        64: shrink(WORKLOADS["medium"], H=3, T=5, Hg=30, Wg=31, k=11, block=64)}       # N = 4650: 73 blocks
+
 
 class Call:
     """A library call with the buffers it reads (`reads`, with two sets of contents) and writes (`writes`)."""
@@ -150,7 +154,17 @@ CASES = [(n, b) for n in NAMES for b in (128, 64)] + [(n, 128) for n in ("quanti
 
 @pytest.mark.parametrize("name,block", CASES)
 def test_inputs_written_just_before_a_call(name, block):
-    c = Call(name, W[block])
+    _check(Call(name, W[block]))
+
+
+@pytest.mark.parametrize("name,block", [(n, b) for n in ("block_select", "block_select_mass", "block_select_noalloc", "block_select_e4m3",
+                                                         "block_select_pooled", "step", "step_remainder", "step_e4m3") for b in (128, 64)] +
+                         [("step_4bit", 128)])
+def test_inputs_written_just_before_a_call_of_many_blocks(name, block):
+    _check(Call(name, LONG[block]))
+
+
+def _check(c):
     want = []
     for i in range(2):
         c.fill(i)

@@ -11,25 +11,38 @@ from paper_2606_23743_b200.workloads import WORKLOADS, shrink
 pytestmark = pytest.mark.gpu
 
 
-def _case(rng):
+def _case(rng, many=False):
     block = int(rng.choice([64, 128])); d = int(rng.choice([64, 128])); fp8 = bool(rng.integers(0, 2))
     T, Hg, Wg = int(rng.integers(1, 7)), int(rng.integers(1, 12)), int(rng.integers(1, 40))
+    if many:                                                  # 65 to 224 blocks per head, every other time frames of whole blocks
+        T = int(rng.integers(5, 9))
+        Hg, Wg = (block, int(rng.integers(13, 29))) if rng.random() < 0.5 else (block // 2, int(rng.integers(27, 57)))
     N = T * Hg * Wg
     Nb = -(-N // block)
     kw = dict(B=int(rng.integers(1, 3)), H=int(rng.integers(1, 4)), T=T, Hg=Hg, Wg=Wg, block=block, d=d,
               mode=int(rng.integers(0, 2)), k=int(rng.integers(1, 12)), tau=float(rng.choice([0.5, 0.9, 0.99, 1.0])),
               fp8=fp8, sigma_f=float(rng.choice([0.3, 0.65, 1.0])), sigma_w=float(rng.choice([0.0, 0.5])),
               qk_mult=float(rng.choice([1.0, 1.5, 3.0])), win_t=-1, win_s=-1)
-    if rng.random() < 0.25 and N % block == 0 and Nb % T == 0:
+    if rng.random() < (0.7 if many else 0.25) and N % block == 0 and Nb % T == 0:
         kw.update(win_t=int(rng.integers(0, 2)), win_s=int(rng.integers(0, 2)))
     return shrink(WORKLOADS["medium"], **kw), rng.random() < 0.2
 
 
 @pytest.mark.parametrize("seed", [1, 2, 3])
 def test_random_configurations(seed):
+    _run(seed, 40)
+
+
+@pytest.mark.parametrize("seed", [4, 5])
+def test_random_configurations_of_many_blocks(seed):
+    """The same above 64 blocks per head, where scores and selection are kernels of their own."""
+    _run(seed, 12, many=True)
+
+
+def _run(seed, cases, many=False):
     rng = np.random.default_rng(seed)
-    for case in range(40):
-        w, dense = _case(rng)
+    for case in range(cases):
+        w, dense = _case(rng, many)
         what = f"seed {seed} case {case}: {w}"
         (q, k, v), (qb, kb, vb) = U.host_inputs(w, seed=1000 * seed + case)
         qd, kd, vd = U.dev(q), U.dev(k), U.dev(v)

@@ -19,6 +19,9 @@ CASES = {
     "window": shrink(WORKLOADS["xl"], B=2, H=2, T=6),                                # 3x3 forced, k=37
     "window_gt_k": shrink(WORKLOADS["xl"], B=1, H=2, T=4, k=5),                      # |F| up to 9 > k
     "window_mass": shrink(WORKLOADS["xl"], B=1, H=2, T=4, mode=1, k=20, tau=0.5),
+    "window_gt_k_72_blocks": shrink(WORKLOADS["xl"], B=1, H=2, T=6, k=5),
+    "window_mass_72_blocks": shrink(WORKLOADS["xl"], B=1, H=2, T=6, mode=1, k=20, tau=0.5),
+    "window_mass_204_blocks": shrink(WORKLOADS["xl"], B=1, H=1, T=17, mode=1, k=60, tau=0.7),
     "block64_d128": shrink(WORKLOADS["medium"], H=2, T=2, block=64, k=8),
     "k_ge_nb": shrink(WORKLOADS["tiny"], k=99),
     "k1": shrink(WORKLOADS["medium"], H=2, T=2, k=1),
@@ -187,7 +190,8 @@ def test_threshold_search_on_awkward_scores(nb, mode):
                 assert ci[rp[r]:rp[r + 1]].tolist() == want, (h, k)
 
 
-@pytest.mark.parametrize("nb,k,window", [(16, 4, False), (16, 16, False), (40, 33, False), (129, 70, False), (16, 9, True)])
+@pytest.mark.parametrize("nb,k,window", [(16, 4, False), (16, 16, False), (40, 33, False), (129, 70, False), (16, 9, True), (68, 9, True),
+                                         (132, 20, True)])
 def test_rows_of_a_known_length_are_written_whole(nb, k, window):
     """A NaN score is never selected, so a row of top-k can find fewer than the k blocks its row_ptr covers: the entries left
     over are block 0, whatever col_idx held before."""
@@ -234,9 +238,15 @@ def test_rows_of_a_known_length_are_written_whole(nb, k, window):
     (2, 9, 64, 128, 128, False, 1, 9, False, "packed", "normal"),
     (1, 24, 17, 128, 128, False, 0, 2, False, "heads", "ties"),
     (1, 5, 65, 64, 64, False, 1, 9, False, "heads", "normal"),            # the general kernels, one block more
+    (1, 4, 68, 64, 64, False, 1, 12, True, "heads", "normal"),            # ... forced window and mass
+    (1, 3, 72, 128, 128, True, 1, 40, True, "tokens", "normal"),
+    (2, 3, 132, 64, 128, False, 0, 3, True, "tokens", "ties"),            # ... window larger than k, equal scores
+    (1, 4, 68, 64, 128, False, 0, 12, True, "heads", "nan"),              # ... forced window, rows of NaN scores come out short
+    (1, 4, 132, 64, 64, False, 1, 12, True, "packed", "nan"),
+    (1, 2, 100, 64, 64, False, 1, 150, True, "heads", "zero"),
 ])
 def test_routing_of_small_problems(B_, H, Nb, block, d, fp8, mode, k, window, layout, values):
-    """Few blocks per head take kernels of their own, which rank a row's candidates instead of searching a threshold: the lists are what the sequential
+    """Few blocks per head take kernels of their own (the last rows are of the general ones), which rank a row's candidates instead of searching a threshold: the lists are what the sequential
     rule takes from the kernel's own scores, and routing in one call is routing from means that another call has made, byte for byte."""
     N = Nb * block - (37 if Nb % 2 else 0)
     g = torch.Generator(device="cuda").manual_seed(Nb)
@@ -295,7 +305,7 @@ def test_routing_of_small_problems(B_, H, Nb, block, d, fp8, mode, k, window, la
                 break
             kept.append(J)
         want = sorted(kept)
-        if mode == 0 and not window:
+        if mode == 0 and (not window or k >= 9):                          # (a row's count is known: no window larger than k)
             want += [0] * (min(k, Nb) - len(want))                        # (a short row is filled up)
         have = ci[rp[r]:rp[r + 1]].tolist()
         if values == "nan":
@@ -365,3 +375,44 @@ def test_small_problems_where_no_cluster_fits(H, Nb, block, d, fp8, mode):
         B.debug_set_mode(0)
     for x in got + [route(B.block_select)]:
         assert all(torch.equal(a, b) for a, b in zip(want, x))
+
+
+@pytest.mark.parametrize("d,block,fp8", [(64, 64, True), (128, 64, True), (64, 128, True), (128, 128, True), (64, 64, False), (128, 64, False),
+                                         (64, 128, False), (128, 128, False)])
+@pytest.mark.parametrize("run", [3, 0], ids=["run3", "longest"])
+def test_pooling_in_runs_of_blocks(run, d, block, fp8):
+    """A CTA pools a run of blocks, the longer the larger the call, up to 128 KB: the means are those of calls on one head each, which are
+    small enough for a block per CTA, byte for byte, and those of another program."""
+    block_bytes = block * d * (1 if fp8 else 2)
+    blocks = (run or (128 << 10) // block_bytes) * ((16 << 20) // block_bytes)          # of Q and K together
+    H = 40
+    Nb = blocks // (2 * H) + 1
+    Nb += Nb % max(run, 2) == 0                                             # (the last run of a head is a short one)
+    N = Nb * block - 21
+    g = torch.Generator(device="cuda").manual_seed(d + block)
+    q, k = (torch.randn(1, N, H, d, generator=g, device="cuda", dtype=torch.bfloat16).transpose(1, 2) for _ in range(2))
+    scales = [None, None]
+    if fp8:
+        q, k = (x.to(torch.float8_e4m3fn).view(torch.uint8) for x in (q, k))
+        scales = [torch.rand(1, H, Nb, generator=g, device="cuda") + 0.5 for _ in range(2)]
+
+    def pool(h0, h1):
+        part = [x[:, h0:h1] for x in (q, k)]
+        means = [torch.full((1, h1 - h0, Nb, d), float("nan"), device="cuda") for _ in range(2)]
+        B.pool_qk(B.make_problem(*part, None, None, N, block, 0.0, fp8), *part, *means, *(s if s is None else s[:, h0:h1].contiguous() for s in scales))
+        return torch.stack(means)
+
+    got = pool(0, H)
+    assert torch.equal(got, torch.cat([pool(h, h + 1) for h in range(H)], dim=2))
+    h = H - 1
+    for i, x in enumerate((q, k)):
+        y = torch.zeros(Nb * block, d, dtype=torch.float64, device="cuda")
+        y[:N] = (x[0, h].view(torch.float8_e4m3fn) if fp8 else x[0, h]).double()
+        count = torch.full((Nb, 1), float(block), dtype=torch.float64, device="cuda")
+        count[-1] = N - (Nb - 1) * block
+        want = y.reshape(Nb, block, d).sum(1) / count
+        if fp8:
+            want *= scales[i][0, h].double()[:, None]
+        # (sums of at most 128 values in fp32: each addition's error is below 2^-24 of a partial sum, and those stay below sum |y|)
+        bound = 2.0 ** -24 * 130 * y.abs().reshape(Nb, block, d).sum(1) / count * (scales[i][0, h].double()[:, None] if fp8 else 1.0)
+        assert ((got[i, 0, h].double() - want).abs() <= bound + 1e-30).all()

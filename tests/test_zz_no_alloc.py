@@ -50,6 +50,15 @@ def test_noalloc_matches_allocating_entry_point_twice_in_a_row():
     assert torch.equal(a2[1], b2[1])
 
 
+@pytest.mark.parametrize("kw", [dict(k=5), dict(mode=1, k=20, tau=0.5)], ids=["window_gt_k", "window_mass"])
+def test_noalloc_with_a_window_and_many_blocks(kw):
+    """72 blocks per head: scores, selection and compaction are kernels of their own, and all of them use the scratch."""
+    w = shrink(WORKLOADS["xl"], B=1, H=2, T=6, **kw)
+    (q, k, _), _ = U.host_inputs(w)
+    a, b = _both(w, U.dev(q), U.dev(k))
+    assert torch.equal(a[0], b[0]) and torch.equal(a[1], b[1]) and torch.equal(a[2], b[2])
+
+
 def test_noalloc_rejects_problems_beyond_its_scratch():
     w = WORKLOADS["xl"]                                        # pooled means alone are 24 MB
     # describe the full-size problem without allocating it: the size check is host-side and
