@@ -48,7 +48,8 @@ static __device__ __forceinline__ void stage_row(uint8_t* tile, int row, int c0,
 // stores of 32 rows per warp before), and the block means with it.
 // mean_k, mean_v (of the tensors behind tm_k and tm_v; both or neither): the block means that the attention kernel's block-mean tiles read,
 // [B*H][Nbp][128] bf16, rows >= Nb zero.  They are at hand here: without the pass that makes them from K and V again
-// (pool_kv_kernel) a call on the same 20 x 138 blocks is 46 to 53 us shorter.
+// (pool_kv_kernel) a call on the same 20 x 138 blocks is 46 to 53 us shorter.  (fp32 both, but in eight partial sums per column where that kernel has
+// sixteen: a mean whose sums are not exact in fp32 can round to the neighbouring bf16 value.)
 __global__ void __launch_bounds__(128)
 cov_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ct,
            int H, int N, int block, int Nb, __nv_bfloat16* __restrict__ mean_k, __nv_bfloat16* __restrict__ mean_v, int Nbp,

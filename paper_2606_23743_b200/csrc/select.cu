@@ -885,7 +885,9 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
   }
   {
     // 64 x 64 tiles where they give most of the SMs a CTA, else 32 x 32: with few rows the time is one CTA's latency, and
-    // that shrinks with its tile (16 heads of 64 blocks: 16 tiles of 64 x 64 take 6.8 us, 64 of 32 x 32 4.2 us).
+    // that shrinks with its tile.  Routing from means, d = 128, top-k, us, 64 x 64 / 32 x 32: 1 head x 66 blocks 10.4 / 9.1, 2 x 100 9.9 / 8.2, 6 x 128
+    // 10.8 / 10.0, 2 x 192 12.0 / 10.2.  Between 48 and 96 tiles of 64 x 64 neither is the better one throughout, since the time also depends on where the
+    // selection's waiting CTAs have settled: 16 x 80 10.4 / 16.5, 20 x 66 10.5 / 18.0, 6 x 129 16.4 / 12.4, 23 x 100 21.7 / 20.2, 8 x 192 21.3 / 22.5.
     const int heads = m.B * m.H, nt = (m.Nb + 63) / 64;
     rc = nt * nt * heads >= 96 ? launch_scores<D, 8, 4, 8>(qbar, kbar, m.Nb, heads, m.scale, scores, st)
                              : launch_scores<D, 2, 2, 16>(qbar, kbar, m.Nb, heads, m.scale, scores, st);
