@@ -1623,9 +1623,9 @@ int launch_attn_ts(const Dims& m_in, const sva_problem_t* p, const void* q, cons
     }
     // block means of K ([Nbp rows][128], rows >= Nb zero) and of V (transposed tiles), then their maps
     const int run = blocks_per_cta(2LL * m.R, m.block * ts::D * 2);            // (the padding blocks that the grid covers too are not read)
-    if (!with_cov && (rc = launch_dep(m.block == 64 ? pool_kv_kernel<4> : pool_kv_kernel<8>, dim3((L.Nbp + run - 1) / run, m.B * m.H, 2), 256, 0, st, (const __nv_bfloat16*)k,
-                         (const __nv_bfloat16*)v, sk, make_strides(p->v_stride), m.H, m.N, m.block, m.Nb, L.Nbp, run, kp, vtp, vmn ? 1 : 0,
-                         counter)) != SVA_OK)
+    if (!with_cov && (rc = launch_dep(m.block == 64 ? pool_kv_kernel<4> : pool_kv_kernel<8>, dim3((L.Nbp + run - 1) / run, m.B * m.H, 2),
+                                      256, 0, st, (const __nv_bfloat16*)k, (const __nv_bfloat16*)v, sk, make_strides(p->v_stride), m.H, m.N,
+                                      m.block, m.Nb, L.Nbp, run, kp, vtp, vmn ? 1 : 0, counter)) != SVA_OK)
       return rc;
     const cuuint64_t prow = (cuuint64_t)L.Nbp;
     if ((rc = make_map_ts(&tkp, kp, ts::D, prow, m.H, m.B, (cuuint64_t)ts::D * 2, prow * ts::D * 2,

@@ -124,9 +124,10 @@ struct DeviceOnce {
 };
 
 // Consecutive token blocks per CTA of the kernels that stream a tensor's blocks (`blocks` of them over all heads and tensors, of
-// block_bytes) with the next block's loads in flight while they reduce: runs of up to 128 KB, as long as the CTAs' first loads together still
-// come to 16 MB (512 blocks of 32 KB: 3.5 CTAs per SM).  16 heads x 8 192 tokens, pooling of Q and K: one block of 32 KB per CTA 15.5 us, two
-// 14.8, four 14.3; 32 heads x 4 096 tokens in blocks of 16 KB: two 15.8, four 16.1, eight 17.9; 24 x 32 760 in them: two 80.9, four 78.0, eight 74.3.
+// block_bytes) with the next block's loads in flight while they reduce: runs of up to 128 KB, as long as the CTAs' first loads
+// together still come to 16 MB (512 blocks of 32 KB: 3.5 CTAs per SM).  16 heads x 8 192 tokens, pooling of Q and K: one block of
+// 32 KB per CTA 15.5 us, two 14.8, four 14.3; 32 heads x 4 096 tokens in blocks of 16 KB: two 15.8, four 16.1, eight 17.9;
+// 24 x 32 760 in them: two 80.9, four 78.0, eight 74.3.
 inline int blocks_per_cta(long long blocks, int block_bytes) {
   const long long run = blocks * block_bytes >> 24;
   const int most = (128 << 10) / block_bytes;

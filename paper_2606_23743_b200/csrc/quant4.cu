@@ -20,10 +20,11 @@ static constexpr int Q4_THREADS = 256;
 
 // amax[tensor * BH + bh] (as fp32 bits; the launcher zeroes it) = max |x| over the existing tokens
 // From the end of the tensors, which a kernel that has just written them (the prologue) leaves in the L2.
-// A CTA per 128-token block, its second half's loads in flight behind the first half's maxima, and one atomicMax.  (An atomic per warp, 98 304 of
-// them on 48 words, took 100 us for 403 MB.  Runs of blocks per CTA, as pooling has them, are slower: there is no reduction per block to hide.
-// The whole quantiser, us, inputs not in the L2, runs of four / a block per CTA: 24 heads x 32 760 tokens 155.9 / 153.5, 16 x 16 384 61.2 / 56.1, 16 x 8 192
-// 33.3 / 32.8, 8 x 4 096 16.4 / 13.4; inputs in the L2, 16 x 8 192 30.4 / 28.7.)
+// A CTA per 128-token block, its second half's loads in flight behind the first half's maxima, and one atomicMax.  (An atomic per
+// warp, 98 304 of them on 48 words, took 100 us for 403 MB.  Runs of blocks per CTA, as pooling has them, are slower: there is no
+// reduction per block to hide.
+// The whole quantiser, us, inputs not in the L2, runs of four / a block per CTA: 24 heads x 32 760 tokens 155.9 / 153.5,
+// 16 x 16 384 61.2 / 56.1, 16 x 8 192 33.3 / 32.8, 8 x 4 096 16.4 / 13.4; inputs in the L2, 16 x 8 192 30.4 / 28.7.)
 __global__ void __launch_bounds__(Q4_THREADS)
 amax_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k, Strides sq, Strides sk, int H, int N,
             int BH, uint32_t* __restrict__ amax) {

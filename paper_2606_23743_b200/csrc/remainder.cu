@@ -48,8 +48,8 @@ static __device__ __forceinline__ void stage_row(uint8_t* tile, int row, int c0,
 // stores of 32 rows per warp before), and the block means with it.
 // mean_k, mean_v (of the tensors behind tm_k and tm_v; both or neither): the block means that the attention kernel's block-mean tiles read,
 // [B*H][Nbp][128] bf16, rows >= Nb zero.  They are at hand here: without the pass that makes them from K and V again
-// (pool_kv_kernel) a call on the same 20 x 138 blocks is 46 to 53 us shorter.  (fp32 both, but in eight partial sums per column where that kernel has
-// sixteen: a mean whose sums are not exact in fp32 can round to the neighbouring bf16 value.)
+// (pool_kv_kernel) a call on the same 20 x 138 blocks is 46 to 53 us shorter.  (fp32 both, but in eight partial sums per column
+// where that kernel has sixteen: a mean whose sums are not exact in fp32 can round to the neighbouring bf16 value.)
 __global__ void __launch_bounds__(128)
 cov_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ct,
            int H, int N, int block, int Nb, __nv_bfloat16* __restrict__ mean_k, __nv_bfloat16* __restrict__ mean_v, int Nbp,
@@ -87,7 +87,10 @@ cov_kernel(const __grid_constant__ CUtensorMap tm_k, const __grid_constant__ CUt
   if (mean_k) {
     if (J == 0 && bh == 0 && threadIdx.x < 2) row_counter[threadIdx.x] = 0;        // the attention kernel draws its rows from it
     if (J == Nb - 1) {
-      for (int r = Nb; r < Nbp; ++r) mean_k[((long long)bh * Nbp + r) * D + threadIdx.x] = mean_v[((long long)bh * Nbp + r) * D + threadIdx.x] = __float2bfloat16_rn(0.f);
+      for (int r = Nb; r < Nbp; ++r) {
+        const long long at = ((long long)bh * Nbp + r) * D + threadIdx.x;
+        mean_k[at] = mean_v[at] = __float2bfloat16_rn(0.f);
+      }
     }
   }
   if (threadIdx.x == 0) {
@@ -229,10 +232,10 @@ weights_kernel(const float* __restrict__ scores, const int32_t* __restrict__ row
 // Columns: the flattened (e, c) index, in 128 n-tiles of 128.  A operand: W tile [128 I][64 J] K-major; B operand: C^T rows [64 J][128 n]
 // as two 64-element panels, MN-major.  A CTA keeps the W tiles of one or two I-tiles in shared memory and walks through a run of
 // n-tiles, the C^T chunks in a ring, two accumulators per I-tile so that one is read while the next is made.
-// What bounds it is the way from the L2: with W fetched again for every n-tile (a CTA per tile) that was 490 MB for 90 MB read and 90 MB written
-// (20 heads x 138 blocks), 79 us inside the attention call; now 51 (16 heads x 64 blocks: 18.3 -> 16.7).
-// grid (runs, groups of I-tiles, B*H), 192 threads: warps 0-3 read the accumulators and write A^T, one lane of warp 4 loads, one of warp 5
-// issues the MMAs.
+// What bounds it is the way from the L2: with W fetched again for every n-tile (a CTA per tile) that was 490 MB for 90 MB read and
+// 90 MB written (20 heads x 138 blocks), 79 us inside the attention call; now 51 (16 heads x 64 blocks: 18.3 -> 16.7).
+// grid (runs, groups of I-tiles, B*H), 192 threads: warps 0-3 read the accumulators and write A^T, one lane of warp 4 loads, one of
+// warp 5 issues the MMAs.
 namespace agg {
 constexpr uint32_t A_BYTES = 128 * 128, B_PANEL = 64 * 128;           // 16 KB W tile; two 8 KB panels of C^T rows
 constexpr int MAX_STAGES = 6, OUT_STAGE = rem::TILE;
@@ -248,9 +251,10 @@ inline Plan plan(int Nb, int chunks) {
   p.smem = 1024 + w + p.stages * stage + OUT_STAGE;
   return p;
 }
-// Runs of n-tiles per group of I-tiles: the number that gives the shortest longest SM of the B200's 148 (a run costs about two n-tiles to begin), up to
-// an n-tile each: one or two groups -- a call of one or two heads -- would leave most SMs idle otherwise.  The whole call, us, at most 32 runs / so: 1 head x
-// 4 blocks of 128 24.3 / 22.4, x 64 28.0 / 25.6, x 129 42.2 / 37.1, x 256 77.9 / 70.0, 2 heads x 64 29.7 / 28.3, 3 x 64 38.9 / 38.2.
+// Runs of n-tiles per group of I-tiles: the number that gives the shortest longest SM of the B200's 148 (a run costs about two
+// n-tiles to begin), up to an n-tile each: one or two groups -- a call of one or two heads -- would leave most SMs idle otherwise.
+// The whole call, us, at most 32 runs / so: 1 head x 4 blocks of 128 24.3 / 22.4, x 64 28.0 / 25.6, x 129 42.2 / 37.1, x 256
+// 77.9 / 70.0, 2 heads x 64 29.7 / 28.3, 3 x 64 38.9 / 38.2.
 inline int runs(int groups) {
   int best = 1, cost = 1 << 30;
   for (int r = 1; r <= rem::D; ++r) {

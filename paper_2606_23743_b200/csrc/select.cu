@@ -9,8 +9,8 @@
 // scores and selects (route_means_kernel); the smallest problems take one for all three (route_cluster_kernel).
 // select_rows_kernel is one warp per query-block row: it reads the row's scores from that matrix (no shared
 // memory) as order-preserving integer keys, finds the threshold of the rule by narrowing an interval of scores
-// that holds it and emits the kept blocks in ascending order.  When the per-row count is known on the host (top-k with no window larger than k)
-// rows go straight into the CSR; otherwise they are staged and csr_kernel builds it in one launch.
+// that holds it and emits the kept blocks in ascending order.  When the per-row count is known on the host (top-k with no window
+// larger than k) rows go straight into the CSR; otherwise they are staged and csr_kernel builds it in one launch.
 #include <mutex>
 #include <type_traits>
 
@@ -40,13 +40,16 @@ __device__ __forceinline__ void add_vector(const uint4& u, uint64_t (&acc)[8 / E
 // ELEM_BYTES = 2: bf16 input.  ELEM_BYTES = 1: e4m3 codes, multiplied by the block's scale.
 // Bound by the HBM: one pass over Q and K.  A CTA's loads run one block ahead of its sums, across the reduction (two barriers); with a
 // CTA per block nothing was in flight while it reduced.  VECS: 16-byte vectors of a block per thread, so that a step is a whole block
-// whatever its size (with four per step a 128-token block took two steps, and 64-token blocks of e4m3 codes or of d = 64 masked half of the loads).
-// Q and K of 24 heads x 32 760 tokens, d = 128 (403 MB): 75.8 us with a CTA per block, 70.8 with runs of four, two steps a block, 69.1 so (5.8 TB/s);
-// another box, four vectors and runs of four -> a block at a time and runs of up to 128 KB: 24 x 32 760 66.9 -> 61.8 (6.5 TB/s), in 64-token blocks
-// 68.6 -> 65.0, 16 heads x 8 192 14.6 -> 12.3, 20 x 17 550 33.6 -> 30.9, 64 x 47 616 236.5 -> 223.4; d = 64 in 64-token blocks, 16 x 8 192, 11.7 -> 8.0.
-// e4m3 codes (201 MB, converted in pairs) are bound by the sums and the reduction, which half the bytes do not hide: 66.5 -> 58.6 us with the
-// run, 52.6 -> 46.4 (on a faster box) with pairs added in one instruction and partial sums laid out so that no two lanes of a warp meet in a
-// bank, 41.2 with runs of eight; in 64-token blocks 87.4 -> 47.4.
+// whatever its size (with four per step a 128-token block took two steps, and 64-token blocks of e4m3 codes or of d = 64 masked
+// half of the loads).
+// Q and K of 24 heads x 32 760 tokens, d = 128 (403 MB): 75.8 us with a CTA per block, 70.8 with runs of four, two steps a block,
+// 69.1 so (5.8 TB/s);
+// another box, four vectors and runs of four -> a block at a time and runs of up to 128 KB: 24 x 32 760 66.9 -> 61.8 (6.5 TB/s), in
+// 64-token blocks 68.6 -> 65.0, 16 heads x 8 192 14.6 -> 12.3, 20 x 17 550 33.6 -> 30.9, 64 x 47 616 236.5 -> 223.4; d = 64 in
+// 64-token blocks, 16 x 8 192, 11.7 -> 8.0.
+// e4m3 codes (201 MB, converted in pairs) are bound by the sums and the reduction, which half the bytes do not hide: 66.5 -> 58.6
+// us with the run, 52.6 -> 46.4 (on a faster box) with pairs added in one instruction and partial sums laid out so that no two
+// lanes of a warp meet in a bank, 41.2 with runs of eight; in 64-token blocks 87.4 -> 47.4.
 template <int D, int ELEM_BYTES, int VECS>
 __global__ void __launch_bounds__(POOL_THREADS)
 pool_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ k, Strides sq, Strides sk,
@@ -126,22 +129,22 @@ __device__ __forceinline__ float key_score(uint32_t key) {
 // Mass rule: the softmax weights of a row's candidates, in units of 2^-31 (0 where there is none).
 template <int ITEMS>
 __device__ __forceinline__ void mass_weights(const uint32_t (&key)[ITEMS], uint32_t (&wgt)[ITEMS]) {
-      uint32_t km = 0u;
-  #pragma unroll
-      for (int it = 0; it < ITEMS; ++it) km = max(km, key[it]);
-      km = __reduce_max_sync(0xffffffffu, km);
-      const float mx = key_score(km);
-      float z = 0.f, ew[ITEMS];
-  #pragma unroll
-      for (int it = 0; it < ITEMS; ++it) {
-        ew[it] = 0.f;
-        if (key[it]) { ew[it] = expf(key_score(key[it]) - mx); z += ew[it]; }
-      }
-  #pragma unroll
-      for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
-      const float inv_z = 1.0f / z;
-  #pragma unroll
-      for (int it = 0; it < ITEMS; ++it) wgt[it] = __float2uint_rn(ew[it] * inv_z * 2147483648.f);
+  uint32_t km = 0u;
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) km = max(km, key[it]);
+  km = __reduce_max_sync(0xffffffffu, km);
+  const float mx = key_score(km);
+  float z = 0.f, ew[ITEMS];
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) {
+    ew[it] = 0.f;
+    if (key[it]) { ew[it] = expf(key_score(key[it]) - mx); z += ew[it]; }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1) z += __shfl_xor_sync(0xffffffffu, z, o);
+  const float inv_z = 1.0f / z;
+#pragma unroll
+  for (int it = 0; it < ITEMS; ++it) wgt[it] = __float2uint_rn(ew[it] * inv_z * 2147483648.f);
 }
 
 // A row's kept blocks (bit it of `mask`: block it*32 + lane; n of them) in ascending order: straight into the CSR where every row has
@@ -328,8 +331,8 @@ __device__ __forceinline__ void select_and_emit(uint32_t (&key)[ITEMS], const in
 
 // The same rule for short rows: each candidate counts the candidates in front of it (larger score, or equal and a lower index) and, for the
 // mass rule, adds up their mass; it is kept if the sequential rule would still run when its turn comes.  No search, so a row is Nb steps of
-// two or three independent instructions.  Cycles of a CTA's selection phase, threshold search -> this: rows of 16 scores 2 550 -> 1 070, eight rows of
-// 64 scores 4 400 -> 2 650.
+// two or three independent instructions.  Cycles of a CTA's selection phase, threshold search -> this: rows of 16 scores 2 550 ->
+// 1 070, eight rows of 64 scores 4 400 -> 2 650.
 // sk, sw: the row's keys and weights in shared memory (32 * ITEMS words each).
 template <int ITEMS, bool MASS>
 __device__ __forceinline__ void rank_and_emit(uint32_t (&key)[ITEMS], uint32_t* sk, uint32_t* sw, const int I, const int bh,
@@ -508,9 +511,10 @@ select_rows_kernel(const float* __restrict__ scores, SelParams p, int32_t* __res
 // its share of the head's blocks of Q and K (a team of 256 threads per block), writes a key mean into the shared memory of all eight,
 // and then scores and selects its own query blocks.  Sums run in the orders of pool_kernel and block_scores_kernel, so lists and
 // scores are the same bytes.
-// Bound by latency: the launch, the cluster's barriers (about 0.5 us each), the pooling of a block per team (about 1 100 cycles of loads, sums
-// and reduction), and the score and selection phase of a warp per row.  Microseconds of a routing call (top-k), pool_kernel and
-// route_means_kernel / this one: 2 heads x 16 blocks of 64 x 64 7.3 / 5.3, of 128 x 128 7.35 / 6.3; 1 x 8 7.3 / 5.5.
+// Bound by latency: the launch, the cluster's barriers (about 0.5 us each), the pooling of a block per team (about 1 100 cycles of
+// loads, sums and reduction), and the score and selection phase of a warp per row.  Microseconds of a routing call (top-k),
+// pool_kernel and route_means_kernel / this one: 2 heads x 16 blocks of 64 x 64 7.3 / 5.3, of 128 x 128 7.35 / 6.3; 1 x 8
+// 7.3 / 5.5.
 static constexpr int RC_CTAS = 8, RC_TEAMS = 4, RC_TEAM = 256, RC_MAX_NB = 16;
 static constexpr int RC_ROWS = RC_MAX_NB / RC_CTAS;                         // query blocks per CTA at most
 static constexpr int RC_KEYS = 32;                                          // rows of the panel of key means, one per lane
@@ -660,14 +664,16 @@ route_cluster_kernel(const uint8_t* __restrict__ q, const uint8_t* __restrict__ 
 }
 
 // The same tail for block means that are at hand (a pooling or prologue kernel has written them): scores and selection of eight query
-// blocks of a head per CTA, one launch instead of two.  Up to 64 blocks per head, where the key means fit beside one another and a row's rank is
-// counted.  Bound by latency: the means' way from the L2, then as above.  Routing from means, scores and selection kernels -> this one (us, top-k / mass rule with csr_kernel):
-// 16 heads x 64 blocks 8.0 -> 4.9 / 15.2 -> 6.9, 24 x 64 12.3 -> 8.6 / 20.5 -> 11.2, 128 x 64 22.3 -> 15.0 / 27.8 -> 20.8, 2 x 16 6.3 -> 4.9 / 8.4 -> 6.9.
+// blocks of a head per CTA, one launch instead of two.  Up to 64 blocks per head, where the key means fit beside one another and a
+// row's rank is counted.  Bound by latency: the means' way from the L2, then as above.  Routing from means, scores and selection
+// kernels -> this one (us, top-k / mass rule with csr_kernel): 16 heads x 64 blocks 8.0 -> 4.9 / 15.2 -> 6.9, 24 x 64 12.3 ->
+// 8.6 / 20.5 -> 11.2, 128 x 64 22.3 -> 15.0 / 27.8 -> 20.8, 2 x 16 6.3 -> 4.9 / 8.4 -> 6.9.
 static constexpr int RT_ROWS = 8, RT_ITEMS = 2, RT_MAX_NB = 32 * RT_ITEMS;
-// Counting ranks is Nb steps per row where the threshold search takes about log2(Nb) + 2, so with long rows it pays only while the two launches that it
-// saves weigh more than the counting: up to 40 blocks always, beyond that up to a work (CTAs x steps) that 160 heads of 64 blocks come to (187 with the
-// mass rule, whose search carries the masses along).  From means, d = 128, us, scores and selection kernels / this one: top-k, 128 heads x 64 blocks 22.3 / 15.0,
-// 160 x 64 19.4 / 18.3, 200 x 64 20.8 / 22.0, 1 024 x 64 76.6 / 99.2, 220 x 52 19.6 / 19.6, 1 200 x 52 78 / 89, 1 200 x 40 67 / 63; mass rule, 200 x 64 32.9 / 31.0, 300 x 64 40.6 / 44.5.
+// Counting ranks is Nb steps per row where the threshold search takes about log2(Nb) + 2, so with long rows it pays only while the
+// two launches that it saves weigh more than the counting: up to 40 blocks always, beyond that up to a work (CTAs x steps) that 160
+// heads of 64 blocks come to (187 with the mass rule, whose search carries the masses along).  From means, d = 128, us, scores and
+// selection kernels / this one: top-k, 128 heads x 64 blocks 22.3 / 15.0, 160 x 64 19.4 / 18.3, 200 x 64 20.8 / 22.0, 1 024 x 64
+// 76.6 / 99.2, 220 x 52 19.6 / 19.6, 1 200 x 52 78 / 89, 1 200 x 40 67 / 63; mass rule, 200 x 64 32.9 / 31.0, 300 x 64 40.6 / 44.5.
 static bool route_by_rank(const Dims& m, int mode) {
   return m.Nb <= 40 || (m.Nb <= RT_MAX_NB && (long long)m.B * m.H * ((m.Nb + RT_ROWS - 1) / RT_ROWS) * m.Nb <= (mode == 1 ? 96000 : 82000));
 }
@@ -790,10 +796,12 @@ static int launch_pool_d(const Dims& m, const sva_problem_t* p, const void* q, c
                     m.H, m.N, m.block, m.Nb, run, qbar, kbar);
 }
 
-// Where the cluster kernel routes.  Up to 14 heads each of its CTAs has an SM to itself (15 or more clusters of eight SMs do not fit at once), and up to
-// 16 blocks (RC_MAX_NB) a CTA pools in one round.  Beyond that pooling over all SMs and route_means_kernel are faster (us, them / a cluster): 12 heads x 20 blocks
-// of 128 x 128 7.3 / 7.9, 12 x 44 9.8 / 12.2, 16 x 16 7.2 / 8.0 (with two CTAs per SM), 6 x 64 8.5 / 13.4.
-// Where the device cannot hold such a cluster -- the largest cluster shrinks in a partition of too few SMs -- those two serve these sizes too.
+// Where the cluster kernel routes.  Up to 14 heads each of its CTAs has an SM to itself (15 or more clusters of eight SMs do not
+// fit at once), and up to 16 blocks (RC_MAX_NB) a CTA pools in one round.  Beyond that pooling over all SMs and route_means_kernel
+// are faster (us, them / a cluster): 12 heads x 20 blocks of 128 x 128 7.3 / 7.9, 12 x 44 9.8 / 12.2, 16 x 16 7.2 / 8.0 (with two
+// CTAs per SM), 6 x 64 8.5 / 13.4.
+// Where the device cannot hold such a cluster -- the largest cluster shrinks in a partition of too few SMs -- those two serve these
+// sizes too.
 static int g_debug_route = 0;
 void route_set_debug_mode(int v) { g_debug_route = v; }
 static bool route_in_cluster(const Dims& m) { return m.Nb <= RC_MAX_NB && m.B * m.H <= 14; }
@@ -872,8 +880,9 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
   if (route_by_rank(m, s->mode)) {
     constexpr int smem = 4 * ((RT_MAX_NB + RT_ROWS) * (D + 4) + 2 * RT_ROWS * RT_MAX_NB);      // (below the 48 KB that need no attribute)
     static_assert(smem <= 48 * 1024, "");
-    rc = launch_dep(s->mode == 1 ? route_means_kernel<D, true> : route_means_kernel<D, false>, dim3((m.Nb + RT_ROWS - 1) / RT_ROWS, m.B * m.H),
-                    RT_ROWS * 32, smem, st, (const float*)qbar, (const float*)kbar, m.scale, sp, block_scores, row_ptr, col_idx, tmp_idx, counts, m.R);
+    rc = launch_dep(s->mode == 1 ? route_means_kernel<D, true> : route_means_kernel<D, false>,
+                    dim3((m.Nb + RT_ROWS - 1) / RT_ROWS, m.B * m.H), RT_ROWS * 32, smem, st, (const float*)qbar, (const float*)kbar,
+                    m.scale, sp, block_scores, row_ptr, col_idx, tmp_idx, counts, m.R);
     return rc != SVA_OK ? rc : csr();
   }
   // scores: into the caller's matrix if it wants one, else into the workspace (after the staging arrays)
@@ -885,9 +894,10 @@ static int launch_select_d(const Dims& m, const sva_problem_t* p, const sva_sele
   }
   {
     // 64 x 64 tiles where they give most of the SMs a CTA, else 32 x 32: with few rows the time is one CTA's latency, and
-    // that shrinks with its tile.  Routing from means, d = 128, top-k, us, 64 x 64 / 32 x 32: 1 head x 66 blocks 10.4 / 9.1, 2 x 100 9.9 / 8.2, 6 x 128
-    // 10.8 / 10.0, 2 x 192 12.0 / 10.2.  Between 48 and 96 tiles of 64 x 64 neither is the better one throughout, since the time also depends on where the
-    // selection's waiting CTAs have settled: 16 x 80 10.4 / 16.5, 20 x 66 10.5 / 18.0, 6 x 129 16.4 / 12.4, 23 x 100 21.7 / 20.2, 8 x 192 21.3 / 22.5.
+    // that shrinks with its tile.  Routing from means, d = 128, top-k, us, 64 x 64 / 32 x 32: 1 head x 66 blocks 10.4 / 9.1,
+    // 2 x 100 9.9 / 8.2, 6 x 128 10.8 / 10.0, 2 x 192 12.0 / 10.2.  Between 48 and 96 tiles of 64 x 64 neither is the better one
+    // throughout, since the time also depends on where the selection's waiting CTAs have settled: 16 x 80 10.4 / 16.5, 20 x 66
+    // 10.5 / 18.0, 6 x 129 16.4 / 12.4, 23 x 100 21.7 / 20.2, 8 x 192 21.3 / 22.5.
     const int heads = m.B * m.H, nt = (m.Nb + 63) / 64;
     rc = nt * nt * heads >= 96 ? launch_scores<D, 8, 4, 8>(qbar, kbar, m.Nb, heads, m.scale, scores, st)
                              : launch_scores<D, 2, 2, 16>(qbar, kbar, m.Nb, heads, m.scale, scores, st);
